@@ -159,8 +159,9 @@ struct amg_coarse {
   float* tc5_xs = nullptr;    // their power-of-two scale per site,
   float* tc5_ds = nullptr;    // the power-of-two scale of every FP32 stencil block,
   void* tc5_d16 = nullptr;    // and the FP16 storage as planes with rotated pieces
-  void* fU = nullptr;         // fine operator (amg_setup_fine): links [V][4][3][3] in vec_prec
-  void* fC = nullptr;         // clover [V][2][6][6] in vec_prec (aliases clover for FP64)
+  void* fU = nullptr;         // fine operator (amg_setup_fine): links, FP64 [V][4][3][3], FP32 in block order (fine.cu)
+  void* fC = nullptr;         // its clover: FP64 the handle's clover itself, FP32 block-order words of 2 C
+  cudaMemPool_t fpool = nullptr;  // FP32 smoother: copies of x and y in block order (stream-ordered)
   void* fwork = nullptr;      // outer FGMRES workspace (fine Krylov basis, Z vectors, sums)
   size_t fwork_bytes = 0;
   // Three levels (level2.cu).  A level-2 handle (level == 2) holds R2 in R64 ([Vc2][2][ntv2]

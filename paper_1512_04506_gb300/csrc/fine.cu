@@ -14,16 +14,21 @@
 // chirality halves with the handle's 6x6 blocks C^{ll}, C^{rr}.
 //
 // The smoother's blocks are the aggregation blocks.  One half sweep (colour c) is one launch: one
-// CTA per (block of colour c, right-hand side), one thread per site.  The CTA forms the residual
-// r = y - D x on its sites (the neighbours outside the block have the other colour and are not
-// written in this launch), runs n_mr MR steps on B e = r with B = D without the hops that cross
-// the block face (rho in shared memory, block-wide sums), and adds e to x.
+// CTA per block of colour c and group of right-hand sides (FP64: per right-hand side), one thread
+// per site.  The CTA forms the residual r = y - D x on its sites (the neighbours outside the block
+// have the other colour and are not written in this launch), runs n_mr MR steps on B e = r with
+// B = D without the hops that cross the block face (rho in shared memory, block-wide sums), and
+// adds e to x.
+//
+// FP32 keeps the links and the clover of the fine lattice in an order of its own (see kLinkQ).
 #include "amg_internal.cuh"
+#include "pipe.cuh"
 
 #include <math.h>
 
 #include <algorithm>
 #include <complex>
+#include <type_traits>
 #include <vector>
 
 namespace {
@@ -109,32 +114,16 @@ __device__ __forceinline__ void hop_u(const C u[9], const C p[12], C out[12]) {
   }
 }
 
-// The 3x3 link at U9 = U + (s 4 + mu) 9.  FP32: 72 bytes from an offset 16-byte aligned for even mu
-// and 8 bytes past that for odd mu (s 4 + mu has the parity of mu), so four 16-byte loads and one
-// 8-byte load.
-template <int mu>
+// The 3x3 link at U9 = U + (s 4 + mu) 9 (FP64)
 __device__ __forceinline__ void load_link(const double2* __restrict__ U9, double2 u[9]) {
 #pragma unroll
   for (int k = 0; k < 9; ++k) u[k] = __ldg(U9 + k);
 }
-template <int mu>
-__device__ __forceinline__ void load_link(const float2* __restrict__ U9, float2 u[9]) {
-  constexpr int o = mu & 1;  // entries before the first 16-byte boundary
-  if (o) u[0] = __ldg(U9);
-  const float4* q = reinterpret_cast<const float4*>(U9 + o);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const float4 f = __ldg(q + k);
-    u[o + 2 * k] = make_float2(f.x, f.y);
-    u[o + 2 * k + 1] = make_float2(f.z, f.w);
-  }
-  if (!o) u[8] = __ldg(U9 + 8);
-}
 
-template <bool FWD, int mu, typename C>
-__device__ __forceinline__ void hop(const C* __restrict__ U, const C p[12], C out[12]) {
-  C u[9];
-  load_link<mu>(U, u);
+template <bool FWD, int mu>
+__device__ __forceinline__ void hop(const double2* __restrict__ U, const double2 p[12], double2 out[12]) {
+  double2 u[9];
+  load_link(U, u);
   hop_u<FWD, mu>(u, p, out);
 }
 
@@ -160,41 +149,165 @@ __device__ __forceinline__ void site_term(const C* __restrict__ Cl, T mass, cons
   }
 }
 
-__host__ __device__ __forceinline__ int tri_index(int a, int b) { return a * 6 - a * (a - 1) / 2 + (b - a); }  // a <= b
+// FP32 links and clover in HBM: per site kLinkQ 16-byte words of links (36 entries, two per word,
+// direction mu at entries 9 mu .. 9 mu + 8) and kClovQ words of clover, block by block: word q of the
+// site with local index t in block b at (b NQ + q) Vb + t.  A block's links (and its clover) are one
+// contiguous run, which one bulk copy moves, and consecutive lanes read consecutive words; with one
+// record per site in lattice order (strides of 288 and 352 bytes) every load of a warp touched up to
+// 32 lines, and the line look-ups in L1 bounded D.
+//
+// The clover of a chirality is [[H, X], [X^dag, -H]] with H = H^dag (spin blocks sigma_m (x) G_m with
+// Hermitian G_m): 27 real numbers instead of 36, as 14 complex words (H00, H11), (H22, 0), H01, H02,
+// H12, X row by row.  All are stored times 2, so that with a mass of 2 (4 + m0) the sums below are
+// 2 D psi with hops of weight one (an exact scaling), halved once at the end.
+constexpr int kLinkQ = 18, kClovQ = 14;
 
-// FP32 clover of one site in HBM as the two Hermitian blocks' upper triangles with the diagonal
-// (21 entries each in tri_index order, one padding entry after each: 44 complex, 352 bytes instead
-// of 576; C_ba = conj(C_ab)), read with 16-byte loads
-constexpr int kClPacked = 44;
-__device__ __forceinline__ void site_term_hp(const float2* __restrict__ Cl, float mass, const float2 p[12],
-                                             float2 out[12]) {
+__device__ __forceinline__ float2 lo2(float4 f) { return make_float2(f.x, f.y); }
+__device__ __forceinline__ float2 hi2(float4 f) { return make_float2(f.z, f.w); }
+// The link of direction mu of a site whose first word is U, words `stride` apart: four 16-byte words
+// and half of a fifth
+template <int mu>
+__device__ __forceinline__ void load_link(const float4* __restrict__ U, int stride, float2 u[9]) {
+  constexpr int e0 = 9 * mu, o = e0 & 1, p0 = e0 >> 1;
+  u[o ? 0 : 8] = __ldg(reinterpret_cast<const float2*>(U + (o ? p0 : p0 + 4) * stride) + o);
 #pragma unroll
-  for (int hh = 0; hh < 2; ++hh) {
-    float2 c[22];
-    const float4* q = reinterpret_cast<const float4*>(Cl + hh * 22);
+  for (int k = 0; k < 4; ++k) {
+    const float4 f = __ldg(U + (p0 + o + k) * stride);
+    u[o + 2 * k] = lo2(f);
+    u[o + 2 * k + 1] = hi2(f);
+  }
+}
+
+// N 16-byte words, `stride` words apart, of shared memory or (load_words) read-only global memory
+template <int N>
+__device__ __forceinline__ void put_words(float4* S, int stride, const float2 p[2 * N]) {
 #pragma unroll
-    for (int k = 0; k < 11; ++k) {
-      const float4 f = __ldg(q + k);
-      c[2 * k] = make_float2(f.x, f.y);
-      c[2 * k + 1] = make_float2(f.z, f.w);
-    }
+  for (int k = 0; k < N; ++k) S[k * stride] = make_float4(p[2 * k].x, p[2 * k].y, p[2 * k + 1].x, p[2 * k + 1].y);
+}
+template <int N>
+__device__ __forceinline__ void get_words(const float4* S, int stride, float2 p[2 * N]) {
 #pragma unroll
-    for (int a = 0; a < 6; ++a) {
-      float2 acc = zscale(p[hh * 6 + a], mass);
+  for (int k = 0; k < N; ++k) {
+    const float4 f = S[k * stride];
+    p[2 * k] = lo2(f);
+    p[2 * k + 1] = hi2(f);
+  }
+}
+template <int N>
+__device__ __forceinline__ void load_words(const float4* __restrict__ G, int stride, float2 p[2 * N]) {
 #pragma unroll
-      for (int b = 0; b < 6; ++b) {
-        if (a <= b) zfma(acc, c[tri_index(a, b)], p[hh * 6 + b]);
-        else zfmac(acc, c[tri_index(b, a)], p[hh * 6 + b]);
-      }
-      out[hh * 6 + a] = acc;
+  for (int k = 0; k < N; ++k) {
+    const float4 f = __ldg(G + k * stride);
+    p[2 * k] = lo2(f);
+    p[2 * k + 1] = hi2(f);
+  }
+}
+// 16-byte global -> shared copy that bypasses the registers (and L1)
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() {
+  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+}
+
+// h = (1 -+ g_mu) p on the upper half: u - A d (FWD), u + A d; h[3 s + colour]
+template <bool FWD, int mu>
+__device__ __forceinline__ void half_spinor(const float2 p[12], float2 h[6]) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    float2 a0, a1;
+    amul(mu, p[6 + c], p[9 + c], a0, a1);
+    h[c] = FWD ? zsub(p[c], a0) : zadd(p[c], a0);
+    h[3 + c] = FWD ? zsub(p[3 + c], a1) : zadd(p[3 + c], a1);
+  }
+}
+// row a of U h (FWD) or U^dag h for both spins
+template <bool FWD>
+__device__ __forceinline__ void colour_row(const float2* u, const float2 h[6], int a, float2& w0, float2& w1) {
+  w0 = w1 = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    if (FWD) {
+      zfma(w0, u[a * 3 + b], h[b]);
+      zfma(w1, u[a * 3 + b], h[3 + b]);
+    } else {
+      zfmac(w0, u[b * 3 + a], h[b]);
+      zfmac(w1, u[b * 3 + a], h[3 + b]);
     }
   }
 }
-// the site term of site s: FP32 from the packed clover, FP64 from the full [2][6][6] blocks
-template <typename C, typename T>
-__device__ __forceinline__ void site_term_at(const C* __restrict__ Cl, long long s, T mass, const C p[12], C out[12]) {
-  if constexpr (sizeof(C) == 8) site_term_hp(Cl + s * kClPacked, mass, p, out);
-  else site_term(Cl + s * 72, mass, p, out);
+// o += -(1 -+ g_mu)-hop of twice D for colour a of the product w: -w on the upper half, +- A^dag w on
+// the lower
+template <bool FWD, int mu>
+__device__ __forceinline__ void add_hop(float2 w0, float2 w1, int a, float2 o[12]) {
+  float2 d0, d1;
+  adagmul(mu, w0, w1, d0, d1);
+  o[a] = zsub(o[a], w0);
+  o[3 + a] = zsub(o[3 + a], w1);
+  o[6 + a] = FWD ? zadd(o[6 + a], d0) : zsub(o[6 + a], d0);
+  o[9 + a] = FWD ? zadd(o[9 + a], d1) : zsub(o[9 + a], d1);
+}
+template <bool FWD, int mu>
+__device__ __forceinline__ void hop2(const float2* u, const float2 p[12], float2 o[12]) {
+  float2 h[6], w0, w1;
+  half_spinor<FWD, mu>(p, h);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    colour_row<FWD>(u, h, a, w0, w1);
+    add_hop<FWD, mu>(w0, w1, a, o);
+  }
+}
+
+// out = (mass2 + 2 C) p from the site's clover words c (14 complex per chirality, times 2)
+__device__ __forceinline__ void site_term2(const float2 c[2 * kClovQ], float mass2, const float2 p[12], float2 out[12]) {
+#pragma unroll
+  for (int hh = 0; hh < 2; ++hh) {
+    const float2* k = c + hh * kClovQ;
+    const float2 *u = p + hh * 6, *d = u + 3;
+    const float dg[3] = {k[0].x, k[0].y, k[1].x};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      float2 s0 = zscale(u[a], mass2), s1 = zscale(d[a], mass2);
+      s0.x = fmaf(dg[a], u[a].x, s0.x);
+      s0.y = fmaf(dg[a], u[a].y, s0.y);
+      s1.x = fmaf(-dg[a], d[a].x, s1.x);
+      s1.y = fmaf(-dg[a], d[a].y, s1.y);
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        if (a < b) {
+          const float2 hab = k[1 + a + b];  // H01, H02, H12 at words 2, 3, 4
+          zfma(s0, hab, u[b]);
+          zfma(s1, zneg(hab), d[b]);
+        } else if (a > b) {
+          const float2 hba = k[1 + a + b];
+          zfmac(s0, hba, u[b]);
+          zfmac(s1, zneg(hba), d[b]);
+        }
+        zfma(s0, k[5 + 3 * a + b], d[b]);
+        zfmac(s1, k[5 + 3 * b + a], u[b]);
+      }
+      out[hh * 6 + a] = s0;
+      out[hh * 6 + 3 + a] = s1;
+    }
+  }
+}
+// Division by an invariant d of n < 2^31: n / d = (mulhi(m, n) + n) >> l with l = ceil(log2 d) and
+// m = floor(2^32 (2^l - d) / d) + 1 (Granlund and Montgomery 1994)
+struct FastDiv {
+  unsigned d, m, l;
+};
+FastDiv fast_div(unsigned d) {
+  FastDiv f{d, 0, 0};
+  while ((1ull << f.l) < d) ++f.l;
+  f.m = (unsigned)((((1ull << f.l) - d) << 32) / d + 1);
+  return f;
+}
+// n / d; rem: n % d
+__device__ __forceinline__ unsigned divide(unsigned n, const FastDiv& f, int& rem) {
+  const unsigned q = (__umulhi(f.m, n) + n) >> f.l;
+  rem = (int)(n - q * f.d);
+  return q;
 }
 
 struct FineGeom {
@@ -203,19 +316,27 @@ struct FineGeom {
   int B[4];
   int Lc[4];
   int Vb;
+  FastDiv dL[3], dB[3], dLc[3], dVb;
 };
 
-__device__ __forceinline__ void site_coords(const FineGeom& g, long long s, int x[4]) {
-  x[0] = (int)(s % g.L[0]);
-  s /= g.L[0];
-  x[1] = (int)(s % g.L[1]);
-  s /= g.L[1];
-  x[2] = (int)(s % g.L[2]);
-  x[3] = (int)(s / g.L[2]);
+__device__ __forceinline__ void coords_of(unsigned s, const FastDiv d[3], int x[4]) {
+#pragma unroll
+  for (int mu = 0; mu < 3; ++mu) s = divide(s, d[mu], x[mu]);
+  x[3] = (int)s;
 }
+__device__ __forceinline__ void site_coords(const FineGeom& g, long long s, int x[4]) { coords_of((unsigned)s, g.dL, x); }
 
 __device__ __forceinline__ long long site_of(const FineGeom& g, const int x[4]) {
   return (((long long)x[3] * g.L[2] + x[2]) * g.L[1] + x[1]) * g.L[0] + x[0];
+}
+
+// Lattice site of local index t in the block at coordinates X
+__device__ __forceinline__ long long local_site(const FineGeom& g, const int X[4], int t) {
+  int c[4];
+  coords_of((unsigned)t, g.dB, c);
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) c[mu] += X[mu] * g.B[mu];
+  return site_of(g, c);
 }
 
 template <typename C>
@@ -246,11 +367,10 @@ __device__ __forceinline__ long long nbr_site(const FineGeom& g, long long s, co
   return x[mu] > 0 ? s - st : s + st * (g.L[mu] - 1);
 }
 
-// out += all 8 hops of D at site s (neighbour spinors from v)
-template <typename C>
-__device__ __forceinline__ void all_hops(const FineGeom& g, const C* __restrict__ U, const C* __restrict__ v,
-                                         long long s, const int x[4], int nrhs, int r, C o[12]) {
-  C p[12];
+// out += all 8 hops of D at site s (neighbour spinors from v), FP64
+__device__ __forceinline__ void all_hops(const FineGeom& g, const double2* __restrict__ U, const double2* __restrict__ v,
+                                         long long s, const int x[4], int nrhs, int r, double2 o[12]) {
+  double2 p[12];
 #define AMG_HOPS(MU)                                      \
   {                                                       \
     const long long sf = nbr_site<MU, 1>(g, s, x);        \
@@ -267,15 +387,11 @@ __device__ __forceinline__ void all_hops(const FineGeom& g, const C* __restrict_
 #undef AMG_HOPS
 }
 
-// out = D psi (SUB: out = y - D psi), one thread per (site, right-hand side)
-template <typename T, bool SUB>
-__global__ void __launch_bounds__(128) dirac_kernel(const typename Cx<T>::type* __restrict__ U,
-                                                    const typename Cx<T>::type* __restrict__ Cl,
-                                                    const typename Cx<T>::type* __restrict__ psi,
-                                                    const typename Cx<T>::type* __restrict__ y,
-                                                    typename Cx<T>::type* __restrict__ out, FineGeom g, T mass,
-                                                    int nrhs) {
-  using C = typename Cx<T>::type;
+// out = D psi (SUB: out = y - D psi), one thread per (site, right-hand side); FP64
+template <bool SUB>
+__global__ void __launch_bounds__(128) dirac_kernel(const double2* __restrict__ U, const double2* __restrict__ Cl,
+                                                    const double2* __restrict__ psi, const double2* __restrict__ y,
+                                                    double2* __restrict__ out, FineGeom g, double mass, int nrhs) {
   const long long total = g.V * nrhs;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
        e += (long long)gridDim.x * blockDim.x) {
@@ -283,9 +399,9 @@ __global__ void __launch_bounds__(128) dirac_kernel(const typename Cx<T>::type* 
     const int r = (int)(e % nrhs);
     int x[4];
     site_coords(g, s, x);
-    C p[12], o[12];
+    double2 p[12], o[12];
     load12(psi, s, nrhs, r, p);
-    site_term_at(Cl, s, mass, p, o);
+    site_term(Cl + s * 72, mass, p, o);
     all_hops(g, U, psi, s, x, nrhs, r, o);
     if (SUB) {
       load12(y, s, nrhs, r, p);
@@ -297,13 +413,194 @@ __global__ void __launch_bounds__(128) dirac_kernel(const typename Cx<T>::type* 
   }
 }
 
+// Block coordinates of block k, and the block one step along mu
+__device__ __forceinline__ int block_of(const FineGeom& g, const int X[4]) {
+  return ((X[3] * g.Lc[2] + X[2]) * g.Lc[1] + X[1]) * g.Lc[0] + X[0];
+}
+template <int mu, int dir>
+__device__ __forceinline__ int block_next(const FineGeom& g, const int X[4]) {
+  int Y[4] = {X[0], X[1], X[2], X[3]};
+  Y[mu] = dir > 0 ? (X[mu] + 1 < g.Lc[mu] ? X[mu] + 1 : 0) : (X[mu] > 0 ? X[mu] - 1 : g.Lc[mu] - 1);
+  return block_of(g, Y);
+}
+
+// First word of the site below along mu (its link of direction mu carries the backward hop)
+template <int mu>
+__device__ __forceinline__ const float4* link_below(const FineGeom& g, const float4* U, const float4* Us, const int X[4],
+                                                    const int lc[4], int t, int stride) {
+  if (lc[mu] > 0) return Us - stride;
+  return U + (long long)block_next<mu, -1>(g, X) * kLinkQ * g.Vb + t + (g.B[mu] - 1) * stride;
+}
+
+// The same in FP32, several columns: lanes over (site in block order, group of NC columns), so that the
+// columns of a site are read together and its links and clover are broadcast.  With an even number of
+// columns a thread takes two (16-byte loads, half as many link and clover loads per column;
+// 16^3 x 32 and 12 columns: 162 us against 179 with one).  FAST: fewer than 2^31 threads.
+template <int NC>
+__device__ __forceinline__ void load_cols(const float2* __restrict__ v, long long site, int nrhs, int r, float2 p[NC][12]) {
+  if constexpr (NC == 1) {
+    load12(v, site, nrhs, r, p[0]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      const float4 f = __ldg(reinterpret_cast<const float4*>(v + (site * 12 + k) * nrhs + r));
+      p[0][k] = lo2(f);
+      p[1][k] = hi2(f);
+    }
+  }
+}
+template <bool SUB, bool FAST, int NC>
+__global__ void __launch_bounds__(128, NC == 1 ? 4 : 3) dirac32_kernel(const float4* __restrict__ U,
+                                                                       const float4* __restrict__ Cl,
+                                                                       const float2* __restrict__ psi,
+                                                                       const float2* __restrict__ y,
+                                                                       float2* __restrict__ out, FineGeom g, float mass2,
+                                                                       FastDiv dn) {
+  const int groups = (int)dn.d, nrhs = groups * NC;
+  const long long total = g.V * groups;
+  const int Vb = g.Vb;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
+       e += (long long)gridDim.x * blockDim.x) {
+    int r, t, X[4], lc[4], x[4];
+    unsigned i;
+    if (FAST) {
+      i = divide((unsigned)e, dn, r);
+    } else {
+      i = (unsigned)(e / groups);
+      r = (int)(e % groups);
+    }
+    r *= NC;
+    const unsigned b = divide(i, g.dVb, t);
+    coords_of(b, g.dLc, X);
+    coords_of((unsigned)t, g.dB, lc);
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) x[mu] = X[mu] * g.B[mu] + lc[mu];
+    const long long s = site_of(g, x);
+    float2 p[NC][12], o[NC][12];
+    load_cols<NC>(psi, s, nrhs, r, p);
+    {
+      float2 c[2 * kClovQ];
+      load_words<kClovQ>(Cl + (long long)b * kClovQ * Vb + t, Vb, c);
+#pragma unroll
+      for (int k = 0; k < NC; ++k) site_term2(c, mass2, p[k], o[k]);
+    }
+    const float4* Us = U + (long long)b * kLinkQ * Vb + t;
+    int stride = 1;
+#define AMG_HOPS2(MU)                                                                              \
+  {                                                                                                \
+    float2 u[9];                                                                                   \
+    load_cols<NC>(psi, nbr_site<MU, 1>(g, s, x), nrhs, r, p);                                      \
+    load_link<MU>(Us, Vb, u);                                                                      \
+    _Pragma("unroll") for (int k = 0; k < NC; ++k) hop2<true, MU>(u, p[k], o[k]);                  \
+    load_cols<NC>(psi, nbr_site<MU, -1>(g, s, x), nrhs, r, p);                                     \
+    load_link<MU>(link_below<MU>(g, U, Us, X, lc, t, stride), Vb, u);                              \
+    _Pragma("unroll") for (int k = 0; k < NC; ++k) hop2<false, MU>(u, p[k], o[k]);                 \
+    stride *= g.B[MU];                                                                             \
+  }
+    AMG_HOPS2(0)
+    AMG_HOPS2(1)
+    AMG_HOPS2(2)
+    AMG_HOPS2(3)
+#undef AMG_HOPS2
+    if (SUB) load_cols<NC>(y, s, nrhs, r, p);
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+      for (int k = 0; k < 12; ++k) {
+        o[c][k] = zscale(o[c][k], 0.5f);
+        if (SUB) o[c][k] = zsub(p[c][k], o[c][k]);
+      }
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      float2* q = out + (s * 12 + k) * nrhs + r;
+      if constexpr (NC == 1) *q = o[0][k];
+      else *reinterpret_cast<float4*>(q) = make_float4(o[0][k].x, o[0][k].y, o[1][k].x, o[1][k].y);
+    }
+  }
+}
+
+// One column: a CTA takes nb whole blocks (at most kDiracSites sites, one thread each, in the block order
+// of the links and the clover).  Their spinors are copied to shared memory in runs and serve the hops
+// inside a block; a neighbour across a block face is read from global memory, through the same
+// (generic) load, so that the hops have no branches and their loads overlap.  The links and the clover
+// are read as they are needed, consecutive words by consecutive lanes.  The result goes out through
+// the spinor tile.
+//
+// Bounds: HBM (816 bytes per site), reached as far as two CTAs per SM cover each other's waits.
+// 32^3 x 64: 310 us, 81 % of the copy bandwidth.  One thread per site in lattice order with records of 288 and 352 bytes took
+// 509 us (3,150 line look-ups in L1 per warp of sites).
+constexpr int kDiracSites = 256;
+constexpr int kRec = 7;  // words per record in the tile: 16-byte accesses of 8 consecutive sites hit all banks
+template <bool SUB>
+__global__ void __launch_bounds__(kDiracSites, 2) dirac32_block_kernel(const float4* __restrict__ U,
+                                                                       const float4* __restrict__ Cl, const float2* psi,
+                                                                       const float2* __restrict__ y, float2* out,
+                                                                       FineGeom g, float mass2, int nb, int nblocks) {
+  __shared__ float4 tile[kDiracSites * kRec];
+  __shared__ unsigned lex[kDiracSites];
+  const int Vb = g.Vb, b0 = blockIdx.x * nb, n = min(nb, nblocks - b0) * Vb, i = threadIdx.x;
+  const bool act = i < n;
+  int t, X[4], lc[4], x[4];
+  const int b = b0 + (int)divide((unsigned)(act ? i : 0), g.dVb, t);
+  coords_of((unsigned)b, g.dLc, X);
+  coords_of((unsigned)t, g.dB, lc);
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) x[mu] = X[mu] * g.B[mu] + lc[mu];
+  const long long s = site_of(g, x);
+  if (act) lex[i] = (unsigned)s;
+  __syncthreads();
+  for (int e = i; e < n * 6; e += blockDim.x)
+    cp_async16(tile + e / 6 * kRec + e % 6, reinterpret_cast<const float4*>(psi) + (long long)lex[e / 6] * 6 + e % 6);
+  float2 o[12], p[12];
+  float2 c[2 * kClovQ];
+  load_words<kClovQ>(Cl + (long long)b * kClovQ * Vb + t, Vb, c);
+  cp_async_wait_all();
+  __syncthreads();
+  if (act) {
+    const float4* own = tile + i * kRec;
+    get_words<6>(own, 1, p);
+    site_term2(c, mass2, p, o);
+    const float4* Us = U + (long long)b * kLinkQ * Vb + t;
+    int stride = 1;
+#define AMG_HOPS2(MU)                                                                                          \
+  {                                                                                                            \
+    float2 u[9];                                                                                               \
+    const float4* q = lc[MU] + 1 < g.B[MU] ? own + stride * kRec                                               \
+                                           : reinterpret_cast<const float4*>(psi + nbr_site<MU, 1>(g, s, x) * 12); \
+    load_link<MU>(Us, Vb, u);                                                                                  \
+    get_words<6>(q, 1, p);                                                                                     \
+    hop2<true, MU>(u, p, o);                                                                                   \
+    q = lc[MU] > 0 ? own - stride * kRec : reinterpret_cast<const float4*>(psi + nbr_site<MU, -1>(g, s, x) * 12); \
+    load_link<MU>(link_below<MU>(g, U, Us, X, lc, t, stride), Vb, u);                                          \
+    get_words<6>(q, 1, p);                                                                                     \
+    hop2<false, MU>(u, p, o);                                                                                  \
+    stride *= g.B[MU];                                                                                         \
+  }
+    AMG_HOPS2(0)
+    AMG_HOPS2(1)
+    AMG_HOPS2(2)
+    AMG_HOPS2(3)
+#undef AMG_HOPS2
+#pragma unroll
+    for (int k = 0; k < 12; ++k) o[k] = zscale(o[k], 0.5f);
+    if (SUB) {
+      load12(y, s, 1, 0, p);
+#pragma unroll
+      for (int k = 0; k < 12; ++k) o[k] = zsub(p[k], o[k]);
+    }
+  }
+  __syncthreads();
+  if (act) put_words<6>(tile + i * kRec, 1, o);
+  __syncthreads();
+  for (int e = i; e < n * 6; e += blockDim.x)
+    reinterpret_cast<float4*>(out)[(long long)lex[e / 6] * 6 + e % 6] = tile[e / 6 * kRec + e % 6];
+}
+
 // MR coefficient alpha = <p, rho> / <p, p> from per-thread partial sums v = (<p,p>, Re, Im <p,rho>):
-// warp sums, then the CTA sum and the division by one thread, all in the vector precision (FP64
-// is slow on this GPU: every thread summing and dividing in FP64 had kept the FP64 pipe busy, and
-// one thread's FP64 division held the whole CTA at the barrier), alpha broadcast through shared
-// memory.  ok = false when <p, p> = 0.  red: 3 doubles per warp + 3 doubles.
-template <typename T, typename C>
-__device__ __forceinline__ void cta_alpha(T v[3], double* red, C& al, bool& ok) {
+// warp sums, then the CTA sum and the division by one thread (FP64 is slow on this GPU: every thread
+// summing and dividing would keep the FP64 pipe busy), alpha broadcast through shared memory.
+// ok = false when <p, p> = 0.  red: 3 doubles per warp + 3 doubles.  FP64.
+__device__ __forceinline__ void cta_alpha(double v[3], double* red, double2& al, bool& ok) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
 #pragma unroll
   for (int k = 0; k < 3; ++k)
@@ -311,27 +608,27 @@ __device__ __forceinline__ void cta_alpha(T v[3], double* red, C& al, bool& ok) 
     for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
   __syncthreads();  // red may still be read by the previous call
   if (lane == 0)
-    for (int k = 0; k < 3; ++k) red[warp * 3 + k] = (double)v[k];
+    for (int k = 0; k < 3; ++k) red[warp * 3 + k] = v[k];
   __syncthreads();
   double* out = red + 3 * nw;
   if (threadIdx.x == 0) {
-    T sp = 0, sr = 0, si = 0;
+    double sp = 0, sr = 0, si = 0;
     for (int w = 0; w < nw; ++w) {
-      sp += (T)red[w * 3];
-      sr += (T)red[w * 3 + 1];
-      si += (T)red[w * 3 + 2];
+      sp += red[w * 3];
+      sr += red[w * 3 + 1];
+      si += red[w * 3 + 2];
     }
-    out[0] = sp > 0 ? (double)(sr / sp) : 0.0;
-    out[1] = sp > 0 ? (double)(si / sp) : 0.0;
+    out[0] = sp > 0 ? sr / sp : 0.0;
+    out[1] = sp > 0 ? si / sp : 0.0;
     red[3 * nw + 2] = sp > 0 ? 1.0 : 0.0;
   }
   __syncthreads();
-  al.x = (T)out[0];
-  al.y = (T)out[1];
+  al.x = out[0];
+  al.y = out[1];
   ok = out[2] != 0.0;
 }
 
-// The same coefficient with one barrier: each warp's lane 0 writes the warp's partial sums to its
+// The same coefficient in FP32 with one barrier: each warp's lane 0 writes the warp's partial sums to its
 // slot of red (3 values per warp, FP32), and after the barrier every thread sums the slots in warp
 // order and divides, so that all threads hold the same alpha (the order and the arithmetic of
 // cta_alpha, hence the same value).  Callers alternate between two red buffers from one step to the
@@ -357,11 +654,12 @@ __device__ __forceinline__ void cta_alpha_all(float v[3], float* red, float2& al
 }
 
 // Intra-block hops of the block operator B at local site t: neighbours' rho from shared memory
-// (component-major: rho[q * Vb + t]), links from global memory.
-template <int mu, typename C>
-__device__ __forceinline__ void block_hops_mu(const FineGeom& g, const C* __restrict__ U, const C* rho, int t,
-                                              long long s, const int x[4], const int lc[4], int stride, C o[12]) {
-  C p[12];
+// (component-major: rho[q * Vb + t]), links from global memory; FP64.
+template <int mu>
+__device__ __forceinline__ void block_hops_mu(const FineGeom& g, const double2* __restrict__ U, const double2* rho,
+                                              int t, long long s, const int x[4], const int lc[4], int stride,
+                                              double2 o[12]) {
+  double2 p[12];
   if (lc[mu] + 1 < g.B[mu]) {
 #pragma unroll
     for (int q = 0; q < 12; ++q) p[q] = rho[q * g.Vb + t + stride];
@@ -375,29 +673,31 @@ __device__ __forceinline__ void block_hops_mu(const FineGeom& g, const C* __rest
   }
 }
 
+// Coordinates of the k-th block of a colour: rows of Lc[0] / 2 blocks, X of the colour's parity in
+// each row
+__device__ __forceinline__ void colour_block(const FineGeom& g, int k, int colour, int X[4]) {
+  const int half = g.Lc[0] / 2;
+  int row = k / half;
+  X[1] = row % g.Lc[1];
+  row /= g.Lc[1];
+  X[2] = row % g.Lc[2];
+  X[3] = row / g.Lc[2];
+  X[0] = 2 * (k % half) + ((colour + X[1] + X[2] + X[3]) & 1);
+}
+
 // One SAP half sweep on the blocks of one colour: x += MR_{n_mr}(B_b, (y - D x)|_b) per block.
 // grid (Vc / 2, nrhs); blockDim >= Vb (threads past Vb only join the sums); dynamic smem: rho
 // [12][Vb] + 3 doubles per warp + 3 doubles.
-template <typename T>
-__global__ void __launch_bounds__(256) sap_kernel(const typename Cx<T>::type* __restrict__ U,
-                                                  const typename Cx<T>::type* __restrict__ Cl,
-                                                  const typename Cx<T>::type* __restrict__ y,
-                                                  typename Cx<T>::type* __restrict__ x, FineGeom g, T mass,
-                                                  int nrhs, int colour, int n_mr) {
-  using C = typename Cx<T>::type;
+__global__ void __launch_bounds__(256) sap_kernel(const double2* __restrict__ U, const double2* __restrict__ Cl,
+                                                  const double2* __restrict__ y, double2* __restrict__ x, FineGeom g,
+                                                  double mass, int nrhs, int colour, int n_mr) {
+  using C = double2;
   extern __shared__ __align__(16) unsigned char smem[];
   C* rho = reinterpret_cast<C*>(smem);
   double* red = reinterpret_cast<double*>(smem + (size_t)g.Vb * 12 * sizeof(C));
   const int r = blockIdx.y;
-  // the k-th block of this colour: rows of Lc[0] / 2 blocks, X of the colour's parity in each row
-  const long long k = blockIdx.x;
-  const int half = g.Lc[0] / 2;
-  long long row = k / half;
-  const int Y = (int)(row % g.Lc[1]);
-  row /= g.Lc[1];
-  const int Z = (int)(row % g.Lc[2]);
-  const int Tt = (int)(row / g.Lc[2]);
-  const int X = 2 * (int)(k % half) + ((colour + Y + Z + Tt) & 1);
+  int X[4];
+  colour_block(g, blockIdx.x, colour, X);
   const int t = threadIdx.x;
   const bool act = t < g.Vb;
   int lc[4] = {0, 0, 0, 0}, xs[4] = {0, 0, 0, 0};
@@ -407,10 +707,8 @@ __global__ void __launch_bounds__(256) sap_kernel(const typename Cx<T>::type* __
     lc[1] = (t / g.B[0]) % g.B[1];
     lc[2] = (t / (g.B[0] * g.B[1])) % g.B[2];
     lc[3] = t / (g.B[0] * g.B[1] * g.B[2]);
-    xs[0] = X * g.B[0] + lc[0];
-    xs[1] = Y * g.B[1] + lc[1];
-    xs[2] = Z * g.B[2] + lc[2];
-    xs[3] = Tt * g.B[3] + lc[3];
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) xs[mu] = X[mu] * g.B[mu] + lc[mu];
     s = site_of(g, xs);
   }
   const int st1 = g.B[0], st2 = g.B[0] * g.B[1], st3 = g.B[0] * g.B[1] * g.B[2];
@@ -419,7 +717,7 @@ __global__ void __launch_bounds__(256) sap_kernel(const typename Cx<T>::type* __
   if (act) {
     C p[12];
     load12(x, s, nrhs, r, p);
-    site_term_at(Cl, s, mass, p, o);
+    site_term(Cl + s * 72, mass, p, o);
     all_hops(g, U, x, s, xs, nrhs, r, o);
     load12(y, s, nrhs, r, p);
 #pragma unroll
@@ -432,12 +730,12 @@ __global__ void __launch_bounds__(256) sap_kernel(const typename Cx<T>::type* __
 #pragma unroll 1
   for (int it = 0; it < n_mr; ++it) {
     // p = B rho at this site: site term plus the hops that stay inside the block
-    T v[3] = {0, 0, 0};
+    double v[3] = {0, 0, 0};
     C rr[12];
     if (act) {
 #pragma unroll
       for (int q = 0; q < 12; ++q) rr[q] = rho[q * g.Vb + t];
-      site_term_at(Cl, s, mass, rr, o);
+      site_term(Cl + s * 72, mass, rr, o);
       block_hops_mu<0>(g, U, rho, t, s, xs, lc, 1, o);
       block_hops_mu<1>(g, U, rho, t, s, xs, lc, st1, o);
       block_hops_mu<2>(g, U, rho, t, s, xs, lc, st2, o);
@@ -472,238 +770,355 @@ __global__ void __launch_bounds__(256) sap_kernel(const typename Cx<T>::type* __
   }
 }
 
-// The same half sweep with the block's links and clover staged in shared memory once, so that
-// the MR steps read no global memory (FP32; a 4^4 block takes 74 KB of links, 90 KB of clover and
-// 25 KB of rho).  Every staged record keeps its HBM order in pairs of entries, one float4 per pair,
-// laid out [pair][Vb]: the threads of a warp (one site each) then read 512 consecutive bytes with
-// 16-byte loads, and the staging copies the 16-byte pieces as they lie in HBM (cp.async, no
-// register round trip).  Links [18][Vb] (the site's 36 entries, 9 per direction); clover [22][Vb]
-// (per chirality the upper triangle with the diagonal, 21 entries padded to 22: the blocks are
-// Hermitian, C_ba = conj(C_ab)); rho [6][Vb].
-__device__ __forceinline__ float2 lo2(float4 f) { return make_float2(f.x, f.y); }
-__device__ __forceinline__ float2 hi2(float4 f) { return make_float2(f.z, f.w); }
-// Entry e of a staged record at local site t (the low or high half of pair e / 2)
-__device__ __forceinline__ float2 staged_entry(const float4* S, int Vb, int t, int e) {
-  return reinterpret_cast<const float2*>(S + (size_t)(e >> 1) * Vb + t)[e & 1];
+// The same half sweep in FP32.  A thread holds its site's four links and its clover (128 registers)
+// while it sweeps a group of nr right-hand sides.  A backward hop needs the link of the neighbour it
+// comes from, which another thread holds: that thread multiplies, U_mu^dag (1 + g_mu) rho with its
+// own link and rho, and hands the half spinor over in shared memory (48 bytes; the link and the
+// spinor would be 168).  The hops that cross the block face appear in the residual only: a list of
+// face sites, spread over all threads, fetches the outside neighbours; forward ones leave their half
+// spinors in halo, backward ones the finished product in the hand-over buffer.
+//
+// One persistent CTA of Vb threads (255 registers: one per SM at 4^4) takes (block, group) items.  The
+// next item's links and clover come by bulk copy into shared memory while the MR steps of the current
+// one run.  x and y are in the block order of the links (BLOCKED): bulk copies, and 16-byte words of
+// consecutive sites for the face neighbours; otherwise in the caller's order, entry by entry.
+//
+// Bounds: the FP32 pipes (about 1,330 operations per site and application of D or B, five of them:
+// 13 K cycles per block and column) at two warps per sub-partition; of 41 K cycles per block (32^4)
+// the MR steps take 6.4 K each, the hops across the faces 7 K (4 K when their lines are in L2).
+// Half sweep with 4 MR steps: 277 us at 32^4 and one column, 379 us at 16^3 x 32 and 12 columns;
+// staging the links and the clover in shared memory once per block and column instead (189 KB, every
+// MR step reading them back) took 367 and 1,424 us.
+//
+// Shared memory (float4 words): x [6][Vb] (12 entries), rho [6][Vb], the hand-over buffer [4 mu][3][Vb],
+// the next links [18][Vb] and clover [14][Vb].  Between the load of the links into registers and the
+// end of the residual the latter two hold halo ([3][f] per direction, f its face sites) and y [6][Vb].
+__host__ __device__ inline int face_sites(const FineGeom& g, int mu) { return g.Vb / g.B[mu]; }
+constexpr int kSapRed = 12;  // words of the MR coefficient's warp sums: 2 buffers x 3 sums x 8 warps of floats
+inline size_t sap_smem(const FineGeom& g) {
+  return amgpipe::kPipeBytes + (size_t)(kSapRed + (24 + kLinkQ + kClovQ) * g.Vb) * sizeof(float4);
 }
-// The link of direction mu at local site t: entries 9 mu .. 9 mu + 8, four pairs and one half
-template <int mu>
-__device__ __forceinline__ void staged_link(const float4* Us, int Vb, int t, float2 u[9]) {
-  constexpr int e0 = 9 * mu, o = e0 & 1, p0 = e0 >> 1;
-  if (o) u[0] = staged_entry(Us, Vb, t, e0);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const float4 f = Us[(size_t)(p0 + o + k) * Vb + t];
-    u[o + 2 * k] = lo2(f);
-    u[o + 2 * k + 1] = hi2(f);
-  }
-  if (!o) u[8] = staged_entry(Us, Vb, t, e0 + 8);
-}
-__device__ __forceinline__ void staged_spinor(const float4* R, int Vb, int t, float2 p[12]) {
-#pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    const float4 f = R[(size_t)k * Vb + t];
-    p[2 * k] = lo2(f);
-    p[2 * k + 1] = hi2(f);
-  }
-}
-__device__ __forceinline__ void store_spinor(float4* R, int Vb, int t, const float2 p[12]) {
-#pragma unroll
-  for (int k = 0; k < 6; ++k) R[(size_t)k * Vb + t] = make_float4(p[2 * k].x, p[2 * k].y, p[2 * k + 1].x, p[2 * k + 1].y);
-}
-// 16-byte global -> shared copy that bypasses the registers (and L1)
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-}
-
-__device__ __forceinline__ void site_term_packed(const float4* Cs, int Vb, int t, float mass, const float2 p[12],
-                                                 float2 out[12]) {
-#pragma unroll
-  for (int hh = 0; hh < 2; ++hh) {
-    float2 c[21];
-#pragma unroll
-    for (int k = 0; k < 10; ++k) {
-      const float4 f = Cs[(size_t)(hh * 11 + k) * Vb + t];
-      c[2 * k] = lo2(f);
-      c[2 * k + 1] = hi2(f);
-    }
-    c[20] = staged_entry(Cs, Vb, t, hh * 22 + 20);
-#pragma unroll
-    for (int a = 0; a < 6; ++a) {
-      float2 acc = zscale(p[hh * 6 + a], mass);
-#pragma unroll
-      for (int b = 0; b < 6; ++b) {
-        if (a <= b) zfma(acc, c[tri_index(a, b)], p[hh * 6 + b]);
-        else zfmac(acc, c[tri_index(b, a)], p[hh * 6 + b]);
-      }
-      out[hh * 6 + a] = acc;
-    }
-  }
-}
-
-template <int mu>
-__device__ __forceinline__ void block_hops_smem(const float4* Us, const float4* rho, int Vb, int t, const int lc[4],
-                                                int bmu, int stride, float2 o[12]) {
-  float2 p[12], u[9];
-  if (lc[mu] + 1 < bmu) {
-    staged_spinor(rho, Vb, t + stride, p);
-    staged_link<mu>(Us, Vb, t, u);
-    hop_u<true, mu>(u, p, o);
-  }
-  if (lc[mu] > 0) {
-    staged_spinor(rho, Vb, t - stride, p);
-    staged_link<mu>(Us, Vb, t - stride, u);
-    hop_u<false, mu>(u, p, o);
-  }
-}
-
-// Both hops of direction mu of the full D at site s (neighbour spinors from global memory), links
-// from the staged block where they lie in it: the forward link always, the backward one unless the
-// neighbour is outside the block.
-template <int mu>
-__device__ __forceinline__ void residual_hops(const FineGeom& g, const float2* __restrict__ U, const float4* Us,
-                                              const float2* __restrict__ v, long long s, const int x[4], const int lc[4],
-                                              int Vb, int t, int stride, int nrhs, int r, float2 o[12]) {
-  float2 p[12], u[9];
-  load12(v, nbr_site<mu, 1>(g, s, x), nrhs, r, p);
-  staged_link<mu>(Us, Vb, t, u);
-  hop_u<true, mu>(u, p, o);
-  const long long sb = nbr_site<mu, -1>(g, s, x);
-  load12(v, sb, nrhs, r, p);
-  if (lc[mu] > 0) {
-    staged_link<mu>(Us, Vb, t - stride, u);
+// Column r of x and y: in block order word q of (block b, site t) at r V 6 + (b 6 + q) Vb + t, else
+// entry k of lattice site s at (s 12 + k) nrhs + r
+template <bool BLOCKED>
+__device__ __forceinline__ void load_site(const FineGeom& g, const float2* __restrict__ v, int b, const int X[4], int t,
+                                          int nrhs, int r, float2 p[12]) {
+  if (BLOCKED) {
+    const float4* q = reinterpret_cast<const float4*>(v) + r * g.V * 6 + (long long)b * 6 * g.Vb + t;
+    load_words<6>(q, g.Vb, p);
   } else {
-    load_link<mu>(U + (sb * 4 + mu) * 9, u);
+    load12(v, local_site(g, X, t), nrhs, r, p);
   }
-  hop_u<false, mu>(u, p, o);
 }
 
-__global__ void __launch_bounds__(256, 1) sap_smem_kernel(const float2* __restrict__ U, const float2* __restrict__ Cl,
-                                                          const float2* __restrict__ y, float2* __restrict__ x,
-                                                          FineGeom g, float mass, int nrhs, int colour, int n_mr) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int Vb = g.Vb;
-  float4* Us = reinterpret_cast<float4*>(smem);
-  float4* Cs = Us + (size_t)18 * Vb;
-  float4* rho = Cs + (size_t)22 * Vb;
-  // two buffers of the MR coefficient's warp sums, 3 floats per warp each
-  float* redf = reinterpret_cast<float*>(rho + (size_t)6 * Vb);
-  const int r = blockIdx.y;
-  const long long k = blockIdx.x;
-  const int half = g.Lc[0] / 2;
-  long long row = k / half;
-  const int Y = (int)(row % g.Lc[1]);
-  row /= g.Lc[1];
-  const int Z = (int)(row % g.Lc[2]);
-  const int Tt = (int)(row / g.Lc[2]);
-  const int X = 2 * (int)(k % half) + ((colour + Y + Z + Tt) & 1);
-  const int t = threadIdx.x;
-  const bool act = t < Vb;
-  int lc[4] = {0, 0, 0, 0}, xs[4] = {0, 0, 0, 0};
-  long long s = 0;
-  if (act) {
-    lc[0] = t % g.B[0];
-    lc[1] = (t / g.B[0]) % g.B[1];
-    lc[2] = (t / (g.B[0] * g.B[1])) % g.B[2];
-    lc[3] = t / (g.B[0] * g.B[1] * g.B[2]);
-    xs[0] = X * g.B[0] + lc[0];
-    xs[1] = Y * g.B[1] + lc[1];
-    xs[2] = Z * g.B[2] + lc[2];
-    xs[3] = Tt * g.B[3] + lc[3];
-    s = site_of(g, xs);
-  }
-  const int st1 = g.B[0], st2 = g.B[0] * g.B[1], st3 = g.B[0] * g.B[1] * g.B[2];
-  float2 o[12], e[12];
-  if (act) {
-    // stage this site's links (288 bytes) and packed clover (352 bytes) as they lie in HBM
-    const float4* U4 = reinterpret_cast<const float4*>(U + s * 36);
+// The hops of face site f of direction mu to its outside neighbours on both sides.  t: its local index
+// at lc[mu] = 0; the block's site at lc[mu] = B - 1 is (B - 1) stride further.
+template <int mu, bool BLOCKED>
+__device__ __forceinline__ void face_hops(const FineGeom& g, const float4* __restrict__ U, const float2* __restrict__ x,
+                                          const int X[4], int f, int stride, int nrhs, int r, float4* ex, float4* halo) {
+  const int Vb = g.Vb, nf = face_sites(g, mu);
+  const int t = f / stride * (stride * g.B[mu]) + f % stride, tt = t + (g.B[mu] - 1) * stride;
+  int Xf[4] = {X[0], X[1], X[2], X[3]}, Xb[4] = {X[0], X[1], X[2], X[3]};
+  Xf[mu] = X[mu] + 1 < g.Lc[mu] ? X[mu] + 1 : 0;
+  Xb[mu] = X[mu] > 0 ? X[mu] - 1 : g.Lc[mu] - 1;
+  const int bf = block_of(g, Xf), bb = block_of(g, Xb);
+  float2 pf[12], pb[12], h[6], u[9], w[6];
+  load_site<BLOCKED>(g, x, bf, Xf, t, nrhs, r, pf);
+  load_site<BLOCKED>(g, x, bb, Xb, tt, nrhs, r, pb);
+  load_link<mu>(U + (long long)bb * kLinkQ * Vb + tt, Vb, u);
+  half_spinor<true, mu>(pf, h);
+  put_words<3>(halo + f, nf, h);
+  half_spinor<false, mu>(pb, h);
 #pragma unroll
-    for (int q = 0; q < 18; ++q) cp_async16(Us + (size_t)q * Vb + t, U4 + q);
-    const float4* C4 = reinterpret_cast<const float4*>(Cl + s * kClPacked);
-#pragma unroll
-    for (int q = 0; q < 22; ++q) cp_async16(Cs + (size_t)q * Vb + t, C4 + q);
+  for (int a = 0; a < 3; ++a) colour_row<false>(u, h, a, w[a], w[3 + a]);
+  put_words<3>(ex + mu * 3 * Vb + t, Vb, w);
+}
+// body(direction, face site, offset of the direction's halo) for every face site of the block
+template <typename F>
+__device__ __forceinline__ void for_faces(const int nf[4], F&& body) {
+  const int n = nf[0] + nf[1] + nf[2] + nf[3];
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    int f = i;
+    if (f < nf[0]) body(std::integral_constant<int, 0>(), f, 0);
+    else if ((f -= nf[0]) < nf[1]) body(std::integral_constant<int, 1>(), f, 3 * nf[0]);
+    else if ((f -= nf[1]) < nf[2]) body(std::integral_constant<int, 2>(), f, 3 * (nf[0] + nf[1]));
+    else body(std::integral_constant<int, 3>(), f - nf[2], 3 * (nf[0] + nf[1] + nf[2]));
   }
-  cp_async_wait_all();
-  __syncthreads();  // links and clover staged
-  if (act) {
-    // residual r = y - D x on this site (full D: neighbours outside the block have the other colour);
-    // the clover, the forward links and the backward links inside the block from shared memory
+}
+
+// The thread's half spinors U_mu^dag (1 + g_mu) p for its forward neighbours in the block
+template <int mu>
+__device__ __forceinline__ void hand_over(const float2 u[36], const float2 p[12], bool inside, int Vb, int t, int stride,
+                                          float4* ex) {
+  if (!inside) return;
+  float2 h[6], w[6];
+  half_spinor<false, mu>(p, h);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) colour_row<false>(u + 9 * mu, h, a, w[a], w[3 + a]);
+  put_words<3>(ex + mu * 3 * Vb + t + stride, Vb, w);
+}
+template <int mu>
+__device__ __forceinline__ void take_over(const float4* ex, int Vb, int t, float2 o[12]) {
+  float2 w[6];
+  get_words<3>(ex + mu * 3 * Vb + t, Vb, w);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) add_hop<false, mu>(w[a], w[3 + a], a, o);
+}
+// forward hop from the half spinor h
+template <int mu>
+__device__ __forceinline__ void forward_half(const float2 u[36], const float2 h[6], float2 o[12]) {
+  float2 w0, w1;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    colour_row<true>(u + 9 * mu, h, a, w0, w1);
+    add_hop<true, mu>(w0, w1, a, o);
+  }
+}
+// both hops of direction mu of the full D: neighbours in the block from xs, outside ones from halo
+template <int mu>
+__device__ __forceinline__ void full_hops(const float2 u[36], const float4* xs, const float4* ex, const float4* halo,
+                                          int nf, int f, bool inside, int Vb, int t, int stride, float2 o[12]) {
+  float2 h[6];
+  if (inside) {
     float2 p[12];
-    load12(x, s, nrhs, r, p);
-    site_term_packed(Cs, Vb, t, mass, p, o);
-    residual_hops<0>(g, U, Us, x, s, xs, lc, Vb, t, 1, nrhs, r, o);
-    residual_hops<1>(g, U, Us, x, s, xs, lc, Vb, t, st1, nrhs, r, o);
-    residual_hops<2>(g, U, Us, x, s, xs, lc, Vb, t, st2, nrhs, r, o);
-    residual_hops<3>(g, U, Us, x, s, xs, lc, Vb, t, st3, nrhs, r, o);
-    load12(y, s, nrhs, r, p);
+    get_words<6>(xs + t + stride, Vb, p);
+    half_spinor<true, mu>(p, h);
+  } else {
+    get_words<3>(halo + f, nf, h);
+  }
+  forward_half<mu>(u, h, o);
+  take_over<mu>(ex, Vb, t, o);
+}
+// both hops of direction mu of the block operator
+template <int mu>
+__device__ __forceinline__ void block_hops(const float2 u[36], const float4* rho, const float4* ex, bool inside, bool below,
+                                           int Vb, int t, int stride, float2 o[12]) {
+  if (inside) {
+    float2 p[12], h[6];
+    get_words<6>(rho + t + stride, Vb, p);
+    half_spinor<true, mu>(p, h);
+    forward_half<mu>(u, h, o);
+  }
+  if (below) take_over<mu>(ex, Vb, t, o);
+}
+
+template <bool BLOCKED>
+__global__ void __launch_bounds__(256, 1) sap_reg_kernel(const float4* __restrict__ U, const float4* __restrict__ Cl,
+                                                         const float2* __restrict__ y, float2* x, FineGeom g, float mass2,
+                                                         int nrhs, int nr, int groups, int items, int colour, int n_mr,
+                                                         unsigned* err) {
+  using namespace amgpipe;
+  extern __shared__ __align__(128) unsigned char sm[];
+  Pipe* pp = reinterpret_cast<Pipe*>(sm);  // full[0]: links and clover, full[1]: x and y
+  const int Vb = g.Vb;
+  float* red = reinterpret_cast<float*>(sm + kPipeBytes);
+  float4* xs = reinterpret_cast<float4*>(sm + kPipeBytes) + kSapRed;
+  float4* rho = xs + 6 * Vb;
+  float4* ex = rho + 6 * Vb;
+  float4* us = ex + 12 * Vb;
+  float4* cs = us + kLinkQ * Vb;
+  float4 *halo = us, *ys = cs;
+  const int nf[4] = {face_sites(g, 0), face_sites(g, 1), face_sites(g, 2), face_sites(g, 3)};
+  const int t = threadIdx.x, ta = t < Vb ? t : 0;
+  const bool act = t < Vb;
+  const int st[4] = {1, g.B[0], g.B[0] * g.B[1], g.B[0] * g.B[1] * g.B[2]};
+  bool in[4], below[4];  // neighbour in the block forward, backward
+  int fi[4];             // index among the face sites of a direction
+  {
+    int lc[4];
+    coords_of((unsigned)ta, g.dB, lc);
 #pragma unroll
-    for (int q = 0; q < 12; ++q) {
-      p[q] = zsub(p[q], o[q]);
-      e[q] = zzero<float2>();
+    for (int mu = 0; mu < 4; ++mu) {
+      in[mu] = act && lc[mu] + 1 < g.B[mu];
+      below[mu] = lc[mu] > 0;
+      fi[mu] = t / (st[mu] * g.B[mu]) * st[mu] + t % st[mu];
     }
-    store_spinor(rho, Vb, t, p);
+  }
+  auto load_links = [&](int item) {  // one thread: the item's links and clover
+    int X[4];
+    colour_block(g, item / groups, colour, X);
+    const long long b = block_of(g, X);
+    mbar_expect_tx(&pp->full[0], (unsigned)((kLinkQ + kClovQ) * Vb * sizeof(float4)));
+    bulk_load(us, U + b * kLinkQ * Vb, (unsigned)(kLinkQ * Vb * sizeof(float4)), &pp->full[0]);
+    bulk_load(cs, Cl + b * kClovQ * Vb, (unsigned)(kClovQ * Vb * sizeof(float4)), &pp->full[0]);
+  };
+  if (t == 0) {
+    mbar_init(&pp->full[0], 1);
+    mbar_init(&pp->full[1], 1);
+    pp->abort = 0;
+    fence_mbar_init();
+    load_links(blockIdx.x);
   }
   __syncthreads();
+  unsigned phl = 0, phx = 0;
+  // items: (block, group of columns), the groups of a block next to each other (they share its
+  // lines in L2)
+  for (int item = blockIdx.x; item < items; item += gridDim.x) {
+    const int r0 = item % groups * nr, r1 = min(nrhs, r0 + nr);
+    int X[4];
+    colour_block(g, item / groups, colour, X);
+    const int b = block_of(g, X);
+    if (!wait_phase(&pp->full[0], phl, pp)) abort_cta(pp, err);
+    phl ^= 1u;
+    float2 u[36], cl[2 * kClovQ];
+    get_words<kLinkQ>(us + ta, Vb, u);
+    get_words<kClovQ>(cs + ta, Vb, cl);
+    for (int r = r0; r < r1; ++r) {
+      float2 p[12], o[12], e[12];
+      // x and y on the block, and the hops from outside it
+      __syncthreads();  // us, cs (first column) and xs (later ones) are read
+      if (pp->abort) return;
+      if (BLOCKED) {
+        if (t == 0) {
+          const unsigned bytes = (unsigned)(6 * Vb * sizeof(float4));
+          const long long at = r * g.V * 6 + (long long)b * 6 * Vb;
+          mbar_expect_tx(&pp->full[1], 2 * bytes);
+          bulk_load(xs, reinterpret_cast<const float4*>(x) + at, bytes, &pp->full[1]);
+          bulk_load(ys, reinterpret_cast<const float4*>(y) + at, bytes, &pp->full[1]);
+        }
+      } else if (act) {
+        const long long s = local_site(g, X, t);
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+          reinterpret_cast<float2*>(xs + (k >> 1) * Vb + t)[k & 1] = x[(s * 12 + k) * nrhs + r];
+          reinterpret_cast<float2*>(ys + (k >> 1) * Vb + t)[k & 1] = y[(s * 12 + k) * nrhs + r];
+        }
+      }
+      for_faces(nf, [&](auto mu, int f, int off) {
+        face_hops<mu, BLOCKED>(g, U, x, X, f, st[mu], nrhs, r, ex, halo + off);
+      });
+      if (BLOCKED) {
+        if (!wait_phase(&pp->full[1], phx, pp)) abort_cta(pp, err);
+        phx ^= 1u;
+      }
+      get_words<6>(xs + ta, Vb, p);
+      hand_over<0>(u, p, in[0], Vb, t, st[0], ex);
+      hand_over<1>(u, p, in[1], Vb, t, st[1], ex);
+      hand_over<2>(u, p, in[2], Vb, t, st[2], ex);
+      hand_over<3>(u, p, in[3], Vb, t, st[3], ex);
+      __syncthreads();
+      if (pp->abort) return;
+      if (act) {
+        // rho = y - D x
+        site_term2(cl, mass2, p, o);
+        full_hops<0>(u, xs, ex, halo, nf[0], fi[0], in[0], Vb, t, st[0], o);
+        full_hops<1>(u, xs, ex, halo + 3 * nf[0], nf[1], fi[1], in[1], Vb, t, st[1], o);
+        full_hops<2>(u, xs, ex, halo + 3 * (nf[0] + nf[1]), nf[2], fi[2], in[2], Vb, t, st[2], o);
+        full_hops<3>(u, xs, ex, halo + 3 * (nf[0] + nf[1] + nf[2]), nf[3], fi[3], in[3], Vb, t, st[3], o);
+        get_words<6>(ys + t, Vb, p);
+#pragma unroll
+        for (int q = 0; q < 12; ++q) {
+          p[q].x = fmaf(-0.5f, o[q].x, p[q].x);
+          p[q].y = fmaf(-0.5f, o[q].y, p[q].y);
+          e[q] = zzero<float2>();
+        }
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // halo and y before the next copies
+      __syncthreads();  // the hand-over buffer, halo and y are read
+      if (t == 0 && r + 1 == r1 && item + (int)gridDim.x < items) load_links(item + gridDim.x);
 #pragma unroll 1
-  for (int it = 0; it < n_mr; ++it) {
-    // p = B rho at this site: site term plus the hops that stay inside the block
-    float v[3] = {0, 0, 0};
-    float2 rr[12];
-    if (act) {
-      staged_spinor(rho, Vb, t, rr);
-      site_term_packed(Cs, Vb, t, mass, rr, o);
-      block_hops_smem<0>(Us, rho, Vb, t, lc, g.B[0], 1, o);
-      block_hops_smem<1>(Us, rho, Vb, t, lc, g.B[1], st1, o);
-      block_hops_smem<2>(Us, rho, Vb, t, lc, g.B[2], st2, o);
-      block_hops_smem<3>(Us, rho, Vb, t, lc, g.B[3], st3, o);
+      for (int it = 0; it < n_mr; ++it) {
+        // p holds rho on this site
+        if (act) put_words<6>(rho + t, Vb, p);
+        hand_over<0>(u, p, in[0], Vb, t, st[0], ex);
+        hand_over<1>(u, p, in[1], Vb, t, st[1], ex);
+        hand_over<2>(u, p, in[2], Vb, t, st[2], ex);
+        hand_over<3>(u, p, in[3], Vb, t, st[3], ex);
+        __syncthreads();
+        float v[3] = {0, 0, 0};
+        if (act) {
+          site_term2(cl, mass2, p, o);  // o = 2 B rho
+          block_hops<0>(u, rho, ex, in[0], below[0], Vb, t, st[0], o);
+          block_hops<1>(u, rho, ex, in[1], below[1], Vb, t, st[1], o);
+          block_hops<2>(u, rho, ex, in[2], below[2], Vb, t, st[2], o);
+          block_hops<3>(u, rho, ex, in[3], below[3], Vb, t, st[3], o);
 #pragma unroll
-      for (int q = 0; q < 12; ++q) {
-        v[0] += o[q].x * o[q].x + o[q].y * o[q].y;        // <p, p>
-        v[1] += o[q].x * rr[q].x + o[q].y * rr[q].y;      // Re <p, rho>
-        v[2] += o[q].x * rr[q].y - o[q].y * rr[q].x;      // Im <p, rho>
+          for (int q = 0; q < 12; ++q) {
+            v[0] += o[q].x * o[q].x + o[q].y * o[q].y;  // <o, o>
+            v[1] += o[q].x * p[q].x + o[q].y * p[q].y;  // Re <o, rho>
+            v[2] += o[q].x * p[q].y - o[q].y * p[q].x;  // Im <o, rho>
+          }
+        }
+        float2 al;
+        bool ok;
+        // the barrier inside also orders every read of rho and ex before the next step's writes
+        cta_alpha_all(v, red + (it & 1) * 24, al, ok);
+        if (ok) {  // al = alpha / 2 (o = 2 B rho): e += alpha rho, rho -= alpha B rho
+          const float2 al2 = make_float2(2.f * al.x, 2.f * al.y);
+#pragma unroll
+          for (int q = 0; q < 12; ++q) {
+            zfma(e[q], al2, p[q]);
+            float2 ap = zzero<float2>();
+            zfma(ap, al, o[q]);
+            p[q] = zsub(p[q], ap);
+          }
+        }
       }
-    }
-    float2 al;
-    bool ok;
-    // also orders every read of rho before the writes below
-    cta_alpha_all(v, redf + (it & 1) * 3 * ((blockDim.x + 31) >> 5), al, ok);
-    if (act && ok) {
-      float2 nr[12];
+      if (act) {
+        get_words<6>(xs + t, Vb, p);
 #pragma unroll
-      for (int q = 0; q < 12; ++q) {
-        zfma(e[q], al, rr[q]);
-        float2 ap = zzero<float2>();
-        zfma(ap, al, o[q]);
-        nr[q] = zsub(rr[q], ap);
-      }
-      store_spinor(rho, Vb, t, nr);
-    }
-    __syncthreads();
-  }
-  if (act) {
-    if (nrhs == 1) {  // one column: the site's 96 bytes as six 16-byte words
-      float4* x4 = reinterpret_cast<float4*>(x + s * 12);
+        for (int k = 0; k < 12; ++k) p[k] = zadd(p[k], e[k]);
+        if (BLOCKED) {
+          put_words<6>(reinterpret_cast<float4*>(x) + r * g.V * 6 + (long long)b * 6 * Vb + t, Vb, p);
+        } else {
+          const long long s = local_site(g, X, t);
 #pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        float4 f = x4[k];
-        f.x += e[2 * k].x;
-        f.y += e[2 * k].y;
-        f.z += e[2 * k + 1].x;
-        f.w += e[2 * k + 1].y;
-        x4[k] = f;
-      }
-    } else {
-#pragma unroll
-      for (int q = 0; q < 12; ++q) {
-        const long long idx = (s * 12 + q) * nrhs + r;
-        x[idx] = zadd(x[idx], e[q]);
+          for (int k = 0; k < 12; ++k) x[(s * 12 + k) * nrhs + r] = p[k];
+        }
       }
     }
   }
+}
+
+// Columns j0 .. j0 + N groups - 1 of v ([V][12][nrhs]) <-> w ([column][block][6 words][Vb], block order).
+// One CTA per kTileSites sites of a block and N columns, through shared memory: v is read and written
+// in runs (the B[0] sites of a row; N neighbouring columns), w in runs of consecutive sites.  Bound:
+// HBM; many small CTAs keep it busy (32^4, one column: 36 us a copy, 5.6 TB/s; a CTA per block with the
+// site index computed by divisions took 86 us).
+constexpr int kTileSites = 64;
+template <bool TO, int N>
+__global__ void __launch_bounds__(256) blocked_kernel(float2* __restrict__ v, float2* __restrict__ w, Geom g, int nrhs,
+                                                      int j0, int groups) {
+  constexpr int P = kTileSites + 1;
+  __shared__ float2 sc[N * 12 * P];  // [column][entry][site]
+  const int Vb = (int)g.Vb, chunks = (Vb + kTileSites - 1) / kTileSites;
+  const int grp = (int)(blockIdx.x % groups), q0 = (int)(blockIdx.x / groups), t0 = q0 % chunks * kTileSites;
+  const long long b = q0 / chunks, origin = block_origin(g, b);
+  const int ts = min(kTileSites, Vb - t0);
+  const int* soff = g.soff + t0;
+  float4* wb = reinterpret_cast<float4*>(w) + (long long)grp * N * g.V * 6 + b * 6 * Vb + t0;
+  auto caller = [&](auto&& body) {  // e = (site, entry, column), the column fastest
+#pragma unroll 6
+    for (int e = threadIdx.x; e < ts * 12 * N; e += 256) {
+      const int c = e % N, k = e / N % 12, t = e / (12 * N);
+      body(v + ((origin + __ldg(soff + t)) * 12 + k) * nrhs + j0 + grp * N + c, sc + (c * 12 + k) * P + t);
+    }
+  };
+  auto caller_words = [&](auto&& body) {  // one column: e = (site, word)
+#pragma unroll 2
+    for (int e = threadIdx.x; e < ts * 6; e += 256)
+      body(reinterpret_cast<float4*>(v) + (origin + __ldg(soff + e / 6)) * 6 + e % 6, sc + e % 6 * 2 * P + e / 6);
+  };
+  auto blocked = [&](auto&& body) {  // e = (column, word, site)
+#pragma unroll 2
+    for (int e = threadIdx.x; e < N * 6 * kTileSites; e += 256) {
+      const int t = e % kTileSites, q = e / kTileSites % 6, c = e / (6 * kTileSites);
+      if (t < ts) body(wb + (long long)c * g.V * 6 + q * Vb + t, sc + (c * 12 + 2 * q) * P + t);
+    }
+  };
+  auto word_in = [](const float4* a, float2* s) {
+    const float4 f = *a;
+    s[0] = lo2(f);
+    s[P] = hi2(f);
+  };
+  auto word_out = [](float4* a, const float2* s) { *a = make_float4(s[0].x, s[0].y, s[P].x, s[P].y); };
+  if (!TO) blocked(word_in);
+  else if (N == 1 && nrhs == 1) caller_words(word_in);
+  else caller([](const float2* a, float2* s) { *s = *a; });
+  __syncthreads();
+  if (TO) blocked(word_out);
+  else if (N == 1 && nrhs == 1) caller_words(word_out);
+  else caller([](float2* a, const float2* s) { *a = *s; });
 }
 
 // ------------------------------------------------------------------ outer FGMRES vector kernels
@@ -867,91 +1282,223 @@ FineGeom fine_geom(const amg_coarse* h) {
   }
   g.V = h->g.V;
   g.Vb = (int)h->g.Vb;
+  for (int mu = 0; mu < 3; ++mu) {
+    g.dL[mu] = fast_div(g.L[mu]);
+    g.dB[mu] = fast_div(g.B[mu]);
+    g.dLc[mu] = fast_div(g.Lc[mu]);
+  }
+  g.dVb = fast_div(g.Vb);
   return g;
 }
 
-// FP64 clover blocks [V][2][6][6] -> FP32 packed upper triangles [V][2][22] (tri_index order, the last
-// entry of each chirality zero)
-__global__ void clover_pack_kernel(const double2* __restrict__ in, float2* __restrict__ out, long long V) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < V * 44; e += (long long)gridDim.x * blockDim.x) {
-    const long long s = e / 44;
-    const int hh = (int)(e % 44) / 22, k = (int)(e % 22);
-    float2 v = make_float2(0.f, 0.f);
-    if (k < 21) {
-      int a = 0;
-      while (tri_index(a, 5) < k) ++a;  // row of entry k: the first row whose last entry is >= k
-      const int b = a + (k - tri_index(a, a));
-      const double2 d = in[(s * 2 + hh) * 36 + a * 6 + b];
-      v = make_float2((float)d.x, (float)d.y);
-    }
-    out[e] = v;
+// Links [V][36] and clover blocks [V][2][6][6] in FP64 -> the FP32 words in block order (see kLinkQ)
+__global__ void links_words_kernel(const double2* __restrict__ in, float4* __restrict__ out, Geom g) {
+  const long long n = g.V * kLinkQ;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
+    const long long b = e / (kLinkQ * g.Vb);
+    const int q = (int)(e / g.Vb % kLinkQ);
+    const double2* U = in + block_site_fast(g, block_origin(g, b), (int)(e % g.Vb)) * 36 + 2 * q;
+    out[e] = make_float4((float)U[0].x, (float)U[0].y, (float)U[1].x, (float)U[1].y);
   }
 }
-
-template <typename T>
-__global__ void to_prec_kernel(const double2* __restrict__ in, typename Cx<T>::type* __restrict__ out, long long n) {
+__global__ void clover_words_kernel(const double2* __restrict__ in, float4* __restrict__ out, Geom g) {
+  const long long n = g.V * kClovQ;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    typename Cx<T>::type v;
-    v.x = (T)in[e].x;
-    v.y = (T)in[e].y;
-    out[e] = v;
+    const long long b = e / (kClovQ * g.Vb);
+    const int q = (int)(e / g.Vb % kClovQ), hh = q / 7;
+    const double2* C = in + (block_site_fast(g, block_origin(g, b), (int)(e % g.Vb)) * 2 + hh) * 36;
+    float2 v[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int w = 2 * (q % 7) + k;  // complex word of the chirality
+      if (w < 2) {
+        v[k].x = 2.f * (float)C[w * 2 * 7].x;                      // H00, H22
+        v[k].y = w == 0 ? 2.f * (float)C[7].x : 0.f;               // H11
+      } else {
+        const int a = w < 5 ? (w == 4 ? 1 : 0) : (w - 5) / 3;
+        const int c = w < 5 ? (w == 2 ? 1 : 2) : 3 + (w - 5) % 3;
+        v[k] = make_float2(2.f * (float)C[a * 6 + c].x, 2.f * (float)C[a * 6 + c].y);
+      }
+    }
+    out[e] = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
   }
 }
 
 bool fine_fp64(const amg_coarse* h) { return h->p.vec_prec == AMG_FP64; }
 
-template <typename T>
-amg_status launch_dirac(amg_coarse* h, const void* psi, const void* y, void* out, int nrhs, cudaStream_t st) {
-  using C = typename Cx<T>::type;
+template <int NC>
+auto* pick_dirac32(bool sub, bool fast) {
+  return sub ? (fast ? dirac32_kernel<true, true, NC> : dirac32_kernel<true, false, NC>)
+             : (fast ? dirac32_kernel<false, true, NC> : dirac32_kernel<false, false, NC>);
+}
+
+amg_status dirac_any(amg_coarse* h, const void* psi, const void* y, void* out, int nrhs, cudaStream_t st) {
   const long long total = h->g.V * nrhs;
   const long long want = (total + 127) / 128;
   const int grid = (int)(want < 16LL * amg_sm_count() ? want : 16LL * amg_sm_count());
-  const T mass = (T)(4.0 + h->p.m0);
-  if (y)
-    dirac_kernel<T, true><<<grid, 128, 0, st>>>((const C*)h->fU, (const C*)h->fC, (const C*)psi, (const C*)y, (C*)out,
-                                                 fine_geom(h), mass, nrhs);
-  else
-    dirac_kernel<T, false><<<grid, 128, 0, st>>>((const C*)h->fU, (const C*)h->fC, (const C*)psi, nullptr, (C*)out,
-                                                  fine_geom(h), mass, nrhs);
+  const FineGeom g = fine_geom(h);
+  if (fine_fp64(h)) {
+    const double mass = 4.0 + h->p.m0;
+    auto* U = (const double2*)h->fU;
+    auto* C = (const double2*)h->fC;
+    if (y)
+      dirac_kernel<true><<<grid, 128, 0, st>>>(U, C, (const double2*)psi, (const double2*)y, (double2*)out, g, mass, nrhs);
+    else
+      dirac_kernel<false><<<grid, 128, 0, st>>>(U, C, (const double2*)psi, nullptr, (double2*)out, g, mass, nrhs);
+  } else {
+    const float mass2 = 2.f * (float)(4.0 + h->p.m0);
+    auto* U = (const float4*)h->fU;
+    auto* C = (const float4*)h->fC;
+    const float2 *p = (const float2*)psi, *yy = (const float2*)y;
+    const int nb = g.Vb <= kDiracSites ? kDiracSites / g.Vb : 0, nblocks = (int)h->g.Vc;
+    const int ctas = nb ? (nblocks + nb - 1) / nb : 0;
+    // fewer tiles than SMs: one thread per site in lattice order spreads over more of them
+    if (nrhs == 1 && ctas >= amg_sm_count()) {
+      const int threads = (nb * g.Vb + 31) / 32 * 32;
+      auto* k = y ? dirac32_block_kernel<true> : dirac32_block_kernel<false>;
+      k<<<ctas, threads, 0, st>>>(U, C, p, yy, (float2*)out, g, mass2, nb, nblocks);
+    } else {
+      const int nc = nrhs % 2 ? 1 : 2, groups = nrhs / nc;
+      const FastDiv dn = fast_div(groups);
+      const long long threads = h->g.V * groups;
+      auto* k = nc == 1 ? pick_dirac32<1>(y != nullptr, threads < (1LL << 31)) : pick_dirac32<2>(y != nullptr, threads < (1LL << 31));
+      k<<<(unsigned)std::min((threads + 127) / 128, 16LL * amg_sm_count()), 128, 0, st>>>(U, C, p, yy, (float2*)out, g, mass2, dn);
+    }
+  }
   AMG_LAUNCH_CHECK();
   h->launches++;
   return AMG_OK;
 }
 
-amg_status dirac_any(amg_coarse* h, const void* psi, const void* y, void* out, int nrhs, cudaStream_t st) {
-  return fine_fp64(h) ? launch_dirac<double>(h, psi, y, out, nrhs, st) : launch_dirac<float>(h, psi, y, out, nrhs, st);
+// CTAs of the FP32 half sweep resident at once: the register file holds 256 of its threads
+int sap_slots(int threads, size_t smem) {
+  return amg_sm_count() * std::max(1, std::min(256 / threads, (int)(227 * 1024 / smem)));
 }
 
-template <typename T>
-amg_status launch_sap(amg_coarse* h, const void* y, void* x, int nrhs, int n_cycles, int n_mr, cudaStream_t st) {
-  using C = typename Cx<T>::type;
-  const int threads = (h->g.Vb + 31) / 32 * 32;
-  if (sizeof(T) == 4) {
-    // links, clover and rho of a block, then two buffers of the MR coefficient's warp sums
-    const size_t sm2 = (size_t)h->g.Vb * (18 + 22 + 6) * sizeof(float4) + (size_t)(threads / 32) * 2 * 3 * sizeof(float);
-    if (threads <= 256 && sm2 <= 227 * 1024) {
-      AMG_CUDA_TRY(cudaFuncSetAttribute(sap_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2));
-      const dim3 grid((unsigned)(h->g.Vc / 2), (unsigned)nrhs);
-      const float mass = (float)(4.0 + h->p.m0);
-      for (int c = 0; c < n_cycles; ++c)
-        for (int colour = 0; colour < 2; ++colour) {
-          sap_smem_kernel<<<grid, threads, sm2, st>>>((const float2*)h->fU, (const float2*)h->fC, (const float2*)y,
-                                                      (float2*)x, fine_geom(h), mass, nrhs, colour, n_mr);
-          AMG_LAUNCH_CHECK();
-          h->launches++;
-        }
-      return AMG_OK;
+// Columns per item of the FP32 half sweep: an item loads its block's links and clover once and sweeps a
+// group of columns with them (about a quarter of a column's time), so larger groups repeat fewer
+// loads and smaller ones fill the last wave; the group with the least waves x (load + columns).
+int sap_columns(long long nblk, int nrhs, int slots) {
+  int best = 1;
+  double best_cost = 0;
+  for (int c = 1; c <= nrhs; ++c) {
+    const long long ctas = nblk * ((nrhs + c - 1) / c);
+    const double cost = (double)((ctas + slots - 1) / slots) * (0.25 + c);
+    if (c == 1 || cost < best_cost) {
+      best = c;
+      best_cost = cost;
     }
   }
-  const size_t smem = (size_t)h->g.Vb * 12 * sizeof(C) + (size_t)(threads / 32 + 1) * 3 * sizeof(double);
+  return best;
+}
+
+template <bool BLOCKED>
+amg_status sweep32(amg_coarse* h, const float2* y, float2* x, int nrhs, int n_cycles, int n_mr, cudaStream_t st) {
+  const FineGeom g = fine_geom(h);
+  const int threads = (g.Vb + 31) / 32 * 32;
+  const size_t smem = sap_smem(g);
   if (threads > 256 || smem > 227 * 1024) return AMG_ERR_UNSUPPORTED;
-  AMG_CUDA_TRY(cudaFuncSetAttribute(sap_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const dim3 grid((unsigned)(h->g.Vc / 2), (unsigned)nrhs);
-  const T mass = (T)(4.0 + h->p.m0);
+  AMG_CUDA_TRY(cudaFuncSetAttribute(sap_reg_kernel<BLOCKED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const long long nblk = h->g.Vc / 2;
+  const int slots = sap_slots(threads, smem);
+  const int nr = sap_columns(nblk, nrhs, slots), groups = (nrhs + nr - 1) / nr;
+  const int items = (int)(nblk * groups);
+  const float mass2 = 2.f * (float)(4.0 + h->p.m0);
   for (int c = 0; c < n_cycles; ++c)
     for (int colour = 0; colour < 2; ++colour) {
-      sap_kernel<T><<<grid, threads, smem, st>>>((const C*)h->fU, (const C*)h->fC, (const C*)y, (C*)x, fine_geom(h),
-                                                 mass, nrhs, colour, n_mr);
+      sap_reg_kernel<BLOCKED><<<std::min(items, slots), threads, smem, st>>>((const float4*)h->fU, (const float4*)h->fC, y, x,
+                                                                            g, mass2, nrhs, nr, groups, items, colour, n_mr,
+                                                                            h->err);
+      AMG_LAUNCH_CHECK();
+      h->launches++;
+    }
+  return AMG_OK;
+}
+
+// The sweeps run on copies of x and y in block order, one vector per column; x is copied back.  The
+// copies come from the handle's pool, at most kColBytes at a time (columns are independent).  While
+// the stream is captured, or without memory for them, the sweeps work on the caller's vectors.
+constexpr size_t kColBytes = (size_t)2 << 30;
+int sap_copy_columns(const amg_coarse* h, int nrhs) {
+  return (int)std::max<size_t>(1, std::min<size_t>(nrhs, kColBytes / (2 * h->g.V * 12 * sizeof(float2))));
+}
+size_t sap_copy_bytes(const amg_coarse* h, int nrhs) {
+  return 2 * (size_t)h->g.V * 12 * sizeof(float2) * sap_copy_columns(h, nrhs);
+}
+
+// Columns j0 .. j0 + nc - 1 of v to (TO) or from w; four columns per CTA (a 32-byte sector), the rest
+// in a launch of their own
+template <bool TO>
+amg_status blocked_copy(amg_coarse* h, const float2* v, const float2* w, int nrhs, int j0, int nc, cudaStream_t st) {
+  float2 *vv = const_cast<float2*>(v), *ww = const_cast<float2*>(w);
+  const unsigned tiles = (unsigned)(h->g.Vc * ((h->g.Vb + kTileSites - 1) / kTileSites));
+  const int groups = nc / 4, rest = nc % 4;
+  if (groups) blocked_kernel<TO, 4><<<tiles * groups, 256, 0, st>>>(vv, ww, h->g, nrhs, j0, groups);
+  j0 += 4 * groups;
+  ww += (size_t)4 * groups * h->g.V * 12;
+  if (rest == 1) blocked_kernel<TO, 1><<<tiles, 256, 0, st>>>(vv, ww, h->g, nrhs, j0, 1);
+  else if (rest == 2) blocked_kernel<TO, 2><<<tiles, 256, 0, st>>>(vv, ww, h->g, nrhs, j0, 1);
+  else if (rest == 3) blocked_kernel<TO, 3><<<tiles, 256, 0, st>>>(vv, ww, h->g, nrhs, j0, 1);
+  h->launches += (groups > 0) + (rest > 0);
+  AMG_LAUNCH_CHECK();
+  return AMG_OK;
+}
+
+// The pool, with the copies of max_nrhs columns allocated once here rather than in the first sweep; kept
+// until the handle goes.  Without it (a device without pools) the sweeps do without copies.
+void sap_pool(amg_coarse* h, cudaStream_t st) {
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  uint64_t keep = kColBytes;
+  void* w = nullptr;
+  if (cudaGetDevice(&props.location.id) != cudaSuccess || cudaMemPoolCreate(&h->fpool, &props) != cudaSuccess) {
+    h->fpool = nullptr;
+  } else if (cudaMemPoolSetAttribute(h->fpool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess &&
+             cudaMallocFromPoolAsync(&w, sap_copy_bytes(h, h->p.max_nrhs), h->fpool, st) == cudaSuccess) {
+    cudaFreeAsync(w, st);
+  }
+  cudaGetLastError();
+}
+
+amg_status launch_sap32(amg_coarse* h, const void* yv, void* xv, int nrhs, int n_cycles, int n_mr, cudaStream_t st) {
+  const float2* y = (const float2*)yv;
+  float2* x = (float2*)xv;
+  const size_t n = (size_t)h->g.V * 12;
+  if (n_cycles < 1) return AMG_OK;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  AMG_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
+  const int chunk = sap_copy_columns(h, nrhs);
+  float2* w = nullptr;
+  if (h->fpool && cap == cudaStreamCaptureStatusNone &&
+      cudaMallocFromPoolAsync((void**)&w, sap_copy_bytes(h, nrhs), h->fpool, st) != cudaSuccess) {
+    cudaGetLastError();
+    w = nullptr;
+  }
+  if (!w) return sweep32<false>(h, y, x, nrhs, n_cycles, n_mr, st);
+  float2* wx = w + n * chunk;
+  amg_status s = AMG_OK;
+  for (int j0 = 0; j0 < nrhs && s == AMG_OK; j0 += chunk) {
+    const int nc = std::min(chunk, nrhs - j0);
+    s = blocked_copy<true>(h, y, w, nrhs, j0, nc, st);
+    if (s == AMG_OK) s = blocked_copy<true>(h, x, wx, nrhs, j0, nc, st);
+    if (s == AMG_OK) s = sweep32<true>(h, w, wx, nc, n_cycles, n_mr, st);
+    if (s == AMG_OK) s = blocked_copy<false>(h, x, wx, nrhs, j0, nc, st);
+  }
+  cudaFreeAsync(w, st);
+  return s;
+}
+
+amg_status launch_sap64(amg_coarse* h, const void* y, void* x, int nrhs, int n_cycles, int n_mr, cudaStream_t st) {
+  const int threads = (h->g.Vb + 31) / 32 * 32;
+  const size_t smem = (size_t)h->g.Vb * 12 * sizeof(double2) + (size_t)(threads / 32 + 1) * 3 * sizeof(double);
+  if (threads > 256 || smem > 227 * 1024) return AMG_ERR_UNSUPPORTED;
+  AMG_CUDA_TRY(cudaFuncSetAttribute(sap_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const dim3 grid((unsigned)(h->g.Vc / 2), (unsigned)nrhs);
+  for (int c = 0; c < n_cycles; ++c)
+    for (int colour = 0; colour < 2; ++colour) {
+      sap_kernel<<<grid, threads, smem, st>>>((const double2*)h->fU, (const double2*)h->fC, (const double2*)y,
+                                              (double2*)x, fine_geom(h), 4.0 + h->p.m0, nrhs, colour, n_mr);
       AMG_LAUNCH_CHECK();
       h->launches++;
     }
@@ -959,8 +1506,7 @@ amg_status launch_sap(amg_coarse* h, const void* y, void* x, int nrhs, int n_cyc
 }
 
 amg_status sap_any(amg_coarse* h, const void* y, void* x, int nrhs, int n_cycles, int n_mr, cudaStream_t st) {
-  return fine_fp64(h) ? launch_sap<double>(h, y, x, nrhs, n_cycles, n_mr, st)
-                      : launch_sap<float>(h, y, x, nrhs, n_cycles, n_mr, st);
+  return fine_fp64(h) ? launch_sap64(h, y, x, nrhs, n_cycles, n_mr, st) : launch_sap32(h, y, x, nrhs, n_cycles, n_mr, st);
 }
 
 amg_status check_fine(amg_coarse* h, const void* a, const void* b, int nrhs) {
@@ -1266,6 +1812,8 @@ void amg_internal_free_fine(amg_coarse* h) {
   cudaFree(h->fU);
   if (h->fC != (void*)h->clover) cudaFree(h->fC);
   cudaFree(h->fwork);
+  if (h->fpool) cudaMemPoolDestroy(h->fpool);
+  h->fpool = nullptr;
   h->fU = h->fC = h->fwork = nullptr;
   h->fwork_bytes = 0;
 }
@@ -1285,11 +1833,16 @@ amg_status amg_setup_fine(amg_handle h, const void* d_U, void* stream) {
     AMG_CUDA_TRY(cudaMemcpyAsync(h->fU, d_U, nU * sizeof(double2), cudaMemcpyDeviceToDevice, st));
     h->fC = h->clover;
   } else {
-    AMG_CUDA_TRY(cudaMalloc(&h->fU, nU * sizeof(float2)));
-    AMG_CUDA_TRY(cudaMalloc(&h->fC, h->g.V * kClPacked * sizeof(float2)));
-    to_prec_kernel<float><<<4 * amg_sm_count(), 256, 0, st>>>((const double2*)d_U, (float2*)h->fU, nU);
+    AMG_CUDA_TRY(cudaMalloc(&h->fU, h->g.V * kLinkQ * sizeof(float4)));
+    if (cudaMalloc(&h->fC, h->g.V * kClovQ * sizeof(float4)) != cudaSuccess) {
+      cudaGetLastError();
+      amg_internal_free_fine(h);
+      return AMG_ERR_OOM;
+    }
+    sap_pool(h, st);
+    links_words_kernel<<<8 * amg_sm_count(), 256, 0, st>>>((const double2*)d_U, (float4*)h->fU, h->g);
     AMG_LAUNCH_CHECK();
-    clover_pack_kernel<<<4 * amg_sm_count(), 256, 0, st>>>(h->clover, (float2*)h->fC, h->g.V);
+    clover_words_kernel<<<8 * amg_sm_count(), 256, 0, st>>>(h->clover, (float4*)h->fC, h->g);
     AMG_LAUNCH_CHECK();
     h->launches += 2;
   }
