@@ -864,6 +864,104 @@ __global__ void __launch_bounds__(256) restrict_kernel(const ST* __restrict__ R,
   }
 }
 
+// Several columns in FP32 (restriction and prolongation): a thread works on pairs of consecutive dofs
+// 2q, 2q + 1 of an aggregate, whose NR columns are NR 16-byte pieces (piece p: values 2p, 2p + 1 of
+// [dof][column]).  In shared memory the pieces of pair q are stored with their index xor'ed by swz(q),
+// so that the same piece of eight consecutive pairs lies in eight different bank groups for every NR.
+template <int NR>
+__device__ __forceinline__ int swz(int q) {
+  constexpr int g = NR % 8 == 0 ? 8 : (NR % 4 == 0 ? 4 : (NR % 2 == 0 ? 2 : 1));
+  return (q / (8 / g)) & (g - 1);
+}
+// An even split of n columns into chunks of at most `most` (the last may be short)
+struct ColumnChunks {
+  int size, count;
+};
+inline ColumnChunks column_chunks(int n, int most) {
+  const int count = (n + most - 1) / most, size = (n + count - 1) / count;
+  return {size, (n + size - 1) / size};
+}
+
+// Restriction: NR (2 .. 4) columns and TM rows per warp.  With one row per warp every value of y came from
+// shared memory once per row (and 4 columns were 64 bytes apart from lane to lane, so that eight lanes
+// met in two banks); TM rows share it.
+//
+// One CTA per (block, chunk of NR columns), the chunks of a block next to each other: they read the
+// same rows at about the same time, so R leaves HBM once and the other chunks find it in L2.  A short
+// last chunk repeats its last column and drops the copies.
+//
+// Bounds: HBM (R once, y once) and, from 8 columns on, nearly the FP32 pipes.  24^3 x 48, Ntv 20,
+// 8 columns: 400 us; one launch per 4 columns with a row per warp took 2 x 831 us.
+template <int NR, int TM>
+__global__ void __launch_bounds__(256, 2) restrict_cols_kernel(const float2* __restrict__ R, const float2* __restrict__ y,
+                                                               float2* __restrict__ yc, Geom g, int ld, int chunks) {
+  extern __shared__ float4 ysm[];  // [h][pair][NR] pieces
+  const int nagg = g.nagg, ntv = g.ntv, npair = nagg / 2, Vb = (int)g.Vb;
+  const long long blk = blockIdx.x / chunks;
+  const int r0 = (int)(blockIdx.x % chunks) * NR;
+  const long long origin = block_origin(g, blk);
+  if (NR % 2 == 0 && ld % 2 == 0) {  // 16-byte copies; r0 and ld even, a short chunk ends at an even column
+    for (int e = threadIdx.x; e < Vb * 6 * NR; e += 256) {
+      const int c = e % (NR / 2), dof = e / (NR / 2) % 12, sl = e / (6 * NR);
+      const int hh = dof / 6, n = sl * 6 + dof % 6, q = n >> 1, p = (n & 1) * (NR / 2) + c;
+      cp_async_elem(reinterpret_cast<double2*>(ysm + ((size_t)hh * npair + q) * NR + (p ^ swz<NR>(q))),
+                    reinterpret_cast<const double2*>(y + (block_site_fast(g, origin, sl) * 12 + dof) * ld +
+                                                     min(r0 + 2 * c, ld - 2)));
+    }
+  } else {
+    float2* ys = reinterpret_cast<float2*>(ysm);
+    for (int e = threadIdx.x; e < Vb * 12 * NR; e += 256) {
+      const int r = e % NR, dof = e / NR % 12, sl = e / (12 * NR);
+      const int hh = dof / 6, n = sl * 6 + dof % 6, q = n >> 1, v = (n & 1) * NR + r;
+      cp_async_elem(ys + (((size_t)hh * npair + q) * NR + ((v >> 1) ^ swz<NR>(q))) * 2 + (v & 1),
+                    y + (block_site_fast(g, origin, sl) * 12 + dof) * ld + min(r0 + r, ld - 1));
+    }
+  }
+  cp_async_commit();
+  cp_async_wait_all();
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, hh = warp & 1;
+  const float4* yh = ysm + (size_t)hh * npair * NR;
+  for (int j0 = (warp >> 1) * TM; j0 < ntv; j0 += 4 * TM) {
+    const float4* Rj[TM];  // rows past the last are read again and dropped
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+      Rj[i] = reinterpret_cast<const float4*>(R + ((blk * 2 + hh) * ntv + min(j0 + i, ntv - 1)) * (long long)nagg);
+    float2 acc[TM][NR];
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int r = 0; r < NR; ++r) acc[i][r] = make_float2(0.f, 0.f);
+#pragma unroll 2
+    for (int q = lane; q < npair; q += 32) {
+      float4 v[TM];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) v[i] = __ldcg(Rj[i] + q);
+      float2 yv[2 * NR];
+#pragma unroll
+      for (int p = 0; p < NR; ++p) {
+        const float4 f = yh[(size_t)q * NR + (p ^ swz<NR>(q))];
+        yv[2 * p] = make_float2(f.x, f.y);
+        yv[2 * p + 1] = make_float2(f.z, f.w);
+      }
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          cfma(acc[i][r], make_float2(v[i].x, v[i].y), yv[r]);
+          cfma(acc[i][r], make_float2(v[i].z, v[i].w), yv[NR + r]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const float2 sum = warp_csum(acc[i][r]);
+        if (lane == 0 && j0 + i < ntv && r0 + r < ld) yc[((blk * 2 + hh) * ntv + j0 + i) * ld + r0 + r] = sum;
+      }
+  }
+}
+
 // ------------------------------------------------------------------ prolongation
 // Item = block; chunk = (h, n0): rows j = 0..ntv-1 of R_i^h restricted to n0 .. n0+nch-1, one bulk
 // copy per row into stage [j][nch].  Consumer warp w owns stage w; lane l computes
@@ -1121,22 +1219,51 @@ amg_status launch_restrict(amg_coarse* h, const ST* R, const ST* y, ST* yc, int 
   return AMG_OK;
 }
 
+template <int NR, int TM>
+amg_status launch_restrict_cols(amg_coarse* h, const float2* R, const float2* y, float2* yc, int ld, int chunks,
+                                cudaStream_t st) {
+  const size_t smem = (size_t)h->g.nagg * NR * sizeof(float4);
+  AMG_CUDA_TRY(cudaFuncSetAttribute(restrict_cols_kernel<NR, TM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  restrict_cols_kernel<NR, TM><<<(unsigned)(h->g.Vc * chunks), 256, smem, st>>>(R, y, yc, h->g, ld, chunks);
+  AMG_LAUNCH_CHECK();
+  h->launches++;
+  return AMG_OK;
+}
+// rows per warp: the rows of a chirality over four warps in as few passes of at most 6 as they need
+template <int NR>
+amg_status launch_restrict_rows(amg_coarse* h, const float2* R, const float2* y, float2* yc, int ld, int chunks,
+                                cudaStream_t st) {
+  const int per = (h->g.ntv + 3) / 4, passes = (per + 5) / 6;
+  switch ((per + passes - 1) / passes) {
+    case 1: return launch_restrict_cols<NR, 1>(h, R, y, yc, ld, chunks, st);
+    case 2: return launch_restrict_cols<NR, 2>(h, R, y, yc, ld, chunks, st);
+    case 3: return launch_restrict_cols<NR, 3>(h, R, y, yc, ld, chunks, st);
+    case 4: return launch_restrict_cols<NR, 4>(h, R, y, yc, ld, chunks, st);
+    case 5: return launch_restrict_cols<NR, 5>(h, R, y, yc, ld, chunks, st);
+    default: return launch_restrict_cols<NR, 6>(h, R, y, yc, ld, chunks, st);
+  }
+}
+
 // Largest nch dividing 6 Vb, a multiple of 6 (whole sites), with ntv * nch * sizeof(ST) <= 24 KB.
-// Prolongation for FP32 R (one pass for nrhs <= 4 columns): one CTA per block, like the
-// restriction.  R is stored row-major per test vector ([block][2 Ntv rows][nagg dofs]), so the
-// output dofs read R by column: a thread owns two consecutive dofs n, n + 1 of one chirality half
-// (the same site: a site has 6 dofs per half) and reads their 16 bytes of every row j < Ntv, a warp
-// covering 512 contiguous bytes per row; x_c of the block sits in shared memory.  The rows are
-// read with the streaming hint (read once) and x is written with one 16-byte streaming store per
-// pair (1 RHS).  Measured 93 % of the copy bandwidth against 90 % for the bulk-copy ring form
-// (prolong_tma_kernel, kept for FP64), whose single-dof lanes stored 8 bytes each.
+// Prolongation for FP32 R: one CTA per block and chunk of NR <= 4 columns, like the restriction (the
+// chunks of a block next to each other, a short last one repeats its last column and drops the
+// copies).  R is stored row-major per test vector ([block][2 Ntv rows][nagg dofs]), so the output dofs
+// read R by column: a thread owns two consecutive dofs n, n + 1 of one chirality half (the same site: a
+// site has 6 dofs per half) and reads their 16 bytes of every row j < Ntv, a warp covering 512
+// contiguous bytes per row; x_c of the block sits in shared memory.  One column reads the rows with the
+// streaming hint (read once) and writes x with one 16-byte streaming store per pair: 93 % of the copy
+// bandwidth against 90 % for the bulk-copy ring form (prolong_tma_kernel, kept for FP64), whose
+// single-dof lanes stored 8 bytes each.  24^3 x 48, Ntv 20, 8 columns: 368 us against 2 x 311 us for
+// one launch per 4 columns; chunks of 8 with the results leaving through shared memory took 379 us.
 template <int NR>
 __global__ void __launch_bounds__(256) prolong_pair_kernel(const float2* __restrict__ R, const float2* __restrict__ xc,
-                                                           float2* __restrict__ x, Geom g, int ld, int r0) {
+                                                           float2* __restrict__ x, Geom g, int ld, int chunks) {
   __shared__ float2 xs[2 * AMG_MAX_NTV * NR];
-  const long long blk = blockIdx.x;
+  const long long blk = NR == 1 ? blockIdx.x : blockIdx.x / chunks;
+  const int r0 = NR == 1 ? 0 : (int)(blockIdx.x % chunks) * NR;
   const int nagg = g.nagg, ntv = g.ntv, npair = nagg / 2;
-  for (int e = threadIdx.x; e < 2 * ntv * NR; e += blockDim.x) xs[e] = xc[(blk * 2 * ntv + e / NR) * ld + r0 + e % NR];
+  for (int e = threadIdx.x; e < 2 * ntv * NR; e += blockDim.x)
+    xs[e] = xc[(blk * 2 * ntv + e / NR) * ld + min(r0 + e % NR, ld - 1)];
   __syncthreads();
   const long long origin = block_origin(g, blk);
   for (int p = threadIdx.x; p < 2 * npair; p += blockDim.x) {
@@ -1148,7 +1275,8 @@ __global__ void __launch_bounds__(256) prolong_pair_kernel(const float2* __restr
     for (int r = 0; r < NR; ++r) a0[r] = a1[r] = make_float2(0.f, 0.f);
 #pragma unroll 5
     for (int j = 0; j < ntv; ++j) {
-      const float4 v = __ldcs(reinterpret_cast<const float4*>(Rp + (size_t)j * nagg));
+      const float4* row = reinterpret_cast<const float4*>(Rp + (size_t)j * nagg);
+      const float4 v = NR == 1 ? __ldcs(row) : __ldcg(row);
       const float2 v0 = make_float2(v.x, v.y), v1 = make_float2(v.z, v.w);
 #pragma unroll
       for (int r = 0; r < NR; ++r) {
@@ -1160,12 +1288,20 @@ __global__ void __launch_bounds__(256) prolong_pair_kernel(const float2* __restr
     float2* xo = x + (block_site_fast(g, origin, sl) * 12 + dof) * ld + r0;
     if (NR == 1 && ld == 1) {
       __stcs(reinterpret_cast<float4*>(xo), make_float4(a0[0].x, a0[0].y, a1[0].x, a1[0].y));
+    } else if (NR % 2 == 0 && ld % 2 == 0) {  // r0 and ld even: two columns per store
+#pragma unroll
+      for (int r = 0; r + 1 < NR; r += 2)
+        if (r0 + r < ld) {
+          __stcs(reinterpret_cast<float4*>(xo + r), make_float4(a0[r].x, a0[r].y, a0[r + 1].x, a0[r + 1].y));
+          __stcs(reinterpret_cast<float4*>(xo + ld + r), make_float4(a1[r].x, a1[r].y, a1[r + 1].x, a1[r + 1].y));
+        }
     } else {
 #pragma unroll
-      for (int r = 0; r < NR; ++r) {
-        xo[r] = a0[r];
-        xo[ld + r] = a1[r];
-      }
+      for (int r = 0; r < NR; ++r)
+        if (r0 + r < ld) {
+          xo[r] = a0[r];
+          xo[ld + r] = a1[r];
+        }
     }
   }
 }
@@ -1180,9 +1316,9 @@ int prolong_chunk(const Geom& g) {
 }
 
 template <int NR>
-amg_status launch_prolong_pair(amg_coarse* h, const float2* R, const float2* xc, float2* x, int ld, int r0,
+amg_status launch_prolong_pair(amg_coarse* h, const float2* R, const float2* xc, float2* x, int ld, int chunks,
                                cudaStream_t st) {
-  prolong_pair_kernel<NR><<<(unsigned)h->g.Vc, 256, 0, st>>>(R, xc, x, h->g, ld, r0);
+  prolong_pair_kernel<NR><<<(unsigned)(h->g.Vc * chunks), 256, 0, st>>>(R, xc, x, h->g, ld, chunks);
   AMG_LAUNCH_CHECK();
   h->launches++;
   return AMG_OK;
@@ -1252,12 +1388,22 @@ amg_status amg_internal_restrict(amg_coarse* h, const void* y, void* yc, int nrh
     });
   }
   if (h->p.vec_prec == AMG_FP32 && h->p.r_prec == AMG_FP32) {
-    const float2* R = (const float2*)h->Rq;
-    return for_rhs_chunks(nrhs, [&](int r0, int nr) {
-      if (nr == 4) return launch_restrict<float2, 4>(h, R, (const float2*)y, (float2*)yc, nrhs, r0, s);
-      if (nr == 2) return launch_restrict<float2, 2>(h, R, (const float2*)y, (float2*)yc, nrhs, r0, s);
-      return launch_restrict<float2, 1>(h, R, (const float2*)y, (float2*)yc, nrhs, r0, s);
-    });
+    const float2 *R = (const float2*)h->Rq, *yf = (const float2*)y;
+    float2* out = (float2*)yc;
+    if (nrhs == 1) return launch_restrict<float2, 1>(h, R, yf, out, 1, 0, s);
+    // Blocks of fewer than 32 sites (two columns: 64): a warp's lanes run over a row's dof pairs once or a
+    // few times, and many small CTAs with a row per warp hide more (16^4 in 2^4 blocks, Ntv 11, 8 columns:
+    // 111 us against 132; in 2^3 4 blocks, Ntv 16: 29 against 31 with 2 columns, 131 against 70 with 8)
+    if (h->g.Vb < (nrhs == 2 ? 64 : 32))
+      return for_rhs_chunks(nrhs, [&](int r0, int nr) {
+        if (nr == 4) return launch_restrict<float2, 4>(h, R, yf, out, nrhs, r0, s);
+        if (nr == 2) return launch_restrict<float2, 2>(h, R, yf, out, nrhs, r0, s);
+        return launch_restrict<float2, 1>(h, R, yf, out, nrhs, r0, s);
+      });
+    const ColumnChunks c = column_chunks(nrhs, 4);
+    if (c.size == 4) return launch_restrict_rows<4>(h, R, yf, out, nrhs, c.count, s);
+    if (c.size == 3) return launch_restrict_rows<3>(h, R, yf, out, nrhs, c.count, s);
+    return launch_restrict_rows<2>(h, R, yf, out, nrhs, c.count, s);
   }
   return AMG_ERR_UNSUPPORTED;
 }
@@ -1273,12 +1419,15 @@ amg_status amg_internal_prolong(amg_coarse* h, const void* xc, void* x, int nrhs
     });
   }
   if (h->p.vec_prec == AMG_FP32 && h->p.r_prec == AMG_FP32) {
-    const float2* R = (const float2*)h->Rq;
-    return for_rhs_chunks(nrhs, [&](int r0, int nr) {
-      if (nr == 4) return launch_prolong_pair<4>(h, R, (const float2*)xc, (float2*)x, nrhs, r0, s);
-      if (nr == 2) return launch_prolong_pair<2>(h, R, (const float2*)xc, (float2*)x, nrhs, r0, s);
-      return launch_prolong_pair<1>(h, R, (const float2*)xc, (float2*)x, nrhs, r0, s);
-    });
+    const float2 *R = (const float2*)h->Rq, *xf = (const float2*)xc;
+    float2* out = (float2*)x;
+    const ColumnChunks c = column_chunks(nrhs, 4);
+    switch (c.size) {
+      case 1: return launch_prolong_pair<1>(h, R, xf, out, nrhs, c.count, s);
+      case 2: return launch_prolong_pair<2>(h, R, xf, out, nrhs, c.count, s);
+      case 3: return launch_prolong_pair<3>(h, R, xf, out, nrhs, c.count, s);
+      default: return launch_prolong_pair<4>(h, R, xf, out, nrhs, c.count, s);
+    }
   }
   return AMG_ERR_UNSUPPORTED;
 }
