@@ -211,6 +211,14 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
 }
 
+// load_link from shared memory
+template <int mu>
+__device__ __forceinline__ void shared_link(const float4* U, int stride, float2 u[9]) {
+  constexpr int e0 = 9 * mu, o = e0 & 1, p0 = e0 >> 1;
+  u[o ? 0 : 8] = reinterpret_cast<const float2*>(U + (o ? p0 : p0 + 4) * stride)[o];
+  get_words<4>(U + (p0 + o) * stride, stride, u + o);
+}
+
 // h = (1 -+ g_mu) p on the upper half: u - A d (FWD), u + A d; h[3 s + colour]
 template <bool FWD, int mu>
 __device__ __forceinline__ void half_spinor(const float2 p[12], float2 h[6]) {
@@ -653,6 +661,16 @@ __device__ __forceinline__ void cta_alpha_all(float v[3], float* red, float2& al
   al.y = ok ? si / sp : 0.f;
 }
 
+// The same for `lanes` lanes of a warp (a power of two) that hold a whole block
+__device__ __forceinline__ void lanes_alpha(float v[3], int lanes, float2& al, bool& ok) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    for (int o = lanes / 2; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+  ok = v[0] > 0;
+  al.x = ok ? v[1] / v[0] : 0.f;
+  al.y = ok ? v[2] / v[0] : 0.f;
+}
+
 // Intra-block hops of the block operator B at local site t: neighbours' rho from shared memory
 // (component-major: rho[q * Vb + t]), links from global memory; FP64.
 template <int mu>
@@ -770,34 +788,45 @@ __global__ void __launch_bounds__(256) sap_kernel(const double2* __restrict__ U,
   }
 }
 
-// The same half sweep in FP32.  A thread holds its site's four links and its clover (128 registers)
-// while it sweeps a group of nr right-hand sides.  A backward hop needs the link of the neighbour it
-// comes from, which another thread holds: that thread multiplies, U_mu^dag (1 + g_mu) rho with its
-// own link and rho, and hands the half spinor over in shared memory (48 bytes; the link and the
-// spinor would be 168).  The hops that cross the block face appear in the residual only: a list of
-// face sites, spread over all threads, fetches the outside neighbours; forward ones leave their half
-// spinors in halo, backward ones the finished product in the hand-over buffer.
+// The same half sweep in FP32: a CTA takes a block of the colour and a group of nr right-hand sides, one
+// thread per site.  The block's links and clover come to shared memory by bulk copy, once for the
+// group; residual and MR steps read them, rho and the neighbours' rho from there.  The hops across the
+// block face appear in the residual only: a list of face sites, spread over all threads, fetches the
+// outside neighbours and leaves half spinors (from above) and finished products (from below) in
+// halo, so that no lane of the residual waits for a gather of its own.  x and y are in the block order
+// of the links (BLOCKED): one bulk copy, and 16-byte words of consecutive sites for the face
+// neighbours; otherwise in the caller's order, entry by entry.  LANES: blocks of up to 16 sites,
+// several in a warp (`lanes` lanes and a part of shared memory each), their sums by shuffles.
 //
-// One persistent CTA of Vb threads (255 registers: one per SM at 4^4) takes (block, group) items.  The
-// next item's links and clover come by bulk copy into shared memory while the MR steps of the current
-// one run.  x and y are in the block order of the links (BLOCKED): bulk copies, and 16-byte words of
-// consecutive sites for the face neighbours; otherwise in the caller's order, entry by entry.
+// Bounds: the FP32 pipes (about 1,330 operations per site and application of D or B, five of them: 13 K
+// cycles per block of 4^4 and column) and shared memory (1.4 KB read per site and application, 2.9 K
+// cycles), of which two warps per sub-partition (the registers, at 4^4 also shared memory) overlap
+// little: 5.8 K cycles per MR step.  Half sweep with 4 MR steps: 273 us at 32^4 and one column, 340 us at
+// 16^3 x 32 and 12 columns, 37 us at 24^2 8 20 in 2^4 blocks.  Links and clover staged again for every block
+// and column from records gathered site by site, the neighbours by each thread: 367, 1,424, 56 us.
+// Measured and not kept (32^4 / 12 columns): links in registers, backward hops handed over as half
+// spinors, the next block's links fetched ahead 270 / 364 and slower for small blocks; links and
+// clover in registers 277 / 379; two threads per site 314 / 397; own links in registers 278 / 344.
 //
-// Bounds: the FP32 pipes (about 1,330 operations per site and application of D or B, five of them:
-// 13 K cycles per block and column) at two warps per sub-partition; of 41 K cycles per block (32^4)
-// the MR steps take 6.4 K each, the hops across the faces 7 K (4 K when their lines are in L2).
-// Half sweep with 4 MR steps: 277 us at 32^4 and one column, 379 us at 16^3 x 32 and 12 columns;
-// staging the links and the clover in shared memory once per block and column instead (189 KB, every
-// MR step reading them back) took 367 and 1,424 us.
-//
-// Shared memory (float4 words): x [6][Vb] (12 entries), rho [6][Vb], the hand-over buffer [4 mu][3][Vb],
-// the next links [18][Vb] and clover [14][Vb].  Between the load of the links into registers and the
-// end of the residual the latter two hold halo ([3][f] per direction, f its face sites) and y [6][Vb].
+// Shared memory (float4 words) per block: x, then rho [6][Vb] (12 entries), links [18][Vb], clover
+// [14][Vb], and per direction the hops from outside ([3][f] half spinors, [3][f] products, f: its face
+// sites).
 __host__ __device__ inline int face_sites(const FineGeom& g, int mu) { return g.Vb / g.B[mu]; }
-constexpr int kSapRed = 12;  // words of the MR coefficient's warp sums: 2 buffers x 3 sums x 8 warps of floats
-inline size_t sap_smem(const FineGeom& g) {
-  return amgpipe::kPipeBytes + (size_t)(kSapRed + (24 + kLinkQ + kClovQ) * g.Vb) * sizeof(float4);
+__host__ __device__ inline int sap_words(const FineGeom& g) {
+  return (6 + kLinkQ + kClovQ) * g.Vb +
+         6 * (face_sites(g, 0) + face_sites(g, 1) + face_sites(g, 2) + face_sites(g, 3));
 }
+constexpr int kSapRed = 12;  // words of the MR coefficient's warp sums: 2 buffers x 3 sums x 8 warps of floats
+inline size_t sap_smem(const FineGeom& g, int subs) {
+  return amgpipe::kPipeBytes + (size_t)(kSapRed + subs * sap_words(g)) * sizeof(float4);
+}
+inline int sap_lanes(const FineGeom& g) {  // lanes per block, a power of two; 0: one block per CTA
+  if (g.Vb > 16) return 0;
+  int w = 4;
+  while (w < g.Vb) w *= 2;
+  return w;
+}
+
 // Column r of x and y: in block order word q of (block b, site t) at r V 6 + (b 6 + q) Vb + t, else
 // entry k of lattice site s at (s 12 + k) nrhs + r
 template <bool BLOCKED>
@@ -811,11 +840,12 @@ __device__ __forceinline__ void load_site(const FineGeom& g, const float2* __res
   }
 }
 
-// The hops of face site f of direction mu to its outside neighbours on both sides.  t: its local index
-// at lc[mu] = 0; the block's site at lc[mu] = B - 1 is (B - 1) stride further.
+// The hops of face site f of direction mu to its outside neighbours on both sides (t: its local index
+// at lc[mu] = 0; the block's site at lc[mu] = B - 1 is (B - 1) stride further): the half spinor from
+// above to halo[f], the product from below to halo[3 nf + f]
 template <int mu, bool BLOCKED>
 __device__ __forceinline__ void face_hops(const FineGeom& g, const float4* __restrict__ U, const float2* __restrict__ x,
-                                          const int X[4], int f, int stride, int nrhs, int r, float4* ex, float4* halo) {
+                                          const int X[4], int f, int stride, int nrhs, int r, float4* halo) {
   const int Vb = g.Vb, nf = face_sites(g, mu);
   const int t = f / stride * (stride * g.B[mu]) + f % stride, tt = t + (g.B[mu] - 1) * stride;
   int Xf[4] = {X[0], X[1], X[2], X[3]}, Xb[4] = {X[0], X[1], X[2], X[3]};
@@ -831,279 +861,242 @@ __device__ __forceinline__ void face_hops(const FineGeom& g, const float4* __res
   half_spinor<false, mu>(pb, h);
 #pragma unroll
   for (int a = 0; a < 3; ++a) colour_row<false>(u, h, a, w[a], w[3 + a]);
-  put_words<3>(ex + mu * 3 * Vb + t, Vb, w);
+  put_words<3>(halo + 3 * nf + f, nf, w);
 }
-// body(direction, face site, offset of the direction's halo) for every face site of the block
-template <typename F>
-__device__ __forceinline__ void for_faces(const int nf[4], F&& body) {
-  const int n = nf[0] + nf[1] + nf[2] + nf[3];
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    int f = i;
-    if (f < nf[0]) body(std::integral_constant<int, 0>(), f, 0);
-    else if ((f -= nf[0]) < nf[1]) body(std::integral_constant<int, 1>(), f, 3 * nf[0]);
-    else if ((f -= nf[1]) < nf[2]) body(std::integral_constant<int, 2>(), f, 3 * (nf[0] + nf[1]));
-    else body(std::integral_constant<int, 3>(), f - nf[2], 3 * (nf[0] + nf[1] + nf[2]));
-  }
-}
-
-// The thread's half spinors U_mu^dag (1 + g_mu) p for its forward neighbours in the block
-template <int mu>
-__device__ __forceinline__ void hand_over(const float2 u[36], const float2 p[12], bool inside, int Vb, int t, int stride,
-                                          float4* ex) {
-  if (!inside) return;
-  float2 h[6], w[6];
-  half_spinor<false, mu>(p, h);
-#pragma unroll
-  for (int a = 0; a < 3; ++a) colour_row<false>(u + 9 * mu, h, a, w[a], w[3 + a]);
-  put_words<3>(ex + mu * 3 * Vb + t + stride, Vb, w);
-}
-template <int mu>
-__device__ __forceinline__ void take_over(const float4* ex, int Vb, int t, float2 o[12]) {
-  float2 w[6];
-  get_words<3>(ex + mu * 3 * Vb + t, Vb, w);
-#pragma unroll
-  for (int a = 0; a < 3; ++a) add_hop<false, mu>(w[a], w[3 + a], a, o);
-}
-// forward hop from the half spinor h
-template <int mu>
-__device__ __forceinline__ void forward_half(const float2 u[36], const float2 h[6], float2 o[12]) {
-  float2 w0, w1;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    colour_row<true>(u + 9 * mu, h, a, w0, w1);
-    add_hop<true, mu>(w0, w1, a, o);
-  }
-}
-// both hops of direction mu of the full D: neighbours in the block from xs, outside ones from halo
-template <int mu>
-__device__ __forceinline__ void full_hops(const float2 u[36], const float4* xs, const float4* ex, const float4* halo,
-                                          int nf, int f, bool inside, int Vb, int t, int stride, float2 o[12]) {
-  float2 h[6];
-  if (inside) {
-    float2 p[12];
-    get_words<6>(xs + t + stride, Vb, p);
-    half_spinor<true, mu>(p, h);
-  } else {
-    get_words<3>(halo + f, nf, h);
-  }
-  forward_half<mu>(u, h, o);
-  take_over<mu>(ex, Vb, t, o);
-}
-// both hops of direction mu of the block operator
-template <int mu>
-__device__ __forceinline__ void block_hops(const float2 u[36], const float4* rho, const float4* ex, bool inside, bool below,
-                                           int Vb, int t, int stride, float2 o[12]) {
-  if (inside) {
-    float2 p[12], h[6];
-    get_words<6>(rho + t + stride, Vb, p);
-    half_spinor<true, mu>(p, h);
-    forward_half<mu>(u, h, o);
-  }
-  if (below) take_over<mu>(ex, Vb, t, o);
-}
-
+// face_hops of every face site of the block, spread over its threads (t of threads)
 template <bool BLOCKED>
-__global__ void __launch_bounds__(256, 1) sap_reg_kernel(const float4* __restrict__ U, const float4* __restrict__ Cl,
-                                                         const float2* __restrict__ y, float2* x, FineGeom g, float mass2,
-                                                         int nrhs, int nr, int groups, int items, int colour, int n_mr,
-                                                         unsigned* err) {
+__device__ __forceinline__ void all_face_hops(const FineGeom& g, const float4* __restrict__ U, const float2* __restrict__ x,
+                                              const int X[4], const int nf[4], const int st[4], int nrhs, int r, int t,
+                                              int threads, float4* halo) {
+  const int n = nf[0] + nf[1] + nf[2] + nf[3];
+  for (int i = t; i < n; i += threads) {
+    int f = i;
+    if (f < nf[0]) face_hops<0, BLOCKED>(g, U, x, X, f, st[0], nrhs, r, halo);
+    else if ((f -= nf[0]) < nf[1]) face_hops<1, BLOCKED>(g, U, x, X, f, st[1], nrhs, r, halo + 6 * nf[0]);
+    else if ((f -= nf[1]) < nf[2]) face_hops<2, BLOCKED>(g, U, x, X, f, st[2], nrhs, r, halo + 6 * (nf[0] + nf[1]));
+    else face_hops<3, BLOCKED>(g, U, x, X, f - nf[2], st[3], nrhs, r, halo + 6 * (nf[0] + nf[1] + nf[2]));
+  }
+}
+// both hops of direction mu: neighbours in the block from R with the links in us; from outside the
+// half spinors and products in halo (FULL), or none
+template <int mu, bool FULL>
+__device__ __forceinline__ void site_hops(const float4* us, const float4* R, const float4* halo, int nf, int f, bool inside,
+                                           bool below, int Vb, int t, int stride, float2 o[12]) {
+  float2 p[12], h[6], u[9], w0, w1;
+  if (FULL || inside) {
+    if (!FULL || inside) {
+      get_words<6>(R + t + stride, Vb, p);
+      half_spinor<true, mu>(p, h);
+    } else {
+      get_words<3>(halo + f, nf, h);
+    }
+    shared_link<mu>(us + t, Vb, u);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      colour_row<true>(u, h, a, w0, w1);
+      add_hop<true, mu>(w0, w1, a, o);
+    }
+  }
+  if (below) {
+    get_words<6>(R + t - stride, Vb, p);
+    shared_link<mu>(us + t - stride, Vb, u);
+    hop2<false, mu>(u, p, o);
+  } else if (FULL) {
+    get_words<3>(halo + 3 * nf + f, nf, h);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) add_hop<false, mu>(h[a], h[3 + a], a, o);
+  }
+}
+
+template <bool BLOCKED, bool LANES>
+__global__ void __launch_bounds__(256, 1) sap32_kernel(const float4* __restrict__ U, const float4* __restrict__ Cl,
+                                                       const float2* __restrict__ y, float2* x, FineGeom g, float mass2,
+                                                       int nrhs, int nr, int groups, int nblk, int lanes, int colour,
+                                                       int n_mr, unsigned* err) {
   using namespace amgpipe;
   extern __shared__ __align__(128) unsigned char sm[];
-  Pipe* pp = reinterpret_cast<Pipe*>(sm);  // full[0]: links and clover, full[1]: x and y
-  const int Vb = g.Vb;
+  Pipe* pp = reinterpret_cast<Pipe*>(sm);  // full[0]: links and clover, full[1]: x
+  const int Vb = g.Vb, W = LANES ? lanes : (int)blockDim.x, subs = LANES ? 32 / lanes : 1;
+  const int t = LANES ? (int)threadIdx.x & (lanes - 1) : (int)threadIdx.x, sub = LANES ? (int)threadIdx.x / lanes : 0;
+  const int ta = t < Vb ? t : 0, item = blockIdx.x;
   float* red = reinterpret_cast<float*>(sm + kPipeBytes);
-  float4* xs = reinterpret_cast<float4*>(sm + kPipeBytes) + kSapRed;
-  float4* rho = xs + 6 * Vb;
-  float4* ex = rho + 6 * Vb;
-  float4* us = ex + 12 * Vb;
+  float4* xr = reinterpret_cast<float4*>(sm + kPipeBytes) + kSapRed + sub * sap_words(g);
+  float4* us = xr + 6 * Vb;
   float4* cs = us + kLinkQ * Vb;
-  float4 *halo = us, *ys = cs;
+  float4* halo = cs + kClovQ * Vb;
   const int nf[4] = {face_sites(g, 0), face_sites(g, 1), face_sites(g, 2), face_sites(g, 3)};
-  const int t = threadIdx.x, ta = t < Vb ? t : 0;
-  const bool act = t < Vb;
   const int st[4] = {1, g.B[0], g.B[0] * g.B[1], g.B[0] * g.B[1] * g.B[2]};
-  bool in[4], below[4];  // neighbour in the block forward, backward
-  int fi[4];             // index among the face sites of a direction
+  const int k = item / groups * subs + sub;  // block of the colour (past the last: the last, not written)
+  int X[4];
+  colour_block(g, min(k, nblk - 1), colour, X);
+  const int b = block_of(g, X);
+  if (threadIdx.x == 0) {
+    mbar_init(&pp->full[0], subs);
+    mbar_init(&pp->full[1], subs);
+    pp->abort = 0;
+    fence_mbar_init();
+  }
+  __syncthreads();
+  if (t == 0) {
+    mbar_expect_tx(&pp->full[0], (unsigned)((kLinkQ + kClovQ) * Vb * sizeof(float4)));
+    bulk_load(us, U + (long long)b * kLinkQ * Vb, (unsigned)(kLinkQ * Vb * sizeof(float4)), &pp->full[0]);
+    bulk_load(cs, Cl + (long long)b * kClovQ * Vb, (unsigned)(kClovQ * Vb * sizeof(float4)), &pp->full[0]);
+  }
+  const bool act = t < Vb && k < nblk;
+  bool in[4], below[4];
+  int fi[4];
   {
     int lc[4];
     coords_of((unsigned)ta, g.dB, lc);
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
-      in[mu] = act && lc[mu] + 1 < g.B[mu];
+      in[mu] = lc[mu] + 1 < g.B[mu];
       below[mu] = lc[mu] > 0;
-      fi[mu] = t / (st[mu] * g.B[mu]) * st[mu] + t % st[mu];
+      fi[mu] = ta / (st[mu] * g.B[mu]) * st[mu] + ta % st[mu];
     }
   }
-  auto load_links = [&](int item) {  // one thread: the item's links and clover
-    int X[4];
-    colour_block(g, item / groups, colour, X);
-    const long long b = block_of(g, X);
-    mbar_expect_tx(&pp->full[0], (unsigned)((kLinkQ + kClovQ) * Vb * sizeof(float4)));
-    bulk_load(us, U + b * kLinkQ * Vb, (unsigned)(kLinkQ * Vb * sizeof(float4)), &pp->full[0]);
-    bulk_load(cs, Cl + b * kClovQ * Vb, (unsigned)(kClovQ * Vb * sizeof(float4)), &pp->full[0]);
-  };
-  if (t == 0) {
-    mbar_init(&pp->full[0], 1);
-    mbar_init(&pp->full[1], 1);
-    pp->abort = 0;
-    fence_mbar_init();
-    load_links(blockIdx.x);
-  }
-  __syncthreads();
-  unsigned phl = 0, phx = 0;
-  // items: (block, group of columns), the groups of a block next to each other (they share its
-  // lines in L2)
-  for (int item = blockIdx.x; item < items; item += gridDim.x) {
-    const int r0 = item % groups * nr, r1 = min(nrhs, r0 + nr);
-    int X[4];
-    colour_block(g, item / groups, colour, X);
-    const int b = block_of(g, X);
-    if (!wait_phase(&pp->full[0], phl, pp)) abort_cta(pp, err);
-    phl ^= 1u;
-    float2 u[36], cl[2 * kClovQ];
-    get_words<kLinkQ>(us + ta, Vb, u);
-    get_words<kClovQ>(cs + ta, Vb, cl);
-    for (int r = r0; r < r1; ++r) {
-      float2 p[12], o[12], e[12];
-      // x and y on the block, and the hops from outside it
-      __syncthreads();  // us, cs (first column) and xs (later ones) are read
-      if (pp->abort) return;
-      if (BLOCKED) {
-        if (t == 0) {
-          const unsigned bytes = (unsigned)(6 * Vb * sizeof(float4));
-          const long long at = r * g.V * 6 + (long long)b * 6 * Vb;
-          mbar_expect_tx(&pp->full[1], 2 * bytes);
-          bulk_load(xs, reinterpret_cast<const float4*>(x) + at, bytes, &pp->full[1]);
-          bulk_load(ys, reinterpret_cast<const float4*>(y) + at, bytes, &pp->full[1]);
-        }
-      } else if (act) {
-        const long long s = local_site(g, X, t);
+  const int r0 = item % groups * nr, r1 = min(nrhs, r0 + nr);
+  unsigned phx = 0;
+  for (int r = r0; r < r1; ++r) {
+    float2 p[12], o[12], e[12], x0[12];
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // rho before the next copy of x
+    __syncthreads();  // the previous column's rho is read
+    if (BLOCKED) {
+      if (t == 0) {
+        const unsigned bytes = (unsigned)(6 * Vb * sizeof(float4));
+        mbar_expect_tx(&pp->full[1], bytes);
+        bulk_load(xr, reinterpret_cast<const float4*>(x) + r * g.V * 6 + (long long)b * 6 * Vb, bytes, &pp->full[1]);
+      }
+    } else if (act) {
+      const long long s = local_site(g, X, t);
 #pragma unroll
-        for (int k = 0; k < 12; ++k) {
-          reinterpret_cast<float2*>(xs + (k >> 1) * Vb + t)[k & 1] = x[(s * 12 + k) * nrhs + r];
-          reinterpret_cast<float2*>(ys + (k >> 1) * Vb + t)[k & 1] = y[(s * 12 + k) * nrhs + r];
-        }
-      }
-      for_faces(nf, [&](auto mu, int f, int off) {
-        face_hops<mu, BLOCKED>(g, U, x, X, f, st[mu], nrhs, r, ex, halo + off);
-      });
-      if (BLOCKED) {
-        if (!wait_phase(&pp->full[1], phx, pp)) abort_cta(pp, err);
-        phx ^= 1u;
-      }
-      get_words<6>(xs + ta, Vb, p);
-      hand_over<0>(u, p, in[0], Vb, t, st[0], ex);
-      hand_over<1>(u, p, in[1], Vb, t, st[1], ex);
-      hand_over<2>(u, p, in[2], Vb, t, st[2], ex);
-      hand_over<3>(u, p, in[3], Vb, t, st[3], ex);
+      for (int q = 0; q < 12; ++q) reinterpret_cast<float2*>(xr + (q >> 1) * Vb + t)[q & 1] = x[(s * 12 + q) * nrhs + r];
+    }
+    // the hops across the faces: half spinors from above, products from below
+    all_face_hops<BLOCKED>(g, U, x, X, nf, st, nrhs, r, t, W, halo);
+    load_site<BLOCKED>(g, y, b, X, ta, nrhs, r, e);
+    if (BLOCKED && !wait_phase(&pp->full[1], phx, pp)) abort_cta(pp, err);
+    phx ^= 1u;
+    if (r == r0 && !wait_phase(&pp->full[0], 0, pp)) abort_cta(pp, err);
+    __syncthreads();
+    if (pp->abort) return;
+    const float4 *h0 = halo, *h1 = h0 + 6 * nf[0], *h2 = h1 + 6 * nf[1], *h3 = h2 + 6 * nf[2];
+    {
+      float2 cl[2 * kClovQ];
+      get_words<kClovQ>(cs + ta, Vb, cl);
+      get_words<6>(xr + ta, Vb, x0);
+      site_term2(cl, mass2, x0, o);
+    }
+    site_hops<0, true>(us, xr, h0, nf[0], fi[0], in[0], below[0], Vb, ta, st[0], o);
+    site_hops<1, true>(us, xr, h1, nf[1], fi[1], in[1], below[1], Vb, ta, st[1], o);
+    site_hops<2, true>(us, xr, h2, nf[2], fi[2], in[2], below[2], Vb, ta, st[2], o);
+    site_hops<3, true>(us, xr, h3, nf[3], fi[3], in[3], below[3], Vb, ta, st[3], o);
+#pragma unroll
+    for (int q = 0; q < 12; ++q) {  // rho = y - D x
+      p[q] = make_float2(fmaf(-0.5f, o[q].x, e[q].x), fmaf(-0.5f, o[q].y, e[q].y));
+      e[q] = zzero<float2>();
+    }
+    __syncthreads();  // x is read
+#pragma unroll 1
+    for (int it = 0; it < n_mr; ++it) {
+      if (act) put_words<6>(xr + t, Vb, p);
       __syncthreads();
-      if (pp->abort) return;
-      if (act) {
-        // rho = y - D x
-        site_term2(cl, mass2, p, o);
-        full_hops<0>(u, xs, ex, halo, nf[0], fi[0], in[0], Vb, t, st[0], o);
-        full_hops<1>(u, xs, ex, halo + 3 * nf[0], nf[1], fi[1], in[1], Vb, t, st[1], o);
-        full_hops<2>(u, xs, ex, halo + 3 * (nf[0] + nf[1]), nf[2], fi[2], in[2], Vb, t, st[2], o);
-        full_hops<3>(u, xs, ex, halo + 3 * (nf[0] + nf[1] + nf[2]), nf[3], fi[3], in[3], Vb, t, st[3], o);
-        get_words<6>(ys + t, Vb, p);
+      {
+        float2 cl[2 * kClovQ];
+        get_words<kClovQ>(cs + ta, Vb, cl);
+        site_term2(cl, mass2, p, o);  // o = 2 B rho
+      }
+      site_hops<0, false>(us, xr, h0, 0, 0, in[0], below[0], Vb, ta, st[0], o);
+      site_hops<1, false>(us, xr, h1, 0, 0, in[1], below[1], Vb, ta, st[1], o);
+      site_hops<2, false>(us, xr, h2, 0, 0, in[2], below[2], Vb, ta, st[2], o);
+      site_hops<3, false>(us, xr, h3, 0, 0, in[3], below[3], Vb, ta, st[3], o);
+      float v[3] = {0, 0, 0};
+      if (t < Vb) {
 #pragma unroll
         for (int q = 0; q < 12; ++q) {
-          p[q].x = fmaf(-0.5f, o[q].x, p[q].x);
-          p[q].y = fmaf(-0.5f, o[q].y, p[q].y);
-          e[q] = zzero<float2>();
+          v[0] += o[q].x * o[q].x + o[q].y * o[q].y;  // <o, o>
+          v[1] += o[q].x * p[q].x + o[q].y * p[q].y;  // Re <o, rho>
+          v[2] += o[q].x * p[q].y - o[q].y * p[q].x;  // Im <o, rho>
         }
       }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // halo and y before the next copies
-      __syncthreads();  // the hand-over buffer, halo and y are read
-      if (t == 0 && r + 1 == r1 && item + (int)gridDim.x < items) load_links(item + gridDim.x);
-#pragma unroll 1
-      for (int it = 0; it < n_mr; ++it) {
-        // p holds rho on this site
-        if (act) put_words<6>(rho + t, Vb, p);
-        hand_over<0>(u, p, in[0], Vb, t, st[0], ex);
-        hand_over<1>(u, p, in[1], Vb, t, st[1], ex);
-        hand_over<2>(u, p, in[2], Vb, t, st[2], ex);
-        hand_over<3>(u, p, in[3], Vb, t, st[3], ex);
-        __syncthreads();
-        float v[3] = {0, 0, 0};
-        if (act) {
-          site_term2(cl, mass2, p, o);  // o = 2 B rho
-          block_hops<0>(u, rho, ex, in[0], below[0], Vb, t, st[0], o);
-          block_hops<1>(u, rho, ex, in[1], below[1], Vb, t, st[1], o);
-          block_hops<2>(u, rho, ex, in[2], below[2], Vb, t, st[2], o);
-          block_hops<3>(u, rho, ex, in[3], below[3], Vb, t, st[3], o);
-#pragma unroll
-          for (int q = 0; q < 12; ++q) {
-            v[0] += o[q].x * o[q].x + o[q].y * o[q].y;  // <o, o>
-            v[1] += o[q].x * p[q].x + o[q].y * p[q].y;  // Re <o, rho>
-            v[2] += o[q].x * p[q].y - o[q].y * p[q].x;  // Im <o, rho>
-          }
-        }
-        float2 al;
-        bool ok;
-        // the barrier inside also orders every read of rho and ex before the next step's writes
+      float2 al;
+      bool ok;
+      // the barrier (inside) also orders every read of rho before the next step's writes
+      if (LANES) {
+        lanes_alpha(v, lanes, al, ok);
+        __syncwarp();
+      } else {
         cta_alpha_all(v, red + (it & 1) * 24, al, ok);
-        if (ok) {  // al = alpha / 2 (o = 2 B rho): e += alpha rho, rho -= alpha B rho
-          const float2 al2 = make_float2(2.f * al.x, 2.f * al.y);
+      }
+      if (ok) {  // al = alpha / 2 (o = 2 B rho): e += alpha rho, rho -= alpha B rho
+        const float2 al2 = make_float2(2.f * al.x, 2.f * al.y);
 #pragma unroll
-          for (int q = 0; q < 12; ++q) {
-            zfma(e[q], al2, p[q]);
-            float2 ap = zzero<float2>();
-            zfma(ap, al, o[q]);
-            p[q] = zsub(p[q], ap);
-          }
+        for (int q = 0; q < 12; ++q) {
+          zfma(e[q], al2, p[q]);
+          float2 ap = zzero<float2>();
+          zfma(ap, al, o[q]);
+          p[q] = zsub(p[q], ap);
         }
       }
-      if (act) {
-        get_words<6>(xs + t, Vb, p);
+    }
+    if (act) {
 #pragma unroll
-        for (int k = 0; k < 12; ++k) p[k] = zadd(p[k], e[k]);
-        if (BLOCKED) {
-          put_words<6>(reinterpret_cast<float4*>(x) + r * g.V * 6 + (long long)b * 6 * Vb + t, Vb, p);
-        } else {
-          const long long s = local_site(g, X, t);
+      for (int q = 0; q < 12; ++q) p[q] = zadd(x0[q], e[q]);
+      if (BLOCKED) {
+        put_words<6>(reinterpret_cast<float4*>(x) + r * g.V * 6 + (long long)b * 6 * Vb + t, Vb, p);
+      } else {
+        const long long s = local_site(g, X, t);
 #pragma unroll
-          for (int k = 0; k < 12; ++k) x[(s * 12 + k) * nrhs + r] = p[k];
-        }
+        for (int q = 0; q < 12; ++q) x[(s * 12 + q) * nrhs + r] = p[q];
       }
     }
   }
 }
 
 // Columns j0 .. j0 + N groups - 1 of v ([V][12][nrhs]) <-> w ([column][block][6 words][Vb], block order).
-// One CTA per kTileSites sites of a block and N columns, through shared memory: v is read and written
+// One CTA per kTileSites sites (in block order) and N columns, through shared memory: v is read and written
 // in runs (the B[0] sites of a row; N neighbouring columns), w in runs of consecutive sites.  Bound:
 // HBM; many small CTAs keep it busy (32^4, one column: 36 us a copy, 5.6 TB/s; a CTA per block with the
 // site index computed by divisions took 86 us).
 constexpr int kTileSites = 64;
 template <bool TO, int N>
-__global__ void __launch_bounds__(256) blocked_kernel(float2* __restrict__ v, float2* __restrict__ w, Geom g, int nrhs,
-                                                      int j0, int groups) {
+__global__ void __launch_bounds__(256) blocked_kernel(float2* __restrict__ v, float2* __restrict__ w, FineGeom g,
+                                                      const int* __restrict__ soff, int nrhs, int j0, int groups) {
   constexpr int P = kTileSites + 1;
-  __shared__ float2 sc[N * 12 * P];  // [column][entry][site]
-  const int Vb = (int)g.Vb, chunks = (Vb + kTileSites - 1) / kTileSites;
-  const int grp = (int)(blockIdx.x % groups), q0 = (int)(blockIdx.x / groups), t0 = q0 % chunks * kTileSites;
-  const long long b = q0 / chunks, origin = block_origin(g, b);
-  const int ts = min(kTileSites, Vb - t0);
-  const int* soff = g.soff + t0;
-  float4* wb = reinterpret_cast<float4*>(w) + (long long)grp * N * g.V * 6 + b * 6 * Vb + t0;
+  __shared__ float2 sc[N * 12 * P];           // [column][entry][site]
+  __shared__ unsigned lex[kTileSites];        // the sites' places in the lattice
+  __shared__ long long wof[kTileSites];       // and of their first words in w
+  const int Vb = g.Vb, grp = (int)(blockIdx.x % groups);
+  const long long i0 = (long long)(blockIdx.x / groups) * kTileSites;
+  const int ts = (int)min((long long)kTileSites, g.V - i0);
+  if (threadIdx.x < ts) {
+    int t, X[4];
+    const unsigned b = divide((unsigned)(i0 + threadIdx.x), g.dVb, t);
+    coords_of(b, g.dLc, X);
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) X[mu] *= g.B[mu];
+    lex[threadIdx.x] = (unsigned)(site_of(g, X) + __ldg(soff + t));
+    wof[threadIdx.x] = (long long)b * 6 * Vb + t;
+  }
+  __syncthreads();
+  float4* wg = reinterpret_cast<float4*>(w) + (long long)grp * N * g.V * 6;
   auto caller = [&](auto&& body) {  // e = (site, entry, column), the column fastest
 #pragma unroll 6
     for (int e = threadIdx.x; e < ts * 12 * N; e += 256) {
       const int c = e % N, k = e / N % 12, t = e / (12 * N);
-      body(v + ((origin + __ldg(soff + t)) * 12 + k) * nrhs + j0 + grp * N + c, sc + (c * 12 + k) * P + t);
+      body(v + ((long long)lex[t] * 12 + k) * nrhs + j0 + grp * N + c, sc + (c * 12 + k) * P + t);
     }
   };
   auto caller_words = [&](auto&& body) {  // one column: e = (site, word)
 #pragma unroll 2
     for (int e = threadIdx.x; e < ts * 6; e += 256)
-      body(reinterpret_cast<float4*>(v) + (origin + __ldg(soff + e / 6)) * 6 + e % 6, sc + e % 6 * 2 * P + e / 6);
+      body(reinterpret_cast<float4*>(v) + (long long)lex[e / 6] * 6 + e % 6, sc + e % 6 * 2 * P + e / 6);
   };
   auto blocked = [&](auto&& body) {  // e = (column, word, site)
 #pragma unroll 2
     for (int e = threadIdx.x; e < N * 6 * kTileSites; e += 256) {
       const int t = e % kTileSites, q = e / kTileSites % 6, c = e / (6 * kTileSites);
-      if (t < ts) body(wb + (long long)c * g.V * 6 + q * Vb + t, sc + (c * 12 + 2 * q) * P + t);
+      if (t < ts) body(wg + (long long)c * g.V * 6 + wof[t] + q * Vb, sc + (c * 12 + 2 * q) * P + t);
     }
   };
   auto word_in = [](const float4* a, float2* s) {
@@ -1395,20 +1388,18 @@ int sap_columns(long long nblk, int nrhs, int slots) {
 template <bool BLOCKED>
 amg_status sweep32(amg_coarse* h, const float2* y, float2* x, int nrhs, int n_cycles, int n_mr, cudaStream_t st) {
   const FineGeom g = fine_geom(h);
-  const int threads = (g.Vb + 31) / 32 * 32;
-  const size_t smem = sap_smem(g);
+  const int lanes = sap_lanes(g), subs = lanes ? 32 / lanes : 1, threads = lanes ? 32 : (g.Vb + 31) / 32 * 32;
+  const size_t smem = sap_smem(g, subs);
   if (threads > 256 || smem > 227 * 1024) return AMG_ERR_UNSUPPORTED;
-  AMG_CUDA_TRY(cudaFuncSetAttribute(sap_reg_kernel<BLOCKED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const long long nblk = h->g.Vc / 2;
-  const int slots = sap_slots(threads, smem);
-  const int nr = sap_columns(nblk, nrhs, slots), groups = (nrhs + nr - 1) / nr;
-  const int items = (int)(nblk * groups);
+  auto* k = lanes ? sap32_kernel<BLOCKED, true> : sap32_kernel<BLOCKED, false>;
+  AMG_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int nblk = (int)(h->g.Vc / 2), units = (nblk + subs - 1) / subs;
+  const int nr = sap_columns(units, nrhs, sap_slots(threads, smem)), groups = (nrhs + nr - 1) / nr;
   const float mass2 = 2.f * (float)(4.0 + h->p.m0);
   for (int c = 0; c < n_cycles; ++c)
     for (int colour = 0; colour < 2; ++colour) {
-      sap_reg_kernel<BLOCKED><<<std::min(items, slots), threads, smem, st>>>((const float4*)h->fU, (const float4*)h->fC, y, x,
-                                                                            g, mass2, nrhs, nr, groups, items, colour, n_mr,
-                                                                            h->err);
+      k<<<units * groups, threads, smem, st>>>((const float4*)h->fU, (const float4*)h->fC, y, x, g, mass2, nrhs, nr, groups,
+                                              nblk, lanes, colour, n_mr, h->err);
       AMG_LAUNCH_CHECK();
       h->launches++;
     }
@@ -1431,14 +1422,16 @@ size_t sap_copy_bytes(const amg_coarse* h, int nrhs) {
 template <bool TO>
 amg_status blocked_copy(amg_coarse* h, const float2* v, const float2* w, int nrhs, int j0, int nc, cudaStream_t st) {
   float2 *vv = const_cast<float2*>(v), *ww = const_cast<float2*>(w);
-  const unsigned tiles = (unsigned)(h->g.Vc * ((h->g.Vb + kTileSites - 1) / kTileSites));
+  const unsigned tiles = (unsigned)((h->g.V + kTileSites - 1) / kTileSites);
   const int groups = nc / 4, rest = nc % 4;
-  if (groups) blocked_kernel<TO, 4><<<tiles * groups, 256, 0, st>>>(vv, ww, h->g, nrhs, j0, groups);
+  const FineGeom g = fine_geom(h);
+  const int* so = h->soff;
+  if (groups) blocked_kernel<TO, 4><<<tiles * groups, 256, 0, st>>>(vv, ww, g, so, nrhs, j0, groups);
   j0 += 4 * groups;
   ww += (size_t)4 * groups * h->g.V * 12;
-  if (rest == 1) blocked_kernel<TO, 1><<<tiles, 256, 0, st>>>(vv, ww, h->g, nrhs, j0, 1);
-  else if (rest == 2) blocked_kernel<TO, 2><<<tiles, 256, 0, st>>>(vv, ww, h->g, nrhs, j0, 1);
-  else if (rest == 3) blocked_kernel<TO, 3><<<tiles, 256, 0, st>>>(vv, ww, h->g, nrhs, j0, 1);
+  if (rest == 1) blocked_kernel<TO, 1><<<tiles, 256, 0, st>>>(vv, ww, g, so, nrhs, j0, 1);
+  else if (rest == 2) blocked_kernel<TO, 2><<<tiles, 256, 0, st>>>(vv, ww, g, so, nrhs, j0, 1);
+  else if (rest == 3) blocked_kernel<TO, 3><<<tiles, 256, 0, st>>>(vv, ww, g, so, nrhs, j0, 1);
   h->launches += (groups > 0) + (rest > 0);
   AMG_LAUNCH_CHECK();
   return AMG_OK;
