@@ -3,11 +3,11 @@
 // coarse layout [Vc][2][ntv][nrhs]; all scalars (Hessenberg matrix, rotations, residual
 // estimates, convergence flags) live on the device, so the host only launches kernels.
 //
-// One Arnoldi step is two launches for nrhs in {1, 2, 4, 8, 16}: w = D_c V_j (the application
-// reads the unnormalised vector times 1/h_{j,j-1} and stores V_j on the way), then the
-// cooperative k_arnoldi (dots <V_i, w>, column j of H, w -= sum H_ij V_i with |w|^2, Givens
-// rotation and convergence test, phases separated by grid barriers).  Other column counts take
-// three launches (k_dots, then k_update, each ending in a last-CTA reduction).  Once every
+// One Arnoldi step is two launches: w = D_c V_j (the application reads the unnormalised vector times
+// 1/h_{j,j-1} and stores V_j on the way), then the cooperative k_arnoldi (dots <V_i, w>, column j of
+// H, w -= sum H_ij V_i with |w|^2, Givens rotation and convergence test, phases separated by grid
+// barriers).  Where a cooperative launch cannot hold its CTAs resident, k_dots and k_update take its
+// place, each ending in a last-CTA reduction.  Grids follow the vectors' length.  Once every
 // right-hand side has converged the device flag `done` makes every later kernel return at once
 // and a mapped host word receives the solve's ticket; the host reads it after the next
 // application is queued (so the GPU never waits for the host) or, without polling, launches the
@@ -139,13 +139,13 @@ __device__ inline double2 shfl_d2(double2 v, int src) {
 // entries are c_i carry_i + s_i col[i+1].  The carries are a prefix composition of the complex
 // affine maps x -> A_i + B_i x, taken as a warp scan (five shuffle rounds per 32 rotations)
 // instead of a chain of j dependent steps.
-__device__ inline void givens_scan_half(const double2& ci, const double2& si, const double2& b, bool valid, double2 x0,
-                                        double2& carry_i, double2& carry_next) {
+// n: rotations in this half; a scan over n of them needs ceil(log2 n) rounds
+__device__ inline void givens_scan_half(const double2& ci, const double2& si, const double2& b, bool valid, int n,
+                                        double2 x0, double2& carry_i, double2& carry_next) {
   const int lane = threadIdx.x & 31;
   double2 A = valid ? cmulc(ci, b) : make_double2(0, 0);               // conj(c_i) b
   double2 Bm = valid ? make_double2(-si.x, si.y) : make_double2(1, 0);  // -conj(s_i)
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
+  for (int o = 1; o < n && o < 32; o <<= 1) {
     const double2 Ap = make_double2(__shfl_up_sync(0xffffffffu, A.x, o), __shfl_up_sync(0xffffffffu, A.y, o));
     const double2 Bp = make_double2(__shfl_up_sync(0xffffffffu, Bm.x, o), __shfl_up_sync(0xffffffffu, Bm.y, o));
     if (lane >= o) {
@@ -178,7 +178,6 @@ __device__ void arnoldi_step_warp(FState& s, int r, int j, double n2, int* any) 
     if (lane == 0) s.invh[r] = 0;
     return;
   }
-  const double hnext = sqrt(n2);
   // col[i + 1] for rotation i = lane (first half) and i = lane + 32 (second half)
   const double2 c32 = shfl_d2(col1, 0);
   double2 b0 = make_double2(__shfl_down_sync(0xffffffffu, col0.x, 1), __shfl_down_sync(0xffffffffu, col0.y, 1));
@@ -186,18 +185,21 @@ __device__ void arnoldi_step_warp(FState& s, int r, int j, double n2, int* any) 
   const double2 b1 = make_double2(__shfl_down_sync(0xffffffffu, col1.x, 1), __shfl_down_sync(0xffffffffu, col1.y, 1));
   const double2 x0 = shfl_d2(col0, 0);
   double2 ci0, cn0, carry = x0, f0 = z, f1 = z;
-  givens_scan_half(c0, s0, b0, lane < j, x0, ci0, cn0);
+  givens_scan_half(c0, s0, b0, lane < j, j, x0, ci0, cn0);
   if (lane < j) f0 = cadd(cmul(c0, ci0), cmul(s0, b0));
   if (j > 0 && j <= 32) carry = shfl_d2(cn0, j - 1);
   if (j > 32) {
     const double2 x32 = shfl_d2(cn0, 31);
     double2 ci1, cn1;
-    givens_scan_half(c1, s1, b1, lane + 32 < j, x32, ci1, cn1);
+    givens_scan_half(c1, s1, b1, lane + 32 < j, j - 32, x32, ci1, cn1);
     if (lane + 32 < j) f1 = cadd(cmul(c1, ci1), cmul(s1, b1));
     carry = shfl_d2(cn1, j - 33);
   }
   const double den2 = carry.x * carry.x + carry.y * carry.y + n2;
-  const double inv_den = den2 > 0 ? 1.0 / sqrt(den2) : 0.0;
+  // sqrt and 1 / sqrt of n2 and den2, one in the even lanes, the other in the odd ones
+  const double root = sqrt(lane & 1 ? den2 : n2), inv_root = 1.0 / root;
+  const double hnext = __shfl_sync(0xffffffffu, root, 0), inv_hnext = __shfl_sync(0xffffffffu, inv_root, 0);
+  const double inv_den = den2 > 0 ? __shfl_sync(0xffffffffu, inv_root, 1) : 0.0;
   const double den = den2 * inv_den;
   const double2 c = den2 > 0 ? cscale(cconj(carry), inv_den) : make_double2(1, 0);
   const double2 sv = make_double2(hnext * inv_den, 0);
@@ -219,7 +221,7 @@ __device__ void arnoldi_step_warp(FState& s, int r, int j, double n2, int* any) 
       s.active[r] = 0;
       s.invh[r] = 0;
     } else {
-      s.invh[r] = 1.0 / hnext;
+      s.invh[r] = inv_hnext;
       atomicOr(any, 1);
     }
   }
@@ -304,73 +306,16 @@ __global__ void __launch_bounds__(ST_T) k_update(FState s, CT* __restrict__ w, c
   if (threadIdx.x == 0 && !any) mark_done(s);
 }
 
-template <typename CT>
-__global__ void __launch_bounds__(ST_T) k_dots_flat(FState s, const CT* __restrict__ w, const CT* __restrict__ V,
-                                                    long long vstride, int j) {
-  if (*s.done) return;
-  const int i = blockIdx.y;
-  const CT* Vi = V + i * vstride;
-  const long long n = s.rows * s.nrhs;
-  CT a = CT{0, 0};
-  for (long long e = blockIdx.x * (long long)ST_T + threadIdx.x; e < n; e += (long long)s.nblk * ST_T)
-    cfmac(a, Vi[e], w[e]);
-  cta_col_sum_store(to_d(a), s.nrhs, s.part + ((long long)i * s.nblk + blockIdx.x) * s.nrhs);
-  if (!last_block(s.counter, s.nblk * (j + 1))) return;
-  const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int t = warp; t < (j + 1) * s.nrhs; t += nw) {
-    const double2 sum = warp_sum_partials(s.part, s.nblk, s.nrhs, t);
-    const int ii = t / s.nrhs, r = t % s.nrhs;
-    if ((threadIdx.x & 31) == 0) s.H[((long long)r * (s.m + 1) + ii) * s.m + j] = s.active[r] ? sum : make_double2(0, 0);
-  }
-}
-
-template <typename CT>
-__global__ void __launch_bounds__(ST_T) k_update_flat(FState s, CT* __restrict__ w, const CT* __restrict__ V,
-                                                      long long vstride, int j) {
-  if (*s.done) return;
-  __shared__ CT hc[AMG_MAX_NTV + 1][MAXR];
-  for (int e = threadIdx.x; e < (j + 1) * s.nrhs; e += ST_T) {
-    const int i = e / s.nrhs, r = e % s.nrhs;
-    hc[i][r] = from_d<CT>(ld_cg(s.H + ((long long)r * (s.m + 1) + i) * s.m + j));
-  }
-  __syncthreads();
-  const int col = threadIdx.x % s.nrhs;
-  const long long n = s.rows * s.nrhs;
-  decltype(CT{}.x) acc = 0;
-  for (long long e = blockIdx.x * (long long)ST_T + threadIdx.x; e < n; e += (long long)s.nblk * ST_T) {
-    CT v = w[e];
-    for (int i = 0; i <= j; ++i) {
-      const CT q = V[i * vstride + e];
-      const CT c = hc[i][col];
-      v.x -= c.x * q.x - c.y * q.y;
-      v.y -= c.x * q.y + c.y * q.x;
-    }
-    w[e] = v;
-    acc += v.x * v.x + v.y * v.y;
-  }
-  cta_col_sum_store(make_double2((double)acc, 0.0), s.nrhs, s.part + (long long)blockIdx.x * s.nrhs);
-  if (!last_block(s.counter, s.nblk)) return;
-  __shared__ int any;
-  __shared__ double n2s[MAXR];
-  if (threadIdx.x == 0) any = 0;
-  for (int r = threadIdx.x >> 5; r < s.nrhs; r += blockDim.x >> 5) {
-    const double2 v = warp_sum_partials(s.part, s.nblk, s.nrhs, r);
-    if ((threadIdx.x & 31) == 0) n2s[r] = v.x;
-  }
-  __syncthreads();
-  for (int r = threadIdx.x >> 5; r < s.nrhs; r += ST_T / 32) arnoldi_step_warp(s, r, j, n2s[r], &any);
-  __syncthreads();
-  if (threadIdx.x == 0 && !any) mark_done(s);
-}
-
-// ---- fused Arnoldi step for nrhs in {1, 2, 4, 8, 16} (flat element loops as above): one
-// cooperative launch, one CTA per SM, does the dots, the Hessenberg column, the update with |w|^2
-// and the Givens step, with two grid barriers in place of a kernel boundary and a last-CTA
-// hand-off.  With one or a few columns the coarse vectors are small (Vc * 2 Ntv rows, about a
+// ---- fused Arnoldi step: one cooperative launch of at most one CTA per SM does the dots, the
+// Hessenberg column, the update with |w|^2 and the Givens step, with two grid barriers in place of a
+// kernel boundary and a last-CTA hand-off.  The element loops are flat: with nrhs dividing 32 (POW2)
+// as above, otherwise the CTA uses a multiple of nrhs threads, so that a thread again meets one
+// column, and column sums go through shared memory (the row-per-thread form of k_dots / k_update,
+// which served these counts, took 31 and 38 us a launch for 12 columns at 16^3 x 32).  With one or a few columns the coarse vectors are small (Vc * 2 Ntv rows, about a
 // megabyte), each phase is a few memory round trips and the launch and barrier latencies set the
 // time; with 16 columns they reach hundreds of megabytes and the phases stream, which is what the
 // round shapes below are for.
-constexpr int AR_T = 512;
+constexpr int AR_T = 512;  // most threads of a CTA
 constexpr int AR_W = AR_T / 32;
 template <typename CT>
 constexpr int ar_ic() { return sizeof(CT) == 8 ? 8 : 4; }  // dot products reduced per CTA round
@@ -416,17 +361,64 @@ __device__ bool grid_sync(unsigned* bar, unsigned* err, unsigned extra) {
   return ok != 0;
 }
 
-template <typename CT, int AR_IC, int AR_U, int KQ>
+// Sum over the CTA's threads of equal column (thread t < per has column t % nr) of v[thread] by one warp;
+// valid in lane 0.  FP32 partial sums are added as pairs of floats (TwoSum), which loses nothing
+// against sums in FP64 and stays off the scarce FP64 pipe.
+__device__ inline void pair_sum(float& h, float& l, float h2, float l2) {
+  const float t = __fadd_rn(h, h2), v = __fsub_rn(t, h);
+  l = __fadd_rn(l, __fadd_rn(l2, __fadd_rn(__fsub_rn(h, __fsub_rn(t, v)), __fsub_rn(h2, v))));
+  h = t;
+}
+__device__ inline double2 column_sum(const float2* v, int per, int nr, int r) {
+  float hx = 0, lx = 0, hy = 0, ly = 0;
+  for (int k = r + (threadIdx.x & 31) * nr; k < per; k += 32 * nr) {
+    pair_sum(hx, lx, v[k].x, 0.f);
+    pair_sum(hy, ly, v[k].y, 0.f);
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    pair_sum(hx, lx, __shfl_xor_sync(0xffffffffu, hx, o), __shfl_xor_sync(0xffffffffu, lx, o));
+    pair_sum(hy, ly, __shfl_xor_sync(0xffffffffu, hy, o), __shfl_xor_sync(0xffffffffu, ly, o));
+  }
+  return make_double2((double)hx + (double)lx, (double)hy + (double)ly);
+}
+__device__ inline double2 column_sum(const double2* v, int per, int nr, int r) {
+  double2 t = make_double2(0, 0);
+  for (int k = r + (threadIdx.x & 31) * nr; k < per; k += 32 * nr) t = cadd(t, v[k]);
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
+    t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
+  }
+  return t;
+}
+
+// Sum of v[0 .. W - 1] (W <= 32) by one warp; valid in lane 0
+__device__ inline double2 warps_sum(const double2* v, int W) {
+  const int lane = threadIdx.x & 31;
+  double2 t = lane < W ? v[lane] : make_double2(0, 0);
+  for (int o = W > 1 ? 1 << (31 - __clz(W - 1)) : 0; o; o >>= 1) {
+    t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
+    t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
+  }
+  return t;
+}
+
+template <typename CT, int AR_IC, int AR_U, int KQ, bool POW2>
 __global__ void __launch_bounds__(AR_T) k_arnoldi(FState s, CT* __restrict__ w, const CT* __restrict__ V,
                                                   long long vstride, int j) {
   using RT = decltype(CT{}.x);
   if (*s.done) return;
-  __shared__ double2 red[AR_IC][AR_W][MAXR];
+  __shared__ double2 red[POW2 ? AR_IC : 1][MAXR][AR_W + 1];
+  __shared__ CT tred[POW2 ? 1 : AR_IC][AR_T];
   __shared__ CT hc[AMG_MAX_NTV + 1][MAXR];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nr = s.nrhs, G = gridDim.x;
-  const long long n = s.rows * nr;
-  const long long e0 = (long long)blockIdx.x * AR_T + threadIdx.x, es = (long long)G * AR_T;
-  // 1. per-CTA partial sums of <V_i, w>, i = 0..j (lane l only ever meets column l % nr)
+  const int T = blockDim.x, W = T >> 5;
+  const int per = POW2 ? T : T / nr * nr;  // threads that take elements
+  const long long n = s.rows * nr, es = (long long)G * per;
+  const long long e0 = threadIdx.x < per ? (long long)blockIdx.x * per + threadIdx.x : n;
+  const bool one = G == 1 && s.bar_extra == 0;  // a single CTA needs no grid barrier
+  // 1. per-CTA partial sums of <V_i, w>, i = 0..j (a thread only ever meets column e0 % nr)
   for (int i0 = 0; i0 <= j; i0 += AR_IC) {
     const int ni = min(AR_IC, j + 1 - i0);
     CT a[AR_IC];
@@ -444,47 +436,67 @@ __global__ void __launch_bounds__(AR_T) k_arnoldi(FState s, CT* __restrict__ w, 
           vv[ii][u] = (ii < ni && eb + u * es < n) ? V[(i0 + ii) * vstride + eb + u * es] : CT{0, 0};
 #pragma unroll
       for (int ii = 0; ii < AR_IC; ++ii)
+        if (ii < ni)
 #pragma unroll
-        for (int u = 0; u < AR_U; ++u) cfmac(a[ii], vv[ii][u], wv[u]);
+          for (int u = 0; u < AR_U; ++u) cfmac(a[ii], vv[ii][u], wv[u]);
     }
     // warp sums in the vectors' own precision (FP64 arithmetic is scarce on this GPU), then FP64
+    if constexpr (!POW2) {
 #pragma unroll
-    for (int ii = 0; ii < AR_IC; ++ii) {
-      if (ii < ni) {
-        CT v = a[ii];
-        for (int o = 16; o >= nr; o >>= 1) {
-          v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-          v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+      for (int ii = 0; ii < AR_IC; ++ii) tred[ii][threadIdx.x] = a[ii];
+      __syncthreads();
+      for (int t = warp; t < ni * nr; t += W) {
+        const double2 sum = column_sum(tred[t / nr], per, nr, t % nr);
+        if (lane == 0) s.part[((long long)(i0 + t / nr) * G + blockIdx.x) * nr + t % nr] = sum;
+      }
+    } else {
+#pragma unroll
+      for (int ii = 0; ii < AR_IC; ++ii) {
+        if (ii < ni) {
+          CT v = a[ii];
+          for (int o = 16; o >= nr; o >>= 1) {
+            v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+            v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+          }
+          if (lane < nr) red[ii][lane][warp] = to_d(v);
         }
-        if (lane < nr) red[ii][warp][lane] = to_d(v);
+      }
+      __syncthreads();
+      for (int t = warp; t < ni * nr; t += W) {  // the warps' sums
+        const double2 sum = warps_sum(red[t / nr][t % nr], W);
+        if (lane == 0) s.part[((long long)(i0 + t / nr) * G + blockIdx.x) * nr + t % nr] = sum;
       }
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < ni * nr; t += AR_T) {
-      const int ii = t / nr, r = t % nr;
-      double2 sum = make_double2(0, 0);
-      for (int wp = 0; wp < AR_W; ++wp) sum = cadd(sum, red[ii][wp][r]);
-      s.part[((long long)(i0 + ii) * G + blockIdx.x) * nr + r] = sum;
-    }
-    __syncthreads();
   }
-  if (!grid_sync(s.bar, s.err, s.bar_extra)) return;
-  // 2. column j of H: one warp per (i, r) sums the G partials
+  if (one) __syncthreads();
+  else if (!grid_sync(s.bar, s.err, s.bar_extra)) return;
+  // 2. column j of H: one warp per (i, r) sums the G partials.  A few sums are taken by every CTA for
+  // itself, which costs less than another grid barrier (2 us).
   const int P = (j + 1) * nr;
-  for (int t = blockIdx.x * AR_W + warp; t < P; t += G * AR_W) {
-    const double2 sum = warp_sum_partials(s.part, G, nr, t);
+  const bool each = P <= 8;
+  for (int t = each ? warp : blockIdx.x * W + warp; t < P; t += each ? W : G * W) {
     const int i = t / nr, r = t % nr;
-    if (lane == 0) s.H[((long long)r * (s.m + 1) + i) * s.m + j] = __ldcg(s.active + r) ? sum : make_double2(0, 0);
+    double2 sum = warp_sum_partials(s.part, G, nr, t);
+    if (!__ldcg(s.active + r)) sum = make_double2(0, 0);
+    if (lane == 0) {
+      if (each) hc[i][r] = from_d<CT>(sum);
+      if (!each || blockIdx.x == 0) s.H[((long long)r * (s.m + 1) + i) * s.m + j] = sum;
+    }
   }
-  if (!grid_sync(s.bar, s.err, s.bar_extra)) return;
-  // 3. w -= sum_i H[r][i][j] V_i and the partial sums of |w|^2 (into row 0 of the partials,
-  // whose reads in 2. are complete)
-  for (int t = threadIdx.x; t < P; t += AR_T) {
-    const int i = t / nr, r = t % nr;
-    hc[i][r] = from_d<CT>(ld_cg(s.H + ((long long)r * (s.m + 1) + i) * s.m + j));
+  if (!each) {
+    if (one) __syncthreads();
+    else if (!grid_sync(s.bar, s.err, s.bar_extra)) return;
+    for (int t = threadIdx.x; t < P; t += T) {
+      const int i = t / nr, r = t % nr;
+      hc[i][r] = from_d<CT>(ld_cg(s.H + ((long long)r * (s.m + 1) + i) * s.m + j));
+    }
   }
   __syncthreads();
-  const int col = lane % nr;
+  // 3. w -= sum_i H[r][i][j] V_i and the partial sums of |w|^2 (into row j + 1 of the partials: with
+  // `each`, a slower CTA may still read the dots in rows 0 .. j)
+  const int col = (int)threadIdx.x % nr;
+  double2* n2part = s.part + (long long)(j + 1) * G * nr;
   RT acc = 0;
   for (long long eb = e0; eb < n; eb += AR_U * es) {
     CT v[AR_U];
@@ -526,25 +538,33 @@ __global__ void __launch_bounds__(AR_T) k_arnoldi(FState s, CT* __restrict__ w, 
         acc += v[u].x * v[u].x + v[u].y * v[u].y;
       }
   }
-  for (int o = 16; o >= nr; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane < nr) red[0][warp][lane] = make_double2((double)acc, 0);
-  __syncthreads();
-  if (threadIdx.x < nr) {
-    double sum = 0;
-    for (int wp = 0; wp < AR_W; ++wp) sum += red[0][wp][threadIdx.x].x;
-    s.part[(long long)blockIdx.x * nr + threadIdx.x] = make_double2(sum, 0);
+  if (!POW2) {
+    tred[0][threadIdx.x] = CT{acc, 0};
+    __syncthreads();
+    for (int r = warp; r < nr; r += W) {
+      const double2 sum = column_sum(tred[0], per, nr, r);
+      if (lane == 0) n2part[(long long)blockIdx.x * nr + r] = sum;
+    }
+  } else {
+    for (int o = 16; o >= nr; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane < nr) red[0][lane][warp] = make_double2((double)acc, 0);
+    __syncthreads();
+    for (int r = warp; r < nr; r += W) {
+      const double2 sum = warps_sum(red[0][r], W);
+      if (lane == 0) n2part[(long long)blockIdx.x * nr + r] = sum;
+    }
   }
   // 4. the last CTA: |w|^2 per column and the Givens step, one warp per right-hand side
   if (!last_block(s.counter, G)) return;
   __shared__ int any;
   __shared__ double n2s[MAXR];
   if (threadIdx.x == 0) any = 0;
-  for (int r = warp; r < nr; r += AR_W) {
-    const double2 v = warp_sum_partials(s.part, G, nr, r);
+  for (int r = warp; r < nr; r += W) {
+    const double2 v = warp_sum_partials(n2part, G, nr, r);
     if (lane == 0) n2s[r] = v.x;
   }
   __syncthreads();
-  for (int r = warp; r < nr; r += AR_W) arnoldi_step_warp(s, r, j, n2s[r], &any);
+  for (int r = warp; r < nr; r += W) arnoldi_step_warp(s, r, j, n2s[r], &any);
   __syncthreads();
   if (threadIdx.x == 0 && !any) mark_done(s);
 }
@@ -657,10 +677,12 @@ template <typename CT>
 __global__ void __launch_bounds__(ST_T) k_residual(FState s, CT* __restrict__ w, const CT* __restrict__ b, int first,
                                                    CT* __restrict__ xzero) {
   if (*s.done) return;
-  if (32 % s.nrhs == 0) {  // flat, coalesced (see k_dots_flat; one column included)
-    const long long n = s.rows * s.nrhs, es = (long long)s.nblk * ST_T;
-    decltype(CT{}.x) acc = 0;
-    for (long long eb = blockIdx.x * (long long)ST_T + threadIdx.x; eb < n; eb += 4 * es) {  // 4 elements per round
+  const bool pow2 = 32 % s.nrhs == 0;  // flat, coalesced, a thread meets one column (see k_arnoldi)
+  const int per = pow2 ? ST_T : ST_T / s.nrhs * s.nrhs;
+  decltype(CT{}.x) acc = 0;
+  {
+    const long long n = s.rows * s.nrhs, es = (long long)s.nblk * per;
+    for (long long eb = threadIdx.x < per ? blockIdx.x * (long long)per + threadIdx.x : n; eb < n; eb += 4 * es) {  // 4 a round
       CT v[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
@@ -682,31 +704,17 @@ __global__ void __launch_bounds__(ST_T) k_residual(FState s, CT* __restrict__ w,
         }
       }
     }
+  }
+  if (pow2) {
     cta_col_sum_store(make_double2((double)acc, 0.0), s.nrhs, s.part + (long long)blockIdx.x * s.nrhs);
   } else {
-    CT a[MAXR];
-#pragma unroll
-    for (int r = 0; r < MAXR; ++r) a[r] = CT{0, 0};
-    for (long long row = blockIdx.x * (long long)ST_T + threadIdx.x; row < s.rows;
-         row += (long long)s.nblk * ST_T) {
-#pragma unroll
-      for (int r = 0; r < MAXR; ++r) {
-        if (r >= s.nrhs) break;
-        CT v = b[row * s.nrhs + r];
-        if (!first) {
-          const CT q = w[row * s.nrhs + r];
-          v.x -= q.x;
-          v.y -= q.y;
-        }
-        w[row * s.nrhs + r] = v;
-        if (xzero) xzero[row * s.nrhs + r] = CT{0, 0};
-        a[r].x += v.x * v.x + v.y * v.y;
-      }
+    __shared__ CT tred[ST_T];
+    tred[threadIdx.x] = CT{acc, 0};
+    __syncthreads();
+    for (int r = threadIdx.x >> 5; r < s.nrhs; r += ST_T / 32) {
+      const double2 sum = column_sum(tred, per, s.nrhs, r);
+      if ((threadIdx.x & 31) == 0) s.part[(long long)blockIdx.x * s.nrhs + r] = sum;
     }
-    double2 acc[MAXR];
-#pragma unroll
-    for (int r = 0; r < MAXR; ++r) acc[r] = to_d(a[r]);
-    cta_sum_store(acc, s.nrhs, s.part + (long long)blockIdx.x * s.nrhs);
   }
   if (!last_block(s.counter, s.nblk)) return;
   __shared__ int any;
@@ -745,7 +753,14 @@ __global__ void __launch_bounds__(ST_T) k_residual(FState s, CT* __restrict__ w,
   if (threadIdx.x == 0 && !any) mark_done(s);
 }
 
-// Grid of the cooperative k_arnoldi: one CTA per SM (at most solve_nblk(), the partial-sum rows'
+template <typename CT>
+const void* arnoldi_kernel(bool is_long, bool pow2) {
+  if (is_long)
+    return pow2 ? (const void*)k_arnoldi<CT, 2, ar_ulong<CT>(), 1, true> : (const void*)k_arnoldi<CT, 2, ar_ulong<CT>(), 1, false>;
+  return pow2 ? (const void*)k_arnoldi<CT, ar_ic<CT>(), 4, 4, true> : (const void*)k_arnoldi<CT, ar_ic<CT>(), 4, 4, false>;
+}
+
+// Largest grid of the cooperative k_arnoldi: one CTA per SM (at most solve_nblk(), the partial-sum rows'
 // length); 0 when the device cannot hold it resident.  Found once per device.
 template <typename CT>
 int arnoldi_grid() {
@@ -760,12 +775,14 @@ int arnoldi_grid() {
   if (dev >= 64) dev = 63;
   int& g = cache[dev];
   if (g < 0) {
-    int per = 0, coop = 0;
+    int coop = 0, per = 1 << 30;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-    int per_long = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_arnoldi<CT, ar_ic<CT>(), 4, 4>, AR_T, 0);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_long, k_arnoldi<CT, 2, ar_ulong<CT>(), 1>, AR_T, 0);
-    per = std::min(per, per_long);
+    for (const void* k : {arnoldi_kernel<CT>(false, true), arnoldi_kernel<CT>(false, false), arnoldi_kernel<CT>(true, true),
+                          arnoldi_kernel<CT>(true, false)}) {
+      int p = 0;
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, k, AR_T, 0);
+      per = std::min(per, p);
+    }
     g = (coop && per > 0) ? std::min(amg_sm_count(), solve_nblk()) : 0;
   }
   return g;
@@ -778,13 +795,18 @@ template <typename CT>
 amg_status solve_impl(amg_coarse* h, long long rows, amg_apply_fn op, const CT* b, CT* x, int nrhs, double tol, int m,
                       int max_applies, cudaStream_t st, double* info, unsigned char* ws, bool poll) {
   const long long vstride = rows * nrhs;
-  const bool flat = nrhs > 1 && 32 % nrhs == 0;  // coalesced flat loops (see k_dots_flat)
-  const int ar_grid = 32 % nrhs == 0 ? arnoldi_grid<CT>() : 0;  // fused step (k_arnoldi) when > 0
+  // Grids: a round of 4 elements per thread where the vector is short, so that a coarse lattice of a few
+  // sites pays no barriers and no sums of CTAs and warps without work (FP64 instructions are scarce: one
+  // warp instruction in 16 cycles per SM).  4^4 in 2^4 blocks, 256 elements in FP64: a coarse-grid
+  // correction takes 97 us, 117 with a CTA of 16 warps, 130 with 152 CTAs.
+  const long long rounds = (vstride + 4 * AR_T - 1) / (4 * AR_T);
+  const int ar_grid = (int)std::min<long long>(arnoldi_grid<CT>(), rounds);  // fused step (k_arnoldi) when > 0
+  const int ar_threads = (int)std::min<long long>(AR_T, (vstride + 127) / 128 * 32);
   SolveWork& sw = h->sw;
   FState s;
   s.m = m;
   s.nrhs = nrhs;
-  const int nblk = solve_nblk();
+  const int nblk = (int)std::min<long long>(solve_nblk(), (vstride + 4 * ST_T - 1) / (4 * ST_T));
   s.nblk = nblk;
   s.rows = rows;
   s.tol = tol;
@@ -794,7 +816,7 @@ amg_status solve_impl(amg_coarse* h, long long rows, amg_apply_fn op, const CT* 
   CT* nxt = cur + vstride;                  // D_c V_j, orthogonalised in place
   p += align256((size_t)(m + 3) * vstride * sizeof(CT));
   s.part = (double2*)p;
-  p += align256((size_t)(m + 1) * nblk * nrhs * sizeof(double2));
+  p += align256((size_t)(m + 1) * solve_nblk() * nrhs * sizeof(double2));
   double2* d2 = (double2*)p;
   s.H = d2;
   d2 += (size_t)nrhs * (m + 1) * m;
@@ -821,7 +843,7 @@ amg_status solve_impl(amg_coarse* h, long long rows, amg_apply_fn op, const CT* 
   s.bar_extra = sw.test_extra_arrivals;
   if (poll) sw.ticket = sw.ticket >= (1 << 30) ? 1 : sw.ticket + 1;  // never 0, the word's initial value
   s.ticket = poll ? sw.ticket : 0;
-  const unsigned egrid = 4 * amg_sm_count();
+  const unsigned egrid = (unsigned)std::min<long long>(4 * amg_sm_count(), (vstride + 4 * ST_T - 1) / (4 * ST_T));
   AMG_CUDA_TRY(cudaMemsetAsync(fl, 0, (4 * (size_t)nrhs + 8) * sizeof(int), st));
   k_residual<CT><<<nblk, ST_T, 0, st>>>(s, cur, b, 1, x);  // also x = 0
   AMG_LAUNCH_CHECK();
@@ -860,18 +882,12 @@ amg_status solve_impl(amg_coarse* h, long long rows, amg_apply_fn op, const CT* 
         const CT* Vr = V;
         int jj = j;
         void* args[] = {&s, &nxt, &Vr, (void*)&vstride, &jj};
-        const void* kern = rows * nrhs > AR_LONG ? (const void*)k_arnoldi<CT, 2, ar_ulong<CT>(), 1>
-                                                 : (const void*)k_arnoldi<CT, ar_ic<CT>(), 4, 4>;
-        AMG_CUDA_TRY(cudaLaunchCooperativeKernel(kern, dim3(ar_grid), dim3(AR_T), args, 0, st));
+        const void* kern = arnoldi_kernel<CT>(rows * nrhs > AR_LONG, 32 % nrhs == 0);
+        AMG_CUDA_TRY(cudaLaunchCooperativeKernel(kern, dim3(ar_grid), dim3(ar_threads), args, 0, st));
         h->launches += 1;
       } else {
-        if (flat) {
-          k_dots_flat<CT><<<dim3(nblk, j + 1), ST_T, 0, st>>>(s, nxt, V, vstride, j);
-          k_update_flat<CT><<<nblk, ST_T, 0, st>>>(s, nxt, V, vstride, j);
-        } else {
-          k_dots<CT><<<dim3(nblk, j + 1), ST_T, 0, st>>>(s, nxt, V, vstride, j);
-          k_update<CT><<<nblk, ST_T, 0, st>>>(s, nxt, V, vstride, j);
-        }
+        k_dots<CT><<<dim3(nblk, j + 1), ST_T, 0, st>>>(s, nxt, V, vstride, j);
+        k_update<CT><<<nblk, ST_T, 0, st>>>(s, nxt, V, vstride, j);
         AMG_LAUNCH_CHECK();
         h->launches += 2;
       }
