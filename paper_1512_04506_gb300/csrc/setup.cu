@@ -10,6 +10,7 @@
 
 #include <stdio.h>
 #include <stdlib.h>
+#include <algorithm>
 #include <vector>
 
 namespace {
@@ -155,28 +156,40 @@ __global__ void clover_kernel(const double2* __restrict__ U, double2* __restrict
 }
 
 // ------------------------------------------------------------------ block reductions
-template <int K>
-__device__ inline void block_sum(double2 (&v)[K], double2* sm) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+// Sum of NV values (a power of two, at most 32) over the warp's lanes; lane l gets the total of value
+// l >> (5 - log2 NV).  Halving the values with the distance takes NV - 1 + (5 - log2 NV) FP64 additions
+// instead of 5 NV.
+template <int NV>
+__device__ inline double warp_totals(double (&v)[NV]) {
+  const int lane = threadIdx.x & 31;
+  int o = 16;
 #pragma unroll
-  for (int k = 0; k < K; ++k)
+  for (int n = NV / 2; n > 0; n /= 2, o >>= 1) {
+    const bool up = lane & o;
 #pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      v[k].x += __shfl_xor_sync(0xffffffffu, v[k].x, o);
-      v[k].y += __shfl_xor_sync(0xffffffffu, v[k].y, o);
-    }
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < K; ++k) sm[warp * K + k] = v[k];
-  __syncthreads();
-  if (threadIdx.x < K) {
-    double2 t = make_double2(0, 0);
-    for (int w = 0; w < nw; ++w) t = cadd(t, sm[w * K + threadIdx.x]);
-    sm[32 * K + threadIdx.x] = t;
+    for (int i = 0; i < NV / 2; ++i)
+      if (i < n) {
+        const double give = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+      }
   }
+  for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  return v[0];
+}
+// CTA sums of NV values: left in out[0 .. NV - 1] (shared; valid after this call's last barrier).
+// sm: [warps][NV]
+template <int NV>
+__device__ inline void block_totals(double (&v)[NV], double* sm, double* out) {
+  constexpr int sh = NV == 32 ? 0 : NV == 16 ? 1 : NV == 8 ? 2 : NV == 4 ? 3 : NV == 2 ? 4 : 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const double t = warp_totals<NV>(v);
+  if ((lane & ((1 << sh) - 1)) == 0) sm[warp * NV + (lane >> sh)] = t;
   __syncthreads();
-#pragma unroll
-  for (int k = 0; k < K; ++k) v[k] = sm[32 * K + k];
+  if (threadIdx.x < NV) {
+    double sum = 0;
+    for (int w = 0; w < nw; ++w) sum += sm[w * NV + threadIdx.x];
+    out[threadIdx.x] = sum;
+  }
   __syncthreads();
 }
 
@@ -184,23 +197,30 @@ __device__ inline void block_sum(double2 (&v)[K], double2* sm) {
 // One CTA per aggregate (blk, h).  The aggregate's test vectors (6 Vb x ntv) are processed in
 // column blocks of NB = 4: each block is projected against all earlier columns with classical
 // Gram-Schmidt (all coefficients from the same vectors), twice, then orthonormalised column by
-// column, again classically and twice.  Element n of the aggregate lives in thread n mod T.
-// Output row j of R_i^h = conj(q_j).
+// column, again classically and twice.  Element n of the aggregate lives in thread n mod T, E elements
+// per thread.  Output row j of R_i^h = conj(q_j).
+//
+// Bound: the FP64 pipes (one warp instruction in 64 cycles per sub-partition): 4 instructions per element and pair
+// of columns in every dot and every update, and as little else as possible: updates add the negated
+// coefficients, sums halve their values as they go down the lanes, one warp takes the roots and
+// reciprocals.  16^4, Ntv 20: 5.5 ms; with a multiplication, a fused one and a subtraction per update,
+// 5 additions per value and lane and roots in every thread 8.8 ms.
 constexpr int GS_NB = 4;
 constexpr int GS_EMAX = 8;
 
+template <int E>
 __global__ void __launch_bounds__(256) gs_kernel(const double2* __restrict__ tv, double2* __restrict__ R,
                                                  Geom g, unsigned* err) {
-  __shared__ double2 red[32 * 16 + 16];
-  __shared__ double2 coef[AMG_MAX_NTV * GS_NB];
+  __shared__ double sm[8 * 32], tot[32], n0[GS_NB], scal;
+  __shared__ double2 coef[AMG_MAX_NTV * GS_NB];  // minus the coefficients
   const long long agg = blockIdx.x;
   const long long blk = agg >> 1;
   const int h = (int)(agg & 1);
   const int T = blockDim.x, tid = threadIdx.x, ntv = g.ntv, nagg = g.nagg;
-  long long tvoff[GS_EMAX];
-  bool valid[GS_EMAX];
+  long long tvoff[E];
+  bool valid[E];
 #pragma unroll
-  for (int e = 0; e < GS_EMAX; ++e) {
+  for (int e = 0; e < E; ++e) {
     const int n = tid + e * T;
     valid[e] = n < nagg;
     tvoff[e] = 0;
@@ -211,23 +231,25 @@ __global__ void __launch_bounds__(256) gs_kernel(const double2* __restrict__ tv,
     }
   }
   double2* Rblk = R + agg * (long long)ntv * nagg;
-  double2 w[GS_EMAX][GS_NB];
+  double2 w[E][GS_NB];
   for (int j0 = 0; j0 < ntv; j0 += GS_NB) {
     const int nb = min(GS_NB, ntv - j0);
 #pragma unroll
-    for (int e = 0; e < GS_EMAX; ++e)
+    for (int e = 0; e < E; ++e)
 #pragma unroll
       for (int c = 0; c < GS_NB; ++c)
         w[e][c] = (valid[e] && c < nb) ? tv[tvoff[e] + j0 + c] : make_double2(0, 0);
-    double2 n0[GS_NB];
+    {
+      double v[GS_NB];
 #pragma unroll
-    for (int c = 0; c < GS_NB; ++c) {
-      double s = 0;
+      for (int c = 0; c < GS_NB; ++c) {
+        v[c] = 0;
 #pragma unroll
-      for (int e = 0; e < GS_EMAX; ++e) s += w[e][c].x * w[e][c].x + w[e][c].y * w[e][c].y;
-      n0[c] = make_double2(s, 0);
+        for (int e = 0; e < E; ++e) v[c] = fma(w[e][c].x, w[e][c].x, fma(w[e][c].y, w[e][c].y, v[c]));
+      }
+      block_totals<GS_NB>(v, sm, tot);
+      if (tid < GS_NB) n0[tid] = tot[tid];
     }
-    block_sum<GS_NB>(n0, red);
     // projection against the earlier column blocks (block classical GS), twice
     for (int pass = 0; pass < 2 && j0 > 0; ++pass) {
       for (int k0 = 0; k0 < j0; k0 += GS_NB) {
@@ -235,7 +257,7 @@ __global__ void __launch_bounds__(256) gs_kernel(const double2* __restrict__ tv,
 #pragma unroll
         for (int q = 0; q < GS_NB * GS_NB; ++q) d[q] = make_double2(0, 0);
 #pragma unroll
-        for (int e = 0; e < GS_EMAX; ++e) {
+        for (int e = 0; e < E; ++e) {
           if (!valid[e]) continue;
           const int n = tid + e * T;
 #pragma unroll
@@ -245,23 +267,26 @@ __global__ void __launch_bounds__(256) gs_kernel(const double2* __restrict__ tv,
             for (int c = 0; c < GS_NB; ++c) cfma(d[kk * GS_NB + c], r, w[e][c]);
           }
         }
-        block_sum<GS_NB * GS_NB>(d, red);
-        if (tid < GS_NB * GS_NB) coef[k0 * GS_NB + tid] = d[tid];
+        double v[2 * GS_NB * GS_NB];
+#pragma unroll
+        for (int q = 0; q < GS_NB * GS_NB; ++q) {
+          v[2 * q] = d[q].x;
+          v[2 * q + 1] = d[q].y;
+        }
+        block_totals<2 * GS_NB * GS_NB>(v, sm, tot);
+        if (tid < GS_NB * GS_NB) coef[k0 * GS_NB + tid] = make_double2(-tot[2 * tid], -tot[2 * tid + 1]);
+        __syncthreads();
       }
-      __syncthreads();
       for (int k0 = 0; k0 < j0; k0 += GS_NB) {
 #pragma unroll
-        for (int e = 0; e < GS_EMAX; ++e) {
+        for (int e = 0; e < E; ++e) {
           if (!valid[e]) continue;
           const int n = tid + e * T;
 #pragma unroll
           for (int kk = 0; kk < GS_NB; ++kk) {
-            const double2 q = cconj(Rblk[(long long)(k0 + kk) * nagg + n]);
+            const double2 r = Rblk[(long long)(k0 + kk) * nagg + n];
 #pragma unroll
-            for (int c = 0; c < GS_NB; ++c) {
-              const double2 cf = coef[(k0 + kk) * GS_NB + c];
-              w[e][c] = csub(w[e][c], cmul(q, cf));
-            }
+            for (int c = 0; c < GS_NB; ++c) cfmac(w[e][c], r, coef[(k0 + kk) * GS_NB + c]);  // w -= q_k coef
           }
         }
       }
@@ -272,37 +297,44 @@ __global__ void __launch_bounds__(256) gs_kernel(const double2* __restrict__ tv,
     for (int c = 0; c < GS_NB; ++c) {
       if (c >= nb) break;
       for (int pass = 0; pass < 2 && c > 0; ++pass) {
-        double2 d[GS_NB];
+        double v[2 * GS_NB];
 #pragma unroll
         for (int cp = 0; cp < GS_NB; ++cp) {
-          d[cp] = make_double2(0, 0);
+          double2 d = make_double2(0, 0);
           if (cp < c)
 #pragma unroll
-            for (int e = 0; e < GS_EMAX; ++e) cfmac(d[cp], w[e][cp], w[e][c]);
+            for (int e = 0; e < E; ++e) cfmac(d, w[e][cp], w[e][c]);
+          v[2 * cp] = d.x;
+          v[2 * cp + 1] = d.y;
         }
-        block_sum<GS_NB>(d, red);
+        block_totals<2 * GS_NB>(v, sm, tot);
 #pragma unroll
-        for (int e = 0; e < GS_EMAX; ++e)
+        for (int cp = 0; cp < GS_NB; ++cp)
+          if (cp < c) {
+            const double2 m = make_double2(-tot[2 * cp], -tot[2 * cp + 1]);
 #pragma unroll
-          for (int cp = 0; cp < GS_NB; ++cp)
-            if (cp < c) w[e][c] = csub(w[e][c], cmul(w[e][cp], d[cp]));
+            for (int e = 0; e < E; ++e) cfma(w[e][c], w[e][cp], m);
+          }
+        __syncthreads();  // tot is read
       }
-      double2 nn[1];
-      double s = 0;
+      double v[1] = {0};
 #pragma unroll
-      for (int e = 0; e < GS_EMAX; ++e) s += w[e][c].x * w[e][c].x + w[e][c].y * w[e][c].y;
-      nn[0] = make_double2(s, 0);
-      block_sum<1>(nn, red);
-      const double nrm = sqrt(nn[0].x);
-      if (!(nrm > 1e-12 * sqrt(n0[c].x))) {
-        if (tid == 0) atomicOr(err, AMG_EBIT_RANK);
+      for (int e = 0; e < E; ++e) v[0] = fma(w[e][c].x, w[e][c].x, fma(w[e][c].y, w[e][c].y, v[0]));
+      block_totals<1>(v, sm, tot);
+      if (tid < 32) {
+        const double nrm = sqrt(tot[0]);
+        if (tid == 0) {
+          if (!(nrm > 1e-12 * sqrt(n0[c]))) atomicOr(err, AMG_EBIT_RANK);
+          scal = nrm > 0 ? 1.0 / nrm : 0.0;
+        }
       }
-      const double inv = nrm > 0 ? 1.0 / nrm : 0.0;
+      __syncthreads();
+      const double inv = scal;
 #pragma unroll
-      for (int e = 0; e < GS_EMAX; ++e) w[e][c] = cscale(w[e][c], inv);
+      for (int e = 0; e < E; ++e) w[e][c] = cscale(w[e][c], inv);
     }
 #pragma unroll
-    for (int e = 0; e < GS_EMAX; ++e) {
+    for (int e = 0; e < E; ++e) {
       if (!valid[e]) continue;
       const int n = tid + e * T;
 #pragma unroll
@@ -322,12 +354,57 @@ __global__ void __launch_bounds__(256) gs_kernel(const double2* __restrict__ tv,
 // the +mu face to F_mu.  Job 4 sums P(x)^dagger ((4+m0) + C(x)) P(x) with both chiralities
 // stacked in the same 6 rows (only the chirality-diagonal quadrants are kept).
 // b_mu: -i sigma_x, -i sigma_y, -i sigma_z, 1.
-__device__ inline double2 bmat(int mu, int a, int b) {
-  if (mu == 0) return (a != b) ? make_double2(0, -1) : make_double2(0, 0);
-  if (mu == 1) return (a == 0 && b == 1) ? make_double2(-1, 0) : ((a == 1 && b == 0) ? make_double2(1, 0) : make_double2(0, 0));
-  if (mu == 2) return (a == b) ? make_double2(0, a == 0 ? -1 : 1) : make_double2(0, 0);
-  return (a == b) ? make_double2(1, 0) : make_double2(0, 0);
+//
+// Bound: the FP64 pipes (one warp instruction in 64 cycles per SM sub-partition), so what counts is the
+// number of FP64 warp instructions per sub-partition.  Each thread keeps a TA x TC tile of the sum; the
+// CTA has a multiple of four warps, and where the tiles fill fewer, groups of warps share out the
+// sites; the tile shape is the one that needs the fewest instructions so, links leaving through the face come last so that one set of
+// accumulators serves S_mu and F_mu, the self job works on the tiles that its quadrants need, and the
+// factors b_mu (+-1, +-i) only move words and flip signs in the integer pipe.  16^4, Ntv 20: 21.9 ms;
+// 2 x 4 tiles in two accumulator sets, all tiles of the self job and b_mu as products took 30.1 ms.
+__device__ inline double flip(double v) {  // -v off the FP64 pipe
+  return __hiloint2double(__double2hiint(v) ^ (int)0x80000000, __double2loint(v));
 }
+__device__ inline double2 conj_i(double2 z) { return make_double2(z.x, flip(z.y)); }
+// row a of -b_mu z, z the entry of spin b(a) = 1 - a (mu < 2), a (mu >= 2)
+__device__ inline double2 neg_b(int mu, int a, double2 z) {
+  if (mu == 0 || (mu == 2 && a == 0)) return make_double2(flip(z.y), z.x);  // i z
+  if (mu == 2) return make_double2(z.y, flip(z.x));                         // -i z
+  if (mu == 1 && a == 0) return z;
+  return make_double2(flip(z.x), flip(z.y));
+}
+// visiting order t -> local site: the sites with l_mu = B_mu - 1 last
+__device__ inline int face_last(int t, int nface, int stride, int Bmu) {
+  const int lmu = t / nface, r = t % nface;
+  return (r / stride) * (stride * Bmu) + lmu * stride + (r % stride);
+}
+
+// The TA x TC tiles of the nc x nc sum that a job needs: all, or (self) those that meet a
+// chirality-diagonal quadrant
+struct Tiles {
+  int nta, ntc, TA, TC, ntv;
+  bool self;
+  __host__ __device__ int first(int ta) const { return self && ta * TA >= ntv ? ntv / TC : 0; }
+  __host__ __device__ int last(int ta) const { return self && ta * TA + TA <= ntv ? (ntv + TC - 1) / TC : ntc; }
+  __host__ __device__ int count() const {
+    if (!self) return nta * ntc;
+    int n = 0;
+    for (int ta = 0; ta < nta; ++ta) n += last(ta) - first(ta);
+    return n;
+  }
+  __host__ __device__ bool at(int k, int& ta, int& tc) const {  // the k-th of them
+    tc = 0;
+    for (ta = 0; ta < nta; ++ta) {
+      const int n = last(ta) - first(ta);
+      if (k < n) {
+        tc = first(ta) + k;
+        return true;
+      }
+      k -= n;
+    }
+    return false;
+  }
+};
 
 template <int TA, int TC>
 __global__ void __launch_bounds__(256) assemble_kernel(const double2* __restrict__ R, const double2* __restrict__ U,
@@ -339,157 +416,141 @@ __global__ void __launch_bounds__(256) assemble_kernel(const double2* __restrict
   const int nc = g.nc, ntv = g.ntv, nagg = g.nagg, Vb = (int)g.Vb;
   double2* As = smem;                        // [sb][6][ncp]
   double2* Bs = smem + (size_t)sb_max * 6 * ncp;
-  const int ntc = ncp / TC, nta = ncp / TA, ntiles = ntc * nta;
-  const int tid = threadIdx.x;
-  const int ta = tid / ntc, tc = tid % ntc;
-  double2 acc0[TA][TC], acc1[TA][TC];
+  const int nta = (nc + TA - 1) / TA, ntc = (nc + TC - 1) / TC;
+  const int tid = threadIdx.x, nwarp = blockDim.x >> 5;
+  // tiles of this job over tw warps; the CTA's warps form KG groups that share out the sites
+  const Tiles need{nta, ntc, TA, TC, ntv, job == 4};
+  const int tw = (need.count() + 31) / 32, KG = max(1, nwarp / tw), kg = (tid >> 5) / tw, lt = tid - kg * tw * 32;
+  int ta, tc;
+  const bool active = need.at(lt, ta, tc) && kg < KG;
+  double2 acc[TA][TC];
 #pragma unroll
   for (int i = 0; i < TA; ++i)
 #pragma unroll
-    for (int j = 0; j < TC; ++j) acc0[i][j] = acc1[i][j] = make_double2(0, 0);
+    for (int j = 0; j < TC; ++j) acc[i][j] = make_double2(0, 0);
+  double2* P0 = part + ((blk * 5 + job) * 2 + 0) * (long long)nc * nc;
+  auto write = [&](double2* P) {  // sum over the groups (through shared memory), then out; clears the tiles
+    if (active && kg > 0)
+#pragma unroll
+      for (int i = 0; i < TA; ++i)
+#pragma unroll
+        for (int jj = 0; jj < TC; ++jj) smem[(((kg - 1) * TA + i) * TC + jj) * tw * 32 + lt] = acc[i][jj];
+    __syncthreads();
+    for (int q = 1; active && kg == 0 && q < KG; ++q)
+#pragma unroll
+      for (int i = 0; i < TA; ++i)
+#pragma unroll
+        for (int jj = 0; jj < TC; ++jj) acc[i][jj] = cadd(acc[i][jj], smem[(((q - 1) * TA + i) * TC + jj) * tw * 32 + lt]);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < TA; ++i)
+#pragma unroll
+      for (int jj = 0; jj < TC; ++jj) {
+        const int a = ta * TA + i, c = tc * TC + jj;
+        if (active && kg == 0 && a < nc && c < nc) P[a * nc + c] = acc[i][jj];
+        acc[i][jj] = make_double2(0, 0);
+      }
+  };
   // coarse coordinates of this block and stride of direction mu inside a block
-  int Xc[4];
+  int X[4];
   {
     long long r = blk;
     for (int m = 0; m < 4; ++m) {
-      Xc[m] = (int)(r % g.Lc[m]);
+      X[m] = (int)(r % g.Lc[m]);
       r /= g.Lc[m];
     }
   }
   const int mu = job < 4 ? job : 0;
   int stride_mu = 1;
   for (int m = 0; m < mu; ++m) stride_mu *= g.B[m];
-  long long blk_fwd;
-  {
-    int X[4] = {Xc[0], Xc[1], Xc[2], Xc[3]};
-    X[mu] = (X[mu] + 1) % g.Lc[mu];
-    blk_fwd = ((long long)(X[3] * g.Lc[2] + X[2]) * g.Lc[1] + X[1]) * g.Lc[0] + X[0];
+  X[mu] = (X[mu] + 1) % g.Lc[mu];
+  const long long blk_fwd = ((long long)(X[3] * g.Lc[2] + X[2]) * g.Lc[1] + X[1]) * g.Lc[0] + X[0];
+  const int Bmu = g.B[mu], nface = job < 4 ? Vb / Bmu : 0;
+  int end = Vb - nface;  // the links inside the block first
+  if (end == 0) {
+    write(P0);  // S_mu of a block of extent 1: none
+    end = Vb;
   }
-  for (int s0 = 0; s0 < Vb; s0 += sb_max) {
-    const int nsb = min(sb_max, Vb - s0);
-    for (int pr = tid; pr < sb_max * ncp; pr += blockDim.x) {
+  for (int s0 = 0, nsb = 0; s0 < Vb; s0 += nsb) {
+    nsb = min(sb_max, end - s0);
+    for (int pr = tid; pr < nsb * ncp; pr += blockDim.x) {
       const int sb = pr / ncp, c = pr % ncp;
-      double2 A[6], Bt[6];
+      double2 *Ao = As + (size_t)sb * 6 * ncp + c, *Bo = Bs + (size_t)sb * 6 * ncp + c;
+      if (c >= nc) {
 #pragma unroll
-      for (int k = 0; k < 6; ++k) A[k] = Bt[k] = make_double2(0, 0);
-      if (sb < nsb && c < nc) {
-        const int sl = s0 + sb;
-        const long long site = block_site(g, blk, sl);
-        const int hc = c / ntv, j = c % ntv;
-        const double2* Rc = R + ((blk * 2 + hc) * (long long)ntv + j) * nagg + sl * 6;
-        double2 q[6];
-#pragma unroll
-        for (int k = 0; k < 6; ++k) q[k] = cconj(Rc[k]);
-        if (job < 4) {
-          // A = u^dagger P(x): l columns keep the l rows, r columns give -b_mu P_r
-          if (hc == 0) {
-#pragma unroll
-            for (int k = 0; k < 6; ++k) A[k] = q[k];
-          } else {
-#pragma unroll
-            for (int a = 0; a < 2; ++a)
-#pragma unroll
-              for (int col = 0; col < 3; ++col) {
-                double2 t = make_double2(0, 0);
-#pragma unroll
-                for (int b = 0; b < 2; ++b) cfma(t, bmat(mu, a, b), q[b * 3 + col]);
-                A[a * 3 + col] = cscale(t, -1.0);
-              }
-          }
-          // neighbour x + mu and its block
-          const int lmu = (sl / stride_mu) % g.B[mu];
-          const bool face = lmu == g.B[mu] - 1;
-          const int sn = face ? sl - (g.B[mu] - 1) * stride_mu : sl + stride_mu;
-          const long long bn = face ? blk_fwd : blk;
-          const double2* Rn = R + ((bn * 2 + hc) * (long long)ntv + j) * nagg + sn * 6;
-          double2 qn[6];
-#pragma unroll
-          for (int k = 0; k < 6; ++k) qn[k] = cconj(Rn[k]);
-          const double2* Ul = U + (site * 4 + mu) * 9;
-          double2 z[6];
-#pragma unroll
-          for (int b = 0; b < 2; ++b)
-#pragma unroll
-            for (int col = 0; col < 3; ++col) {
-              double2 t = make_double2(0, 0);
-#pragma unroll
-              for (int cp = 0; cp < 3; ++cp) cfma(t, Ul[col * 3 + cp], qn[b * 3 + cp]);
-              z[b * 3 + col] = t;
-            }
-          if (hc == 0) {
-#pragma unroll
-            for (int k = 0; k < 6; ++k) Bt[k] = z[k];
-          } else {
-#pragma unroll
-            for (int a = 0; a < 2; ++a)
-#pragma unroll
-              for (int col = 0; col < 3; ++col) {
-                double2 t = make_double2(0, 0);
-#pragma unroll
-                for (int b = 0; b < 2; ++b) cfma(t, bmat(mu, a, b), z[b * 3 + col]);
-                Bt[a * 3 + col] = cscale(t, -1.0);
-              }
-          }
-        } else {
-          const double2* C6 = clov + (site * 2 + hc) * 36;
-#pragma unroll
-          for (int k = 0; k < 6; ++k) {
-            A[k] = q[k];
-            double2 t = cscale(q[k], 4.0 + m0);
-#pragma unroll
-            for (int kp = 0; kp < 6; ++kp) cfma(t, C6[k * 6 + kp], q[kp]);
-            Bt[k] = t;
-          }
-        }
+        for (int k = 0; k < 6; ++k) Ao[k * ncp] = Bo[k * ncp] = make_double2(0, 0);
+        continue;
       }
+      const int sl = job < 4 ? face_last(s0 + sb, nface, stride_mu, Bmu) : s0 + sb;
+      const long long site = block_site(g, blk, sl);
+      const int hc = c / ntv, j = c % ntv;
+      const double2* Rc = R + ((blk * 2 + hc) * (long long)ntv + j) * nagg + sl * 6;
+      double2 q[6];
 #pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        As[((size_t)sb * 6 + k) * ncp + c] = A[k];
-        Bs[((size_t)sb * 6 + k) * ncp + c] = Bt[k];
+      for (int k = 0; k < 6; ++k) q[k] = conj_i(Rc[k]);
+      if (job < 4) {
+        // A = u^dagger P(x): l columns keep the l rows, r columns give -b_mu P_r; Bt the same of
+        // U_mu(x) P(x + mu), with the neighbour and its block
+        const bool face = s0 + sb >= Vb - nface;
+        const int sn = face ? sl - (Bmu - 1) * stride_mu : sl + stride_mu;
+        const double2* Rn = R + (((face ? blk_fwd : blk) * 2 + hc) * (long long)ntv + j) * nagg + sn * 6;
+        const double2* Ul = U + (site * 4 + mu) * 9;
+        double2 qn[6], z[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) qn[k] = conj_i(Rn[k]);
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+          for (int col = 0; col < 3; ++col) {
+            double2 t = make_double2(0, 0);
+#pragma unroll
+            for (int cp = 0; cp < 3; ++cp) cfma(t, Ul[col * 3 + cp], qn[b * 3 + cp]);
+            z[b * 3 + col] = t;
+          }
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+          for (int col = 0; col < 3; ++col) {
+            const int k = a * 3 + col, kb = (1 - a) * 3 + col;
+            Ao[k * ncp] = hc == 0 ? q[k] : neg_b(mu, a, mu < 2 ? q[kb] : q[k]);
+            Bo[k * ncp] = hc == 0 ? z[k] : neg_b(mu, a, mu < 2 ? z[kb] : z[k]);
+          }
+      } else {
+        const double2* C6 = clov + (site * 2 + hc) * 36;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+          Ao[k * ncp] = q[k];
+          double2 t = cscale(q[k], 4.0 + m0);
+#pragma unroll
+          for (int kp = 0; kp < 6; ++kp) cfma(t, C6[k * 6 + kp], q[kp]);
+          Bo[k * ncp] = t;
+        }
       }
     }
     __syncthreads();
-    if (tid < ntiles) {
-      for (int sb = 0; sb < nsb; ++sb) {
-        const int sl = s0 + sb;
-        const bool face = job < 4 && ((sl / stride_mu) % g.B[mu]) == g.B[mu] - 1;
-#pragma unroll
+    if (active) {
+      for (int sb = kg; sb < nsb; sb += KG) {
+#pragma unroll 1
         for (int k = 0; k < 6; ++k) {
           double2 av[TA], bv[TC];
 #pragma unroll
           for (int i = 0; i < TA; ++i) av[i] = As[((size_t)sb * 6 + k) * ncp + ta * TA + i];
 #pragma unroll
           for (int jj = 0; jj < TC; ++jj) bv[jj] = Bs[((size_t)sb * 6 + k) * ncp + tc * TC + jj];
-          if (face) {
 #pragma unroll
-            for (int i = 0; i < TA; ++i)
+          for (int i = 0; i < TA; ++i)
 #pragma unroll
-              for (int jj = 0; jj < TC; ++jj) cfmac(acc1[i][jj], av[i], bv[jj]);
-          } else {
-#pragma unroll
-            for (int i = 0; i < TA; ++i)
-#pragma unroll
-              for (int jj = 0; jj < TC; ++jj) cfmac(acc0[i][jj], av[i], bv[jj]);
-          }
+            for (int jj = 0; jj < TC; ++jj) cfmac(acc[i][jj], av[i], bv[jj]);
         }
       }
     }
     __syncthreads();
+    if (s0 + nsb == end && end < Vb) {
+      write(P0);  // S_mu
+      end = Vb;
+    }
   }
-  if (tid < ntiles) {
-    double2* P0 = part + ((blk * 5 + job) * 2 + 0) * (long long)nc * nc;
-    double2* P1 = P0 + (long long)nc * nc;
-#pragma unroll
-    for (int i = 0; i < TA; ++i)
-#pragma unroll
-      for (int jj = 0; jj < TC; ++jj) {
-        const int a = ta * TA + i, c = tc * TC + jj;
-        if (a < nc && c < nc) {
-          P0[a * nc + c] = acc0[i][jj];
-          P1[a * nc + c] = acc1[i][jj];
-        }
-      }
-  }
+  write(job < 4 ? P0 + (long long)nc * nc : P0);  // F_mu, or the self block
 }
 
 // D_c blocks from the partial sums:
@@ -588,6 +649,60 @@ __global__ void r_to_fp32_kernel(const double2* __restrict__ R, float2* __restri
 // ------------------------------------------------------------------ host driver
 static int round_up(int a, int b) { return (a + b - 1) / b * b; }
 
+// Warps of the assembly's CTA: the hop jobs' tiles, rounded up to a multiple of four
+static int assemble_warps(int nc, int ta, int tc) {
+  return round_up((((nc + ta - 1) / ta) * ((nc + tc - 1) / tc) + 31) / 32, 4);
+}
+
+template <int TA, int TC>
+static amg_status launch_assemble_tile(const Geom& g, const double2* R, const double2* U, const double2* clov,
+                                       double2* part, double m0, cudaStream_t st) {
+  const int ncp = std::max(round_up(g.nc, TA), round_up(g.nc, TC));
+  const int nta = (g.nc + TA - 1) / TA, ntc = (g.nc + TC - 1) / TC, W = assemble_warps(g.nc, TA, TC), T = 32 * W;
+  if (T > 256) return AMG_ERR_UNSUPPORTED;
+  int sb = 8;  // sites per chunk: several CTAs per SM, so that one builds while others contract
+  while (sb > 4 && (size_t)sb * 12 * ncp * sizeof(double2) > 40 * 1024) sb >>= 1;
+  size_t words = (size_t)sb * 12 * ncp;
+  for (int self = 0; self < 2; ++self) {  // the groups' tiles on their way to the first group
+    const int tw = (Tiles{nta, ntc, TA, TC, g.ntv, self != 0}.count() + 31) / 32;
+    words = std::max(words, (size_t)(std::max(1, W / tw) - 1) * TA * TC * tw * 32);
+  }
+  const size_t sm = words * sizeof(double2);
+  AMG_CUDA_TRY(cudaFuncSetAttribute(assemble_kernel<TA, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  assemble_kernel<TA, TC><<<dim3((unsigned)g.Vc, 5), T, sm, st>>>(R, U, clov, part, g, m0, ncp, sb);
+  AMG_LAUNCH_CHECK();
+  return AMG_OK;
+}
+
+// The tile shape with the fewest FP64 instructions per row and sub-partition (2 Ntv = 40: 5 x 5, two groups
+// of two warps; 48: 3 x 6, four warps; 16: 2 x 4, four groups of one warp).
+static amg_status launch_assemble(const Geom& g, const double2* R, const double2* U, const double2* clov, double2* part,
+                                  double m0, cudaStream_t st) {
+  constexpr int shapes[][2] = {{5, 5}, {6, 4}, {4, 4}, {3, 6}, {2, 4}, {3, 2}, {2, 2}};
+  int best = -1;
+  double cost = 0;
+  for (int k = 0; k < 7; ++k) {
+    const int ta = shapes[k][0], tc = shapes[k][1], W = assemble_warps(g.nc, ta, tc);
+    if (W > 8) continue;
+    const int tw = (((g.nc + ta - 1) / ta) * ((g.nc + tc - 1) / tc) + 31) / 32;
+    const double c = (double)(W / 4) * ta * tc / (W / tw);
+    if (best < 0 || c < cost) {
+      best = k;
+      cost = c;
+    }
+  }
+  switch (best) {
+    case 0: return launch_assemble_tile<5, 5>(g, R, U, clov, part, m0, st);
+    case 1: return launch_assemble_tile<6, 4>(g, R, U, clov, part, m0, st);
+    case 2: return launch_assemble_tile<4, 4>(g, R, U, clov, part, m0, st);
+    case 3: return launch_assemble_tile<3, 6>(g, R, U, clov, part, m0, st);
+    case 4: return launch_assemble_tile<2, 4>(g, R, U, clov, part, m0, st);
+    case 5: return launch_assemble_tile<3, 2>(g, R, U, clov, part, m0, st);
+    case 6: return launch_assemble_tile<2, 2>(g, R, U, clov, part, m0, st);
+    default: return AMG_ERR_UNSUPPORTED;
+  }
+}
+
 // The setup's steps; the caller owns the timing events and frees `part` if a step fails.
 static amg_status setup_body(amg_coarse* h, const double2* U, const double2* tv, cudaStream_t st, cudaEvent_t (&ev)[5],
                              double2*& part) {
@@ -607,7 +722,9 @@ static amg_status setup_body(amg_coarse* h, const double2* U, const double2* tv,
   if (gs_pair == AMG_ERR_UNSUPPORTED) {
     int T = round_up(g.nagg < 256 ? g.nagg : 256, 32);
     if ((g.nagg + T - 1) / T > GS_EMAX) return AMG_ERR_UNSUPPORTED;
-    gs_kernel<<<(unsigned)(g.Vc * 2), T, 0, st>>>(tv, h->R64, g, h->err);
+    void (*const gs[GS_EMAX])(const double2*, double2*, Geom, unsigned*) = {
+        gs_kernel<1>, gs_kernel<2>, gs_kernel<3>, gs_kernel<4>, gs_kernel<5>, gs_kernel<6>, gs_kernel<7>, gs_kernel<8>};
+    gs[(g.nagg + T - 1) / T - 1]<<<(unsigned)(g.Vc * 2), T, 0, st>>>(tv, h->R64, g, h->err);
     AMG_LAUNCH_CHECK();
   } else if (gs_pair != AMG_OK) {
     return gs_pair;
@@ -619,25 +736,7 @@ static amg_status setup_body(amg_coarse* h, const double2* U, const double2* tv,
   if (h->p.setup_arith == AMG_SETUP_F32PAIR) {
     AMG_TRY_INTERNAL(amg_internal_assemble_pair(g, h->R64, U, h->clover, part, h->p.m0, h->err, st));
   } else {
-    // 2x4 register tiles up to 2 ntv = 40, 4x4 tiles up to 2 ntv = 64; at most 256 threads
-    const bool big = g.nc > 40;
-    const int TA = big ? 4 : 2, TC = 4;
-    const int ncp = round_up(g.nc, 4);
-    const int ntiles = (ncp / TA) * (ncp / TC);
-    const int T = round_up(ntiles < 128 ? 128 : ntiles, 32);
-    if (T > 256) return AMG_ERR_UNSUPPORTED;
-    int sb = 8;
-    while (sb > 1 && (size_t)sb * 12 * ncp * sizeof(double2) > 96 * 1024) sb >>= 1;
-    const size_t sm = (size_t)sb * 12 * ncp * sizeof(double2);
-    dim3 grid((unsigned)g.Vc, 5);
-    if (big) {
-      AMG_CUDA_TRY(cudaFuncSetAttribute(assemble_kernel<4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-      assemble_kernel<4, 4><<<grid, T, sm, st>>>(h->R64, U, h->clover, part, g, h->p.m0, ncp, sb);
-    } else {
-      AMG_CUDA_TRY(cudaFuncSetAttribute(assemble_kernel<2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-      assemble_kernel<2, 4><<<grid, T, sm, st>>>(h->R64, U, h->clover, part, g, h->p.m0, ncp, sb);
-    }
-    AMG_LAUNCH_CHECK();
+    AMG_TRY_INTERNAL(launch_assemble(g, h->R64, U, h->clover, part, h->p.m0, st));
   }
   {
     const long long total = g.Vc * 9LL * g.nc * g.nc;

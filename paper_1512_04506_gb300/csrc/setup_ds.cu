@@ -89,6 +89,11 @@ __device__ __forceinline__ void lacc_fmac(lacc& s, const pc& a, const pc& b) {
   pair_fma(s.ih, s.il, a.rh, a.rl, b.ih, b.il);
   pair_fma(s.ih, s.il, -a.ih, -a.il, b.rh, b.rl);
 }
+// s.r += |a|^2
+__device__ __forceinline__ void lacc_norm(lacc& s, const pc& a) {
+  pair_fma(s.rh, s.rl, a.rh, a.rl, a.rh, a.rl);
+  pair_fma(s.rh, s.rl, a.ih, a.il, a.ih, a.il);
+}
 __device__ __forceinline__ pc lacc_value(const lacc& s) {  // normalised pair (|l| <= ulp(h) / 2)
   pc r;
   two_sum(s.rh, s.rl, r.rh, r.rl);
@@ -449,7 +454,11 @@ assemble_pair_ws_kernel(const double2* __restrict__ R, const double2* __restrict
 // applied twice, then the block's columns one by one, again twice) with every value a pair of
 // floats.  One CTA of up to 512 threads per aggregate; element n of the aggregate in thread n mod T
 // (at most GS_PE elements per thread).  Block sums: pair sums per thread, warp shuffles with pair
-// additions (TwoSum on both parts), then one warp over the warps' partial sums.
+// additions (TwoSum on both parts), then the warps' partial sums (pair_totals).
+//
+// Bound: the FP32 pipes (12 operations per real multiply-add).  16^3 x 32, Ntv 24: 6.4 ms; with every sum
+// taken down all 32 lanes (more additions than the dots themselves), the warps' sums one after the
+// other by one warp and roots in every thread 11.0 ms.
 constexpr int GS_PNB = 4;  // columns per block
 constexpr int GS_PKG = 2;  // earlier columns per dot-product round
 constexpr int GS_PE = 3;   // elements per thread: aggregates of up to 3 x 512 = 1536 = 6 x 4^4 entries
@@ -462,51 +471,40 @@ __device__ __forceinline__ void pair_add(float& h, float& l, float h2, float l2)
   two_sum(s, t, h, l);
   l = __fadd_rn(l, w);
 }
-__device__ __forceinline__ void pc_add(pc& a, const pc& b) {
-  pair_add(a.rh, a.rl, b.rh, b.rl);
-  pair_add(a.ih, a.il, b.ih, b.il);
-}
-__device__ __forceinline__ pc pc_shfl_xor(const pc& a, int o) {
-  return pc{__shfl_xor_sync(0xffffffffu, a.rh, o), __shfl_xor_sync(0xffffffffu, a.ih, o),
-            __shfl_xor_sync(0xffffffffu, a.rl, o), __shfl_xor_sync(0xffffffffu, a.il, o)};
-}
-// CTA sum of K complex pairs; every thread gets the sums.  red: [32][K] float4.
-template <int K>
-__device__ inline void pc_block_sum(pc (&v)[K], float4* red) {
+// CTA sums of NV pairs (a power of two, 2 <= NV <= 32, at most 16 warps): left in out[0 .. NV - 1] (shared,
+// valid after the call).  red: [16][NV].  The values are halved as they go down the lanes (NV - 1 pair
+// additions and shuffles, then the rest plainly, instead of 5 NV), and the warps' sums are added by 16
+// lanes per value at once instead of value after value in one warp.
+template <int NV>
+__device__ inline void pair_totals(float (&h)[NV], float (&l)[NV], float2* red, float2* out) {
+  constexpr int sh = NV == 32 ? 0 : NV == 16 ? 1 : NV == 8 ? 2 : NV == 4 ? 3 : 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  int o = 16;
 #pragma unroll
-  for (int k = 0; k < K; ++k)
+  for (int n = NV / 2; n > 0; n /= 2, o >>= 1) {
+    const bool up = lane & o;
 #pragma unroll
-    for (int o = 16; o; o >>= 1) pc_add(v[k], pc_shfl_xor(v[k], o));
-  __syncthreads();  // red may still be read by the previous call
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < K; ++k) red[warp * K + k] = make_float4(v[k].rh, v[k].ih, v[k].rl, v[k].il);
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      pc t = pc{0.f, 0.f, 0.f, 0.f};
-      if (lane < nw) {
-        const float4 f = red[lane * K + k];
-        t = pc{f.x, f.y, f.z, f.w};
+    for (int i = 0; i < NV / 2; ++i)
+      if (i < n) {
+        const float gh = up ? h[i] : h[i + n], gl = up ? l[i] : l[i + n];
+        h[i] = up ? h[i + n] : h[i];
+        l[i] = up ? l[i + n] : l[i];
+        pair_add(h[i], l[i], __shfl_xor_sync(0xffffffffu, gh, o), __shfl_xor_sync(0xffffffffu, gl, o));
       }
+  }
+  for (; o > 0; o >>= 1)
+    pair_add(h[0], l[0], __shfl_xor_sync(0xffffffffu, h[0], o), __shfl_xor_sync(0xffffffffu, l[0], o));
+  if ((lane & ((1 << sh) - 1)) == 0) red[warp * NV + (lane >> sh)] = make_float2(h[0], l[0]);
+  __syncthreads();
+  for (int t = threadIdx.x; t < 16 * NV; t += blockDim.x) {
+    const int v = t >> 4, w = t & 15;
+    float2 f = w < nw ? red[w * NV + v] : make_float2(0.f, 0.f);
 #pragma unroll
-      for (int o = 16; o; o >>= 1) pc_add(t, pc_shfl_xor(t, o));
-      v[k] = t;
-    }
+    for (int q = 8; q; q >>= 1)
+      pair_add(f.x, f.y, __shfl_xor_sync(0xffffffffu, f.x, q), __shfl_xor_sync(0xffffffffu, f.y, q));
+    if (w == 0) out[v] = f;
   }
   __syncthreads();
-  if (warp == 0)
-#pragma unroll
-    for (int k = 0; k < K; ++k)
-      if (lane == k) red[32 * K + k] = make_float4(v[k].rh, v[k].ih, v[k].rl, v[k].il);
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const float4 f = red[32 * K + k];
-    v[k] = pc{f.x, f.y, f.z, f.w};
-  }
 }
 __device__ __forceinline__ pc pc_mul_sub(const pc& w, const pc& q, const pc& cf) {  // w - q cf
   lacc s{w.rh, w.rl, w.ih, w.il};
@@ -516,8 +514,9 @@ __device__ __forceinline__ pc pc_mul_sub(const pc& w, const pc& q, const pc& cf)
 
 __global__ void __launch_bounds__(512) gs_pair_kernel(const double2* __restrict__ tv, double2* __restrict__ R, Geom g,
                                                       unsigned* err) {
-  __shared__ float4 red[32 * GS_PKG * GS_PNB + GS_PKG * GS_PNB];
+  __shared__ float2 red[16 * 2 * GS_PKG * GS_PNB], tot[2 * GS_PKG * GS_PNB];
   __shared__ float4 coef[AMG_MAX_NTV * GS_PNB];
+  __shared__ float2 scal;
   const long long agg = blockIdx.x;
   const long long blk = agg >> 1;
   const int h = (int)(agg & 1);
@@ -546,17 +545,17 @@ __global__ void __launch_bounds__(512) gs_pair_kernel(const double2* __restrict_
       for (int c = 0; c < GS_PNB; ++c) w[e][c] = (valid[e] && c < nb) ? split_c(tv[tvoff[e] + j0 + c]) : zero;
     double n0[GS_PNB];
     {
-      pc nn[GS_PNB];
+      float nh[GS_PNB], nl[GS_PNB];
 #pragma unroll
       for (int c = 0; c < GS_PNB; ++c) {
         lacc s{0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int e = 0; e < GS_PE; ++e) lacc_fmac(s, w[e][c], w[e][c]);
-        nn[c] = lacc_value(s);
+        for (int e = 0; e < GS_PE; ++e) lacc_norm(s, w[e][c]);
+        two_sum(s.rh, s.rl, nh[c], nl[c]);
       }
-      pc_block_sum<GS_PNB>(nn, red);
+      pair_totals<GS_PNB>(nh, nl, red, tot);
 #pragma unroll
-      for (int c = 0; c < GS_PNB; ++c) n0[c] = (double)nn[c].rh + (double)nn[c].rl;
+      for (int c = 0; c < GS_PNB; ++c) n0[c] = (double)tot[c].x + (double)tot[c].y;
     }
     // projection against the earlier columns (all coefficients from the same vectors), twice
     for (int pass = 0; pass < 2 && j0 > 0; ++pass) {
@@ -576,13 +575,15 @@ __global__ void __launch_bounds__(512) gs_pair_kernel(const double2* __restrict_
             for (int c = 0; c < GS_PNB; ++c) lacc_fma(da[kk * GS_PNB + c], r, w[e][c]);
           }
         }
-        pc d[GS_PKG * GS_PNB];
+        float dh[2 * GS_PKG * GS_PNB], dl[2 * GS_PKG * GS_PNB];
 #pragma unroll
-        for (int q = 0; q < GS_PKG * GS_PNB; ++q) d[q] = lacc_value(da[q]);
-        pc_block_sum<GS_PKG * GS_PNB>(d, red);
-#pragma unroll
-        for (int q = 0; q < GS_PKG * GS_PNB; ++q)
-          if (tid == q && k0 + q / GS_PNB < j0) coef[k0 * GS_PNB + q] = make_float4(d[q].rh, d[q].ih, d[q].rl, d[q].il);
+        for (int q = 0; q < GS_PKG * GS_PNB; ++q) {
+          two_sum(da[q].rh, da[q].rl, dh[2 * q], dl[2 * q]);
+          two_sum(da[q].ih, da[q].il, dh[2 * q + 1], dl[2 * q + 1]);
+        }
+        pair_totals<2 * GS_PKG * GS_PNB>(dh, dl, red, tot);
+        if (tid < GS_PKG * GS_PNB && k0 + tid / GS_PNB < j0)
+          coef[k0 * GS_PNB + tid] = make_float4(tot[2 * tid].x, tot[2 * tid + 1].x, tot[2 * tid].y, tot[2 * tid + 1].y);
       }
       __syncthreads();
       // w -= sum_k q_k coef_k in unnormalised pairs, renormalised every 8 columns
@@ -624,40 +625,49 @@ __global__ void __launch_bounds__(512) gs_pair_kernel(const double2* __restrict_
     for (int c = 0; c < GS_PNB; ++c) {
       if (c >= nb) break;
       for (int pass = 0; pass < 2 && c > 0; ++pass) {
-        pc d[GS_PNB];
+        float dh[2 * GS_PNB], dl[2 * GS_PNB];
 #pragma unroll
         for (int cp = 0; cp < GS_PNB; ++cp) {
           lacc s{0.f, 0.f, 0.f, 0.f};
           if (cp < c)
 #pragma unroll
             for (int e = 0; e < GS_PE; ++e) lacc_fmac(s, w[e][cp], w[e][c]);
-          d[cp] = lacc_value(s);
+          two_sum(s.rh, s.rl, dh[2 * cp], dl[2 * cp]);
+          two_sum(s.ih, s.il, dh[2 * cp + 1], dl[2 * cp + 1]);
         }
-        pc_block_sum<GS_PNB>(d, red);
+        pair_totals<2 * GS_PNB>(dh, dl, red, tot);
 #pragma unroll
-        for (int e = 0; e < GS_PE; ++e)
+        for (int cp = 0; cp < GS_PNB; ++cp)
+          if (cp < c) {
+            const pc d{tot[2 * cp].x, tot[2 * cp + 1].x, tot[2 * cp].y, tot[2 * cp + 1].y};
 #pragma unroll
-          for (int cp = 0; cp < GS_PNB; ++cp)
-            if (cp < c) w[e][c] = pc_mul_sub(w[e][c], w[e][cp], d[cp]);
+            for (int e = 0; e < GS_PE; ++e) w[e][c] = pc_mul_sub(w[e][c], w[e][cp], d);
+          }
       }
-      pc nn[1];
       {
+        float nh[2] = {0.f, 0.f}, nl[2] = {0.f, 0.f};
         lacc s{0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int e = 0; e < GS_PE; ++e) lacc_fmac(s, w[e][c], w[e][c]);
-        nn[0] = lacc_value(s);
+        for (int e = 0; e < GS_PE; ++e) lacc_norm(s, w[e][c]);
+        two_sum(s.rh, s.rl, nh[0], nl[0]);
+        pair_totals<2>(nh, nl, red, tot);
       }
-      pc_block_sum<1>(nn, red);
-      const double nrm = sqrt((double)nn[0].rh + (double)nn[0].rl);
-      if (!(nrm > 1e-12 * sqrt(n0[c]))) {
-        if (tid == 0) atomicOr(err, AMG_EBIT_RANK);
+      if (tid < 32) {  // the root and the reciprocal in FP64, by one warp
+        const double nrm = sqrt((double)tot[0].x + (double)tot[0].y);
+        float2 inv;
+        split_double(nrm > 0 ? 1.0 / nrm : 0.0, inv.x, inv.y);
+        if (tid == 0) {
+          if (!(nrm > 1e-12 * sqrt(n0[c]))) atomicOr(err, AMG_EBIT_RANK);
+          scal = inv;
+        }
       }
-      pc inv{0.f, 0.f, 0.f, 0.f};
-      split_double(nrm > 0 ? 1.0 / nrm : 0.0, inv.rh, inv.rl);
+      __syncthreads();
+      const pc inv{scal.x, 0.f, scal.y, 0.f};
 #pragma unroll
       for (int e = 0; e < GS_PE; ++e) {
         lacc s{0.f, 0.f, 0.f, 0.f};
-        lacc_fma(s, inv, w[e][c]);
+        pair_fma(s.rh, s.rl, inv.rh, inv.rl, w[e][c].rh, w[e][c].rl);
+        pair_fma(s.ih, s.il, inv.rh, inv.rl, w[e][c].ih, w[e][c].il);
         w[e][c] = lacc_value(s);
       }
     }
