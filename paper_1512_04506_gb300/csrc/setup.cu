@@ -3,7 +3,8 @@
 //   clover_kernel    C(x) = c_sw (i/4) sum sigma_{mu nu} F_{mu nu}(x), per chirality (Alg. 7's C^{hh})
 //   gs_kernel        block classical Gram-Schmidt per aggregate (Sec. 3, "Gram-Schmidt on aggregates")
 //   assemble_kernel  self and forward blocks of D_c = R D P (Eq. cgo via Alg. 7's D P), as sums
-//                    over links of small rank-6 products
+//                    over links of small rank-6 products: small blocks and few test vectors (the
+//                    others run on the tensor cores, setup_tc.cu)
 //   combine_kernel   D_c blocks from the partial sums; backward blocks by Eq. dagger
 //   quantize_*       D_c and R to the storage precisions of the applies (Sec. 3: half precision D_c)
 #include "amg_internal.cuh"
@@ -703,6 +704,17 @@ static amg_status launch_assemble(const Geom& g, const double2* R, const double2
   }
 }
 
+// Whether the assembly runs on the tensor cores (setup_tc.cu).  That kernel has a fixed cost of about 10 us per block
+// and job and grows slowly with Ntv; the tiled ones grow with Vb Ntv^2.  In FP64 the two meet near
+// Vb Ntv^2 = 1800 (tiled / slices in ms, 10^4 sites: Vb 16, Ntv 8: 1.44 / 1.50, Ntv 11: 2.41 / 1.94; Vb 81, Ntv 4: 0.75 /
+// 0.85, Ntv 6: 1.10 / 0.87; Vb 8, Ntv 12: 2.13 / 2.26, Ntv 16: 3.08 / 2.46).  In pairs of FP32 numbers the tiles are
+// several times cheaper and good at Ntv 11 and below (Vb 54, Ntv 11: 1.05 / 1.16; Vb 81, Ntv 11: 1.07 / 1.00; Vb 16, Ntv 12:
+// 1.36 / 1.90, Ntv 16: 2.15 / 2.10; Vb 8, Ntv 16: 1.84 / 2.39, Ntv 20: 3.12 / 2.97).
+static bool assemble_by_slices(const Geom& g, bool pair) {
+  const long long work = g.Vb * g.ntv * g.ntv;
+  return pair ? g.Vb >= 64 || (g.ntv >= 16 && work >= 3200) : work >= 1800;
+}
+
 // The setup's steps; the caller owns the timing events and frees `part` if a step fails.
 static amg_status setup_body(amg_coarse* h, const double2* U, const double2* tv, cudaStream_t st, cudaEvent_t (&ev)[5],
                              double2*& part) {
@@ -731,9 +743,13 @@ static amg_status setup_body(amg_coarse* h, const double2* U, const double2* tv,
   }
   AMG_CUDA_TRY(cudaEventRecord(ev[2], st));
   // assembly
-  const size_t part_elems = (size_t)g.Vc * 5 * 2 * g.nc * g.nc;
-  AMG_CUDA_TRY(cudaMallocAsync((void**)&part, part_elems * sizeof(double2), st));
-  if (h->p.setup_arith == AMG_SETUP_F32PAIR) {
+  const size_t part_elems = (size_t)g.Vc * 5 * 2 * g.nc * g.nc, exps = (size_t)g.Vc * (9 + 2 * g.ntv);
+  const bool pair = h->p.setup_arith == AMG_SETUP_F32PAIR, slices = assemble_by_slices(g, pair);
+  AMG_CUDA_TRY(cudaMallocAsync((void**)&part, part_elems * sizeof(double2) + (slices ? exps * sizeof(int) : 0), st));
+  if (slices) {
+    AMG_TRY_INTERNAL(amg_internal_assemble_tc(g, h->R64, U, h->clover, (int*)(part + part_elems), part, h->p.m0, pair,
+                                              h->err, st));
+  } else if (pair) {
     AMG_TRY_INTERNAL(amg_internal_assemble_pair(g, h->R64, U, h->clover, part, h->p.m0, h->err, st));
   } else {
     AMG_TRY_INTERNAL(launch_assemble(g, h->R64, U, h->clover, part, h->p.m0, st));

@@ -41,9 +41,11 @@
 // timeout bit of the error word, after which every role leaves its loop, the MMA thread waits
 // (bounded) for its last commit, and tensor memory is freed.
 #include "tc_body.cuh"
+#include "tcgen05.cuh"
 
 namespace {
 using namespace amgtc;
+using namespace amgtc5;
 
 constexpr int kT5Threads = 704;  // 16 builder warps, 4 epilogue warps, the copy warp, the MMA warp
 constexpr int kT5Cols = 512;       // tensor-memory columns allocated
@@ -62,29 +64,6 @@ struct T5Bars {
 constexpr int kT5BarBytes = 256;
 static_assert(sizeof(T5Bars) <= kT5BarBytes, "barrier block");
 
-__device__ inline void tc5_alloc(uint32_t* dst) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(dst)),
-               "r"(kT5Cols)
-               : "memory");
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ inline void tc5_dealloc(uint32_t taddr) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(kT5Cols) : "memory");
-}
-__device__ inline void tc5_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ inline void tc5_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ inline void tc5_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(bar))
-               : "memory");
-}
-// D[tmem] (+)= A[tmem] B[smem], FP16 operands, FP32 accumulator
-__device__ inline void tc5_mma(uint32_t d, uint32_t a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(d),
-      "r"(a), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
 __device__ inline void tc5_ld32(uint32_t taddr, uint32_t (&v)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
@@ -96,25 +75,6 @@ __device__ inline void tc5_ld32(uint32_t taddr, uint32_t (&v)[32]) {
       : "r"(taddr)
       : "memory");
 }
-__device__ inline void tc5_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-__device__ inline void tc5_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ inline void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-// Shared-memory matrix descriptor, K-major without swizzle: start, leading-dimension byte offset
-// (between core matrices adjacent in K), stride-dimension byte offset (adjacent in M / N), and
-// the descriptor version bit of this architecture (bit 46).
-__device__ inline uint64_t tc5_desc(const void* p, uint32_t lbo, uint32_t sbo) {
-  uint64_t d = (uint64_t)((smem_addr(p) & 0x3FFFFu) >> 4);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;
-  return d;
-}
-// Instruction descriptor of kind::f16: FP32 accumulator, FP16 A and B, both K-major, N, M = 128.
-__host__ __device__ constexpr uint32_t tc5_idesc(int n) {
-  return (1u << 4) | (0u << 7) | (0u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-}
-
 __device__ inline bool t5_wait(uint64_t* bar, unsigned parity, Pipe* pp, unsigned* err) {
   if (wait_phase(bar, parity, pp)) return true;
   abort_cta(pp, err);
@@ -228,7 +188,7 @@ __global__ void __launch_bounds__(kT5Threads, 1) apply_tc5_kernel(const T5Args a
     mbar_init(&tb->done, 1);
     fence_mbar_init();
   }
-  if (warp == 21) tc5_alloc(&tb->tmem_base);
+  if (warp == 21) tc5_alloc(&tb->tmem_base, kT5Cols);
   tc5_fence_before();
   __syncthreads();
   tc5_fence_after();
@@ -481,7 +441,7 @@ __global__ void __launch_bounds__(kT5Threads, 1) apply_tc5_kernel(const T5Args a
   tc5_fence_before();
   __syncthreads();
   tc5_fence_after();
-  if (warp == 21) tc5_dealloc(tmem);
+  if (warp == 21) tc5_dealloc(tmem, kT5Cols);
 }
 
 // FP32 coarse vector x (times xscale[r]; the scaled vector also to vout) -> FP32 rows of
