@@ -1,13 +1,14 @@
 // Setup of the restriction and the coarse-grid operator (Alg. 5), in FP64.
 //
 //   clover_kernel    C(x) = c_sw (i/4) sum sigma_{mu nu} F_{mu nu}(x), per chirality (Alg. 7's C^{hh})
-//   gs_kernel        block classical Gram-Schmidt per aggregate (Sec. 3, "Gram-Schmidt on aggregates")
+//   gs_kernel        block classical Gram-Schmidt per aggregate (Sec. 3, "Gram-Schmidt on aggregates"), where
+//                    those in fixed point (setup_gs.cu) and in pairs of floats (setup_ds.cu) do not serve
 //   assemble_kernel  self and forward blocks of D_c = R D P (Eq. cgo via Alg. 7's D P), as sums
 //                    over links of small rank-6 products: small blocks and few test vectors (the
 //                    others run on the tensor cores, setup_tc.cu)
 //   combine_kernel   D_c blocks from the partial sums; backward blocks by Eq. dagger
 //   quantize_*       D_c and R to the storage precisions of the applies (Sec. 3: half precision D_c)
-#include "amg_internal.cuh"
+#include "fixed.cuh"
 
 #include <stdio.h>
 #include <stdlib.h>
@@ -15,6 +16,7 @@
 #include <vector>
 
 namespace {
+using namespace amgfix;
 
 // ------------------------------------------------------------------ clover term
 // Products of links in fixed point: entry = (h 2^31 + l) 2^(e - 60) with |h| <= 2^29, |l| <= 2^30 and one exponent for
@@ -23,18 +25,6 @@ struct I3 {
   int2 re[9], im[9];
   int e;
 };
-__device__ __forceinline__ int2 words31(long long x) {
-  x += 1 << 30;
-  return make_int2((int)(x >> 31), (int)((unsigned)x & 0x7FFFFFFFu) - (1 << 30));
-}
-// (-1)^neg v 2^(60 - e) cut to an integer, for |v| < 2^e; neg: the sign bit's mask
-__device__ __forceinline__ long long fixed60(double v, int e, int neg) {
-  const int hi = __double2hiint(v), lo = __double2loint(v), f = (hi >> 20) & 0x7FF;
-  const unsigned mh = (((unsigned)hi << 10) & 0x3FFFFFFFu) | 0x40000000u | (unsigned)lo >> 22;  // mantissa 2^10
-  const unsigned long long m = (unsigned long long)mh << 32 | (unsigned)lo << 10;
-  const long long x = (long long)(m >> min(1025 + e - f, 63)), s = (hi ^ neg) >> 31;
-  return (x ^ s) - s;
-}
 // U, or its adjoint; `bad` is set if an entry is not finite
 __device__ __forceinline__ I3 load_link(const double2* __restrict__ p, bool dagger, bool& bad) {
   double2 u[9];
@@ -52,8 +42,8 @@ __device__ __forceinline__ I3 load_link(const double2* __restrict__ p, bool dagg
   m.e = max(f - 1022, -900);
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
-    m.re[k] = words31(fixed60(u[k].x, m.e, 0));
-    m.im[k] = words31(fixed60(u[k].y, m.e, dagger ? (int)0x80000000 : 0));
+    m.re[k] = words31(fixed<60>(u[k].x, m.e));
+    m.im[k] = words31(fixed<60>(u[k].y, m.e, dagger ? (int)0x80000000 : 0));
   }
   return m;
 }
@@ -64,16 +54,11 @@ __device__ __forceinline__ void mul(const I3& a, const I3& b, long long (&re)[9]
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       long long hr = 0, lr = 0, hi = 0, li = 0;
-      auto mac = [](long long& h, long long& l, int2 u, int2 x) {
-        h += (long long)u.x * x.x;
-        l += (long long)u.x * x.y;
-        l += (long long)u.y * x.x;
-      };
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
         const int2 ar = a.re[i * 3 + k], ai = a.im[i * 3 + k], br = b.re[k * 3 + j], bi = b.im[k * 3 + j];
         mac(hr, lr, ar, br);
-        mac(hr, lr, make_int2(-ai.x, -ai.y), bi);
+        mac(hr, lr, minus(ai), bi);
         mac(hi, li, ar, bi);
         mac(hi, li, ai, br);
       }
@@ -277,7 +262,8 @@ __device__ inline void block_totals(double (&v)[NV], double* sm, double* out) {
 // Bound: the FP64 pipes (one warp instruction in 64 cycles per sub-partition): 4 instructions per element and pair
 // of columns in every dot and every update, and as little else as possible: updates add the negated
 // coefficients, sums halve their values as they go down the lanes, one warp takes the roots and
-// reciprocals.  16^4, Ntv 20: 5.5 ms; with a multiplication, a fused one and a subtraction per update,
+// reciprocals.  It serves up to 4 test vectors of large aggregates and those beyond the fixed-point kernel (setup_gs.cu).
+// 16^4, Ntv 2: 0.105 ms; Ntv 20: 5.5 ms; with a multiplication, a fused one and a subtraction per update,
 // 5 additions per value and lane and roots in every thread 8.8 ms.
 constexpr int GS_NB = 4;
 constexpr int GS_EMAX = 8;
@@ -802,22 +788,23 @@ static amg_status setup_body(amg_coarse* h, const double2* U, const double2* tv,
   }
   AMG_CUDA_TRY(cudaEventRecord(ev[1], st));
   // Gram-Schmidt, one CTA per aggregate
-  amg_status gs_pair = AMG_ERR_UNSUPPORTED;
-  if (h->p.setup_arith == AMG_SETUP_F32PAIR) gs_pair = amg_internal_gs_pair(g, tv, h->R64, h->err, st);
-  if (gs_pair == AMG_ERR_UNSUPPORTED) {
+  const bool pair = h->p.setup_arith == AMG_SETUP_F32PAIR;
+  amg_status gs = amg_internal_gs_fixed(g, tv, h->R64, pair, h->err, st);
+  if (gs == AMG_ERR_UNSUPPORTED && pair) gs = amg_internal_gs_pair(g, tv, h->R64, h->err, st);
+  if (gs == AMG_ERR_UNSUPPORTED) {
     int T = round_up(g.nagg < 256 ? g.nagg : 256, 32);
     if ((g.nagg + T - 1) / T > GS_EMAX) return AMG_ERR_UNSUPPORTED;
-    void (*const gs[GS_EMAX])(const double2*, double2*, Geom, unsigned*) = {
+    void (*const kernels[GS_EMAX])(const double2*, double2*, Geom, unsigned*) = {
         gs_kernel<1>, gs_kernel<2>, gs_kernel<3>, gs_kernel<4>, gs_kernel<5>, gs_kernel<6>, gs_kernel<7>, gs_kernel<8>};
-    gs[(g.nagg + T - 1) / T - 1]<<<(unsigned)(g.Vc * 2), T, 0, st>>>(tv, h->R64, g, h->err);
+    kernels[(g.nagg + T - 1) / T - 1]<<<(unsigned)(g.Vc * 2), T, 0, st>>>(tv, h->R64, g, h->err);
     AMG_LAUNCH_CHECK();
-  } else if (gs_pair != AMG_OK) {
-    return gs_pair;
+  } else if (gs != AMG_OK) {
+    return gs;
   }
   AMG_CUDA_TRY(cudaEventRecord(ev[2], st));
   // assembly
   const size_t part_elems = (size_t)g.Vc * 5 * 2 * g.nc * g.nc, exps = (size_t)g.Vc * (9 + 2 * g.ntv);
-  const bool pair = h->p.setup_arith == AMG_SETUP_F32PAIR, slices = assemble_by_slices(g, pair);
+  const bool slices = assemble_by_slices(g, pair);
   AMG_CUDA_TRY(cudaMallocAsync((void**)&part, part_elems * sizeof(double2) + (slices ? exps * sizeof(int) : 0), st));
   if (slices) {
     AMG_TRY_INTERNAL(amg_internal_assemble_tc(g, h->R64, U, h->clover, (int*)(part + part_elems), part, h->p.m0, pair,

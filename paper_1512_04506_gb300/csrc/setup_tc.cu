@@ -38,12 +38,14 @@
 // of FP32 numbers on the FP32 pipes 11.4 ms); Ntv 20, DIG 8, 3.5 ms (in FP64 22.0 ms); error of D_c against 64-bit
 // references 2.0e-15 with DIG 8 as with sums in FP64.  Measured slower: U_mu P in FP64 (2 x), the block's coefficients
 // converted by each item (1.2 x), 8 warps on the sums and 11 or 12 builders (1.04 x).
+#include "fixed.cuh"
 #include "tcgen05.cuh"
 
 #include <limits.h>
 #include <string.h>
 
 namespace {
+using namespace amgfix;
 using namespace amgtc5;
 
 constexpr int kExact = 5;          // accumulators s < kExact hold exact integers
@@ -144,21 +146,7 @@ __global__ void __launch_bounds__(256) tc_bounds_kernel(const double2* __restric
   for (int i = threadIdx.x; i < n; i += blockDim.x) exps[blk * n + i] = bound_exp(__longlong_as_double((long long)red[i]));
 }
 
-// ------------------------------------------------------------------ fixed point
-// (-1)^neg v 2^(BITS - e) cut to an integer, for |v| < 2^e, BITS <= 63; neg: the sign bit's mask
-template <int BITS>
-__device__ __forceinline__ long long fixed(double v, int e, int neg = 0) {
-  const int hi = __double2hiint(v), lo = __double2loint(v), f = (hi >> 20) & 0x7FF;
-  const unsigned mh = (((unsigned)hi << 10) & 0x3FFFFFFFu) | 0x40000000u | (unsigned)lo >> 22;  // mantissa 2^10
-  const unsigned long long m = (unsigned long long)mh << 32 | (unsigned)lo << 10;
-  const long long x = (long long)(m >> min(1085 - BITS + e - f, 63)), s = (hi ^ neg) >> 31;
-  return (x ^ s) - s;
-}
-// words of x = h 2^31 + l, |l| <= 2^30
-__device__ __forceinline__ int2 words31(long long x) {
-  x += 1 << 30;
-  return make_int2((int)(x >> 31), (int)((unsigned)x & 0x7FFFFFFFu) - (1 << 30));
-}
+// ------------------------------------------------------------------ digits
 // The factor of -b_mu in row a (see setup.cu), i, -i, -1 or 1: whether it swaps the parts, and the sign bits of
 // the new real and imaginary part
 struct Phase {
@@ -393,14 +381,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) assemble_tc_kernel(const TcArgs
 #pragma unroll
         for (int col = 0; col < 3; ++col) {
           long long hr = 0, hi = 0, lr = 0, li = 0;  // high x high, high x low words
-          auto mac = [](long long& h, long long& l, int2 u, int2 x) {
-            h += (long long)u.x * x.x;
-            l += (long long)u.x * x.y;
-            l += (long long)u.y * x.x;
-          };
           auto cmac = [&](int2 ur, int2 ui, int2 x, int2 y) {
             mac(hr, lr, ur, x);
-            mac(hr, lr, make_int2(-ui.x, -ui.y), y);
+            mac(hr, lr, minus(ui), y);
             mac(hi, li, ur, y);
             mac(hi, li, ui, x);
           };
@@ -411,7 +394,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) assemble_tc_kernel(const TcArgs
               cmac(make_int2(w.x, w.y), make_int2(w.z, w.w), rx[k], ry[k]);
             }
           } else {
-            auto signed_words = [](int2 u, bool minus) { return minus ? make_int2(-u.x, -u.y) : u; };
+            auto signed_words = [](int2 u, bool neg) { return neg ? minus(u) : u; };
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
               if (k == col) {
