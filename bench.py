@@ -56,8 +56,8 @@ TRAFFIC_MRHS_FP32 = 1449390080
 # (profiles/batch_kernel_small_mixed.md); the full launch's traffic is taken in that proportion
 BATCH_TRAFFIC_RATIO = 0.990
 # DRAM traffic / algorithmic bytes of one SAP half sweep, from the 16^4 capture (profiles/sap_16x4.md:
-# 35.56 MB for 65,536 sites x 504 B); the 32^4 launch is taken in proportion
-SAP_TRAFFIC_RATIO = 1.077
+# 31.24 MB for 65,536 sites x 504 B); the 32^4 launch is taken in proportion
+SAP_TRAFFIC_RATIO = 0.946
 METRIC = "coarse-grid correction GB/s & % HBM roofline; batched-mixed vs plain speedup"
 WORKLOAD = "fp32_32^4_b4_ntv20: 32^4 Wilson-clover, 4^4 blocks -> 8^4 coarse, Ntv=20, 1 RHS, " \
            "FP64 setup, FP32 R and D_c; step = R y, FGMRES(30) to 0.05 (<=200 applies), P x_c"
@@ -691,7 +691,8 @@ def run_vcycle(args):
     (two Hermitian 6x6 blocks as upper triangles, 336 B), psi (96 B) and writes out (96 B) = 816 B;
     one SAP half sweep reads, per site of its colour, the links, the clover, y and x and writes x
     (912 B), and reads x on the other colour's sites once (96 B): 504 B per fine site of the
-    lattice."""
+    lattice.  (The kernels read less of the clover, 27 numbers per chirality or 216 B; the model is kept
+    so that figures compare.)  A half sweep is timed as the V-cycle runs it, over its 4 cycles."""
     import torch
     import paper_1512_04506_gb300 as amg
     from synth import device as sd
@@ -714,7 +715,7 @@ def run_vcycle(args):
     applies = info[0][0]
     t, clk = _timed_steps(lambda: amg.amg_vcycle(h, vp, y, x, 1, st), args.steps, args.warmup, st, flush)
     t_d = _kernel_time(lambda: amg.amg_dirac_apply(h, y, x, 1, st), 20, st)
-    t_sap = _kernel_time(lambda: amg.amg_sap(h, y, x, 1, 1, n_mr, st), 10, st) / 2  # one half sweep
+    t_sap = _kernel_time(lambda: amg.amg_sap(h, y, x, 1, n_smoother, n_mr, st), 10, st) / (2 * n_smoother)
     u = torch.empty_like(y)
     t0 = time.perf_counter()
     sinfo = amg.amg_solve(h, vp, y, u, 1, tol=1e-5, restart=30, max_applies=200, stream=st)
@@ -760,7 +761,7 @@ def run_vcycle(args):
                                "(FGMRES(30) to 0.05) + %d SAP cycles of %d MR steps per 4^4 block; FP32" % (n_smoother, n_mr),
                    "bytes_per_step": step_bytes, "coarse_applies": applies, "n_smoother": n_smoother, "n_mr": n_mr,
                    "l2": "256 MB flush before each step"},
-        "roofline": {"bound": "hbm", "kernel": "sap_smem_kernel (one half sweep: residual + %d MR steps per block, "
+        "roofline": {"bound": "hbm", "kernel": "sap32_kernel (one half sweep: residual + %d MR steps per block, "
                      "links and clover in shared memory)" % n_mr, "achieved": round(sap_gbs, 1), "peak": peaks["hbm_gbs"],
                      "unit": "GB/s", "frac": round(sap_gbs / peaks["hbm_gbs"], 4), "peak_source": src,
                      "traffic": round(SAP_TRAFFIC_RATIO * half_bytes) if SAP_TRAFFIC_RATIO and not args.lattice else None,

@@ -69,11 +69,13 @@ typedef enum {
 /* Arithmetic of the Gram-Schmidt and of the D_c = R D P assembly in amg_setup_coarse (the
  * clover field stays FP64). */
 typedef enum {
-    AMG_SETUP_FP64 = 0,     /* doubles on the FP64 pipe                                      */
-    AMG_SETUP_F32PAIR = 1   /* each number an unevaluated sum of two floats (~47 bits), sums by
-                               TwoSum and products by the FMA residual, on the FP32 pipes;
-                               R and D_c agree with FP64 to about 1e-14 relative; aggregates
-                               of more than 1536 entries fall back to the FP64 Gram-Schmidt */
+    AMG_SETUP_FP64 = 0,     /* sums of double accuracy: 64-bit fixed point on the tensor cores and
+                               the integer pipes, or doubles on the FP64 pipe                */
+    AMG_SETUP_F32PAIR = 1   /* sums of at least ~47 bits: 56-bit fixed point on the tensor cores, or
+                               each number an unevaluated sum of two floats (sums by TwoSum,
+                               products by the FMA residual) on the FP32 pipes; R and D_c agree
+                               with FP64 to about 1e-14 relative; aggregates of more than 1536
+                               entries fall back to the FP64 Gram-Schmidt                    */
 } amg_setup_arith;
 
 typedef struct {
