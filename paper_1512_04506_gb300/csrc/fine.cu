@@ -21,9 +21,10 @@
 // adds e to x.
 //
 // FP32 keeps the links and the clover of the fine lattice in an order of its own (see kLinkQ).
-#include "amg_internal.cuh"
+#include "fixed.cuh"
 #include "pipe.cuh"
 
+#include <limits.h>
 #include <math.h>
 
 #include <algorithm>
@@ -703,16 +704,205 @@ __device__ __forceinline__ void colour_block(const FineGeom& g, int k, int colou
   X[0] = 2 * (k % half) + ((colour + X[1] + X[2] + X[3]) & 1);
 }
 
-// One SAP half sweep on the blocks of one colour: x += MR_{n_mr}(B_b, (y - D x)|_b) per block.
+// Words of the links and the clover of an FP64 handle for the MR steps (fixed.cuh), block by block, word q of the site
+// with local index t in block b at (b kFixQ + q) Vb + t: 36 link entries (re, im), then per chirality the diagonal
+// of 4 + m0 + C (6 numbers, two per word), C's entries 01, 02, 12 and its upper right 3 x 3 block (see kClovQ).
+// All of a block relative to 2^exps[b], a bound of every row's and column's sum of |re| + |im|, in units of 2^-61.
+constexpr int kFixQ = 66, kFixClov = 36;
+__global__ void __launch_bounds__(256) fixed_words_kernel(const double2* __restrict__ U, const double2* __restrict__ clov,
+                                                          int4* __restrict__ W, int* __restrict__ exps, FineGeom g,
+                                                          double mass) {
+  __shared__ unsigned long long top;
+  const int b = blockIdx.x;
+  int X[4], row = b;
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    X[mu] = (row % g.Lc[mu]) * g.B[mu];
+    row /= g.Lc[mu];
+  }
+  auto site = [&](int t) {
+    int x[4];
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+      x[mu] = X[mu] + t % g.B[mu];
+      t /= g.B[mu];
+    }
+    return site_of(g, x);
+  };
+  if (threadIdx.x == 0) top = 0;
+  __syncthreads();
+  auto mag = [](double2 z) { return fabs(z.x) + fabs(z.y); };
+  for (int i = threadIdx.x; i < g.Vb * 5; i += blockDim.x) {
+    const int t = i % g.Vb, mu = i / g.Vb;
+    const long long s = site(t);
+    unsigned long long m = 0;
+    auto bound = [&](double v) { m = max(m, (unsigned long long)__double_as_longlong(v)); };  // a NaN wins
+    if (mu < 4) {
+      const double2* u = U + (s * 4 + mu) * 9;
+      for (int k = 0; k < 3; ++k) {
+        bound(mag(u[3 * k]) + mag(u[3 * k + 1]) + mag(u[3 * k + 2]));
+        bound(mag(u[k]) + mag(u[3 + k]) + mag(u[6 + k]));
+      }
+    } else {
+      for (int k = 0; k < 12; ++k) {
+        double v = fabs(mass);
+        for (int q = 0; q < 6; ++q) v += mag(clov[s * 72 + k * 6 + q]);
+        bound(v);
+      }
+    }
+    atomicMax(&top, m);
+  }
+  __syncthreads();
+  const double v = __longlong_as_double((long long)top) * 1.015625;  // |v| < 2^e with room for roundings
+  const int f = (__double2hiint(v) >> 20) & 0x7FF, e = max(f - 1022, -900);
+  if (threadIdx.x == 0) exps[b] = f == 0x7FF ? INT_MAX : e;
+  if (f == 0x7FF) return;
+  for (int i = threadIdx.x; i < g.Vb * kFixQ; i += blockDim.x) {
+    const int t = i % g.Vb, q = i / g.Vb;
+    const long long s = site(t);
+    double2 z;
+    if (q < kFixClov) {
+      z = U[s * 36 + q];
+    } else {
+      const int h = (q - kFixClov) / 15, k = (q - kFixClov) % 15;
+      const double2* c = clov + (s * 2 + h) * 36;
+      if (k < 3)
+        z = make_double2(mass + c[14 * k].x, mass + c[14 * k + 7].x);
+      else
+        z = c[k < 5 ? k - 2 : k == 5 ? 8 : (k - 6) / 3 * 6 + 3 + (k - 6) % 3];
+    }
+    const int2 re = amgfix::words31(amgfix::fixed<61>(z.x, e)), im = amgfix::words31(amgfix::fixed<61>(z.y, e));
+    W[(long long)b * kFixQ * g.Vb + i] = make_int4(re.x, re.y, im.x, im.y);
+  }
+}
+
+struct fx2 {  // complex fixed-point number
+  long long x, y;
+};
+__device__ __forceinline__ fx2 joined(int4 w) {
+  return fx2{amgfix::joined(make_int2(w.x, w.y)), amgfix::joined(make_int2(w.z, w.w))};
+}
+struct FixSum {  // sum of products in units of their high words' products
+  long long h = 0, l = 0;
+  __device__ __forceinline__ void add(int2 a, int2 b) { amgfix::mac(h, l, a, b); }
+  __device__ __forceinline__ long long value() const { return h + ((l + (1 << 30)) >> 31); }
+};
+// out += -(1 -+ g_mu) U p for the hop of one site in fixed point (hop_u without the factor 1/2).  W: the link's words, Vb
+// apart; rho: the neighbour's entries, Vb apart
+template <bool FWD, int mu>
+__device__ __forceinline__ void hop_fixed(const int4* __restrict__ W, const int4* rho, int Vb, fx2 (&out)[12]) {
+  int2 hr[2][3], hi[2][3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    fx2 a0, a1;
+    amul(mu, joined(rho[(6 + c) * Vb]), joined(rho[(9 + c) * Vb]), a0, a1);
+    const fx2 p0 = joined(rho[c * Vb]), p1 = joined(rho[(3 + c) * Vb]);
+    const fx2 h0 = FWD ? zsub(p0, a0) : zadd(p0, a0), h1 = FWD ? zsub(p1, a1) : zadd(p1, a1);
+    hr[0][c] = amgfix::words31(h0.x);
+    hi[0][c] = amgfix::words31(h0.y);
+    hr[1][c] = amgfix::words31(h1.x);
+    hi[1][c] = amgfix::words31(h1.y);
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    FixSum r0, i0, r1, i1;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const int4 u = __ldg(W + (mu * 9 + (FWD ? a * 3 + b : b * 3 + a)) * Vb);
+      const int2 ur = make_int2(u.x, u.y), ui = make_int2(u.z, u.w), ni = amgfix::minus(ui);
+      const int2 pi = FWD ? ui : ni, mi = FWD ? ni : ui;  // backward: conj(u)
+      r0.add(ur, hr[0][b]);
+      r0.add(mi, hi[0][b]);
+      i0.add(ur, hi[0][b]);
+      i0.add(pi, hr[0][b]);
+      r1.add(ur, hr[1][b]);
+      r1.add(mi, hi[1][b]);
+      i1.add(ur, hi[1][b]);
+      i1.add(pi, hr[1][b]);
+    }
+    const fx2 w0{r0.value(), i0.value()}, w1{r1.value(), i1.value()};
+    fx2 d0, d1;
+    adagmul(mu, w0, w1, d0, d1);
+    out[a] = zsub(out[a], w0);
+    out[3 + a] = zsub(out[3 + a], w1);
+    out[6 + a] = FWD ? zadd(out[6 + a], d0) : zsub(out[6 + a], d0);
+    out[9 + a] = FWD ? zadd(out[9 + a], d1) : zsub(out[9 + a], d1);
+  }
+}
+template <int mu>
+__device__ __forceinline__ void block_hops_fixed(const FineGeom& g, const int4* __restrict__ W, const int4* rho, int t,
+                                                 const int lc[4], int stride, fx2 (&out)[12]) {
+  if (lc[mu] + 1 < g.B[mu]) hop_fixed<true, mu>(W + t, rho + t + stride, g.Vb, out);
+  if (lc[mu] > 0) hop_fixed<false, mu>(W + t - stride, rho + t - stride, g.Vb, out);
+}
+// out = 2 (4 + m0 + C) rho at site t
+__device__ __forceinline__ void site_fixed(const int4* __restrict__ W, const int4* rho, int Vb, fx2 (&out)[12]) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    int2 x[6], y[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const int4 p = rho[(6 * h + k) * Vb];
+      x[k] = make_int2(p.x, p.y);
+      y[k] = make_int2(p.z, p.w);
+    }
+    FixSum r[6], i[6];
+    auto cadd = [&](int a, int2 ur, int2 ui, int b) {
+      r[a].add(ur, x[b]);
+      r[a].add(amgfix::minus(ui), y[b]);
+      i[a].add(ur, y[b]);
+      i[a].add(ui, x[b]);
+    };
+    const int4* c = W + (kFixClov + 15 * h) * Vb;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int4 d = __ldg(c + k * Vb), u = __ldg(c + (3 + k) * Vb);
+      r[2 * k].add(make_int2(d.x, d.y), x[2 * k]);
+      i[2 * k].add(make_int2(d.x, d.y), y[2 * k]);
+      r[2 * k + 1].add(make_int2(d.z, d.w), x[2 * k + 1]);
+      i[2 * k + 1].add(make_int2(d.z, d.w), y[2 * k + 1]);
+      const int a = k < 2 ? 0 : 1, b = k < 1 ? 1 : 2;  // G_ab and, conjugated, G_ba; -G for the lower rows
+      const int2 ur = make_int2(u.x, u.y), ui = make_int2(u.z, u.w), nr = amgfix::minus(ur), ni = amgfix::minus(ui);
+      cadd(a, ur, ui, b);
+      cadd(b, ur, ni, a);
+      cadd(3 + a, nr, ni, 3 + b);
+      cadd(3 + b, nr, ui, 3 + a);
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const int4 u = __ldg(c + (6 + a * 3 + b) * Vb);
+        const int2 ur = make_int2(u.x, u.y), ui = make_int2(u.z, u.w);
+        cadd(a, ur, ui, 3 + b);
+        cadd(3 + b, ur, amgfix::minus(ui), a);
+      }
+#pragma unroll
+    for (int a = 0; a < 6; ++a) out[6 * h + a] = fx2{r[a].value() << 1, i[a].value() << 1};
+  }
+}
+
+// One SAP half sweep on the blocks of one colour: x += MR_{n_mr}(B_b, (y - D x)|_b) per block; FP64.
 // grid (Vc / 2, nrhs); blockDim >= Vb (threads past Vb only join the sums); dynamic smem: rho
-// [12][Vb] + 3 doubles per warp + 3 doubles.
+// [12][Vb] + 3 doubles per warp + 3 doubles + 2 ints.
+//
+// Bound: the FP64 pipes (one warp instruction in 64 cycles per sub-partition).  FIXED: the MR steps apply B in fixed
+// point (a multiply-add takes a sixteenth of that): rho as 59-bit integers relative to its largest entry in the block, links and
+// clover as words prepared once, sums of 64 bits; the sums over the block and the updates stay in FP64.  An
+// application is then good to 2^-57 of the block's largest entry.  A block with an entry that is not finite takes
+// the FP64 steps.  12 x 8 x 24 x 16, blocks 3 x 4 x 4 x 2, 3 columns: 447 us a half sweep, in FP64 703 us; 16^4 in
+// 2^4 blocks 497 and 944 us.
+template <bool FIXED>
 __global__ void __launch_bounds__(256) sap_kernel(const double2* __restrict__ U, const double2* __restrict__ Cl,
+                                                  const int4* __restrict__ words, const int* __restrict__ exps,
                                                   const double2* __restrict__ y, double2* __restrict__ x, FineGeom g,
                                                   double mass, int nrhs, int colour, int n_mr) {
   using C = double2;
   extern __shared__ __align__(16) unsigned char smem[];
   C* rho = reinterpret_cast<C*>(smem);
+  int4* rhow = reinterpret_cast<int4*>(smem);
   double* red = reinterpret_cast<double*>(smem + (size_t)g.Vb * 12 * sizeof(C));
+  int* top = reinterpret_cast<int*>(red + 3 * ((blockDim.x + 31) / 32) + 3);  // of rho's exponents, by parity of the step
   const int r = blockIdx.y;
   int X[4];
   colour_block(g, blockIdx.x, colour, X);
@@ -730,54 +920,103 @@ __global__ void __launch_bounds__(256) sap_kernel(const double2* __restrict__ U,
     s = site_of(g, xs);
   }
   const int st1 = g.B[0], st2 = g.B[0] * g.B[1], st3 = g.B[0] * g.B[1] * g.B[2];
+  const int4* W = nullptr;
+  int eb = 0;
+  bool fixed = FIXED;
+  if (FIXED) {
+    const long long b = ((long long)(X[3] * g.Lc[2] + X[2]) * g.Lc[1] + X[1]) * g.Lc[0] + X[0];
+    W = words + b * kFixQ * g.Vb;
+    eb = __ldg(exps + b);
+    fixed = eb != INT_MAX;
+    if (t < 2) top[t] = 0;
+    __syncthreads();
+  }
   // residual r = y - D x on this site (full D: neighbours outside the block have the other colour)
-  C o[12], e[12];
+  C rr[12], e[12];
+#pragma unroll
+  for (int q = 0; q < 12; ++q) rr[q] = e[q] = zzero<C>();
   if (act) {
-    C p[12];
+    C p[12], o[12];
     load12(x, s, nrhs, r, p);
     site_term(Cl + s * 72, mass, p, o);
     all_hops(g, U, x, s, xs, nrhs, r, o);
     load12(y, s, nrhs, r, p);
 #pragma unroll
-    for (int q = 0; q < 12; ++q) {
-      rho[q * g.Vb + t] = zsub(p[q], o[q]);
-      e[q] = zzero<C>();
-    }
+    for (int q = 0; q < 12; ++q) rr[q] = zsub(p[q], o[q]);
   }
-  __syncthreads();
 #pragma unroll 1
   for (int it = 0; it < n_mr; ++it) {
     // p = B rho at this site: site term plus the hops that stay inside the block
-    double v[3] = {0, 0, 0};
-    C rr[12];
+    double v[3] = {0, 0, 0}, unit = 1;
+    C o[12];
+    int er = 0;
+    if (FIXED && fixed) {
+      int f = 0;
+#pragma unroll
+      for (int q = 0; q < 12; ++q)
+        f = max(f, max((__double2hiint(rr[q].x) >> 20) & 0x7FF, (__double2hiint(rr[q].y) >> 20) & 0x7FF));
+      f = __reduce_max_sync(0xffffffffu, f);
+      if ((t & 31) == 0) atomicMax(&top[it & 1], f);
+      __syncthreads();
+      f = top[it & 1];
+      if (t == 0) top[(it + 1) & 1] = 0;  // last read before the previous step's coefficient
+      fixed = f != 0x7FF;
+      er = max(f - 1022, -900);
+    }
+    if (FIXED && fixed) {
+      if (act)
+#pragma unroll
+        for (int q = 0; q < 12; ++q) {
+          const int2 a = amgfix::words31(amgfix::fixed<59>(rr[q].x, er)), b = amgfix::words31(amgfix::fixed<59>(rr[q].y, er));
+          rhow[q * g.Vb + t] = make_int4(a.x, a.y, b.x, b.y);
+        }
+      __syncthreads();
+      unit = scalbn(1.0, eb + er - 59);
+      if (act) {
+        fx2 p[12];
+        site_fixed(W + t, rhow + t, g.Vb, p);
+        block_hops_fixed<0>(g, W, rhow, t, lc, 1, p);
+        block_hops_fixed<1>(g, W, rhow, t, lc, st1, p);
+        block_hops_fixed<2>(g, W, rhow, t, lc, st2, p);
+        block_hops_fixed<3>(g, W, rhow, t, lc, st3, p);
+#pragma unroll
+        for (int q = 0; q < 12; ++q) o[q] = make_double2((double)p[q].x, (double)p[q].y);
+      }
+    } else {
+      if (act)
+#pragma unroll
+        for (int q = 0; q < 12; ++q) rho[q * g.Vb + t] = rr[q];
+      __syncthreads();
+      if (act) {
+        site_term(Cl + s * 72, mass, rr, o);
+        block_hops_mu<0>(g, U, rho, t, s, xs, lc, 1, o);
+        block_hops_mu<1>(g, U, rho, t, s, xs, lc, st1, o);
+        block_hops_mu<2>(g, U, rho, t, s, xs, lc, st2, o);
+        block_hops_mu<3>(g, U, rho, t, s, xs, lc, st3, o);
+      }
+    }
     if (act) {
 #pragma unroll
-      for (int q = 0; q < 12; ++q) rr[q] = rho[q * g.Vb + t];
-      site_term(Cl + s * 72, mass, rr, o);
-      block_hops_mu<0>(g, U, rho, t, s, xs, lc, 1, o);
-      block_hops_mu<1>(g, U, rho, t, s, xs, lc, st1, o);
-      block_hops_mu<2>(g, U, rho, t, s, xs, lc, st2, o);
-      block_hops_mu<3>(g, U, rho, t, s, xs, lc, st3, o);
-#pragma unroll
-      for (int q = 0; q < 12; ++q) {
-        v[0] += o[q].x * o[q].x + o[q].y * o[q].y;        // <p, p>
-        v[1] += o[q].x * rr[q].x + o[q].y * rr[q].y;      // Re <p, rho>
-        v[2] += o[q].x * rr[q].y - o[q].y * rr[q].x;      // Im <p, rho>
+      for (int q = 0; q < 12; ++q) {  // in units of p's
+        v[0] = fma(o[q].x, o[q].x, fma(o[q].y, o[q].y, v[0]));       // <p, p>
+        v[1] = fma(o[q].x, rr[q].x, fma(o[q].y, rr[q].y, v[1]));     // Re <p, rho>
+        v[2] = fma(o[q].x, rr[q].y, fma(-o[q].y, rr[q].x, v[2]));    // Im <p, rho>
       }
+      v[0] = v[0] * unit * unit;
+      v[1] *= unit;
+      v[2] *= unit;
     }
     C al;
     bool ok;
     cta_alpha(v, red, al, ok);  // also orders every read of rho before the writes below
     if (act && ok) {
+      const C na = make_double2(-al.x * unit, -al.y * unit);
 #pragma unroll
       for (int q = 0; q < 12; ++q) {
         zfma(e[q], al, rr[q]);
-        C ap = zzero<C>();
-        zfma(ap, al, o[q]);
-        rho[q * g.Vb + t] = zsub(rr[q], ap);
+        zfma(rr[q], na, o[q]);
       }
     }
-    __syncthreads();
   }
   if (act) {
 #pragma unroll
@@ -1484,14 +1723,16 @@ amg_status launch_sap32(amg_coarse* h, const void* yv, void* xv, int nrhs, int n
 
 amg_status launch_sap64(amg_coarse* h, const void* y, void* x, int nrhs, int n_cycles, int n_mr, cudaStream_t st) {
   const int threads = (h->g.Vb + 31) / 32 * 32;
-  const size_t smem = (size_t)h->g.Vb * 12 * sizeof(double2) + (size_t)(threads / 32 + 1) * 3 * sizeof(double);
+  const size_t smem = (size_t)h->g.Vb * 12 * sizeof(double2) + (size_t)(threads / 32 + 1) * 3 * sizeof(double) + 8;
   if (threads > 256 || smem > 227 * 1024) return AMG_ERR_UNSUPPORTED;
-  AMG_CUDA_TRY(cudaFuncSetAttribute(sap_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  auto* kernel = h->fW ? sap_kernel<true> : sap_kernel<false>;
+  AMG_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const dim3 grid((unsigned)(h->g.Vc / 2), (unsigned)nrhs);
   for (int c = 0; c < n_cycles; ++c)
     for (int colour = 0; colour < 2; ++colour) {
-      sap_kernel<<<grid, threads, smem, st>>>((const double2*)h->fU, (const double2*)h->fC, (const double2*)y,
-                                              (double2*)x, fine_geom(h), 4.0 + h->p.m0, nrhs, colour, n_mr);
+      kernel<<<grid, threads, smem, st>>>((const double2*)h->fU, (const double2*)h->fC, (const int4*)h->fW, h->fE,
+                                          (const double2*)y, (double2*)x, fine_geom(h), 4.0 + h->p.m0, nrhs, colour,
+                                          n_mr);
       AMG_LAUNCH_CHECK();
       h->launches++;
     }
@@ -1805,6 +2046,10 @@ void amg_internal_free_fine(amg_coarse* h) {
   cudaFree(h->fU);
   if (h->fC != (void*)h->clover) cudaFree(h->fC);
   cudaFree(h->fwork);
+  cudaFree(h->fW);
+  cudaFree(h->fE);
+  h->fW = nullptr;
+  h->fE = nullptr;
   if (h->fpool) cudaMemPoolDestroy(h->fpool);
   h->fpool = nullptr;
   h->fU = h->fC = h->fwork = nullptr;
@@ -1825,6 +2070,20 @@ amg_status amg_setup_fine(amg_handle h, const void* d_U, void* stream) {
     AMG_CUDA_TRY(cudaMalloc(&h->fU, nU * sizeof(double2)));
     AMG_CUDA_TRY(cudaMemcpyAsync(h->fU, d_U, nU * sizeof(double2), cudaMemcpyDeviceToDevice, st));
     h->fC = h->clover;
+    // words for the smoother's MR steps; without memory for them these run in FP64
+    if (sap_supported(h)) {
+      if (cudaMalloc(&h->fW, h->g.V * kFixQ * sizeof(int4)) == cudaSuccess &&
+          cudaMalloc(&h->fE, h->g.Vc * sizeof(int)) == cudaSuccess) {
+        fixed_words_kernel<<<(unsigned)h->g.Vc, 256, 0, st>>>((const double2*)h->fU, h->clover, (int4*)h->fW, h->fE,
+                                                              fine_geom(h), 4.0 + h->p.m0);
+        AMG_LAUNCH_CHECK();
+        h->launches++;
+      } else {
+        cudaGetLastError();
+        cudaFree(h->fW);
+        h->fW = nullptr;
+      }
+    }
   } else {
     AMG_CUDA_TRY(cudaMalloc(&h->fU, h->g.V * kLinkQ * sizeof(float4)));
     if (cudaMalloc(&h->fC, h->g.V * kClovQ * sizeof(float4)) != cudaSuccess) {
