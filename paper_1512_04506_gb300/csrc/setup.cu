@@ -160,8 +160,8 @@ __device__ __forceinline__ void field_strength(const double2* __restrict__ U, co
 //
 // Bound: integer multiply-adds and the fixed-point conversions: 72 products of 3 x 3 matrices per site, 12 multiply-adds
 // per complex one (a sixteenth of the time of 4 in FP64 each).  One body for all planes, leaves and steps
-// stays in the instruction cache.  16^3 x 32: 1.09 ms, in FP64 1.99 ms.
-__global__ void __launch_bounds__(128) clover_kernel(const double2* __restrict__ U, double2* __restrict__ C, Geom g,
+// stays in the instruction cache.  16^3 x 32: 1.01 ms (with 255 registers and two CTAs per SM 1.09 ms), in FP64 1.99 ms.
+__global__ void __launch_bounds__(128, 3) clover_kernel(const double2* __restrict__ U, double2* __restrict__ C, Geom g,
                                                      double csw) {
   const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (s >= g.V) return;
