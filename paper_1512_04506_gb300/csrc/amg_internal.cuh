@@ -237,11 +237,14 @@ amg_status amg_internal_assemble_pair(const Geom& g, const double2* R, const dou
 // the same by exact products of slices on the tensor cores; exps: Vc (9 + 2 ntv) ints of scratch
 amg_status amg_internal_assemble_tc(const Geom& g, const double2* R, const double2* U, const double2* clov, int* exps,
                                     double2* part, double m0, bool pair, unsigned* err, cudaStream_t st);
-// Gram-Schmidt per aggregate in fixed point (AMG_ERR_UNSUPPORTED where the other kernels serve)
-amg_status amg_internal_gs_fixed(const Geom& g, const double2* tv, double2* R, bool pair, unsigned* err,
+// Gram-Schmidt per aggregate in fixed point (AMG_ERR_UNSUPPORTED where the other kernels serve); left[agg]: 1 where
+// another kernel has to take the aggregate, else 0
+amg_status amg_internal_gs_fixed(const Geom& g, const double2* tv, double2* R, int* left, bool pair, unsigned* err,
                                  cudaStream_t st);
-// the same in pairs of floats (AMG_ERR_UNSUPPORTED above 1536 entries per aggregate)
-amg_status amg_internal_gs_pair(const Geom& g, const double2* tv, double2* R, unsigned* err, cudaStream_t st);
+// the same in pairs of floats, of the aggregates marked in `only` unless null (AMG_ERR_UNSUPPORTED above 1536 entries
+// per aggregate)
+amg_status amg_internal_gs_pair(const Geom& g, const double2* tv, double2* R, const int* only, unsigned* err,
+                                cudaStream_t st);
 amg_status amg_internal_restrict(amg_coarse* h, const void* y, void* yc, int nrhs, cudaStream_t s);
 amg_status amg_internal_apply(amg_coarse* h, const void* xc, void* yc, int nrhs, cudaStream_t s);
 amg_status amg_internal_prolong(amg_coarse* h, const void* xc, void* x, int nrhs, cudaStream_t s);

@@ -262,7 +262,8 @@ __device__ inline void block_totals(double (&v)[NV], double* sm, double* out) {
 // Bound: the FP64 pipes (one warp instruction in 64 cycles per sub-partition): 4 instructions per element and pair
 // of columns in every dot and every update, and as little else as possible: updates add the negated
 // coefficients, sums halve their values as they go down the lanes, one warp takes the roots and
-// reciprocals.  It serves up to 4 test vectors of large aggregates and those beyond the fixed-point kernel (setup_gs.cu).
+// reciprocals.  It serves up to 4 test vectors of large aggregates, those beyond the fixed-point kernel (setup_gs.cu) and
+// those that it leaves.
 // 16^4, Ntv 2: 0.105 ms; Ntv 20: 5.5 ms; with a multiplication, a fused one and a subtraction per update,
 // 5 additions per value and lane and roots in every thread 8.8 ms.
 constexpr int GS_NB = 4;
@@ -270,7 +271,8 @@ constexpr int GS_EMAX = 8;
 
 template <int E>
 __global__ void __launch_bounds__(256) gs_kernel(const double2* __restrict__ tv, double2* __restrict__ R,
-                                                 Geom g, unsigned* err) {
+                                                 Geom g, const int* __restrict__ only, unsigned* err) {
+  if (only && !only[blockIdx.x]) return;
   __shared__ double sm[8 * 32], tot[32], n0[GS_NB], scal;
   __shared__ double2 coef[AMG_MAX_NTV * GS_NB];  // minus the coefficients
   const long long agg = blockIdx.x;
@@ -789,14 +791,19 @@ static amg_status setup_body(amg_coarse* h, const double2* U, const double2* tv,
   AMG_CUDA_TRY(cudaEventRecord(ev[1], st));
   // Gram-Schmidt, one CTA per aggregate
   const bool pair = h->p.setup_arith == AMG_SETUP_F32PAIR;
-  amg_status gs = amg_internal_gs_fixed(g, tv, h->R64, pair, h->err, st);
-  if (gs == AMG_ERR_UNSUPPORTED && pair) gs = amg_internal_gs_pair(g, tv, h->R64, h->err, st);
+  // what the fixed-point kernel leaves (all, where it does not serve) goes to the kernel of the arithmetic asked for; the
+  // marks, 2 Vc ints, are kept where D_c will be
+  int* left = (int*)h->Dc64;
+  amg_status gs = amg_internal_gs_fixed(g, tv, h->R64, left, pair, h->err, st);
+  if (gs == AMG_ERR_UNSUPPORTED) left = nullptr;
+  else if (gs != AMG_OK) return gs;
+  gs = pair ? amg_internal_gs_pair(g, tv, h->R64, left, h->err, st) : AMG_ERR_UNSUPPORTED;
   if (gs == AMG_ERR_UNSUPPORTED) {
     int T = round_up(g.nagg < 256 ? g.nagg : 256, 32);
     if ((g.nagg + T - 1) / T > GS_EMAX) return AMG_ERR_UNSUPPORTED;
-    void (*const kernels[GS_EMAX])(const double2*, double2*, Geom, unsigned*) = {
+    void (*const kernels[GS_EMAX])(const double2*, double2*, Geom, const int*, unsigned*) = {
         gs_kernel<1>, gs_kernel<2>, gs_kernel<3>, gs_kernel<4>, gs_kernel<5>, gs_kernel<6>, gs_kernel<7>, gs_kernel<8>};
-    kernels[(g.nagg + T - 1) / T - 1]<<<(unsigned)(g.Vc * 2), T, 0, st>>>(tv, h->R64, g, h->err);
+    kernels[(g.nagg + T - 1) / T - 1]<<<(unsigned)(g.Vc * 2), T, 0, st>>>(tv, h->R64, g, left, h->err);
     AMG_LAUNCH_CHECK();
   } else if (gs != AMG_OK) {
     return gs;

@@ -513,7 +513,8 @@ __device__ __forceinline__ pc pc_mul_sub(const pc& w, const pc& q, const pc& cf)
 }
 
 __global__ void __launch_bounds__(512) gs_pair_kernel(const double2* __restrict__ tv, double2* __restrict__ R, Geom g,
-                                                      unsigned* err) {
+                                                      const int* __restrict__ only, unsigned* err) {
+  if (only && !only[blockIdx.x]) return;
   __shared__ float2 red[16 * 2 * GS_PKG * GS_PNB], tot[2 * GS_PKG * GS_PNB];
   __shared__ float4 coef[AMG_MAX_NTV * GS_PNB];
   __shared__ float2 scal;
@@ -760,13 +761,14 @@ amg_status amg_internal_assemble_pair(const Geom& g, const double2* R, const dou
   return AMG_OK;
 }
 
-// Gram-Schmidt of every aggregate in pairs of floats; AMG_ERR_UNSUPPORTED when an aggregate has
-// more than 1536 entries (the FP64 kernel then serves).
-amg_status amg_internal_gs_pair(const Geom& g, const double2* tv, double2* R, unsigned* err, cudaStream_t st) {
+// Gram-Schmidt of every aggregate (of those marked in `only`, unless null) in pairs of floats;
+// AMG_ERR_UNSUPPORTED when an aggregate has more than 1536 entries (the FP64 kernel then serves).
+amg_status amg_internal_gs_pair(const Geom& g, const double2* tv, double2* R, const int* only, unsigned* err,
+                                cudaStream_t st) {
   if (g.nagg > GS_PE * 512) return AMG_ERR_UNSUPPORTED;
   int T = round_up_i((g.nagg + GS_PE - 1) / GS_PE, 32);
   if (T < 64) T = 64;
-  gs_pair_kernel<<<(unsigned)(g.Vc * 2), T, 0, st>>>(tv, R, g, err);
+  gs_pair_kernel<<<(unsigned)(g.Vc * 2), T, 0, st>>>(tv, R, g, only, err);
   AMG_LAUNCH_CHECK();
   return AMG_OK;
 }

@@ -9,12 +9,16 @@
 // its norm where it is projected for the second time.  Products are of words of 31 bits: high x high and the
 // two high x low ones; FULL adds low x low.
 //
+// What is relative to a column's norm loses a site whose entries are far below the column's.  An aggregate where a test
+// vector has such a site (kSiteBits bits or more, entries of 0 apart) is left to the kernels that work in floating
+// point, where every entry is good relative to itself; the others' sites keep at least 47 bits.
+//
 // One CTA of up to 512 threads per aggregate, element n of the aggregate in thread n mod T (E per thread).  Finished
 // columns wait in R as words and become doubles at the end, each element by the thread that wrote it.
 //
 // Bound: integer multiply-adds (12 or, FULL, 16 per complex one, at a quarter of the FP32 rate) and, with one CTA of
 // 128 registers per thread on an SM, the latency of the columns' reads and of the sums' two barriers.  16^4, 4^4 blocks,
-// Ntv 20, FULL: 3.24 ms, in FP64 5.49 ms.
+// Ntv 20, FULL: 3.24 ms, in FP64 5.49 ms; finding what to leave, a pass over the test vectors, 0.08 ms.
 #include "fixed.cuh"
 
 namespace {
@@ -22,6 +26,7 @@ using namespace amgfix;
 
 constexpr int kNB = 4;  // columns per block
 constexpr int kKG = 2;  // earlier columns per round of dots
+constexpr int kSiteBits = 7;  // Gaussian entries: 4 bits between the largest and the smallest of 200,000 sites
 constexpr long long kSmall = 1 << 18;
 
 struct cw {  // complex number in words
@@ -71,9 +76,42 @@ __device__ __forceinline__ void totals(long long (&v)[NV], long long* red, long 
   __syncthreads();
 }
 
+// left[agg]: 1 where a test vector has a site kSiteBits bits or more below its largest entry on the aggregate.  Reads the test
+// vectors once.  One CTA per aggregate; thread t takes column t mod Ntv of every step-th entry.
+__global__ void __launch_bounds__(512) gs_left_kernel(const double2* __restrict__ tv, int* __restrict__ left, Geom g) {
+  extern __shared__ int site[];  // [sites][ntv]: exponent of a column's largest entry at a site
+  __shared__ int top[AMG_MAX_NTV];
+  const long long agg = blockIdx.x, origin = block_origin(g, agg >> 1);
+  const int h = (int)(agg & 1), T = blockDim.x, tid = threadIdx.x, ntv = g.ntv, nagg = g.nagg, n = nagg / 6 * ntv;
+  for (int i = tid; i < n; i += T) site[i] = 0;
+  if (tid < ntv) top[tid] = 0;
+  __syncthreads();
+  const int step = T / ntv, j = tid % ntv;
+  if (tid < step * ntv) {
+    int f = 0;
+#pragma unroll 4
+    for (int i = tid / ntv; i < nagg; i += step) {
+      const double2 v = __ldg(tv + (block_site_fast(g, origin, i / 6) * 12 + 6 * h + i % 6) * ntv + j);
+      const int fe = max((__double2hiint(v.x) >> 20) & 0x7FF, (__double2hiint(v.y) >> 20) & 0x7FF);
+      atomicMax(&site[i / 6 * ntv + j], fe);
+      f = max(f, fe);
+    }
+    atomicMax(&top[j], f);
+  }
+  __syncthreads();
+  bool wide = false;
+  for (int i = tid; i < n; i += T) {
+    const int t = top[i % ntv];
+    wide |= site[i] > 0 && t != 0x7FF && t - site[i] >= kSiteBits;
+  }
+  wide = __syncthreads_or(wide);
+  if (tid == 0) left[agg] = wide;
+}
+
 template <int E, bool FULL>
 __global__ void __launch_bounds__(512) gs_fixed_kernel(const double2* __restrict__ tv, double2* __restrict__ R, Geom g,
-                                                       unsigned* err) {
+                                                       const int* __restrict__ left, unsigned* err) {
+  if (left[blockIdx.x]) return;
   __shared__ long long red[16 * 2 * kKG * kNB], tot[2 * kKG * kNB];
   __shared__ int4 coef[AMG_MAX_NTV * kNB];  // minus the coefficients
   __shared__ int top[kNB];
@@ -350,24 +388,27 @@ __global__ void __launch_bounds__(512) gs_fixed_kernel(const double2* __restrict
 }
 
 template <int E, bool FULL>
-amg_status launch(const Geom& g, const double2* tv, double2* R, unsigned* err, cudaStream_t st) {
+amg_status launch(const Geom& g, const double2* tv, double2* R, int* left, unsigned* err, cudaStream_t st) {
   const int T = (g.nagg + E * 32 - 1) / (E * 32) * 32;
-  gs_fixed_kernel<E, FULL><<<(unsigned)(g.Vc * 2), T, 0, st>>>(tv, R, g, err);
+  gs_left_kernel<<<(unsigned)(g.Vc * 2), 512, (size_t)g.Vb * g.ntv * sizeof(int), st>>>(tv, left, g);
+  AMG_LAUNCH_CHECK();
+  gs_fixed_kernel<E, FULL><<<(unsigned)(g.Vc * 2), T, 0, st>>>(tv, R, g, left, err);
   AMG_LAUNCH_CHECK();
   return AMG_OK;
 }
 }  // namespace
 
-// Gram-Schmidt of every aggregate in fixed point; AMG_ERR_UNSUPPORTED where another kernel serves: above 1536 entries
-// per aggregate, and
+// Gram-Schmidt of every aggregate in fixed point but those marked in `left` (one int per aggregate), which another kernel
+// takes; AMG_ERR_UNSUPPORTED where another kernel serves altogether: above 1536 entries per aggregate, and
 //   in FP64, up to 4 test vectors of large aggregates (16^4, 4^4 blocks, Ntv 2: 0.125 ms, the FP64 kernel 0.105 ms; Ntv
 //     8: 0.75 and 0.97 ms),
 //   in pairs, large aggregates, where FP32 pairs are as fast and need less latency hiding (4^4 blocks, Ntv 24: 3.65 ms,
 //     pairs 3.61 ms; Ntv 8: 0.65 and 0.53 ms; 64-site blocks, Ntv 20: 2.27 and 2.50 ms; 2^4 blocks, Ntv 24: 3.53 and 9.63 ms).
-amg_status amg_internal_gs_fixed(const Geom& g, const double2* tv, double2* R, bool pair, unsigned* err, cudaStream_t st) {
+amg_status amg_internal_gs_fixed(const Geom& g, const double2* tv, double2* R, int* left, bool pair, unsigned* err,
+                                 cudaStream_t st) {
   if (pair && g.nagg <= 512)
-    return g.nagg <= 256 ? launch<1, false>(g, tv, R, err, st) : launch<2, false>(g, tv, R, err, st);
+    return g.nagg <= 256 ? launch<1, false>(g, tv, R, left, err, st) : launch<2, false>(g, tv, R, left, err, st);
   if (pair || g.nagg > 1536 || (g.ntv <= 4 && g.nagg > 512)) return AMG_ERR_UNSUPPORTED;
-  if (g.nagg <= 256) return launch<1, true>(g, tv, R, err, st);
-  return g.nagg <= 1024 ? launch<2, true>(g, tv, R, err, st) : launch<3, true>(g, tv, R, err, st);
+  if (g.nagg <= 256) return launch<1, true>(g, tv, R, left, err, st);
+  return g.nagg <= 1024 ? launch<2, true>(g, tv, R, left, err, st) : launch<3, true>(g, tv, R, left, err, st);
 }
