@@ -231,11 +231,14 @@ inline size_t coarse_elem_bytes(const amg_coarse* h) { return h->p.vec_prec == A
 // two-grid cycle in place of the coarse solve (restriction, one two-grid cycle, prolongation).
 amg_status amg_internal_cgc3(amg_coarse* h, const void* y, void* x, int nrhs, cudaStream_t s);
 amg_status amg_internal_setup(amg_coarse* h, const double2* U, const double2* tv, cudaStream_t s);
-// assembly partial sums ([Vc][5 jobs][2 slots][nc][nc], the layout combine_kernel reads) in pairs of floats
+// assembly partial sums ([Vc][5 jobs][2 slots][nc][nc], the layout combine_kernel reads) in pairs of floats, of the
+// (block, job)s marked in only[blk 5 + job] unless null
 amg_status amg_internal_assemble_pair(const Geom& g, const double2* R, const double2* U, const double2* clov,
-                                      double2* part, double m0, unsigned* err, cudaStream_t st);
-// the same by exact products of slices on the tensor cores; exps: Vc (9 + 2 ntv) ints of scratch
-amg_status amg_internal_assemble_tc(const Geom& g, const double2* R, const double2* U, const double2* clov, int* exps,
+                                      double2* part, double m0, const int* only, unsigned* err, cudaStream_t st);
+// the same by exact products of slices on the tensor cores; work: scratch, whose first 5 Vc ints then mark what another
+// kernel has to take
+size_t amg_internal_assemble_tc_ints(const Geom& g);
+amg_status amg_internal_assemble_tc(const Geom& g, const double2* R, const double2* U, const double2* clov, int* work,
                                     double2* part, double m0, bool pair, unsigned* err, cudaStream_t st);
 // Gram-Schmidt per aggregate in fixed point (AMG_ERR_UNSUPPORTED where the other kernels serve); left[agg]: 1 where
 // another kernel has to take the aggregate, else 0

@@ -471,7 +471,8 @@ struct Tiles {
 template <int TA, int TC>
 __global__ void __launch_bounds__(256) assemble_kernel(const double2* __restrict__ R, const double2* __restrict__ U,
                                 const double2* __restrict__ clov, double2* __restrict__ part, Geom g,
-                                double m0, int ncp, int sb_max) {
+                                double m0, int ncp, int sb_max, const int* __restrict__ only) {
+  if (only && !only[blockIdx.x * 5 + blockIdx.y]) return;
   extern __shared__ double2 smem[];
   const long long blk = blockIdx.x;
   const int job = blockIdx.y;
@@ -718,7 +719,7 @@ static int assemble_warps(int nc, int ta, int tc) {
 
 template <int TA, int TC>
 static amg_status launch_assemble_tile(const Geom& g, const double2* R, const double2* U, const double2* clov,
-                                       double2* part, double m0, cudaStream_t st) {
+                                       double2* part, double m0, const int* only, cudaStream_t st) {
   const int ncp = std::max(round_up(g.nc, TA), round_up(g.nc, TC));
   const int nta = (g.nc + TA - 1) / TA, ntc = (g.nc + TC - 1) / TC, W = assemble_warps(g.nc, TA, TC), T = 32 * W;
   if (T > 256) return AMG_ERR_UNSUPPORTED;
@@ -731,7 +732,7 @@ static amg_status launch_assemble_tile(const Geom& g, const double2* R, const do
   }
   const size_t sm = words * sizeof(double2);
   AMG_CUDA_TRY(cudaFuncSetAttribute(assemble_kernel<TA, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  assemble_kernel<TA, TC><<<dim3((unsigned)g.Vc, 5), T, sm, st>>>(R, U, clov, part, g, m0, ncp, sb);
+  assemble_kernel<TA, TC><<<dim3((unsigned)g.Vc, 5), T, sm, st>>>(R, U, clov, part, g, m0, ncp, sb, only);
   AMG_LAUNCH_CHECK();
   return AMG_OK;
 }
@@ -739,7 +740,7 @@ static amg_status launch_assemble_tile(const Geom& g, const double2* R, const do
 // The tile shape with the fewest FP64 instructions per row and sub-partition (2 Ntv = 40: 5 x 5, two groups
 // of two warps; 48: 3 x 6, four warps; 16: 2 x 4, four groups of one warp).
 static amg_status launch_assemble(const Geom& g, const double2* R, const double2* U, const double2* clov, double2* part,
-                                  double m0, cudaStream_t st) {
+                                  double m0, const int* only, cudaStream_t st) {
   constexpr int shapes[][2] = {{5, 5}, {6, 4}, {4, 4}, {3, 6}, {2, 4}, {3, 2}, {2, 2}};
   int best = -1;
   double cost = 0;
@@ -754,13 +755,13 @@ static amg_status launch_assemble(const Geom& g, const double2* R, const double2
     }
   }
   switch (best) {
-    case 0: return launch_assemble_tile<5, 5>(g, R, U, clov, part, m0, st);
-    case 1: return launch_assemble_tile<6, 4>(g, R, U, clov, part, m0, st);
-    case 2: return launch_assemble_tile<4, 4>(g, R, U, clov, part, m0, st);
-    case 3: return launch_assemble_tile<3, 6>(g, R, U, clov, part, m0, st);
-    case 4: return launch_assemble_tile<2, 4>(g, R, U, clov, part, m0, st);
-    case 5: return launch_assemble_tile<3, 2>(g, R, U, clov, part, m0, st);
-    case 6: return launch_assemble_tile<2, 2>(g, R, U, clov, part, m0, st);
+    case 0: return launch_assemble_tile<5, 5>(g, R, U, clov, part, m0, only, st);
+    case 1: return launch_assemble_tile<6, 4>(g, R, U, clov, part, m0, only, st);
+    case 2: return launch_assemble_tile<4, 4>(g, R, U, clov, part, m0, only, st);
+    case 3: return launch_assemble_tile<3, 6>(g, R, U, clov, part, m0, only, st);
+    case 4: return launch_assemble_tile<2, 4>(g, R, U, clov, part, m0, only, st);
+    case 5: return launch_assemble_tile<3, 2>(g, R, U, clov, part, m0, only, st);
+    case 6: return launch_assemble_tile<2, 2>(g, R, U, clov, part, m0, only, st);
     default: return AMG_ERR_UNSUPPORTED;
   }
 }
@@ -776,7 +777,9 @@ static bool assemble_by_slices(const Geom& g, bool pair) {
   return pair ? g.Vb >= 64 || (g.ntv >= 16 && work >= 3200) : work >= 1800;
 }
 
-// The setup's steps; the caller owns the timing events and frees `part` if a step fails.
+// The setup's steps; the caller owns the timing events and frees `part` if a step fails.  The Gram-Schmidt and the
+// assembly run twice where a fixed-point kernel serves: that one marks the aggregates and (block, job)s whose numbers
+// differ too widely for it, the floating-point kernel of the arithmetic takes these (none: its CTAs return at once).
 static amg_status setup_body(amg_coarse* h, const double2* U, const double2* tv, cudaStream_t st, cudaEvent_t (&ev)[5],
                              double2*& part) {
   const Geom& g = h->g;
@@ -810,17 +813,16 @@ static amg_status setup_body(amg_coarse* h, const double2* U, const double2* tv,
   }
   AMG_CUDA_TRY(cudaEventRecord(ev[2], st));
   // assembly
-  const size_t part_elems = (size_t)g.Vc * 5 * 2 * g.nc * g.nc, exps = (size_t)g.Vc * (9 + 2 * g.ntv);
   const bool slices = assemble_by_slices(g, pair);
-  AMG_CUDA_TRY(cudaMallocAsync((void**)&part, part_elems * sizeof(double2) + (slices ? exps * sizeof(int) : 0), st));
-  if (slices) {
-    AMG_TRY_INTERNAL(amg_internal_assemble_tc(g, h->R64, U, h->clover, (int*)(part + part_elems), part, h->p.m0, pair,
-                                              h->err, st));
-  } else if (pair) {
-    AMG_TRY_INTERNAL(amg_internal_assemble_pair(g, h->R64, U, h->clover, part, h->p.m0, h->err, st));
-  } else {
-    AMG_TRY_INTERNAL(launch_assemble(g, h->R64, U, h->clover, part, h->p.m0, st));
-  }
+  const size_t part_elems = (size_t)g.Vc * 5 * 2 * g.nc * g.nc, work = slices ? amg_internal_assemble_tc_ints(g) : 0;
+  AMG_CUDA_TRY(cudaMallocAsync((void**)&part, part_elems * sizeof(double2) + work * sizeof(int), st));
+  left = slices ? (int*)(part + part_elems) : nullptr;
+  if (slices)
+    AMG_TRY_INTERNAL(amg_internal_assemble_tc(g, h->R64, U, h->clover, left, part, h->p.m0, pair, h->err, st));
+  if (pair)
+    AMG_TRY_INTERNAL(amg_internal_assemble_pair(g, h->R64, U, h->clover, part, h->p.m0, left, h->err, st));
+  else
+    AMG_TRY_INTERNAL(launch_assemble(g, h->R64, U, h->clover, part, h->p.m0, left, st));
   {
     const long long total = g.Vc * 9LL * g.nc * g.nc;
     combine_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(part, h->nbr, h->Dc64, g);

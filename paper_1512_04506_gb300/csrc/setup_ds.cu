@@ -340,7 +340,8 @@ template <int TA, int TC>
 __global__ void __launch_bounds__(512)
 assemble_pair_kernel(const double2* __restrict__ R, const double2* __restrict__ U,
                      const double2* __restrict__ clov, double2* __restrict__ part, Geom g, double m0,
-                     int ncp, int sb_max) {
+                     int ncp, int sb_max, const int* __restrict__ only) {
+  if (only && !only[blockIdx.x * 5 + blockIdx.y]) return;
   extern __shared__ float4 smem4[];
   const int nc = g.nc, Vb = (int)g.Vb;
   float4* As = smem4;  // [sb][6][2 forms][ncp]
@@ -382,7 +383,8 @@ template <int TA, int TC>
 __global__ void __launch_bounds__(512)
 assemble_pair_ws_kernel(const double2* __restrict__ R, const double2* __restrict__ U,
                         const double2* __restrict__ clov, double2* __restrict__ part, Geom g, double m0, int ncp,
-                        int sb, int ncons, unsigned* err) {
+                        int sb, int ncons, const int* __restrict__ only, unsigned* err) {
+  if (only && !only[blockIdx.x * 5 + blockIdx.y]) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   amgpipe::Pipe* pp = reinterpret_cast<amgpipe::Pipe*>(smem_raw);
   float4* buf = reinterpret_cast<float4*>(smem_raw + amgpipe::kPipeBytes);  // [2][A | B][sb][6][2][ncp]
@@ -699,7 +701,7 @@ int lcm_i(int a, int b) {
 
 template <int TA, int TC>
 amg_status launch_ws(const Geom& g, const double2* R, const double2* U, const double2* clov, double2* part,
-                     double m0, unsigned* err, cudaStream_t st) {
+                     double m0, const int* only, unsigned* err, cudaStream_t st) {
   const int ncp = round_up_i(g.nc, lcm_i(TA, TC));
   const int ntiles = (ncp / TA) * (ncp / TC);
   const int ncons = round_up_i(ntiles, 128);
@@ -707,16 +709,17 @@ amg_status launch_ws(const Geom& g, const double2* R, const double2* U, const do
   const size_t sm = amgpipe::kPipeBytes + (size_t)2 * 2 * sb * 12 * ncp * sizeof(float4);
   AMG_CUDA_TRY(cudaFuncSetAttribute(assemble_pair_ws_kernel<TA, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   assemble_pair_ws_kernel<TA, TC><<<dim3((unsigned)g.Vc, 5), ncons + kBuilders, sm, st>>>(R, U, clov, part, g, m0, ncp,
-                                                                                         sb, ncons, err);
+                                                                                         sb, ncons, only, err);
   AMG_LAUNCH_CHECK();
   return AMG_OK;
 }
 
 }  // namespace
 
-// Partial sums of the assembly (the layout the combine step reads) in pairs of floats.
+// Partial sums of the assembly (the layout the combine step reads) in pairs of floats; of the (block, job)s marked in
+// only[blk 5 + job], unless null.
 amg_status amg_internal_assemble_pair(const Geom& g, const double2* R, const double2* U, const double2* clov,
-                                      double2* part, double m0, unsigned* err, cudaStream_t st) {
+                                      double2* part, double m0, const int* only, unsigned* err, cudaStream_t st) {
   if (g.nc <= 48) {
     // tile shape: fewest tile-rows per SM sub-partition (time), at most 384 contraction threads
     struct Shape {
@@ -737,12 +740,12 @@ amg_status amg_internal_assemble_pair(const Geom& g, const double2* R, const dou
       }
     }
     switch (best) {
-      case 0: return launch_ws<2, 3>(g, R, U, clov, part, m0, err, st);
-      case 1: return launch_ws<1, 5>(g, R, U, clov, part, m0, err, st);
-      case 2: return launch_ws<2, 2>(g, R, U, clov, part, m0, err, st);
-      case 3: return launch_ws<1, 4>(g, R, U, clov, part, m0, err, st);
-      case 4: return launch_ws<1, 2>(g, R, U, clov, part, m0, err, st);
-      case 5: return launch_ws<1, 1>(g, R, U, clov, part, m0, err, st);
+      case 0: return launch_ws<2, 3>(g, R, U, clov, part, m0, only, err, st);
+      case 1: return launch_ws<1, 5>(g, R, U, clov, part, m0, only, err, st);
+      case 2: return launch_ws<2, 2>(g, R, U, clov, part, m0, only, err, st);
+      case 3: return launch_ws<1, 4>(g, R, U, clov, part, m0, only, err, st);
+      case 4: return launch_ws<1, 2>(g, R, U, clov, part, m0, only, err, st);
+      case 5: return launch_ws<1, 1>(g, R, U, clov, part, m0, only, err, st);
       default: return AMG_ERR_UNSUPPORTED;
     }
   }
@@ -756,7 +759,7 @@ amg_status amg_internal_assemble_pair(const Geom& g, const double2* R, const dou
   while (sb > 1 && (size_t)sb * 24 * ncp * sizeof(float4) > 200 * 1024) sb >>= 1;
   const size_t sm = (size_t)sb * 24 * ncp * sizeof(float4);
   AMG_CUDA_TRY(cudaFuncSetAttribute(assemble_pair_kernel<2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  assemble_pair_kernel<2, 4><<<dim3((unsigned)g.Vc, 5), T, sm, st>>>(R, U, clov, part, g, m0, ncp, sb);
+  assemble_pair_kernel<2, 4><<<dim3((unsigned)g.Vc, 5), T, sm, st>>>(R, U, clov, part, g, m0, ncp, sb, only);
   AMG_LAUNCH_CHECK();
   return AMG_OK;
 }

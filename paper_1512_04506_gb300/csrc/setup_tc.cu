@@ -11,7 +11,9 @@
 // below 5 x 192 x 128^2 < 2^24, which FP32 holds exactly in any order; every 12 K steps these are added, with
 // their weights, to 64-bit integers in shared memory.  The sums of s >= 5 carry at most 2^-40 of the
 // result each; they stay in FP32 to the end.  Lost are the pairs of s >= DIG, the cut of the columns (56 bits for
-// DIG 7, 64 for DIG 8) and of the 64-bit result.
+// DIG 7, 64 for DIG 8) and of the 64-bit result: about 2^-52 (DIG 8) of the product of the two columns' bounds.  Where the
+// largest product of one site lies far below that, as with test vectors that are small on a face of the block, the (block,
+// job) is left to the kernels that add up in floating point (tc_left_kernel).
 //
 // U_mu P (self: (4 + m0 + C) P) is formed in integers too: coefficients of 62 bits and entries of 61 as two words
 // of 31 bits each, the three leading partial products summed in 64 bits (a 32 x 32 bit multiply-add takes a
@@ -109,25 +111,34 @@ __device__ inline int bound_exp(double v) {
 // inside (face 0) or leave it (1), [8] of |4 + m0| + sum_b |C_ab| over the clover, then [2][ntv] of the columns of
 // P.  Largest magnitude by its bits, so that a NaN wins.
 constexpr int kLinkExps = 9;
+// mags[blk]: [k][site] the exponent of the largest number at a site: k = 0, 1 of P's l and r columns, 2 + mu of the
+// row sums of U_mu, 6 of those of the self term
+constexpr int kMags = 7;
 __global__ void __launch_bounds__(256) tc_bounds_kernel(const double2* __restrict__ R, const double2* __restrict__ U,
-                                                        const double2* __restrict__ clov, int* __restrict__ exps, Geom g,
-                                                        double m0) {
+                                                        const double2* __restrict__ clov, int* __restrict__ exps,
+                                                        int* __restrict__ mags, Geom g, double m0) {
   __shared__ unsigned long long red[kLinkExps + 2 * AMG_MAX_NTV];
+  __shared__ int mag[kMags * kMaxVb];
   const long long blk = blockIdx.x;
-  const int n = kLinkExps + 2 * g.ntv, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n = kLinkExps + 2 * g.ntv, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, Vb = (int)g.Vb;
   for (int i = threadIdx.x; i < n; i += blockDim.x) red[i] = 0;
+  for (int i = threadIdx.x; i < kMags * Vb; i += blockDim.x) mag[i] = 0;
   __syncthreads();
   auto bits = [](double v) { return (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull; };
   for (int row = warp; row < 2 * g.ntv; row += 8) {
     const double2* p = R + (blk * 2 * g.ntv + row) * (long long)g.nagg;
     unsigned long long m = 0;
-    for (int i = lane; i < g.nagg; i += 32) m = max(m, max(bits(p[i].x), bits(p[i].y)));
+    for (int i = lane; i < g.nagg; i += 32) {
+      const unsigned long long v = max(bits(p[i].x), bits(p[i].y));
+      atomicMax(&mag[(row >= g.ntv ? Vb : 0) + i / 6], (int)(v >> 52));
+      m = max(m, v);
+    }
 #pragma unroll
     for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0) red[kLinkExps + row] = m;
   }
   const long long origin = block_origin(g, blk);
-  for (int i = threadIdx.x; i < (int)g.Vb * 24; i += blockDim.x) {  // 12 rows of links, 12 of the clover
+  for (int i = threadIdx.x; i < Vb * 24; i += blockDim.x) {  // 12 rows of links, 12 of the clover
     const int sl = i / 24, q = i % 24;
     const long long s = block_site_fast(g, origin, sl);
     double sum = q < 12 ? 0 : fabs(4.0 + m0);
@@ -141,9 +152,87 @@ __global__ void __launch_bounds__(256) tc_bounds_kernel(const double2* __restric
       slot = 2 * mu + (l % g.B[mu] == g.B[mu] - 1);
     }
     atomicMax(&red[slot], bits(sum));
+    atomicMax(&mag[(q < 12 ? 2 + q / 3 : 6) * Vb + sl], (int)(bits(sum) >> 52));
   }
   __syncthreads();
   for (int i = threadIdx.x; i < n; i += blockDim.x) exps[blk * n + i] = bound_exp(__longlong_as_double((long long)red[i]));
+  for (int i = threadIdx.x; i < kMags * Vb; i += blockDim.x) mags[blk * kMags * Vb + i] = mag[i];
+}
+// left[blk][job]: 1 where, for a pair of chiralities and one kind of links (inside the block, or through the face), the
+// largest product of a site's numbers lies more than kProductBits bits below the product of the largest ones.
+// Gaussian test vectors and SU(3) links: at most 3 bits.  Products that are all 0 are exact, and where a number is not
+// finite the result is not either.
+constexpr int kProductBits = 6;
+__global__ void __launch_bounds__(160) tc_left_kernel(const int* __restrict__ mags, int* __restrict__ left, Geom g) {
+  const int job = threadIdx.x >> 5, lane = threadIdx.x & 31, Vb = (int)g.Vb;
+  const long long blk = blockIdx.x;
+  const int* M = mags + blk * kMags * Vb;
+  auto wide = [](int best, int top, bool finite) {
+    return best > 0 && best < top - kProductBits && finite;
+  };
+  bool any = false;
+  if (job < 4) {
+    int X[4], stride = 1, Bmu = 1;
+    long long r = blk;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      X[m] = (int)(r % g.Lc[m]);
+      r /= g.Lc[m];
+      if (m < job) stride *= g.B[m];
+      if (m == job) {
+        Bmu = g.B[m];
+        X[m] = X[m] + 1 < g.Lc[m] ? X[m] + 1 : 0;
+      }
+    }
+    const long long fwd = ((long long)(X[3] * g.Lc[2] + X[2]) * g.Lc[1] + X[1]) * g.Lc[0] + X[0];
+    for (int p = 0; p < 2; ++p) {  // links inside, links through the face
+      const int *N = p ? mags + fwd * kMags * Vb : M, step = p ? -(Bmu - 1) * stride : stride;
+      int best[2][2] = {}, ta[2] = {}, tb[2] = {}, tu = 0;
+      for (int s = lane; s < Vb; s += 32) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          ta[h] = max(ta[h], M[h * Vb + s]);
+          tb[h] = max(tb[h], N[h * Vb + s]);
+        }
+        if ((s / stride % Bmu == Bmu - 1) != (p == 1)) continue;
+        const int u = M[(2 + job) * Vb + s];
+        tu = max(tu, u);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const int a = M[h * Vb + s], b = N[k * Vb + s + step];
+            if (a > 0 && b > 0 && u > 0) best[h][k] = max(best[h][k], a + b + u);
+          }
+      }
+      tu = __reduce_max_sync(0xffffffffu, tu);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        ta[h] = __reduce_max_sync(0xffffffffu, ta[h]);
+        tb[h] = __reduce_max_sync(0xffffffffu, tb[h]);
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+          any |= wide(__reduce_max_sync(0xffffffffu, best[h][k]), ta[h] + tb[k] + tu, max(max(ta[h], tb[k]), tu) < 0x7FF);
+    }
+  } else {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      int best = 0, ta = 0, tc = 0;
+      for (int s = lane; s < Vb; s += 32) {
+        const int a = M[h * Vb + s], c = M[6 * Vb + s];
+        ta = max(ta, a);
+        tc = max(tc, c);
+        if (a > 0 && c > 0) best = max(best, 2 * a + c);
+      }
+      ta = __reduce_max_sync(0xffffffffu, ta);
+      tc = __reduce_max_sync(0xffffffffu, tc);
+      any |= wide(__reduce_max_sync(0xffffffffu, best), 2 * ta + tc, max(ta, tc) < 0x7FF);
+    }
+  }
+  if (lane == 0) left[blk * 5 + job] = any;
 }
 
 // ------------------------------------------------------------------ digits
@@ -185,7 +274,7 @@ __device__ __forceinline__ void put_digits(long long x0, long long x1, unsigned 
 
 struct TcArgs {
   const double2 *R, *U, *clov;
-  const int* exps;
+  const int *exps, *left;
   double2* part;
   unsigned* err;
   Geom g;
@@ -194,6 +283,7 @@ struct TcArgs {
 
 template <int DIG, bool SELF>
 __global__ void __launch_bounds__(kTcThreads, 1) assemble_tc_kernel(const TcArgs a) {
+  if (a.left[blockIdx.x * 5 + (SELF ? 4 : blockIdx.y)]) return;
   extern __shared__ __align__(128) unsigned char sm[];
   const Geom& g = a.g;
   const int ntv = g.ntv, nc = g.nc, nagg = g.nagg, Vb = (int)g.Vb;
@@ -613,13 +703,21 @@ amg_status launch_tc(const TcArgs& a, cudaStream_t st) {
 }
 }  // namespace
 
-// Partial sums of the assembly (the layout the combine step reads); exps: Vc (9 + 2 ntv) ints of scratch
-amg_status amg_internal_assemble_tc(const Geom& g, const double2* R, const double2* U, const double2* clov, int* exps,
+size_t amg_internal_assemble_tc_ints(const Geom& g) {
+  return (size_t)g.Vc * (5 + kLinkExps + 2 * g.ntv + kMags * g.Vb);
+}
+
+// Partial sums of the assembly (the layout the combine step reads), but those of the (block, job)s marked in work[blk 5 +
+// job], which another kernel takes; work: amg_internal_assemble_tc_ints() ints
+amg_status amg_internal_assemble_tc(const Geom& g, const double2* R, const double2* U, const double2* clov, int* work,
                                     double2* part, double m0, bool pair, unsigned* err, cudaStream_t st) {
   if (g.Vb > kMaxVb || 4 * g.ntv > 128) return AMG_ERR_UNSUPPORTED;
-  tc_bounds_kernel<<<(unsigned)g.Vc, 256, 0, st>>>(R, U, clov, exps, g, m0);
+  int *left = work, *exps = left + g.Vc * 5, *mags = exps + g.Vc * (kLinkExps + 2 * g.ntv);
+  tc_bounds_kernel<<<(unsigned)g.Vc, 256, 0, st>>>(R, U, clov, exps, mags, g, m0);
   AMG_LAUNCH_CHECK();
-  const TcArgs a{R, U, clov, exps, part, err, g, m0};
+  tc_left_kernel<<<(unsigned)g.Vc, 160, 0, st>>>(mags, left, g);
+  AMG_LAUNCH_CHECK();
+  const TcArgs a{R, U, clov, exps, left, part, err, g, m0};
   const amg_status s = pair ? launch_tc<7, false>(a, st) : launch_tc<8, false>(a, st);
   if (s != AMG_OK) return s;
   return pair ? launch_tc<7, true>(a, st) : launch_tc<8, true>(a, st);

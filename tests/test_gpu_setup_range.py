@@ -10,7 +10,7 @@ import pytest
 
 torch = pytest.importorskip("torch")
 
-from oracle import coarse  # noqa: E402
+from oracle import coarse, dirac  # noqa: E402
 from synth import inputs as si  # noqa: E402
 
 import helpers as H  # noqa: E402
@@ -60,3 +60,21 @@ def test_R(B, ntv, kind, arith):
     site = (16, 2, ntv, -1, 6)
     err = np.sqrt((np.abs(R - ref) ** 2).reshape(site).sum((2, 4)))
     assert (err / np.sqrt((np.abs(ref) ** 2).reshape(site).sum((2, 4)))).max() < 1e-12
+
+
+# also an extent of 1 (no link inside), and more columns than the pair tiles with builder warps take
+MORE = CASES + [((1, 4, 4, 5), 12, "spread"), ((4, 3, 3, 3), 26, "faces")]
+
+
+@pytest.mark.parametrize("arith", ["fp64", "pair"])
+@pytest.mark.parametrize("B,ntv,kind", MORE, ids=["%s-%d-%s" % ("x".join(map(str, c[0])), c[1], c[2]) for c in MORE])
+def test_Dc(B, ntv, kind, arith):
+    """Every direction of every site's D_c to 1e-12 of its own norm, the library's bound for a direction."""
+    import paper_1512_04506_gb300 as amg
+    L, Uh, tv = _inputs(B, ntv, kind)
+    U = np.moveaxis(Uh.reshape(H.field_shape(L) + (4, 3, 3)), 4, 0)
+    Q = coarse.orthonormalize(tv.reshape(H.field_shape(L) + (4, 3, ntv)), B)
+    ref = coarse.coarse_operator(U, dirac.clover_field(U, H.CSW), H.M0, Q, L, B)
+    _, Dc = _setup(amg, L, B, ntv, Uh, tv, arith)
+    err = np.sqrt((np.abs(Dc - ref) ** 2).sum((2, 3)) / (np.abs(ref) ** 2).sum((2, 3)))
+    assert err.max() < 1e-12
