@@ -85,10 +85,77 @@ __device__ __forceinline__ I3 scaled(const long long (&re)[9], const long long (
   return m;
 }
 
-// F_{mu nu}(x) = (Q - Q^dagger)/8 with Q the four counter-clockwise leaves at x: leaf l follows the steps
-// +mu, +nu, -mu, -nu from the l-th on, round.  f: imaginary parts of the diagonal, real and imaginary parts of
-// (0,1), (0,2), (1,2); F is anti-Hermitian.
-__device__ __forceinline__ void field_strength(const double2* __restrict__ U, const Geom& g, const int (&x)[4], int mu,
+// Step s of leaf `leaf` of plane (mu, nu) from y: the leaf follows the steps +mu, +nu, -mu, -nu from the leaf-th on, round.
+// Returns the link passed (its adjoint is meant if `back`) and moves y on.
+__device__ __forceinline__ const double2* leaf_link(const double2* __restrict__ U, const Geom& g, int (&y)[4], int mu, int nu,
+                                                    int leaf, int s, bool& back) {
+  const int k = (leaf + s) & 3, d = k & 1 ? nu : mu;
+  back = k >= 2;
+  long long site = 0;
+  int step = 0;
+#pragma unroll
+  for (int m = 3; m >= 0; --m) {
+    const int fwd = y[m] + 1 < g.L[m] ? y[m] + 1 : 0, bwd = y[m] > 0 ? y[m] - 1 : g.L[m] - 1;
+    if (m == d) step = back ? bwd : fwd;
+    if (m == d && back) y[m] = bwd;
+    site = site * g.L[m] + y[m];
+  }
+#pragma unroll
+  for (int m = 0; m < 4; ++m)
+    if (m == d) y[m] = step;
+  return U + (site * 4 + d) * 9;
+}
+
+// field_strength in FP64, where every part keeps the accuracy of its own size.  Out of line: links close to 1, whose F
+// is far below them, are the exception.
+__device__ __noinline__ void field_strength_fp64(const double2* __restrict__ U, const Geom& g, int x0, int x1, int x2, int x3,
+                                                 int mu, int nu, double* f) {
+  double2 q[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) q[k] = make_double2(0, 0);
+#pragma unroll 1
+  for (int leaf = 0; leaf < 4; ++leaf) {
+    int y[4] = {x0, x1, x2, x3};
+    double2 t[9] = {};
+#pragma unroll 1
+    for (int s = 0; s < 4; ++s) {
+      bool back;
+      const double2* p = leaf_link(U, g, y, mu, nu, leaf, s, back);
+      double2 u[9], z[9];
+#pragma unroll
+      for (int k = 0; k < 9; ++k) {
+        u[k] = __ldg(p + (back ? k % 3 * 3 + k / 3 : k));
+        if (back) u[k].y = -u[k].y;
+      }
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          z[i * 3 + j] = make_double2(0, 0);
+#pragma unroll
+          for (int k = 0; k < 3; ++k) cfma(z[i * 3 + j], t[i * 3 + k], u[k * 3 + j]);
+        }
+#pragma unroll
+      for (int k = 0; k < 9; ++k) t[k] = s ? z[k] : u[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 9; ++k) q[k] = cadd(q[k], t[k]);
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) f[i] = 0.25 * q[4 * i].y;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int i = k < 2 ? 0 : 1, j = k < 1 ? 1 : 2;
+    f[3 + 2 * k] = 0.125 * (q[i * 3 + j].x - q[j * 3 + i].x);
+    f[4 + 2 * k] = 0.125 * (q[i * 3 + j].y + q[j * 3 + i].y);
+  }
+}
+
+// F_{mu nu}(x) = (Q - Q^dagger)/8 with Q the four counter-clockwise leaves at x.  f: imaginary parts of the diagonal, real and
+// imaginary parts of (0,1), (0,2), (1,2); F is anti-Hermitian.  The fixed-point sums are good to about 2^-57 of the links'
+// products; returns true if F lies below 2^-kWeakBits of these.
+constexpr int kWeakBits = 7;  // spread 0.2 of the links: F about 0.1
+__device__ __forceinline__ bool field_strength(const double2* __restrict__ U, const Geom& g, const int (&x)[4], int mu,
                                                int nu, double* f) {
   long long qr[9], qi[9];
   int unit = 0;  // of Q
@@ -101,21 +168,9 @@ __device__ __forceinline__ void field_strength(const double2* __restrict__ U, co
     int uz = 0;
 #pragma unroll 1
     for (int s = 0; s < 4; ++s) {
-      const int k = (leaf + s) & 3, d = k & 1 ? nu : mu;
-      const bool back = k >= 2;
-      long long site = 0;
-      int step = 0;
-#pragma unroll
-      for (int m = 3; m >= 0; --m) {
-        const int fwd = y[m] + 1 < g.L[m] ? y[m] + 1 : 0, bwd = y[m] > 0 ? y[m] - 1 : g.L[m] - 1;
-        if (m == d) step = back ? bwd : fwd;
-        if (m == d && back) y[m] = bwd;
-        site = site * g.L[m] + y[m];
-      }
-#pragma unroll
-      for (int m = 0; m < 4; ++m)
-        if (m == d) y[m] = step;
-      const I3 u = load_link(U + (site * 4 + d) * 9, back, bad);
+      bool back;
+      const double2* p = leaf_link(U, g, y, mu, nu, leaf, s, back);
+      const I3 u = load_link(p, back, bad);
       if (s == 0) {
         t = u;
       } else {
@@ -151,6 +206,10 @@ __device__ __forceinline__ void field_strength(const double2* __restrict__ U, co
     f[3 + 2 * k] = value((qr[i * 3 + j] >> 1) - (qr[j * 3 + i] >> 1));
     f[4 + 2 * k] = value((qi[i * 3 + j] >> 1) + (qi[j * 3 + i] >> 1));
   }
+  int top = 0;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) top = max(top, (__double2hiint(f[k]) >> 20) & 0x7FF);
+  return top < unit + 58 - kWeakBits + 1022 && !bad;
 }
 
 // In the chiral basis sigma_{mu nu} = diag(s^l, s^r) with 2x2 blocks
@@ -160,7 +219,7 @@ __device__ __forceinline__ void field_strength(const double2* __restrict__ U, co
 //
 // Bound: integer multiply-adds and the fixed-point conversions: 72 products of 3 x 3 matrices per site, 12 multiply-adds
 // per complex one (a sixteenth of the time of 4 in FP64 each).  One body for all planes, leaves and steps
-// stays in the instruction cache.  16^3 x 32: 1.01 ms (with 255 registers and two CTAs per SM 1.09 ms), in FP64 1.99 ms.
+// stays in the instruction cache (links close to 1 take a second one, in FP64).  16^3 x 32: 1.02 ms (with 255 registers and two CTAs per SM 1.09 ms), in FP64 1.99 ms.
 __global__ void __launch_bounds__(128, 3) clover_kernel(const double2* __restrict__ U, double2* __restrict__ C, Geom g,
                                                      double csw) {
   const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -174,9 +233,14 @@ __global__ void __launch_bounds__(128, 3) clover_kernel(const double2* __restric
   c[2] = (int)(r % g.L[2]);
   c[3] = (int)(r / g.L[2]);
   double F[6][9];  // planes (0,1), (0,2), (1,2), (0,3), (1,3), (2,3)
+  unsigned weak = 0;
 #pragma unroll 1
   for (int p = 0; p < 6; ++p)
-    field_strength(U, g, c, p < 2 ? 0 : p == 2 ? 1 : p - 3, p == 0 ? 1 : p < 3 ? 2 : 3, F[p]);
+    weak |= (unsigned)field_strength(U, g, c, p < 2 ? 0 : p == 2 ? 1 : p - 3, p == 0 ? 1 : p < 3 ? 2 : 3, F[p]) << p;
+#pragma unroll 1
+  for (int p = 0; p < 6; ++p)
+    if (weak >> p & 1)
+      field_strength_fp64(U, g, c[0], c[1], c[2], c[3], p < 2 ? 0 : p == 2 ? 1 : p - 3, p == 0 ? 1 : p < 3 ? 2 : 3, F[p]);
   auto entry = [&](int p, int k) {
     const int i = k / 3, j = k % 3, o = 2 * (i + j) + 1;
     return i == j ? make_double2(0, F[p][i]) : make_double2(i < j ? F[p][o] : -F[p][o], F[p][o + 1]);
