@@ -708,11 +708,14 @@ __device__ __forceinline__ void colour_block(const FineGeom& g, int k, int colou
 // with local index t in block b at (b kFixQ + q) Vb + t: 36 link entries (re, im), then per chirality the diagonal
 // of 4 + m0 + C (6 numbers, two per word), C's entries 01, 02, 12 and its upper right 3 x 3 block (see kClovQ).
 // All of a block relative to 2^exps[b], a bound of every row's and column's sum of |re| + |im|, in units of 2^-61.
+// exps[b] = INT_MAX, and no words: a number that is not finite, or a link more than kFixBits bits below the bound.
 constexpr int kFixQ = 66, kFixClov = 36;
+constexpr int kFixBits = 8;
 __global__ void __launch_bounds__(256) fixed_words_kernel(const double2* __restrict__ U, const double2* __restrict__ clov,
                                                           int4* __restrict__ W, int* __restrict__ exps, FineGeom g,
                                                           double mass) {
   __shared__ unsigned long long top;
+  __shared__ int low;  // exponent of the smallest link
   const int b = blockIdx.x;
   int X[4], row = b;
 #pragma unroll
@@ -729,7 +732,10 @@ __global__ void __launch_bounds__(256) fixed_words_kernel(const double2* __restr
     }
     return site_of(g, x);
   };
-  if (threadIdx.x == 0) top = 0;
+  if (threadIdx.x == 0) {
+    top = 0;
+    low = 0x7FF;
+  }
   __syncthreads();
   auto mag = [](double2 z) { return fabs(z.x) + fabs(z.y); };
   for (int i = threadIdx.x; i < g.Vb * 5; i += blockDim.x) {
@@ -743,6 +749,7 @@ __global__ void __launch_bounds__(256) fixed_words_kernel(const double2* __restr
         bound(mag(u[3 * k]) + mag(u[3 * k + 1]) + mag(u[3 * k + 2]));
         bound(mag(u[k]) + mag(u[3 + k]) + mag(u[6 + k]));
       }
+      if (m > 0) atomicMin(&low, (int)(m >> 52));
     } else {
       for (int k = 0; k < 12; ++k) {
         double v = fabs(mass);
@@ -755,8 +762,9 @@ __global__ void __launch_bounds__(256) fixed_words_kernel(const double2* __restr
   __syncthreads();
   const double v = __longlong_as_double((long long)top) * 1.015625;  // |v| < 2^e with room for roundings
   const int f = (__double2hiint(v) >> 20) & 0x7FF, e = max(f - 1022, -900);
-  if (threadIdx.x == 0) exps[b] = f == 0x7FF ? INT_MAX : e;
-  if (f == 0x7FF) return;
+  const bool none = f == 0x7FF || f - low > kFixBits;
+  if (threadIdx.x == 0) exps[b] = none ? INT_MAX : e;
+  if (none) return;
   for (int i = threadIdx.x; i < g.Vb * kFixQ; i += blockDim.x) {
     const int t = i % g.Vb, q = i / g.Vb;
     const long long s = site(t);
@@ -884,13 +892,14 @@ __device__ __forceinline__ void site_fixed(const int4* __restrict__ W, const int
 
 // One SAP half sweep on the blocks of one colour: x += MR_{n_mr}(B_b, (y - D x)|_b) per block; FP64.
 // grid (Vc / 2, nrhs); blockDim >= Vb (threads past Vb only join the sums); dynamic smem: rho
-// [12][Vb] + 3 doubles per warp + 3 doubles + 2 ints.
+// [12][Vb] + 3 doubles per warp + 3 doubles + 4 ints.
 //
 // Bound: the FP64 pipes (one warp instruction in 64 cycles per sub-partition).  FIXED: the MR steps apply B in fixed
 // point (a multiply-add takes a sixteenth of that): rho as 59-bit integers relative to its largest entry in the block, links and
 // clover as words prepared once, sums of 64 bits; the sums over the block and the updates stay in FP64.  An
-// application is then good to 2^-57 of the block's largest entry.  A block with an entry that is not finite takes
-// the FP64 steps.  12 x 8 x 24 x 16, blocks 3 x 4 x 4 x 2, 3 columns: 447 us a half sweep, in FP64 703 us; 16^4 in
+// application is then good to 2^-57 of the block's largest entry.  A step takes FP64, where every site's sums are good
+// relative to its own terms, if an entry is not finite or a site's largest one (unless 0) lies more than kFixBits
+// bits below the block's.  12 x 8 x 24 x 16, blocks 3 x 4 x 4 x 2, 3 columns: 447 us a half sweep, in FP64 703 us; 16^4 in
 // 2^4 blocks 497 and 944 us.
 template <bool FIXED>
 __global__ void __launch_bounds__(256) sap_kernel(const double2* __restrict__ U, const double2* __restrict__ Cl,
@@ -902,7 +911,8 @@ __global__ void __launch_bounds__(256) sap_kernel(const double2* __restrict__ U,
   C* rho = reinterpret_cast<C*>(smem);
   int4* rhow = reinterpret_cast<int4*>(smem);
   double* red = reinterpret_cast<double*>(smem + (size_t)g.Vb * 12 * sizeof(C));
-  int* top = reinterpret_cast<int*>(red + 3 * ((blockDim.x + 31) / 32) + 3);  // of rho's exponents, by parity of the step
+  // largest exponent of rho, and the smallest of the sites', by parity of the step
+  int *top = reinterpret_cast<int*>(red + 3 * ((blockDim.x + 31) / 32) + 3), *low = top + 2;
   const int r = blockIdx.y;
   int X[4];
   colour_block(g, blockIdx.x, colour, X);
@@ -922,13 +932,16 @@ __global__ void __launch_bounds__(256) sap_kernel(const double2* __restrict__ U,
   const int st1 = g.B[0], st2 = g.B[0] * g.B[1], st3 = g.B[0] * g.B[1] * g.B[2];
   const int4* W = nullptr;
   int eb = 0;
-  bool fixed = FIXED;
+  bool words_ok = FIXED;
   if (FIXED) {
     const long long b = ((long long)(X[3] * g.Lc[2] + X[2]) * g.Lc[1] + X[1]) * g.Lc[0] + X[0];
     W = words + b * kFixQ * g.Vb;
     eb = __ldg(exps + b);
-    fixed = eb != INT_MAX;
-    if (t < 2) top[t] = 0;
+    words_ok = eb != INT_MAX;
+    if (t < 2) {
+      top[t] = 0;
+      low[t] = 0x7FF;
+    }
     __syncthreads();
   }
   // residual r = y - D x on this site (full D: neighbours outside the block have the other colour)
@@ -950,17 +963,25 @@ __global__ void __launch_bounds__(256) sap_kernel(const double2* __restrict__ U,
     double v[3] = {0, 0, 0}, unit = 1;
     C o[12];
     int er = 0;
-    if (FIXED && fixed) {
+    bool fixed = words_ok;
+    if (FIXED && words_ok) {
       int f = 0;
 #pragma unroll
       for (int q = 0; q < 12; ++q)
         f = max(f, max((__double2hiint(rr[q].x) >> 20) & 0x7FF, (__double2hiint(rr[q].y) >> 20) & 0x7FF));
+      const int l = __reduce_min_sync(0xffffffffu, f > 0 ? f : 0x7FF);
       f = __reduce_max_sync(0xffffffffu, f);
-      if ((t & 31) == 0) atomicMax(&top[it & 1], f);
+      if ((t & 31) == 0) {
+        atomicMax(&top[it & 1], f);
+        atomicMin(&low[it & 1], l);
+      }
       __syncthreads();
       f = top[it & 1];
-      if (t == 0) top[(it + 1) & 1] = 0;  // last read before the previous step's coefficient
-      fixed = f != 0x7FF;
+      fixed = f != 0x7FF && f - low[it & 1] <= kFixBits;
+      if (t == 0) {  // last read before the previous step's coefficient
+        top[(it + 1) & 1] = 0;
+        low[(it + 1) & 1] = 0x7FF;
+      }
       er = max(f - 1022, -900);
     }
     if (FIXED && fixed) {
@@ -1723,7 +1744,7 @@ amg_status launch_sap32(amg_coarse* h, const void* yv, void* xv, int nrhs, int n
 
 amg_status launch_sap64(amg_coarse* h, const void* y, void* x, int nrhs, int n_cycles, int n_mr, cudaStream_t st) {
   const int threads = (h->g.Vb + 31) / 32 * 32;
-  const size_t smem = (size_t)h->g.Vb * 12 * sizeof(double2) + (size_t)(threads / 32 + 1) * 3 * sizeof(double) + 8;
+  const size_t smem = (size_t)h->g.Vb * 12 * sizeof(double2) + (size_t)(threads / 32 + 1) * 3 * sizeof(double) + 16;
   if (threads > 256 || smem > 227 * 1024) return AMG_ERR_UNSUPPORTED;
   auto* kernel = h->fW ? sap_kernel<true> : sap_kernel<false>;
   AMG_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
