@@ -226,6 +226,10 @@ amg_status amg_cgc(amg_handle h, const void *d_y, void *d_x, int nrhs, double to
  * amg_setup_fine -- keeps the links d_U ([V][4][3][3] complex double, device, the array given to
  * amg_setup_coarse; not retained) in the handle in vec_prec, with the clover field of the setup,
  * for the fine operator D.  Asynchronous on the stream; may be called again (replaces the copy).
+ * Device memory held until the handle goes: in FP32 512 bytes per site (links and clover) and, where
+ * the smoother can run, its copies of x and y, 192 bytes per site and column of max_nrhs, as many
+ * columns as 2 GB take but one at least; in FP64 576 bytes per site and, where the smoother can run,
+ * 1056 for its fixed-point words (without memory for these or for the copies it works without them).
  */
 amg_status amg_setup_fine(amg_handle h, const void *d_U, void *stream);
 

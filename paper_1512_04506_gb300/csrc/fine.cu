@@ -1667,8 +1667,9 @@ amg_status sweep32(amg_coarse* h, const float2* y, float2* x, int nrhs, int n_cy
 }
 
 // The sweeps run on copies of x and y in block order, one vector per column; x is copied back.  The
-// copies come from the handle's pool, at most kColBytes at a time (columns are independent).  While
-// the stream is captured, or without memory for them, the sweeps work on the caller's vectors.
+// copies come from the handle's pool, at most kColBytes at a time but one column at least (columns are
+// independent).  While the stream is captured, or without memory for them, the sweeps work on the
+// caller's vectors.
 constexpr size_t kColBytes = (size_t)2 << 30;
 int sap_copy_columns(const amg_coarse* h, int nrhs) {
   return (int)std::max<size_t>(1, std::min<size_t>(nrhs, kColBytes / (2 * h->g.V * 12 * sizeof(float2))));
@@ -1697,13 +1698,13 @@ amg_status blocked_copy(amg_coarse* h, const float2* v, const float2* w, int nrh
   return AMG_OK;
 }
 
-// The pool, with the copies of max_nrhs columns allocated once here rather than in the first sweep; kept
-// until the handle goes.  Without it (a device without pools) the sweeps do without copies.
+// The pool, with the copies of max_nrhs columns allocated once here rather than in the first sweep; the pool
+// keeps them until the handle goes.  Without it (a device without pools) the sweeps do without copies.
 void sap_pool(amg_coarse* h, cudaStream_t st) {
   cudaMemPoolProps props = {};
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
-  uint64_t keep = kColBytes;
+  uint64_t keep = sap_copy_bytes(h, h->p.max_nrhs);
   void* w = nullptr;
   if (cudaGetDevice(&props.location.id) != cudaSuccess || cudaMemPoolCreate(&h->fpool, &props) != cudaSuccess) {
     h->fpool = nullptr;
@@ -2112,7 +2113,7 @@ amg_status amg_setup_fine(amg_handle h, const void* d_U, void* stream) {
       amg_internal_free_fine(h);
       return AMG_ERR_OOM;
     }
-    sap_pool(h, st);
+    if (sap_supported(h)) sap_pool(h, st);
     links_words_kernel<<<8 * amg_sm_count(), 256, 0, st>>>((const double2*)d_U, (float4*)h->fU, h->g);
     AMG_LAUNCH_CHECK();
     clover_words_kernel<<<8 * amg_sm_count(), 256, 0, st>>>(h->clover, (float4*)h->fC, h->g);

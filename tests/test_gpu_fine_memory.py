@@ -1,0 +1,58 @@
+"""Device memory that amg_setup_fine holds.
+
+FP32: links and clover (288 and 224 bytes per site) and, where the smoother can run, its copies of max_nrhs columns of x
+and y (192 bytes per site and column, at most 2 GB unless one column takes more), kept between calls.
+"""
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+SLACK = 64 << 20  # granularity of pools and allocations, and what the setup's own pool gives back meanwhile
+
+
+def _held(L, B, max_nrhs, use):
+    import paper_1512_04506_gb300 as amg
+    V = L[0] * L[1] * L[2] * L[3]
+    st = torch.cuda.current_stream()
+    U = torch.eye(3, dtype=torch.complex128, device="cuda").expand(V, 4, 3, 3).contiguous()
+    tv = torch.ones(V, 4, 3, 1, dtype=torch.complex128, device="cuda")
+    p = amg.make_params(L, B, 1, max_nrhs, -0.3, 1.0, amg.AMG_FP32, amg.AMG_FP32, amg.AMG_FP32)
+    h, _ = amg.amg_setup_coarse(p, U, tv, st)
+    try:
+        del tv
+        y = torch.ones(V, 4, 3, 1, dtype=torch.complex64, device="cuda") if use else None
+        x = torch.zeros_like(y) if use else None
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        free = torch.cuda.mem_get_info()[0]
+        amg.amg_setup_fine(h, U, st)
+        torch.cuda.synchronize()
+        if use:
+            amg.amg_sap(h, y, x, 1, 1, 1, st)
+            torch.cuda.synchronize()
+        held = free - torch.cuda.mem_get_info()[0]
+        assert amg.amg_sync_status(h) == amg.AMG_OK
+        return held, V
+    finally:
+        amg.amg_destroy(h)
+        torch.cuda.empty_cache()
+
+
+def test_no_copies_without_the_smoother():
+    """An odd coarse extent: only D can run, and nothing is held for the smoother."""
+    held, V = _held((12, 16, 16, 16), (4, 4, 4, 4), 64, False)
+    assert held < 512 * V + SLACK
+
+
+def test_copies_kept():
+    held, V = _held((16, 16, 16, 16), (4, 4, 4, 4), 16, True)
+    assert abs(held - (512 * V + 192 * 16 * V)) < SLACK
+
+
+def test_large_lattice_keeps_one_column():
+    """Above 11.2 million sites one column's copies exceed 2 GB; they are kept between calls all the same."""
+    held, V = _held((48, 48, 48, 112), (4, 4, 4, 4), 1, True)
+    assert 192 * V > 2 << 30
+    assert abs(held - (512 * V + 192 * V)) < SLACK
