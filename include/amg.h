@@ -229,7 +229,8 @@ amg_status amg_cgc(amg_handle h, const void *d_y, void *d_x, int nrhs, double to
  * Device memory held until the handle goes: in FP32 512 bytes per site (links and clover) and, where
  * the smoother can run, its copies of x and y, 192 bytes per site and column of max_nrhs, as many
  * columns as 2 GB take but one at least; in FP64 576 bytes per site and, where the smoother can run,
- * 1056 for its fixed-point words (without memory for these or for the copies it works without them).
+ * 1056 for its fixed-point words (without memory for these or for the copies it works without them;
+ * amg_solve and amg_adaptive_setup give them back if they run out of memory).
  */
 amg_status amg_setup_fine(amg_handle h, const void *d_U, void *stream);
 

@@ -1772,6 +1772,24 @@ amg_status check_fine(amg_coarse* h, const void* a, const void* b, int nrhs) {
   return AMG_OK;
 }
 
+// Allocates by alloc(), which returns a cudaError_t; where memory runs out once more after giving back what the smoother
+// holds for its speed: the fixed-point words (its steps then take FP64) and the pool's idle copies (the sweeps then
+// allocate them again or do without).
+template <typename F>
+cudaError_t alloc_or_give_back(amg_coarse* h, F&& alloc) {
+  cudaError_t e = alloc();
+  if (e != cudaErrorMemoryAllocation) return e;
+  cudaGetLastError();
+  cudaFree(h->fW);
+  cudaFree(h->fE);
+  h->fW = nullptr;
+  h->fE = nullptr;
+  if (h->fpool) cudaMemPoolTrimTo(h->fpool, 0);
+  e = alloc();
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+
 bool sap_supported(const amg_coarse* h) {
   for (int mu = 0; mu < 4; ++mu)
     if (h->g.Lc[mu] % 2) return false;
@@ -1815,7 +1833,7 @@ amg_status solve_impl(amg_coarse* h, const amg_vcycle_params* vp, const void* f,
     cudaFree(h->fwork);
     h->fwork = nullptr;
     h->fwork_bytes = 0;
-    AMG_CUDA_TRY(cudaMalloc(&h->fwork, need));
+    AMG_CUDA_TRY(alloc_or_give_back(h, [&] { return cudaMalloc(&h->fwork, need); }));
     h->fwork_bytes = need;
   }
   C* Vb = (C*)h->fwork;
@@ -2007,7 +2025,8 @@ amg_status adaptive_impl(amg_coarse* h, const amg_vcycle_params* vp, const doubl
   const long long n12 = h->g.V * 12;
   const size_t vbytes = (size_t)n12 * chunk * sizeof(C);
   void* buf = nullptr;
-  AMG_CUDA_TRY(cudaMallocAsync(&buf, 2 * vbytes + 256 + (size_t)ntv * (sizeof(double) + sizeof(double2)), st));
+  AMG_CUDA_TRY(alloc_or_give_back(
+      h, [&] { return cudaMallocAsync(&buf, 2 * vbytes + 256 + (size_t)ntv * (sizeof(double) + sizeof(double2)), st); }));
   C* y = (C*)buf;
   C* x = y + (size_t)n12 * chunk;
   double* dn = (double*)(x + (size_t)n12 * chunk);

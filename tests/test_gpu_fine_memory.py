@@ -56,3 +56,38 @@ def test_large_lattice_keeps_one_column():
     held, V = _held((48, 48, 48, 112), (4, 4, 4, 4), 1, True)
     assert 192 * V > 2 << 30
     assert abs(held - (512 * V + 192 * V)) < SLACK
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_outer_solve_gets_the_smoothers_memory(prec):
+    """Free memory that holds the outer solve's workspace only together with what the smoother holds for its speed."""
+    import paper_1512_04506_gb300 as amg
+    L, B, restart, max_nrhs = (24, 24, 24, 24), (4, 4, 4, 4), 30, 32 if prec == "fp32" else 1
+    V, z = 24 ** 4, 8 if prec == "fp32" else 16
+    pr, ct = (amg.AMG_FP32, torch.complex64) if prec == "fp32" else (amg.AMG_FP64, torch.complex128)
+    need, held = (2 * restart + 2) * V * 12 * z, 192 * 32 * V if prec == "fp32" else 1056 * V
+    from synth import device as sd
+    st = torch.cuda.current_stream()
+    U, tv, f = sd.links(71, 0.3, L), sd.test_vectors(71, 4, L), sd.fine_rhs(71, 1, L, ct)
+    vp, out = amg.make_vcycle_params(0.05, 30, 50, 1, 2), []
+    for full in (False, True):
+        h, _ = amg.amg_setup_coarse(amg.make_params(L, B, 4, max_nrhs, -0.3, 1.0, pr, pr, pr), U, tv, st)
+        try:
+            amg.amg_setup_fine(h, U, st)
+            u = torch.empty_like(f)
+            amg.amg_vcycle(h, vp, f, u, 1, st)
+            torch.cuda.synchronize()
+            torch.cuda.empty_cache()
+            fill = None
+            if full:
+                fill = torch.empty(torch.cuda.mem_get_info()[0] - need + held // 2, dtype=torch.uint8, device="cuda")
+                assert torch.cuda.mem_get_info()[0] < need
+            info = amg.amg_solve(h, vp, f, u, 1, tol=0.0, restart=restart, max_applies=3, stream=st)
+            del fill
+            out.append((info[0][1], u))
+            assert amg.amg_sync_status(h) == amg.AMG_OK
+        finally:
+            amg.amg_destroy(h)
+            torch.cuda.empty_cache()
+    assert abs(out[1][0] / out[0][0] - 1) < 1e-5
+    assert torch.linalg.vector_norm(out[1][1] - out[0][1]) < 1e-5 * torch.linalg.vector_norm(out[0][1])
