@@ -191,10 +191,13 @@ void amg_note_cuda_error(const char* file, int line, cudaError_t e);
 // Records a printf-style message as the calling thread's last error.
 void amg_note_error(const char* fmt, ...);
 
+// Returns from the caller when a CUDA call fails.  The thread's last error is cleared, so that the next
+// launch is not taken to have failed.
 #define AMG_CUDA_TRY(call)                                \
   do {                                                    \
     cudaError_t e_ = (call);                              \
     if (e_ != cudaSuccess) {                              \
+      cudaGetLastError();                                 \
       amg_note_cuda_error(__FILE__, __LINE__, e_);        \
       return e_ == cudaErrorMemoryAllocation ? AMG_ERR_OOM : AMG_ERR_CUDA; \
     }                                                     \

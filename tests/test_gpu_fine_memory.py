@@ -91,3 +91,30 @@ def test_outer_solve_gets_the_smoothers_memory(prec):
             torch.cuda.empty_cache()
     assert abs(out[1][0] / out[0][0] - 1) < 1e-5
     assert torch.linalg.vector_norm(out[1][1] - out[0][1]) < 1e-5 * torch.linalg.vector_norm(out[0][1])
+
+
+def test_out_of_memory_is_reported_once():
+    """An outer solve without memory for its workspace: the call fails, the next one does not."""
+    import paper_1512_04506_gb300 as amg
+    from synth import device as sd
+    L, st = (24, 24, 24, 24), torch.cuda.current_stream()
+    U, f = sd.links(73, 0.3, L), sd.fine_rhs(73, 1, L, torch.complex128)
+    pr = amg.AMG_FP64
+    h, _ = amg.amg_setup_coarse(amg.make_params(L, (4, 4, 4, 4), 2, 1, -0.3, 1.0, pr, pr, pr), U, sd.test_vectors(73, 2, L), st)
+    try:
+        amg.amg_setup_fine(h, U, st)
+        vp, u = amg.make_vcycle_params(0.05, 30, 50, 1, 2), torch.empty_like(f)
+        amg.amg_vcycle(h, vp, f, u, 1, st)
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        fill = torch.empty(torch.cuda.mem_get_info()[0] - (1 << 30), dtype=torch.uint8, device="cuda")
+        with pytest.raises(amg.AmgError) as e:  # 3.9 GB
+            amg.amg_solve(h, vp, f, u, 1, tol=0.0, restart=30, max_applies=3, stream=st)
+        assert e.value.status == amg.AMG_ERR_OOM
+        amg.amg_dirac_apply(h, f, u, 1, st)
+        amg.amg_vcycle(h, vp, f, u, 1, st)
+        assert amg.amg_sync_status(h) == amg.AMG_OK
+        del fill
+    finally:
+        amg.amg_destroy(h)
+        torch.cuda.empty_cache()
