@@ -159,8 +159,8 @@ struct amg_coarse {
   float* tc5_xs = nullptr;    // their power-of-two scale per site,
   float* tc5_ds = nullptr;    // the power-of-two scale of every FP32 stencil block,
   void* tc5_d16 = nullptr;    // and the FP16 storage as planes with rotated pieces
-  void* fU = nullptr;         // fine operator (amg_setup_fine): links, FP64 [V][4][3][3], FP32 in block order (fine.cu)
-  void* fC = nullptr;         // its clover: FP64 the handle's clover itself, FP32 block-order words of 2 C
+  void* fU = nullptr;         // fine operator (amg_setup_fine): links, FP64 [V][4][3][3], FP32 halved in block order (fine.cu)
+  void* fC = nullptr;         // its clover: FP64 the handle's clover itself, FP32 block-order words
   void* fW = nullptr;         // FP64 smoother: links and clover as fixed-point words (fine.cu),
   int* fE = nullptr;          // their exponent per block
   cudaMemPool_t fpool = nullptr;  // FP32 smoother: copies of x and y in block order (stream-ordered)

@@ -159,8 +159,9 @@ __device__ __forceinline__ void site_term(const C* __restrict__ Cl, T mass, cons
 //
 // The clover of a chirality is [[H, X], [X^dag, -H]] with H = H^dag (spin blocks sigma_m (x) G_m with
 // Hermitian G_m): 27 real numbers instead of 36, as 14 complex words (H00, H11), (H22, 0), H01, H02,
-// H12, X row by row.  All are stored times 2, so that with a mass of 2 (4 + m0) the sums below are
-// 2 D psi with hops of weight one (an exact scaling), halved once at the end.
+// H12, X row by row.  The links are stored halved (exactly), so that the hops have weight one and the
+// sums below are D psi itself: with sums of 2 D psi, halved at the end, D psi and <B rho, B rho> left
+// the FP32 range by a factor of 2 and 4 sooner.
 constexpr int kLinkQ = 18, kClovQ = 14;
 
 __device__ __forceinline__ float2 lo2(float4 f) { return make_float2(f.x, f.y); }
@@ -246,7 +247,7 @@ __device__ __forceinline__ void colour_row(const float2* u, const float2 h[6], i
     }
   }
 }
-// o += -(1 -+ g_mu)-hop of twice D for colour a of the product w: -w on the upper half, +- A^dag w on
+// o += -(1 -+ g_mu)-hop for colour a of the product w: -w on the upper half, +- A^dag w on
 // the lower
 template <bool FWD, int mu>
 __device__ __forceinline__ void add_hop(float2 w0, float2 w1, int a, float2 o[12]) {
@@ -268,8 +269,8 @@ __device__ __forceinline__ void hop2(const float2* u, const float2 p[12], float2
   }
 }
 
-// out = (mass2 + 2 C) p from the site's clover words c (14 complex per chirality, times 2)
-__device__ __forceinline__ void site_term2(const float2 c[2 * kClovQ], float mass2, const float2 p[12], float2 out[12]) {
+// out = (mass + C) p from the site's clover words c (14 complex per chirality)
+__device__ __forceinline__ void site_term_words(const float2 c[2 * kClovQ], float mass, const float2 p[12], float2 out[12]) {
 #pragma unroll
   for (int hh = 0; hh < 2; ++hh) {
     const float2* k = c + hh * kClovQ;
@@ -277,7 +278,7 @@ __device__ __forceinline__ void site_term2(const float2 c[2 * kClovQ], float mas
     const float dg[3] = {k[0].x, k[0].y, k[1].x};
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      float2 s0 = zscale(u[a], mass2), s1 = zscale(d[a], mass2);
+      float2 s0 = zscale(u[a], mass), s1 = zscale(d[a], mass);
       s0.x = fmaf(dg[a], u[a].x, s0.x);
       s0.y = fmaf(dg[a], u[a].y, s0.y);
       s1.x = fmaf(-dg[a], d[a].x, s1.x);
@@ -463,7 +464,7 @@ __global__ void __launch_bounds__(128, NC == 1 ? 4 : 3) dirac32_kernel(const flo
                                                                        const float4* __restrict__ Cl,
                                                                        const float2* __restrict__ psi,
                                                                        const float2* __restrict__ y,
-                                                                       float2* __restrict__ out, FineGeom g, float mass2,
+                                                                       float2* __restrict__ out, FineGeom g, float mass,
                                                                        FastDiv dn) {
   const int groups = (int)dn.d, nrhs = groups * NC;
   const long long total = g.V * groups;
@@ -491,7 +492,7 @@ __global__ void __launch_bounds__(128, NC == 1 ? 4 : 3) dirac32_kernel(const flo
       float2 c[2 * kClovQ];
       load_words<kClovQ>(Cl + (long long)b * kClovQ * Vb + t, Vb, c);
 #pragma unroll
-      for (int k = 0; k < NC; ++k) site_term2(c, mass2, p[k], o[k]);
+      for (int k = 0; k < NC; ++k) site_term_words(c, mass, p[k], o[k]);
     }
     const float4* Us = U + (long long)b * kLinkQ * Vb + t;
     int stride = 1;
@@ -515,10 +516,8 @@ __global__ void __launch_bounds__(128, NC == 1 ? 4 : 3) dirac32_kernel(const flo
 #pragma unroll
     for (int c = 0; c < NC; ++c)
 #pragma unroll
-      for (int k = 0; k < 12; ++k) {
-        o[c][k] = zscale(o[c][k], 0.5f);
+      for (int k = 0; k < 12; ++k)
         if (SUB) o[c][k] = zsub(p[c][k], o[c][k]);
-      }
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
       float2* q = out + (s * 12 + k) * nrhs + r;
@@ -544,7 +543,7 @@ template <bool SUB>
 __global__ void __launch_bounds__(kDiracSites, 2) dirac32_block_kernel(const float4* __restrict__ U,
                                                                        const float4* __restrict__ Cl, const float2* psi,
                                                                        const float2* __restrict__ y, float2* out,
-                                                                       FineGeom g, float mass2, int nb, int nblocks) {
+                                                                       FineGeom g, float mass, int nb, int nblocks) {
   __shared__ float4 tile[kDiracSites * kRec];
   __shared__ unsigned lex[kDiracSites];
   const int Vb = g.Vb, b0 = blockIdx.x * nb, n = min(nb, nblocks - b0) * Vb, i = threadIdx.x;
@@ -568,7 +567,7 @@ __global__ void __launch_bounds__(kDiracSites, 2) dirac32_block_kernel(const flo
   if (act) {
     const float4* own = tile + i * kRec;
     get_words<6>(own, 1, p);
-    site_term2(c, mass2, p, o);
+    site_term_words(c, mass, p, o);
     const float4* Us = U + (long long)b * kLinkQ * Vb + t;
     int stride = 1;
 #define AMG_HOPS2(MU)                                                                                          \
@@ -590,8 +589,6 @@ __global__ void __launch_bounds__(kDiracSites, 2) dirac32_block_kernel(const flo
     AMG_HOPS2(2)
     AMG_HOPS2(3)
 #undef AMG_HOPS2
-#pragma unroll
-    for (int k = 0; k < 12; ++k) o[k] = zscale(o[k], 0.5f);
     if (SUB) {
       load12(y, s, 1, 0, p);
 #pragma unroll
@@ -1170,7 +1167,7 @@ __device__ __forceinline__ void site_hops(const float4* us, const float4* R, con
 
 template <bool BLOCKED, bool LANES>
 __global__ void __launch_bounds__(256, 1) sap32_kernel(const float4* __restrict__ U, const float4* __restrict__ Cl,
-                                                       const float2* __restrict__ y, float2* x, FineGeom g, float mass2,
+                                                       const float2* __restrict__ y, float2* x, FineGeom g, float mass,
                                                        int nrhs, int nr, int groups, int nblk, int lanes, int colour,
                                                        int n_mr, unsigned* err) {
   using namespace amgpipe;
@@ -1245,7 +1242,7 @@ __global__ void __launch_bounds__(256, 1) sap32_kernel(const float4* __restrict_
       float2 cl[2 * kClovQ];
       get_words<kClovQ>(cs + ta, Vb, cl);
       get_words<6>(xr + ta, Vb, x0);
-      site_term2(cl, mass2, x0, o);
+      site_term_words(cl, mass, x0, o);
     }
     site_hops<0, true>(us, xr, h0, nf[0], fi[0], in[0], below[0], Vb, ta, st[0], o);
     site_hops<1, true>(us, xr, h1, nf[1], fi[1], in[1], below[1], Vb, ta, st[1], o);
@@ -1253,7 +1250,7 @@ __global__ void __launch_bounds__(256, 1) sap32_kernel(const float4* __restrict_
     site_hops<3, true>(us, xr, h3, nf[3], fi[3], in[3], below[3], Vb, ta, st[3], o);
 #pragma unroll
     for (int q = 0; q < 12; ++q) {  // rho = y - D x
-      p[q] = make_float2(fmaf(-0.5f, o[q].x, e[q].x), fmaf(-0.5f, o[q].y, e[q].y));
+      p[q] = zsub(e[q], o[q]);
       e[q] = zzero<float2>();
     }
     __syncthreads();  // x is read
@@ -1264,7 +1261,7 @@ __global__ void __launch_bounds__(256, 1) sap32_kernel(const float4* __restrict_
       {
         float2 cl[2 * kClovQ];
         get_words<kClovQ>(cs + ta, Vb, cl);
-        site_term2(cl, mass2, p, o);  // o = 2 B rho
+        site_term_words(cl, mass, p, o);  // o = B rho
       }
       site_hops<0, false>(us, xr, h0, 0, 0, in[0], below[0], Vb, ta, st[0], o);
       site_hops<1, false>(us, xr, h1, 0, 0, in[1], below[1], Vb, ta, st[1], o);
@@ -1288,11 +1285,10 @@ __global__ void __launch_bounds__(256, 1) sap32_kernel(const float4* __restrict_
       } else {
         cta_alpha_all(v, red + (it & 1) * 24, al, ok);
       }
-      if (ok) {  // al = alpha / 2 (o = 2 B rho): e += alpha rho, rho -= alpha B rho
-        const float2 al2 = make_float2(2.f * al.x, 2.f * al.y);
+      if (ok) {  // e += alpha rho, rho -= alpha B rho
 #pragma unroll
         for (int q = 0; q < 12; ++q) {
-          zfma(e[q], al2, p[q]);
+          zfma(e[q], al, p[q]);
           float2 ap = zzero<float2>();
           zfma(ap, al, o[q]);
           p[q] = zsub(p[q], ap);
@@ -1551,7 +1547,7 @@ __global__ void links_words_kernel(const double2* __restrict__ in, float4* __res
     const long long b = e / (kLinkQ * g.Vb);
     const int q = (int)(e / g.Vb % kLinkQ);
     const double2* U = in + block_site_fast(g, block_origin(g, b), (int)(e % g.Vb)) * 36 + 2 * q;
-    out[e] = make_float4((float)U[0].x, (float)U[0].y, (float)U[1].x, (float)U[1].y);
+    out[e] = make_float4(0.5f * (float)U[0].x, 0.5f * (float)U[0].y, 0.5f * (float)U[1].x, 0.5f * (float)U[1].y);
   }
 }
 __global__ void clover_words_kernel(const double2* __restrict__ in, float4* __restrict__ out, Geom g) {
@@ -1565,12 +1561,12 @@ __global__ void clover_words_kernel(const double2* __restrict__ in, float4* __re
     for (int k = 0; k < 2; ++k) {
       const int w = 2 * (q % 7) + k;  // complex word of the chirality
       if (w < 2) {
-        v[k].x = 2.f * (float)C[w * 2 * 7].x;                      // H00, H22
-        v[k].y = w == 0 ? 2.f * (float)C[7].x : 0.f;               // H11
+        v[k].x = (float)C[w * 2 * 7].x;                      // H00, H22
+        v[k].y = w == 0 ? (float)C[7].x : 0.f;               // H11
       } else {
         const int a = w < 5 ? (w == 4 ? 1 : 0) : (w - 5) / 3;
         const int c = w < 5 ? (w == 2 ? 1 : 2) : 3 + (w - 5) % 3;
-        v[k] = make_float2(2.f * (float)C[a * 6 + c].x, 2.f * (float)C[a * 6 + c].y);
+        v[k] = make_float2((float)C[a * 6 + c].x, (float)C[a * 6 + c].y);
       }
     }
     out[e] = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
@@ -1599,7 +1595,7 @@ amg_status dirac_any(amg_coarse* h, const void* psi, const void* y, void* out, i
     else
       dirac_kernel<false><<<grid, 128, 0, st>>>(U, C, (const double2*)psi, nullptr, (double2*)out, g, mass, nrhs);
   } else {
-    const float mass2 = 2.f * (float)(4.0 + h->p.m0);
+    const float mass = (float)(4.0 + h->p.m0);
     auto* U = (const float4*)h->fU;
     auto* C = (const float4*)h->fC;
     const float2 *p = (const float2*)psi, *yy = (const float2*)y;
@@ -1609,13 +1605,13 @@ amg_status dirac_any(amg_coarse* h, const void* psi, const void* y, void* out, i
     if (nrhs == 1 && ctas >= amg_sm_count()) {
       const int threads = (nb * g.Vb + 31) / 32 * 32;
       auto* k = y ? dirac32_block_kernel<true> : dirac32_block_kernel<false>;
-      k<<<ctas, threads, 0, st>>>(U, C, p, yy, (float2*)out, g, mass2, nb, nblocks);
+      k<<<ctas, threads, 0, st>>>(U, C, p, yy, (float2*)out, g, mass, nb, nblocks);
     } else {
       const int nc = nrhs % 2 ? 1 : 2, groups = nrhs / nc;
       const FastDiv dn = fast_div(groups);
       const long long threads = h->g.V * groups;
       auto* k = nc == 1 ? pick_dirac32<1>(y != nullptr, threads < (1LL << 31)) : pick_dirac32<2>(y != nullptr, threads < (1LL << 31));
-      k<<<(unsigned)std::min((threads + 127) / 128, 16LL * amg_sm_count()), 128, 0, st>>>(U, C, p, yy, (float2*)out, g, mass2, dn);
+      k<<<(unsigned)std::min((threads + 127) / 128, 16LL * amg_sm_count()), 128, 0, st>>>(U, C, p, yy, (float2*)out, g, mass, dn);
     }
   }
   AMG_LAUNCH_CHECK();
@@ -1655,10 +1651,10 @@ amg_status sweep32(amg_coarse* h, const float2* y, float2* x, int nrhs, int n_cy
   AMG_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const int nblk = (int)(h->g.Vc / 2), units = (nblk + subs - 1) / subs;
   const int nr = sap_columns(units, nrhs, sap_slots(threads, smem)), groups = (nrhs + nr - 1) / nr;
-  const float mass2 = 2.f * (float)(4.0 + h->p.m0);
+  const float mass = (float)(4.0 + h->p.m0);
   for (int c = 0; c < n_cycles; ++c)
     for (int colour = 0; colour < 2; ++colour) {
-      k<<<units * groups, threads, smem, st>>>((const float4*)h->fU, (const float4*)h->fC, y, x, g, mass2, nrhs, nr, groups,
+      k<<<units * groups, threads, smem, st>>>((const float4*)h->fU, (const float4*)h->fC, y, x, g, mass, nrhs, nr, groups,
                                               nblk, lanes, colour, n_mr, h->err);
       AMG_LAUNCH_CHECK();
       h->launches++;
