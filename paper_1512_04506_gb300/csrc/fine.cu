@@ -1667,6 +1667,7 @@ amg_status sweep32(amg_coarse* h, const float2* y, float2* x, int nrhs, int n_cy
 // independent).  While the stream is captured, or without memory for them, the sweeps work on the
 // caller's vectors.
 constexpr size_t kColBytes = (size_t)2 << 30;
+constexpr size_t kPoolStep = (size_t)64 << 20;  // more than what a pool adds to an allocation (32 MB pieces)
 int sap_copy_columns(const amg_coarse* h, int nrhs) {
   return (int)std::max<size_t>(1, std::min<size_t>(nrhs, kColBytes / (2 * h->g.V * 12 * sizeof(float2))));
 }
@@ -1700,7 +1701,7 @@ void sap_pool(amg_coarse* h, cudaStream_t st) {
   cudaMemPoolProps props = {};
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
-  uint64_t keep = sap_copy_bytes(h, h->p.max_nrhs);
+  uint64_t keep = std::max(kColBytes, sap_copy_bytes(h, h->p.max_nrhs) + kPoolStep);
   void* w = nullptr;
   if (cudaGetDevice(&props.location.id) != cudaSuccess || cudaMemPoolCreate(&h->fpool, &props) != cudaSuccess) {
     h->fpool = nullptr;
