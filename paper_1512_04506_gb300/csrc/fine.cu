@@ -1665,7 +1665,9 @@ amg_status sweep32(amg_coarse* h, const float2* y, float2* x, int nrhs, int n_cy
 // The sweeps run on copies of x and y in block order, one vector per column; x is copied back.  The
 // copies come from the handle's pool, at most kColBytes at a time but one column at least (columns are
 // independent).  While the stream is captured, or without memory for them, the sweeps work on the
-// caller's vectors.
+// caller's vectors; so they do for one cycle of up to three columns, where the copies cost more than
+// they save (us with and without, 4 MR steps: 16^4 and one column 59 and 47, 32^4 672 and 595, 24 16^3
+// and two columns 161 and 157, 16^3 x 32 and three 263 and 264, four 340 and 382).
 constexpr size_t kColBytes = (size_t)2 << 30;
 constexpr size_t kPoolStep = (size_t)64 << 20;  // more than what a pool adds to an allocation (32 MB pieces)
 int sap_copy_columns(const amg_coarse* h, int nrhs) {
@@ -1717,6 +1719,7 @@ amg_status launch_sap32(amg_coarse* h, const void* yv, void* xv, int nrhs, int n
   float2* x = (float2*)xv;
   const size_t n = (size_t)h->g.V * 12;
   if (n_cycles < 1) return AMG_OK;
+  if (n_cycles == 1 && nrhs <= 3) return sweep32<false>(h, y, x, nrhs, n_cycles, n_mr, st);
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   AMG_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
   const int chunk = sap_copy_columns(h, nrhs);

@@ -97,3 +97,19 @@ def test_sap_two_sets_of_copies():
         assert amg.amg_sync_status(h) == amg.AMG_OK
     finally:
         amg.amg_destroy(h)
+
+
+def test_one_cycle_with_and_without_copies():
+    """One cycle of up to three columns works on the caller's vectors, of four on copies: the same bits."""
+    import paper_1512_04506_gb300 as amg
+    c = Fine(amg, (12, 8, 8, 16), (3, 4, 4, 2), 1, 861, "fp32", max_nrhs=4)
+    try:
+        y, x0 = c.dev(c.vec(4, 1)), c.dev(c.vec(4, 2))
+        x = x0.clone()
+        amg.amg_sap(c.h, y, x, 4, 1, 3, c.stream)
+        for n in (1, 2, 3):
+            part = x0[..., :n].contiguous()
+            amg.amg_sap(c.h, y[..., :n].contiguous(), part, n, 1, 3, c.stream)
+            assert torch.equal(part, x[..., :n])
+    finally:
+        c.close()
