@@ -6,8 +6,7 @@
 // One Arnoldi step is two launches: w = D_c V_j (the application reads the unnormalised vector times
 // 1/h_{j,j-1} and stores V_j on the way), then the cooperative k_arnoldi (dots <V_i, w>, column j of
 // H, w -= sum H_ij V_i with |w|^2, Givens rotation and convergence test, phases separated by grid
-// barriers).  Where a cooperative launch cannot hold its CTAs resident, k_dots and k_update take its
-// place, each ending in a last-CTA reduction.  Grids follow the vectors' length.  Once every
+// barriers).  Grids follow the vectors' length.  Once every
 // right-hand side has converged the device flag `done` makes every later kernel return at once
 // and a mapped host word receives the solve's ticket; the host reads it after the next
 // application is queued (so the GPU never waits for the host) or, without polling, launches the
@@ -22,7 +21,7 @@ constexpr int ST_T = 256;
 constexpr int MAXR = 16;
 constexpr int kMaxPartRows = 1024;  // most CTAs of the partial-sum kernels (rows of FState::part)
 
-// CTAs of the partial-sum kernels (k_dots, k_update, k_residual): two per SM.
+// Most CTAs of the kernels that leave partial sums (k_residual; k_arnoldi takes one per SM): two per SM.
 int solve_nblk() { return std::min(2 * amg_sm_count(), kMaxPartRows); }
 
 struct FState {
@@ -54,28 +53,6 @@ template <> __device__ inline float2 from_d<float2>(double2 v) { return make_flo
 template <> __device__ inline double2 from_d<double2>(double2 v) { return v; }
 
 __device__ inline double2 ld_cg(const double2* p) { return __ldcg(p); }
-
-// CTA-wide sum of nrhs complex values per thread; thread r < nrhs writes out[r].
-__device__ inline void cta_sum_store(double2 (&acc)[MAXR], int nrhs, double2* out) {
-  __shared__ double2 sm[ST_T / 32][MAXR];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int r = 0; r < MAXR; ++r) {
-    if (r >= nrhs) break;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      acc[r].x += __shfl_xor_sync(0xffffffffu, acc[r].x, o);
-      acc[r].y += __shfl_xor_sync(0xffffffffu, acc[r].y, o);
-    }
-    if (lane == 0) sm[warp][r] = acc[r];
-  }
-  __syncthreads();
-  if (threadIdx.x < nrhs) {
-    double2 t = make_double2(0, 0);
-    for (int w = 0; w < ST_T / 32; ++w) t = cadd(t, sm[w][threadIdx.x]);
-    out[threadIdx.x] = t;
-  }
-}
 
 // Last-CTA election: every CTA publishes its partial sums, then counts itself in; the CTA that
 // brings the count to `total` sees every partial (threadfence before the count) and resets it.
@@ -227,94 +204,15 @@ __device__ void arnoldi_step_warp(FState& s, int r, int j, double n2, int* any) 
   }
 }
 
-// part[(i * nblk + b) * nrhs + r] = partial <V_i, w> (i = blockIdx.y); the last CTA writes H[.][i][j].
-template <typename CT>
-__global__ void __launch_bounds__(ST_T) k_dots(FState s, const CT* __restrict__ w, const CT* __restrict__ V,
-                                               long long vstride, int j) {
-  if (*s.done) return;
-  const int i = blockIdx.y;
-  const CT* Vi = V + i * vstride;
-  CT a[MAXR];
-#pragma unroll
-  for (int r = 0; r < MAXR; ++r) a[r] = CT{0, 0};
-  for (long long row = blockIdx.x * (long long)ST_T + threadIdx.x; row < s.rows;
-       row += (long long)s.nblk * ST_T) {
-#pragma unroll
-    for (int r = 0; r < MAXR; ++r) {
-      if (r >= s.nrhs) break;
-      cfmac(a[r], Vi[row * s.nrhs + r], w[row * s.nrhs + r]);
-    }
-  }
-  double2 acc[MAXR];
-#pragma unroll
-  for (int r = 0; r < MAXR; ++r) acc[r] = to_d(a[r]);
-  cta_sum_store(acc, s.nrhs, s.part + ((long long)i * s.nblk + blockIdx.x) * s.nrhs);
-  if (!last_block(s.counter, s.nblk * (j + 1))) return;
-  const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int t = warp; t < (j + 1) * s.nrhs; t += nw) {
-    const double2 sum = warp_sum_partials(s.part, s.nblk, s.nrhs, t);
-    const int ii = t / s.nrhs, r = t % s.nrhs;
-    if ((threadIdx.x & 31) == 0) s.H[((long long)r * (s.m + 1) + ii) * s.m + j] = s.active[r] ? sum : make_double2(0, 0);
-  }
-}
-
-// w -= sum_{i<=j} H[r][i][j] V_i and |w|^2; the last CTA does the Givens step (arnoldi_step_warp).
-template <typename CT>
-__global__ void __launch_bounds__(ST_T) k_update(FState s, CT* __restrict__ w, const CT* __restrict__ V,
-                                                 long long vstride, int j) {
-  if (*s.done) return;
-  __shared__ CT hc[AMG_MAX_NTV + 1][MAXR];
-  for (int e = threadIdx.x; e < (j + 1) * s.nrhs; e += ST_T) {
-    const int i = e / s.nrhs, r = e % s.nrhs;
-    hc[i][r] = from_d<CT>(ld_cg(s.H + ((long long)r * (s.m + 1) + i) * s.m + j));
-  }
-  __syncthreads();
-  CT a[MAXR];
-#pragma unroll
-  for (int r = 0; r < MAXR; ++r) a[r] = CT{0, 0};
-  for (long long row = blockIdx.x * (long long)ST_T + threadIdx.x; row < s.rows;
-       row += (long long)s.nblk * ST_T) {
-#pragma unroll
-    for (int r = 0; r < MAXR; ++r) {
-      if (r >= s.nrhs) break;
-      CT v = w[row * s.nrhs + r];
-      for (int i = 0; i <= j; ++i) {
-        const CT q = V[i * vstride + row * s.nrhs + r];
-        const CT c = hc[i][r];
-        v.x -= c.x * q.x - c.y * q.y;
-        v.y -= c.x * q.y + c.y * q.x;
-      }
-      w[row * s.nrhs + r] = v;
-      a[r].x += v.x * v.x + v.y * v.y;
-    }
-  }
-  double2 acc[MAXR];
-#pragma unroll
-  for (int r = 0; r < MAXR; ++r) acc[r] = to_d(a[r]);
-  cta_sum_store(acc, s.nrhs, s.part + (long long)blockIdx.x * s.nrhs);
-  if (!last_block(s.counter, s.nblk)) return;
-  __shared__ int any;
-  __shared__ double n2s[MAXR];
-  if (threadIdx.x == 0) any = 0;
-  for (int r = threadIdx.x >> 5; r < s.nrhs; r += blockDim.x >> 5) {
-    const double2 v = warp_sum_partials(s.part, s.nblk, s.nrhs, r);
-    if ((threadIdx.x & 31) == 0) n2s[r] = v.x;
-  }
-  __syncthreads();
-  for (int r = threadIdx.x >> 5; r < s.nrhs; r += ST_T / 32) arnoldi_step_warp(s, r, j, n2s[r], &any);
-  __syncthreads();
-  if (threadIdx.x == 0 && !any) mark_done(s);
-}
-
 // ---- fused Arnoldi step: one cooperative launch of at most one CTA per SM does the dots, the
 // Hessenberg column, the update with |w|^2 and the Givens step, with two grid barriers in place of a
 // kernel boundary and a last-CTA hand-off.  The element loops are flat: with nrhs dividing 32 (POW2)
 // as above, otherwise the CTA uses a multiple of nrhs threads, so that a thread again meets one
-// column, and column sums go through shared memory (the row-per-thread form of k_dots / k_update,
-// which served these counts, took 31 and 38 us a launch for 12 columns at 16^3 x 32).  With one or a few columns the coarse vectors are small (Vc * 2 Ntv rows, about a
-// megabyte), each phase is a few memory round trips and the launch and barrier latencies set the
-// time; with 16 columns they reach hundreds of megabytes and the phases stream, which is what the
-// round shapes below are for.
+// column, and column sums go through shared memory (a row per thread, in a kernel for the dots and
+// one for the update, took 31 and 38 us a launch for 12 columns at 16^3 x 32).  With one or a few
+// columns the coarse vectors are small (Vc * 2 Ntv rows, about a megabyte), each phase is a few memory
+// round trips and the launch and barrier latencies set the time; with 16 columns they reach hundreds of
+// megabytes and the phases stream, which is what the round shapes below are for.
 constexpr int AR_T = 512;  // most threads of a CTA
 constexpr int AR_W = AR_T / 32;
 template <typename CT>
@@ -761,20 +659,15 @@ const void* arnoldi_kernel(bool is_long, bool pow2) {
 }
 
 // Largest grid of the cooperative k_arnoldi: one CTA per SM (at most solve_nblk(), the partial-sum rows'
-// length); 0 when the device cannot hold it resident.  Found once per device.
+// length); -1 when the device cannot hold it resident.  Found once per device.
 template <typename CT>
 int arnoldi_grid() {
-  static int cache[64];
-  static bool init = false;
-  if (!init) {
-    for (int& c : cache) c = -1;
-    init = true;
-  }
+  static int cache[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) dev = 0;
   if (dev >= 64) dev = 63;
   int& g = cache[dev];
-  if (g < 0) {
+  if (g == 0) {
     int coop = 0, per = 1 << 30;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     for (const void* k : {arnoldi_kernel<CT>(false, true), arnoldi_kernel<CT>(false, false), arnoldi_kernel<CT>(true, true),
@@ -783,7 +676,7 @@ int arnoldi_grid() {
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, k, AR_T, 0);
       per = std::min(per, p);
     }
-    g = (coop && per > 0) ? std::min(amg_sm_count(), solve_nblk()) : 0;
+    g = (coop && per > 0) ? std::min(amg_sm_count(), solve_nblk()) : -1;
   }
   return g;
 }
@@ -800,7 +693,8 @@ amg_status solve_impl(amg_coarse* h, long long rows, amg_apply_fn op, const CT* 
   // warp instruction in 16 cycles per SM).  4^4 in 2^4 blocks, 256 elements in FP64: a coarse-grid
   // correction takes 97 us, 117 with a CTA of 16 warps, 130 with 152 CTAs.
   const long long rounds = (vstride + 4 * AR_T - 1) / (4 * AR_T);
-  const int ar_grid = (int)std::min<long long>(arnoldi_grid<CT>(), rounds);  // fused step (k_arnoldi) when > 0
+  const int ar_grid = (int)std::min<long long>(arnoldi_grid<CT>(), rounds);
+  if (ar_grid < 1) return AMG_ERR_UNSUPPORTED;
   const int ar_threads = (int)std::min<long long>(AR_T, (vstride + 127) / 128 * 32);
   SolveWork& sw = h->sw;
   FState s;
@@ -878,19 +772,12 @@ amg_status solve_impl(amg_coarse* h, long long rows, amg_apply_fn op, const CT* 
         stop = true;
         break;
       }
-      if (ar_grid > 0) {
-        const CT* Vr = V;
-        int jj = j;
-        void* args[] = {&s, &nxt, &Vr, (void*)&vstride, &jj};
-        const void* kern = arnoldi_kernel<CT>(rows * nrhs > AR_LONG, 32 % nrhs == 0);
-        AMG_CUDA_TRY(cudaLaunchCooperativeKernel(kern, dim3(ar_grid), dim3(ar_threads), args, 0, st));
-        h->launches += 1;
-      } else {
-        k_dots<CT><<<dim3(nblk, j + 1), ST_T, 0, st>>>(s, nxt, V, vstride, j);
-        k_update<CT><<<nblk, ST_T, 0, st>>>(s, nxt, V, vstride, j);
-        AMG_LAUNCH_CHECK();
-        h->launches += 2;
-      }
+      const CT* Vr = V;
+      int jj = j;
+      void* args[] = {&s, &nxt, &Vr, (void*)&vstride, &jj};
+      const void* kern = arnoldi_kernel<CT>(rows * nrhs > AR_LONG, 32 % nrhs == 0);
+      AMG_CUDA_TRY(cudaLaunchCooperativeKernel(kern, dim3(ar_grid), dim3(ar_threads), args, 0, st));
+      h->launches += 1;
       std::swap(cur, nxt);
       record();
     }
