@@ -55,9 +55,11 @@ TRAFFIC_MRHS_FP32 = 1449390080
 # DRAM traffic / algorithmic bytes of the fused batch launch, from the reduced-volume capture
 # (profiles/batch_kernel_small_mixed.md); the full launch's traffic is taken in that proportion
 BATCH_TRAFFIC_RATIO = 0.990
-# DRAM traffic / algorithmic bytes of one SAP half sweep, from the 16^4 capture (profiles/sap_16x4.md:
-# 31.24 MB for 65,536 sites x 504 B); the 32^4 launch is taken in proportion
-SAP_TRAFFIC_RATIO = 0.946
+# DRAM traffic / algorithmic bytes of one SAP half sweep, from a 24^4 capture, whose links and clover exceed
+# L2 (profiles/sap_16x4.md: 165.0 MB for 331,776 sites x 444 B); the 32^4 launch is taken in proportion
+SAP_TRAFFIC_RATIO = 1.12
+# FP32 rate that the smoother's operations are held against: 152 SMs x 128 fused multiply-adds x 1.93 GHz
+FP32_TFLOPS = 75.1
 METRIC = "coarse-grid correction GB/s & % HBM roofline; batched-mixed vs plain speedup"
 WORKLOAD = "fp32_32^4_b4_ntv20: 32^4 Wilson-clover, 4^4 blocks -> 8^4 coarse, Ntv=20, 1 RHS, " \
            "FP64 setup, FP32 R and D_c; step = R y, FGMRES(30) to 0.05 (<=200 applies), P x_c"
@@ -687,12 +689,13 @@ def run_vcycle(args):
     followed by 4 SAP cycles (Alg. 3) of 4 MR steps per block; the fine Wilson-clover D on its own;
     and the outer FGMRES(30) preconditioned with the V-cycle to relative residual 1e-5 (Sec. 1).
 
-    Algorithmic bytes (FP32 complex = 8 B) per fine site: D reads 4 links (288 B), the clover
-    (two Hermitian 6x6 blocks as upper triangles, 336 B), psi (96 B) and writes out (96 B) = 816 B;
-    one SAP half sweep reads, per site of its colour, the links, the clover, y and x and writes x
-    (912 B), and reads x on the other colour's sites once (96 B): 504 B per fine site of the
-    lattice.  (The kernels read less of the clover, 27 numbers per chirality or 216 B; the model is kept
-    so that figures compare.)  A half sweep is timed as the V-cycle runs it, over its 4 cycles."""
+    Algorithmic bytes (FP32 complex = 8 B) per fine site: D reads 4 links (288 B), the clover (27 numbers
+    per chirality, 216 B), psi (96 B) and writes out (96 B) = 696 B; one SAP half sweep reads, per site
+    of its colour, the links, the clover, y and x and writes x (792 B), and reads x on the other
+    colour's sites once (96 B): 444 B per fine site of the lattice.  Earlier lines counted the clover as
+    two Hermitian upper triangles (816 and 504 B); `former_bytes` has the figures in that count.
+    Operations of a half sweep: 1 + n_mr applications of D or of its block part on half the sites, 8 per
+    complex multiply-add.  A half sweep is timed as the V-cycle runs it, over its 4 cycles."""
     import torch
     import paper_1512_04506_gb300 as amg
     from synth import device as sd
@@ -746,10 +749,15 @@ def run_vcycle(args):
     amg.amg_destroy(h)
     if status != amg.AMG_OK:
         raise RuntimeError(amg.amg_status_string(status))
+    # the former count of the clover, two Hermitian upper triangles
     d_bytes = V * 816
     half_bytes = V * 504
     cgc_bytes, _ = bytes_model(applies, arnoldi_iterations(applies))
+    former = {"dirac": d_bytes, "sap_half_sweep": half_bytes, "step": cgc_bytes + 2 * n_smoother * half_bytes}
+    # what is read: 27 numbers per chirality
+    d_bytes, half_bytes = V * 696, V * 444
     step_bytes = cgc_bytes + 2 * n_smoother * half_bytes
+    sap_flops = (1 + n_mr) * V // 2 * (8 * (2 * 66 + 36) + 2 * 36 * 8 + 24)
     peaks, src = measured_peaks()
     d_gbs = d_bytes / t_d / 1e9
     sap_gbs = half_bytes / t_sap / 1e9
@@ -761,17 +769,22 @@ def run_vcycle(args):
                                "(FGMRES(30) to 0.05) + %d SAP cycles of %d MR steps per 4^4 block; FP32" % (n_smoother, n_mr),
                    "bytes_per_step": step_bytes, "coarse_applies": applies, "n_smoother": n_smoother, "n_mr": n_mr,
                    "l2": "256 MB flush before each step"},
-        "roofline": {"bound": "hbm", "kernel": "sap32_kernel (one half sweep: residual + %d MR steps per block, "
-                     "links and clover in shared memory)" % n_mr, "achieved": round(sap_gbs, 1), "peak": peaks["hbm_gbs"],
-                     "unit": "GB/s", "frac": round(sap_gbs / peaks["hbm_gbs"], 4), "peak_source": src,
+        "roofline": {"bound": "fp32", "kernel": "sap32_kernel (one half sweep: residual + %d MR steps per block, "
+                     "links and clover in shared memory; the FP32 pipes and shared memory)" % n_mr,
+                     "achieved": round(sap_flops / t_sap / 1e12, 2), "peak": FP32_TFLOPS, "unit": "TFLOP/s",
+                     "frac": round(sap_flops / t_sap / 1e12 / FP32_TFLOPS, 4),
+                     "peak_source": "152 SMs x 128 FP32 fused multiply-adds x 1.93 GHz", "flops_per_launch": sap_flops,
+                     "hbm_gbs": round(sap_gbs, 1), "hbm_frac": round(sap_gbs / peaks["hbm_gbs"], 4), "hbm_peak": peaks["hbm_gbs"],
+                     "hbm_peak_source": src,
                      "traffic": round(SAP_TRAFFIC_RATIO * half_bytes) if SAP_TRAFFIC_RATIO and not args.lattice else None,
-                     "traffic_note": "16^4 capture's traffic / algorithmic bytes x this launch's bytes",
+                     "traffic_note": "24^4 capture's traffic / algorithmic bytes x this launch's bytes",
                      "bytes_per_launch": half_bytes, "avg_launch_us": round(t_sap * 1e6, 2),
                      "step_share": round(2 * n_smoother * t_sap / (t / args.steps), 3)},
         "kernels": {"dirac": {"us": round(t_d * 1e6, 1), "GB/s": round(d_gbs, 1),
                               "frac": round(d_gbs / peaks["hbm_gbs"], 4), "bytes_per_launch": d_bytes},
                     "sap_half_sweep": {"us": round(t_sap * 1e6, 1), "GB/s": round(sap_gbs, 1),
                                        "frac": round(sap_gbs / peaks["hbm_gbs"], 4)}},
+        "former_bytes": former,
         "outer_solve": {"tol": 1e-5, "applies_of_D": sinfo[0][0], "relres": sinfo[0][1],
                         "seconds": round(t_solve, 4), "restart": 30},
         "three_level": {"level2": "%dx%dx%dx%d coarse lattice in 2^4 blocks -> %dx%dx%dx%d, Ntv2 = %d random level-1 "
