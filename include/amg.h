@@ -66,8 +66,11 @@ typedef enum {
     AMG_BF16 = 3
 } amg_prec;
 
-/* Arithmetic of the Gram-Schmidt and of the D_c = R D P assembly in amg_setup_coarse (the
- * clover field stays FP64). */
+/* Arithmetic of the Gram-Schmidt and of the D_c = R D P assembly in amg_setup_coarse.  The clover
+ * field is formed to double accuracy in either: 60-bit fixed point relative to the links' largest
+ * entry, or, for links close to 1, FP64.  Fixed point is relative to the largest entry of a test
+ * vector on its aggregate (of a column of R and P on its block); where the entries differ too widely
+ * between sites the sums are taken in the floating-point arithmetic named. */
 typedef enum {
     AMG_SETUP_FP64 = 0,     /* sums of double accuracy: 64-bit fixed point on the tensor cores and
                                the integer pipes, or doubles on the FP64 pipe                */
@@ -97,15 +100,14 @@ typedef struct {
 typedef struct amg_coarse *amg_handle;
 
 /*
- * amg_setup_coarse -- Alg. 5 on the GPU, in FP64.
+ * amg_setup_coarse -- Alg. 5 on the GPU, to double accuracy (see amg_setup_arith).
  *   d_U  [V][4 mu][3][3] complex double: U_mu(x), the link from x to x+mu.
  *   d_tv [V][4][3][ntv] complex double: the test vectors v_j (Sec. 2.2).
  * Builds the clover field C from d_U, orthonormalises the test vectors on
  * every aggregate A_i^h by block classical Gram-Schmidt (Sec. 3, "Gram-Schmidt
  * on aggregates"), assembles the self block and the four forward blocks of
  * D_c = R D P (Eq. cgo, Alg. 7; all 2 ntv columns of P at once, as
- * Sec. 3 suggests, in FP64 or, with setup_arith = AMG_SETUP_F32PAIR, in pairs
- * of FP32 numbers) and fills the four backward blocks from
+ * Sec. 3 suggests, in the arithmetic setup_arith) and fills the four backward blocks from
  * Eq. dagger, then stores R and D_c in r_prec / link_prec (Sec. 3: D_c may be
  * kept in half precision).  The handle owns every buffer it allocates; the
  * inputs are read only and may be freed once the call returns.  This call
@@ -399,8 +401,8 @@ amg_status amg_batch_test_hook(amg_handle h0, int extra_need);
 /*
  * amg_solve_test_hook -- test hook for the bounded grid barriers of the coarse solve's fused Arnoldi
  * step: the next solves on h expect extra_arrivals more CTAs at each barrier than exist, so every
- * CTA's wait runs out after its limit (about one second), the step ends early and amg_sync_status reports AMG_ERR_TIMEOUT.  extra_arrivals = 0 restores normal
- * operation.  AMG_ERR_INVALID_ARG for a null handle or a negative count.
+ * CTA's wait runs out after its limit (about one second), the step ends early and amg_sync_status
+ * reports AMG_ERR_TIMEOUT.  extra_arrivals = 0 restores normal operation.  AMG_ERR_INVALID_ARG for a null handle or a negative count.
  */
 amg_status amg_solve_test_hook(amg_handle h, int extra_arrivals);
 

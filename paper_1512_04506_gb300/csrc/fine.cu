@@ -534,9 +534,9 @@ __global__ void __launch_bounds__(128, NC == 1 ? 4 : 3) dirac32_kernel(const flo
 // are read as they are needed, consecutive words by consecutive lanes.  The result goes out through
 // the spinor tile.
 //
-// Bounds: HBM (816 bytes per site), reached as far as two CTAs per SM cover each other's waits.
-// 32^3 x 64: 310 us, 81 % of the copy bandwidth.  One thread per site in lattice order with records of 288 and 352 bytes took
-// 509 us (3,150 line look-ups in L1 per warp of sites).
+// Bounds: HBM (696 bytes per site), reached as far as two CTAs per SM cover each other's waits.
+// 32^3 x 64: 305 us, 70 % of the copy bandwidth.  One thread per site in lattice order with records of 288
+// and 352 bytes took 509 us (3,150 line look-ups in L1 per warp of sites).
 constexpr int kDiracSites = 256;
 constexpr int kRec = 7;  // words per record in the tile: 16-byte accesses of 8 consecutive sites hit all banks
 template <bool SUB>

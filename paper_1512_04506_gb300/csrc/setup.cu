@@ -1,11 +1,12 @@
-// Setup of the restriction and the coarse-grid operator (Alg. 5), in FP64.
+// Setup of the restriction and the coarse-grid operator (Alg. 5): the FP64 kernels, the clover in fixed point, and
+// the driver, which chooses between these and the kernels of setup_gs.cu, setup_tc.cu and setup_ds.cu.
 //
 //   clover_kernel    C(x) = c_sw (i/4) sum sigma_{mu nu} F_{mu nu}(x), per chirality (Alg. 7's C^{hh})
 //   gs_kernel        block classical Gram-Schmidt per aggregate (Sec. 3, "Gram-Schmidt on aggregates"), where
 //                    those in fixed point (setup_gs.cu) and in pairs of floats (setup_ds.cu) do not serve
 //   assemble_kernel  self and forward blocks of D_c = R D P (Eq. cgo via Alg. 7's D P), as sums
-//                    over links of small rank-6 products: small blocks and few test vectors (the
-//                    others run on the tensor cores, setup_tc.cu)
+//                    over links of small rank-6 products: small blocks and few test vectors, and
+//                    what the kernel on the tensor cores (setup_tc.cu) leaves of the others
 //   combine_kernel   D_c blocks from the partial sums; backward blocks by Eq. dagger
 //   quantize_*       D_c and R to the storage precisions of the applies (Sec. 3: half precision D_c)
 #include "fixed.cuh"
@@ -486,8 +487,8 @@ __global__ void __launch_bounds__(256) gs_kernel(const double2* __restrict__ tv,
 // CTA has a multiple of four warps, and where the tiles fill fewer, groups of warps share out the
 // sites; the tile shape is the one that needs the fewest instructions so, links leaving through the face come last so that one set of
 // accumulators serves S_mu and F_mu, the self job works on the tiles that its quadrants need, and the
-// factors b_mu (+-1, +-i) only move words and flip signs in the integer pipe.  16^4, Ntv 20: 21.9 ms;
-// 2 x 4 tiles in two accumulator sets, all tiles of the self job and b_mu as products took 30.1 ms.
+// factors b_mu (+-1, +-i) only move words and flip signs in the integer pipe.  16^4 in 2^4 blocks, Ntv 8: 4.5 ms, Ntv 6:
+// 3.2 ms; 2 x 4 tiles in two accumulator sets, all tiles of the self job and b_mu as products took 8.6 and 8.3 ms.
 __device__ inline double flip(double v) {  // -v off the FP64 pipe
   return __hiloint2double(__double2hiint(v) ^ (int)0x80000000, __double2loint(v));
 }
@@ -801,8 +802,8 @@ static amg_status launch_assemble_tile(const Geom& g, const double2* R, const do
   return AMG_OK;
 }
 
-// The tile shape with the fewest FP64 instructions per row and sub-partition (2 Ntv = 40: 5 x 5, two groups
-// of two warps; 48: 3 x 6, four warps; 16: 2 x 4, four groups of one warp).
+// The tile shape with the fewest FP64 instructions per row and sub-partition (2 Ntv = 16: 2 x 4, four groups of one
+// warp; for blocks that the tensor cores leave also 40: 5 x 5, two groups of two warps, and 48: 3 x 6, four warps).
 static amg_status launch_assemble(const Geom& g, const double2* R, const double2* U, const double2* clov, double2* part,
                                   double m0, const int* only, cudaStream_t st) {
   constexpr int shapes[][2] = {{5, 5}, {6, 4}, {4, 4}, {3, 6}, {2, 4}, {3, 2}, {2, 2}};
