@@ -444,8 +444,8 @@ __device__ __forceinline__ const float4* link_below(const FineGeom& g, const flo
 
 // The same in FP32, several columns: lanes over (site in block order, group of NC columns), so that the
 // columns of a site are read together and its links and clover are broadcast.  With an even number of
-// columns a thread takes two (16-byte loads, half as many link and clover loads per column;
-// 16^3 x 32 and 12 columns: 162 us against 179 with one).  FAST: fewer than 2^31 threads.
+// columns a thread takes two (16-byte loads, half as many link and clover loads per column) where that
+// needs less time by waves (dirac32_columns).  FAST: fewer than 2^31 threads.
 template <int NC>
 __device__ __forceinline__ void load_cols(const float2* __restrict__ v, long long site, int nrhs, int r, float2 p[NC][12]) {
   if constexpr (NC == 1) {
@@ -459,8 +459,9 @@ __device__ __forceinline__ void load_cols(const float2* __restrict__ v, long lon
     }
   }
 }
+constexpr int dirac32_ctas(int nc) { return nc == 1 ? 4 : 3; }  // per SM
 template <bool SUB, bool FAST, int NC>
-__global__ void __launch_bounds__(128, NC == 1 ? 4 : 3) dirac32_kernel(const float4* __restrict__ U,
+__global__ void __launch_bounds__(128, dirac32_ctas(NC)) dirac32_kernel(const float4* __restrict__ U,
                                                                        const float4* __restrict__ Cl,
                                                                        const float2* __restrict__ psi,
                                                                        const float2* __restrict__ y,
@@ -1575,6 +1576,19 @@ __global__ void clover_words_kernel(const double2* __restrict__ in, float4* __re
 
 bool fine_fp64(const amg_coarse* h) { return h->p.vec_prec == AMG_FP64; }
 
+// Columns per thread: two if their waves, 1.35 times as long (a thread's loads and sums in series), take less time than
+// those of one.  us with one and two: 8^4 and 2 columns 8.6 and 10.8 (one wave each), 12^4 and 6 18.8 and 21.5 (two
+// each), 8^3 x 16 and 12 15.1 and 12.9 (two and one), 16^3 x 32 and 2 55.6 and 58.4 (four and three), 12 columns 174
+// and 160.
+int dirac32_columns(long long V, int nrhs) {
+  if (nrhs % 2) return 1;
+  auto waves = [&](int nc) {
+    const long long per = 128LL * dirac32_ctas(nc) * amg_sm_count();
+    return (V * (nrhs / nc) + per - 1) / per;
+  };
+  return 1.35 * waves(2) < waves(1) ? 2 : 1;
+}
+
 template <int NC>
 auto* pick_dirac32(bool sub, bool fast) {
   return sub ? (fast ? dirac32_kernel<true, true, NC> : dirac32_kernel<true, false, NC>)
@@ -1607,7 +1621,7 @@ amg_status dirac_any(amg_coarse* h, const void* psi, const void* y, void* out, i
       auto* k = y ? dirac32_block_kernel<true> : dirac32_block_kernel<false>;
       k<<<ctas, threads, 0, st>>>(U, C, p, yy, (float2*)out, g, mass, nb, nblocks);
     } else {
-      const int nc = nrhs % 2 ? 1 : 2, groups = nrhs / nc;
+      const int nc = dirac32_columns(g.V, nrhs), groups = nrhs / nc;
       const FastDiv dn = fast_div(groups);
       const long long threads = h->g.V * groups;
       auto* k = nc == 1 ? pick_dirac32<1>(y != nullptr, threads < (1LL << 31)) : pick_dirac32<2>(y != nullptr, threads < (1LL << 31));

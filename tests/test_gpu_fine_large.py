@@ -113,3 +113,22 @@ def test_one_cycle_with_and_without_copies():
             assert torch.equal(part, x[..., :n])
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("L,B,nrhs", [((8, 8, 8, 8), (4, 4, 4, 4), 2), ((8, 8, 8, 16), (4, 4, 4, 2), 12),
+                                      ((12, 12, 12, 12), (3, 3, 3, 3), 6), ((16, 16, 16, 8), (2, 4, 4, 4), 16)],
+                         ids=["one-2", "two-12", "one-6", "two-16"])
+def test_dirac_even_columns(L, B, nrhs):
+    """One or two columns per thread, by the waves they take."""
+    import paper_1512_04506_gb300 as amg
+    c = Fine(amg, L, B, 1, 863, "fp32", max_nrhs=nrhs)
+    try:
+        psi = c.vec(nrhs, 1)
+        out = torch.empty_like(c.dev(psi))
+        amg.amg_dirac_apply(c.h, c.dev(psi), out, nrhs, c.stream)
+        got = out.cpu().numpy()
+        for r in range(nrhs):
+            ref = dirac.apply_dirac(c.U, c.C, c.m0, c.field(psi[..., r].astype(np.complex128))).reshape(c.V, 4, 3)
+            assert H.rel(got[..., r], ref) < 1e-5
+    finally:
+        c.close()
