@@ -1253,14 +1253,16 @@ amg_status launch_restrict_rows(amg_coarse* h, const float2* R, const float2* y,
 // contiguous bytes per row; x_c of the block sits in shared memory.  One column reads the rows with the
 // streaming hint (read once) and writes x with one 16-byte streaming store per pair: 93 % of the copy
 // bandwidth against 90 % for the bulk-copy ring form (prolong_tma_kernel, kept for FP64), whose
-// single-dof lanes stored 8 bytes each.  24^3 x 48, Ntv 20, 8 columns: 368 us against 2 x 311 us for
+// single-dof lanes stored 8 bytes each.  24^3 x 48, Ntv 20, 8 columns: 371 us against 2 x 311 us for
 // one launch per 4 columns; chunks of 8 with the results leaving through shared memory took 379 us.
-template <int NR>
+// ONE: a single chunk of 1, 3 or 4 columns, where the rows are read once too: with the hint (16^4 in 2^4 blocks,
+// Ntv 16, 4 columns: 33.0 us, 37.7 without; 2 columns are slower so: 16^3 x 32, Ntv 24, 71 us and 66).
+template <int NR, bool ONE>
 __global__ void __launch_bounds__(256) prolong_pair_kernel(const float2* __restrict__ R, const float2* __restrict__ xc,
                                                            float2* __restrict__ x, Geom g, int ld, int chunks) {
   __shared__ float2 xs[2 * AMG_MAX_NTV * NR];
-  const long long blk = NR == 1 ? blockIdx.x : blockIdx.x / chunks;
-  const int r0 = NR == 1 ? 0 : (int)(blockIdx.x % chunks) * NR;
+  const long long blk = ONE ? blockIdx.x : blockIdx.x / chunks;
+  const int r0 = ONE ? 0 : (int)(blockIdx.x % chunks) * NR;
   const int nagg = g.nagg, ntv = g.ntv, npair = nagg / 2;
   for (int e = threadIdx.x; e < 2 * ntv * NR; e += blockDim.x)
     xs[e] = xc[(blk * 2 * ntv + e / NR) * ld + min(r0 + e % NR, ld - 1)];
@@ -1276,7 +1278,7 @@ __global__ void __launch_bounds__(256) prolong_pair_kernel(const float2* __restr
 #pragma unroll 5
     for (int j = 0; j < ntv; ++j) {
       const float4* row = reinterpret_cast<const float4*>(Rp + (size_t)j * nagg);
-      const float4 v = NR == 1 ? __ldcs(row) : __ldcg(row);
+      const float4 v = ONE ? __ldcs(row) : __ldcg(row);
       const float2 v0 = make_float2(v.x, v.y), v1 = make_float2(v.z, v.w);
 #pragma unroll
       for (int r = 0; r < NR; ++r) {
@@ -1318,7 +1320,8 @@ int prolong_chunk(const Geom& g) {
 template <int NR>
 amg_status launch_prolong_pair(amg_coarse* h, const float2* R, const float2* xc, float2* x, int ld, int chunks,
                                cudaStream_t st) {
-  prolong_pair_kernel<NR><<<(unsigned)(h->g.Vc * chunks), 256, 0, st>>>(R, xc, x, h->g, ld, chunks);
+  auto* k = chunks == 1 && NR != 2 ? prolong_pair_kernel<NR, NR != 2> : prolong_pair_kernel<NR, NR == 1>;
+  k<<<(unsigned)(h->g.Vc * chunks), 256, 0, st>>>(R, xc, x, h->g, ld, chunks);
   AMG_LAUNCH_CHECK();
   h->launches++;
   return AMG_OK;
