@@ -1679,11 +1679,18 @@ amg_status sweep32(amg_coarse* h, const float2* y, float2* x, int nrhs, int n_cy
 // The sweeps run on copies of x and y in block order, one vector per column; x is copied back.  The
 // copies come from the handle's pool, at most kColBytes at a time but one column at least (columns are
 // independent).  While the stream is captured, or without memory for them, the sweeps work on the
-// caller's vectors; so they do for one cycle of up to three columns, where the copies cost more than
-// they save (us with and without, 4 MR steps: 16^4 and one column 59 and 47, 32^4 672 and 595, 24 16^3
-// and two columns 161 and 157, 16^3 x 32 and three 263 and 264, four 340 and 382).
+// caller's vectors; so they do where the copies cost more than they save (sap_copies).
 constexpr size_t kColBytes = (size_t)2 << 30;
 constexpr size_t kPoolStep = (size_t)64 << 20;  // more than what a pool adds to an allocation (32 MB pieces)
+// us with and without copies (4 MR steps).  One column gains little from the block order: 32^4 1220 and 1202 for two
+// cycles, 2297 and 2382 for four; in blocks of up to 16 sites 8^4 151 and 145, 16^4 191 and 188, 24^4 893 and 972 for four.
+// One cycle of two columns: 16^4 102 and 98, 32^4 1239 and 1271; of more: 12^4 and three 94 and 90, 8^3 x 16 and eight
+// 65 and 61, but 12^4 and eight 160 and 176, 16^4 and four 177 and 198.  Two cycles of two columns 16^4 171 and 189.
+bool sap_copies(const FineGeom& g, int nrhs, int n_cycles) {
+  constexpr long long kSmall = 1 << 16;  // elements (sites times columns) that one cycle does not copy
+  if (nrhs == 1) return n_cycles > 2 && (sap_lanes(g) == 0 || g.V > kSmall);
+  return n_cycles > 1 || (nrhs > 2 && g.V * nrhs > kSmall);
+}
 int sap_copy_columns(const amg_coarse* h, int nrhs) {
   return (int)std::max<size_t>(1, std::min<size_t>(nrhs, kColBytes / (2 * h->g.V * 12 * sizeof(float2))));
 }
@@ -1733,7 +1740,7 @@ amg_status launch_sap32(amg_coarse* h, const void* yv, void* xv, int nrhs, int n
   float2* x = (float2*)xv;
   const size_t n = (size_t)h->g.V * 12;
   if (n_cycles < 1) return AMG_OK;
-  if (n_cycles == 1 && nrhs <= 3) return sweep32<false>(h, y, x, nrhs, n_cycles, n_mr, st);
+  if (!sap_copies(fine_geom(h), nrhs, n_cycles)) return sweep32<false>(h, y, x, nrhs, n_cycles, n_mr, st);
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   AMG_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
   const int chunk = sap_copy_columns(h, nrhs);

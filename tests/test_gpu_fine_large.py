@@ -99,18 +99,21 @@ def test_sap_two_sets_of_copies():
         amg.amg_destroy(h)
 
 
-def test_one_cycle_with_and_without_copies():
-    """One cycle of up to three columns works on the caller's vectors, of four on copies: the same bits."""
+@pytest.mark.parametrize("L,B,cycles", [((12, 16, 16, 16), (3, 4, 4, 2), 1), ((12, 16, 16, 16), (3, 4, 4, 2), 2),
+                                        ((8, 8, 8, 8), (2, 2, 2, 2), 3), ((8, 8, 8, 8), (4, 4, 4, 4), 1)])
+def test_with_and_without_copies(L, B, cycles):
+    """Few columns or cycles work on the caller's vectors, more on copies: the same bits."""
     import paper_1512_04506_gb300 as amg
-    c = Fine(amg, (12, 8, 8, 16), (3, 4, 4, 2), 1, 861, "fp32", max_nrhs=4)
+    c = Fine(amg, L, B, 1, 861, "fp32", max_nrhs=17)
     try:
-        y, x0 = c.dev(c.vec(4, 1)), c.dev(c.vec(4, 2))
+        n = 4 if c.V > 20000 else 17
+        y, x0 = c.dev(c.vec(n, 1)), c.dev(c.vec(n, 2))
         x = x0.clone()
-        amg.amg_sap(c.h, y, x, 4, 1, 3, c.stream)
-        for n in (1, 2, 3):
-            part = x0[..., :n].contiguous()
-            amg.amg_sap(c.h, y[..., :n].contiguous(), part, n, 1, 3, c.stream)
-            assert torch.equal(part, x[..., :n])
+        amg.amg_sap(c.h, y, x, n, cycles, 3, c.stream)
+        for k in (1, 2, 3):
+            part = x0[..., :k].contiguous()
+            amg.amg_sap(c.h, y[..., :k].contiguous(), part, k, cycles, 3, c.stream)
+            assert torch.equal(part, x[..., :k])
     finally:
         c.close()
 
