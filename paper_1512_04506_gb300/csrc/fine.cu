@@ -1658,12 +1658,17 @@ int sap_columns(long long nblk, int nrhs, int slots) {
 template <bool BLOCKED>
 amg_status sweep32(amg_coarse* h, const float2* y, float2* x, int nrhs, int n_cycles, int n_mr, cudaStream_t st) {
   const FineGeom g = fine_geom(h);
-  const int lanes = sap_lanes(g), subs = lanes ? 32 / lanes : 1, threads = lanes ? 32 : (g.Vb + 31) / 32 * 32;
+  const int nblk = (int)(h->g.Vc / 2);
+  // Small blocks share a warp unless the launch's warps find an SM sub-partition each anyway: then a block's
+  // faces are spread over more lanes (8^4 in 2^4 blocks, one column, 4 cycles: 141 us, 150 with two blocks to a warp).
+  int lanes = sap_lanes(g);
+  while (lanes && lanes < 32 && (long long)nblk * (2 * lanes) / 32 * nrhs <= 4LL * amg_sm_count()) lanes *= 2;
+  const int subs = lanes ? 32 / lanes : 1, threads = lanes ? 32 : (g.Vb + 31) / 32 * 32;
   const size_t smem = sap_smem(g, subs);
   if (threads > 256 || smem > 227 * 1024) return AMG_ERR_UNSUPPORTED;
   auto* k = lanes ? sap32_kernel<BLOCKED, true> : sap32_kernel<BLOCKED, false>;
   AMG_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const int nblk = (int)(h->g.Vc / 2), units = (nblk + subs - 1) / subs;
+  const int units = (nblk + subs - 1) / subs;
   const int nr = sap_columns(units, nrhs, sap_slots(threads, smem)), groups = (nrhs + nr - 1) / nr;
   const float mass = (float)(4.0 + h->p.m0);
   for (int c = 0; c < n_cycles; ++c)
