@@ -1726,6 +1726,7 @@ amg_status blocked_copy(amg_coarse* h, const float2* v, const float2* w, int nrh
 // The pool, with the copies of max_nrhs columns allocated once here rather than in the first sweep; the pool
 // keeps them until the handle goes.  Without it (a device without pools) the sweeps do without copies.
 void sap_pool(amg_coarse* h, cudaStream_t st) {
+  if (h->fpool) return;  // links set again: the lattice, and so the copies' size, are the same
   cudaMemPoolProps props = {};
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
@@ -2107,9 +2108,8 @@ amg_status adaptive_impl(amg_coarse* h, const amg_vcycle_params* vp, const doubl
   return s;
 }
 
-}  // namespace
-
-void amg_internal_free_fine(amg_coarse* h) {
+// All but the pool
+void free_fields(amg_coarse* h) {
   cudaFree(h->fU);
   if (h->fC != (void*)h->clover) cudaFree(h->fC);
   cudaFree(h->fwork);
@@ -2117,10 +2117,16 @@ void amg_internal_free_fine(amg_coarse* h) {
   cudaFree(h->fE);
   h->fW = nullptr;
   h->fE = nullptr;
-  if (h->fpool) cudaMemPoolDestroy(h->fpool);
-  h->fpool = nullptr;
   h->fU = h->fC = h->fwork = nullptr;
   h->fwork_bytes = 0;
+}
+
+}  // namespace
+
+void amg_internal_free_fine(amg_coarse* h) {
+  free_fields(h);
+  if (h->fpool) cudaMemPoolDestroy(h->fpool);
+  h->fpool = nullptr;
 }
 
 extern "C" {
@@ -2131,7 +2137,7 @@ amg_status amg_setup_fine(amg_handle h, const void* d_U, void* stream) {
   if (h->p.vec_prec != AMG_FP64 && h->p.vec_prec != AMG_FP32) return AMG_ERR_UNSUPPORTED;
   cudaStream_t st = (cudaStream_t)stream;
   h->last_stream = st;
-  amg_internal_free_fine(h);
+  free_fields(h);
   const long long nU = h->g.V * 36;
   if (fine_fp64(h)) {
     AMG_CUDA_TRY(cudaMalloc(&h->fU, nU * sizeof(double2)));

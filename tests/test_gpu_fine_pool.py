@@ -36,3 +36,27 @@ def test_nothing_given_back(L, nrhs):
         assert free[-1][0] == free[-1][1]
     finally:
         amg.amg_destroy(h)
+
+
+def test_links_set_again():
+    """amg_setup_fine with other links on the same handle: no more memory held, and results of a new handle."""
+    import paper_1512_04506_gb300 as amg
+    from synth import device as sd
+    L, nrhs, st = (16, 16, 16, 16), 5, torch.cuda.current_stream()
+    Us, tv, y = [sd.links(s, 0.3, L) for s in (81, 82)], sd.test_vectors(81, 2, L), sd.fine_rhs(81, nrhs, L)
+    p = amg.make_params(L, (4, 4, 4, 4), 2, nrhs, -0.3, 1.0, amg.AMG_FP32, amg.AMG_FP32, amg.AMG_FP32)
+    out, held = [], []
+    for first in (0, 1):
+        h, _ = amg.amg_setup_coarse(p, Us[1], tv, st)
+        try:
+            for k in range(first, 2):
+                amg.amg_setup_fine(h, Us[k], st)
+                x = torch.zeros_like(y)
+                amg.amg_sap(h, y, x, nrhs, 2, 3, st)
+                torch.cuda.synchronize()
+                held.append(torch.cuda.mem_get_info()[0])
+            out.append(x)
+        finally:
+            amg.amg_destroy(h)
+    assert torch.equal(out[0], out[1])
+    assert abs(held[0] - held[1]) < 16 << 20
