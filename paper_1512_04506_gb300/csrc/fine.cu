@@ -897,8 +897,8 @@ __device__ __forceinline__ void site_fixed(const int4* __restrict__ W, const int
 // clover as words prepared once, sums of 64 bits; the sums over the block and the updates stay in FP64.  An
 // application is then good to 2^-57 of the block's largest entry.  A step takes FP64, where every site's sums are good
 // relative to its own terms, if an entry is not finite or a site's largest one (unless 0) lies more than kFixBits
-// bits below the block's.  12 x 8 x 24 x 16, blocks 3 x 4 x 4 x 2, 3 columns: 447 us a half sweep, in FP64 703 us; 16^4 in
-// 2^4 blocks 497 and 944 us.
+// bits below the block's.  12 x 8 x 24 x 16, blocks 3 x 4 x 4 x 2, 3 columns: 451 us a half sweep, in FP64 703 us; 16^4 in
+// 2^4 blocks 468 and 944 us.
 template <bool FIXED>
 __global__ void __launch_bounds__(256) sap_kernel(const double2* __restrict__ U, const double2* __restrict__ Cl,
                                                   const int4* __restrict__ words, const int* __restrict__ exps,
